@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <string>
 
@@ -405,6 +406,59 @@ int check_render_opts(const fpo_ctx *ctx, const fpo_frame_opts *opts, uint64_t n
     return FPO_OK;
 }
 
+// cos(pi x) and sin(pi x), exact at multiples of 1/2: x is reduced exactly to
+// [-1, 1] and then to a quarter period.
+static double cospi_h(double x, bool sine)
+{
+    x = std::remainder(x, 2.0);
+    const double q = std::nearbyint(2.0 * x);
+    const double a = (x - 0.5 * q) * 3.14159265358979323846;
+    switch (((int)q + (sine ? 3 : 0)) & 3) {  // sin(y) = cos(y - pi / 2)
+    case 0: return std::cos(a);
+    case 1: return -std::sin(a);
+    case 2: return -std::cos(a);
+    default: return std::sin(a);
+    }
+}
+
+void time_basis(double t, double period_T, int n, float b[32])
+{
+    const double u = t / period_T;
+    for (int i = 0; i < 32; ++i) {
+        if (i >= n) b[i] = 0.0f;
+        else if (!std::isfinite(u)) b[i] = std::numeric_limits<float>::quiet_NaN();
+        else b[i] = (float)((i & 1) ? cospi_h((double)(i + 1) * u, true) : cospi_h((double)i * u, false));
+    }
+}
+
+// The frame's constants: the time basis and, for camera rays, the camera frame.
+static void frame_consts(const FrameParams &fr, int nb, FrameConsts &c)
+{
+    time_basis(fr.t, fr.period_T, nb, c.b);
+    if (fr.mode != FPO_RAYS_CAMERA) return;
+    double f[3], r[3], u[3];
+    for (int k = 0; k < 3; ++k) f[k] = fr.target[k] - fr.eye[k];
+    const double fl = std::sqrt(f[0] * f[0] + f[1] * f[1] + f[2] * f[2]);
+    for (int k = 0; k < 3; ++k) f[k] /= fl;
+    r[0] = f[1] * fr.up[2] - f[2] * fr.up[1];
+    r[1] = f[2] * fr.up[0] - f[0] * fr.up[2];
+    r[2] = f[0] * fr.up[1] - f[1] * fr.up[0];
+    const double rl = std::sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+    for (int k = 0; k < 3; ++k) r[k] /= rl;
+    u[0] = r[1] * f[2] - r[2] * f[1];
+    u[1] = r[2] * f[0] - r[0] * f[2];
+    u[2] = r[0] * f[1] - r[1] * f[0];
+    const double th = std::tan(0.5 * fr.fov_y_deg * 3.14159265358979323846 / 180.0);
+    for (int k = 0; k < 3; ++k) {
+        c.f[k] = (float)f[k];
+        c.r[k] = (float)r[k];
+        c.u[k] = (float)u[k];
+        c.eye[k] = (float)fr.eye[k];
+    }
+    c.sx_scale = (float)(th * (double)fr.width / (double)fr.height);
+    c.sy_scale = (float)th;
+}
+
 // Kernel parameters of one render (or adjoint) call from the context, rays
 // and options.
 TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
@@ -427,6 +481,7 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
     p.fr.ro = rays->o;
     p.fr.rd = rays->d;
     p.fr.rt = rays->t_per_ray;
+    frame_consts(p.fr, ctx->cfg.n1 > ctx->cfg.n2 ? ctx->cfg.n1 : ctx->cfg.n2, p.fc);
     p.nodes = ctx->d_nodes;
     p.root_kind = ctx->root_kind;
     p.depth = ctx->depth;
@@ -493,8 +548,7 @@ int launch_table_pass(const fpo_ctx *ctx, double t, float *table, int max_ctas_p
         lp.b3 = ctx->d_dec_b + 128;
         lp.n1 = ctx->cfg.n1;
         lp.n2 = ctx->cfg.n2;
-        lp.t = t;
-        lp.period_T = ctx->cfg.period_T;
+        time_basis(t, ctx->cfg.period_T, ctx->cfg.n1 > ctx->cfg.n2 ? ctx->cfg.n1 : ctx->cfg.n2, lp.b);
         lp.n_leaves = ctx->n_leaves;
         lp.table = table;
         lp.half_table = ctx->half_table;
@@ -521,8 +575,7 @@ int launch_table_pass(const fpo_ctx *ctx, double t, float *table, int max_ctas_p
     mp.max_ctas_per_sm = max_ctas_per_sm;
     mp.carveout = carveout;
     mp.half_table = ctx->half_table;
-    mp.t = t;
-    mp.period_T = ctx->cfg.period_T;
+    time_basis(t, ctx->cfg.period_T, ctx->cfg.n1 > ctx->cfg.n2 ? ctx->cfg.n1 : ctx->cfg.n2, mp.b);
     mp.status = ctx->d_status;
     mp.test_timeout = test_timeout;
     return launch_materialise(mp, ctx->sm_count, s);

@@ -102,8 +102,21 @@ struct FrameParams {
     const float *ro, *rd, *rt; // explicit rays (device)
 };
 
+// What every CTA of a frame's kernels would otherwise derive in FP64 for
+// itself: Eq. 8 at the frame time and the camera frame, computed once per call
+// on the host in FP64 and rounded to FP32 (the GPU's FP64 rate made the
+// kernels' own prologue some microseconds long).
+struct FrameConsts {
+    float b[32];                     // IDFT_i(t), i < max(n1, n2); 0 beyond
+    float f[3], r[3], u[3], eye[3];  // camera: forward, right, up, eye
+    float sx_scale, sy_scale;        // tan(fov / 2) times the aspect ratio, and plain
+};
+// Eq. 8 at time t for i < n into b (32 values, zero from n on).
+void time_basis(double t, double period_T, int n, float b[32]);
+
 struct TraverseParams {
     FrameParams fr;
+    FrameConsts fc;
     // tree
     const uint32_t *nodes;
     uint32_t root_kind;
@@ -155,7 +168,7 @@ struct MaterialiseParams {
     int pipeline;             // 1: the frame-pipeline shape (materialise_pipeline_shape)
     int max_ctas_per_sm;      // 0: as many as fit
     int carveout;             // preferred shared-memory carveout in percent (0: the driver's default)
-    double t, period_T;
+    float b[32];              // Eq. 8 at the frame time (time_basis)
     uint32_t *status;
     int test_timeout;         // 1: the first wait of each CTA gives up (failure-path test)
 };
@@ -210,7 +223,7 @@ struct LatentParams {
     const uint16_t *w3;       // [n1 + 27 n2][64]
     const float *b3;          // [n1 + 27 n2]
     int n1, n2;
-    double t, period_T;
+    float b[32];              // Eq. 8 at the frame time (time_basis)
     uint32_t n_leaves;
     float *table;             // [n_leaves][TABLE_STRIDE] FP32, or FP16 when half_table
     int half_table;

@@ -58,7 +58,7 @@ namespace fpo {
 namespace {
 
 constexpr int STACK_LEVELS = MAX_DEPTH + 1;
-constexpr int MAX_BASIS = 64;
+constexpr int MAX_BASIS = 32;  // n1 <= 32, n2 <= 16
 
 // Real SH of degree <= 2 at a unit direction, index k = l(l+1)+m
 // (orthonormal; sign convention of the complex SH with Condon-Shortley phase).
@@ -78,13 +78,6 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, float Y[9])
     Y[6] = c3 * (3.0f * z * z - 1.0f);
     Y[7] = -c2 * x * z;
     Y[8] = c4 * (x * x - y * y);
-}
-
-// Eq. 8 at one time, computed in FP64 (cospi/sinpi of i t / T) and rounded.
-__device__ __forceinline__ float basis_fp64(int i, double t, double period)
-{
-    const double u = t / period;
-    return (i & 1) ? (float)sinpi((double)(i + 1) * u) : (float)cospi((double)i * u);
 }
 
 // Eq. 8 from an FP32 time (explicit rays with per-ray times).
@@ -183,7 +176,7 @@ __global__ void __launch_bounds__(MAT_THREADS, 8) materialise_kernel(const __gri
     const uint32_t stage_bytes = sig_bytes + z_bytes + (SCALED ? MAT_CHUNK * 4u : 0u);
     const uint32_t n_chunks = (p.n_leaves + MAT_CHUNK - 1) / MAT_CHUNK;
     const int nb = p.n1 > p.n2 ? p.n1 : p.n2;
-    if (tid < nb) s_b[tid] = basis_fp64(tid, p.t, p.period_T);
+    if (tid < MAX_BASIS) s_b[tid] = tid < nb ? p.b[tid] : 0.0f;
     if (tid == 0) {
         s_fail = 0;
         for (int s = 0; s < S; ++s) ptx::mbar_init(&bars[s], 1);
@@ -444,7 +437,7 @@ __global__ void __launch_bounds__(CH, ST == FPO_STORAGE_F32 ? 4 : 1) materialise
     const uint32_t stage_bytes = sig_bytes + z_bytes + (SCALED ? CH * 4u : 0u);
     const uint32_t n_chunks = (p.n_leaves + CH - 1) / CH;
     const int nb = p.n1 > ML_N2 ? p.n1 : ML_N2;
-    if (tid < MAX_BASIS) s_b[tid] = tid < nb ? basis_fp64(tid, p.t, p.period_T) : 0.0f;
+    if (tid < MAX_BASIS) s_b[tid] = tid < nb ? p.b[tid] : 0.0f;
     if (tid == 0) {
         s_fail = 0;
         for (int s = 0; s < S; ++s) ptx::mbar_init(&bars[s], 1);
@@ -718,9 +711,7 @@ int launch_materialise(const MaterialiseParams &p, int sm_count, void *stream)
 namespace {
 
 struct FrameShared {
-    float b[MAX_BASIS];
-    float f[3], r[3], u[3], eye[3];
-    float sx_scale, sy_scale;
+    float b[MAX_BASIS];  // Eq. 8 at the shared frame time
 };
 
 // Per-lane state of one ray, kept in registers across the warp's step loop.
@@ -752,19 +743,19 @@ __device__ __forceinline__ void write_result(const TraverseParams &p, const RayS
 // Sets up ray `ray` (camera pixel (px, py) or explicit ray): generation,
 // SH basis, clip against the grid cube.  Returns false when the ray misses
 // the tree (its background result is written at once).
-__device__ bool init_ray_geom(const TraverseParams &p, const FrameShared &fs, bool prt, float *s_bray,
+__device__ bool init_ray_geom(const TraverseParams &p, bool prt, float *s_bray,
                               int stride, uint32_t *s_stack, RayState &R, uint32_t ray, int px, int py)
 {
     float ox, oy, oz, dx, dy, dz;
     if (p.fr.mode == FPO_RAYS_CAMERA) {
-        const float sx = (2.0f * ((float)px + 0.5f) / (float)p.fr.width - 1.0f) * fs.sx_scale;
-        const float sy = (1.0f - 2.0f * ((float)py + 0.5f) / (float)p.fr.height) * fs.sy_scale;
-        dx = fs.f[0] + sx * fs.r[0] + sy * fs.u[0];
-        dy = fs.f[1] + sx * fs.r[1] + sy * fs.u[1];
-        dz = fs.f[2] + sx * fs.r[2] + sy * fs.u[2];
-        ox = fs.eye[0];
-        oy = fs.eye[1];
-        oz = fs.eye[2];
+        const float sx = (2.0f * ((float)px + 0.5f) / (float)p.fr.width - 1.0f) * p.fc.sx_scale;
+        const float sy = (1.0f - 2.0f * ((float)py + 0.5f) / (float)p.fr.height) * p.fc.sy_scale;
+        dx = p.fc.f[0] + sx * p.fc.r[0] + sy * p.fc.u[0];
+        dy = p.fc.f[1] + sx * p.fc.r[1] + sy * p.fc.u[1];
+        dz = p.fc.f[2] + sx * p.fc.r[2] + sy * p.fc.u[2];
+        ox = p.fc.eye[0];
+        oy = p.fc.eye[1];
+        oz = p.fc.eye[2];
     } else {
         ox = p.fr.ro[3 * (size_t)ray];
         oy = p.fr.ro[3 * (size_t)ray + 1];
@@ -831,11 +822,11 @@ __device__ bool init_ray_geom(const TraverseParams &p, const FrameShared &fs, bo
 
 // As init_ray_geom; a ray that misses the tree gets its background result.
 template <bool DBG>
-__device__ __forceinline__ bool init_ray(const TraverseParams &p, const FrameShared &fs, bool prt,
+__device__ __forceinline__ bool init_ray(const TraverseParams &p, bool prt,
                                          float *s_bray, int stride, uint32_t *s_stack, RayState &R,
                                          uint32_t ray, int px, int py)
 {
-    if (init_ray_geom(p, fs, prt, s_bray, stride, s_stack, R, ray, px, py)) return true;
+    if (init_ray_geom(p, prt, s_bray, stride, s_stack, R, ray, px, py)) return true;
     write_result(p, R, DBG);
     return false;
 }
@@ -1194,39 +1185,14 @@ __device__ void trace_ray(const TraverseParams &p, const float *bsrc, int bstrid
 
 namespace {
 
-// CTA prologue: stage the top n_smem_nodes nodes in shared memory; the frame
-// basis (Eq. 8 at the shared t, FP64 then FP32) and the camera frame (FP64).
+// CTA prologue: stage the top n_smem_nodes nodes in shared memory, and the
+// frame basis (Eq. 8 at the shared t).
 __device__ void frame_prologue(const TraverseParams &p, uint32_t *s_nodes, FrameShared &fs)
 {
     const uint4 *src = reinterpret_cast<const uint4 *>(p.nodes);
     uint4 *dst = reinterpret_cast<uint4 *>(s_nodes);
     for (uint32_t i = threadIdx.x; i < p.n_smem_nodes * 2; i += blockDim.x) dst[i] = __ldg(src + i);
-    const int nb = p.n1 > p.n2 ? p.n1 : p.n2;
-    if (threadIdx.x < MAX_BASIS)
-        fs.b[threadIdx.x] = (int)threadIdx.x < nb ? basis_fp64(threadIdx.x, p.fr.t, p.fr.period_T) : 0.0f;
-    if (threadIdx.x == MAX_BASIS && p.fr.mode == FPO_RAYS_CAMERA) {
-        double f[3], r[3], u[3];
-        for (int k = 0; k < 3; ++k) f[k] = p.fr.target[k] - p.fr.eye[k];
-        double fl = sqrt(f[0] * f[0] + f[1] * f[1] + f[2] * f[2]);
-        for (int k = 0; k < 3; ++k) f[k] /= fl;
-        r[0] = f[1] * p.fr.up[2] - f[2] * p.fr.up[1];
-        r[1] = f[2] * p.fr.up[0] - f[0] * p.fr.up[2];
-        r[2] = f[0] * p.fr.up[1] - f[1] * p.fr.up[0];
-        double rl = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-        for (int k = 0; k < 3; ++k) r[k] /= rl;
-        u[0] = r[1] * f[2] - r[2] * f[1];
-        u[1] = r[2] * f[0] - r[0] * f[2];
-        u[2] = r[0] * f[1] - r[1] * f[0];
-        const double th = tan(0.5 * p.fr.fov_y_deg * 3.14159265358979323846 / 180.0);
-        for (int k = 0; k < 3; ++k) {
-            fs.f[k] = (float)f[k];
-            fs.r[k] = (float)r[k];
-            fs.u[k] = (float)u[k];
-            fs.eye[k] = (float)p.fr.eye[k];
-        }
-        fs.sx_scale = (float)(th * (double)p.fr.width / (double)p.fr.height);
-        fs.sy_scale = (float)th;
-    }
+    if (threadIdx.x < MAX_BASIS) fs.b[threadIdx.x] = p.fc.b[threadIdx.x];
 }
 
 // Ray k (0..31) of a tile: a camera pixel of a TILE_W x TILE_H block, or an
@@ -1310,7 +1276,7 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
             int px = 0, py = 0;
             if (tile_ray(p, tile, (uint32_t)lane, ray, px, py)) {
                 RayState R;
-                if (init_ray<DBG>(p, fs, prt, my_b, stride, my_stack, R, ray, px, py)) {
+                if (init_ray<DBG>(p, prt, my_b, stride, my_stack, R, ray, px, py)) {
                     trace_ray<TM, DBG, N1, N2>(p, bsrc, bstride, s_nodes, my_stack, stride, R);
                     finish(R);
                 }
@@ -1340,7 +1306,7 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
                         uint32_t ray;
                         int px = 0, py = 0;
                         if (tile_ray(p, cur_tile, cur_next + rank, ray, px, py)) {
-                            active = init_ray<DBG>(p, fs, prt, my_b, stride, my_stack, R, ray, px, py);
+                            active = init_ray<DBG>(p, prt, my_b, stride, my_stack, R, ray, px, py);
                             if (active) cb = locate(p, s_nodes, my_stack, stride, R.P, R.lvl_start);
                         }
                     }
@@ -1606,7 +1572,7 @@ __global__ void __maxnreg__(128) backward_kernel(const __grid_constant__ Backwar
         int px = 0, py = 0;
         if (!tile_ray(p, tile, (uint32_t)lane, ray, px, py)) continue;
         RayState R;
-        if (!init_ray_geom(p, fs, prt, my_b, stride, my_stack, R, ray, px, py)) continue;
+        if (!init_ray_geom(p, prt, my_b, stride, my_stack, R, ray, px, py)) continue;
         backward_ray<N1, N2>(q, bsrc, bstride, s_nodes, my_stack, stride, R);
     }
     if (lane == 0) {
@@ -1820,7 +1786,7 @@ __global__ void __launch_bounds__(128) backward_fp64_kernel(const __grid_constan
         if (!tile_ray(p, tile, (uint32_t)lane, ray, px, py)) continue;
         RayState R0;
         // the FP32 ray as the forward sets it up (it decides the stepping)
-        if (!init_ray_geom(p, fs, false, s_bray + threadIdx.x, stride, my_stack, R0, ray, px, py)) continue;
+        if (!init_ray_geom(p, false, s_bray + threadIdx.x, stride, my_stack, R0, ray, px, py)) continue;
         Ray64 r;
         ray64_setup(p, ray, px, py, r);
         double C[3];

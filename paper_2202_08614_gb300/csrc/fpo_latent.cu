@@ -213,10 +213,7 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
     const int group = tid >> 7, gt = tid & 127;  // warpgroup and thread within it
 
     // --- prologue: basis, weights (bf16 -> f16, core layout), folded layer 3
-    const int nb = p.n1 > p.n2 ? p.n1 : p.n2;
-    if (tid < 32) s_basis[tid] = tid < nb ? (float)((tid & 1) ? sinpi((double)(tid + 1) * (p.t / p.period_T))
-                                                             : cospi((double)tid * (p.t / p.period_T)))
-                                         : 0.0f;
+    if (tid < 32) s_basis[tid] = p.b[tid];
     if (tid == 0) s_range = 0;
     if (tid < LT_GROUPS) {
         s_fail[tid] = 0;
@@ -1279,8 +1276,7 @@ extern "C" int fpo_latent_table(const fpo_decoder *dec, int32_t n1, int32_t n2, 
     p.b3 = dec->b3;
     p.n1 = n1;
     p.n2 = n2;
-    p.t = t;
-    p.period_T = period_T;
+    time_basis(t, period_T, n1 > n2 ? n1 : n2, p.b);
     p.n_leaves = n_leaves;
     p.table = table;
     p.status = status;
