@@ -92,13 +92,6 @@ constexpr int PIPE_TRAV_CTAS = FPO_PIPE_TRAV_CTAS;
 constexpr int PIPE_MAT_SMEM_BUDGET = FPO_PIPE_MAT_SMEM_KB * 1024;  // bytes of coefficient records in flight per SM
 constexpr int PIPE_STATIC_SMEM = 512;            // allowance for each kernel's static shared memory
 constexpr int SMEM_CONFIGS_KB[] = {0, 8, 16, 32, 64, 100, 132, 164, 196, 228};  // per SM, sm_100 family
-// Top-level nodes staged in shared memory per traversal CTA (32 B each); 0
-// with the kernels' default FPO_NODE_SMEM 0, which reads every node slot
-// from global memory.
-#ifndef FPO_SMEM_NODES
-#define FPO_SMEM_NODES 0
-#endif
-constexpr uint32_t SMEM_NODE_BUDGET = FPO_SMEM_NODES;
 constexpr int DEFAULT_TRAVERSE_THREADS = 256;
 constexpr uint32_t DEFAULT_REFILL_MIN = 32;
 constexpr uint32_t DEFAULT_INNER_STEPS = 0xffffffffu;  // a lane runs its ray to the end
@@ -114,7 +107,7 @@ struct fpo_ctx {
     uint32_t *d_status = nullptr;
     // tree
     bool has_tree = false;
-    uint32_t n_leaves = 0, n_nodes = 0, root_kind = ROOT_EMPTY, n_smem_nodes = 0;
+    uint32_t n_leaves = 0, n_nodes = 0, root_kind = ROOT_EMPTY;
     int depth = 0;
     uint32_t max_depth = 0;
     double aabb_min[3] = {0, 0, 0}, aabb_size = 1.0;
@@ -189,7 +182,6 @@ CtxView ctx_view(const fpo_ctx *c)
     v.n_leaves = c->n_leaves;
     v.n_nodes = c->n_nodes;
     v.root_kind = c->root_kind;
-    v.n_smem_nodes = c->n_smem_nodes;
     v.depth = c->depth;
     for (int k = 0; k < 3; ++k) v.aabb_min[k] = c->aabb_min[k];
     v.aabb_size = c->aabb_size;
@@ -333,7 +325,6 @@ int fpo_upload_tree(fpo_ctx *ctx, const fpo_tree_desc *tree)
     ctx->root_kind = pk.root_kind;
     ctx->depth = pk.depth;
     ctx->max_depth = tree->max_depth;
-    ctx->n_smem_nodes = (uint32_t)(n_nodes < SMEM_NODE_BUDGET ? n_nodes : SMEM_NODE_BUDGET);
     for (int k = 0; k < 3; ++k) ctx->aabb_min[k] = tree->aabb_min[k];
     ctx->aabb_size = tree->aabb_size;
     ctx->has_tree = true;
@@ -348,7 +339,7 @@ int fpo_tree_info_get(const fpo_ctx *ctx, fpo_tree_info *out)
     out->n_leaves = ctx->n_leaves;
     out->n_nodes = ctx->n_nodes;
     out->max_depth = ctx->max_depth;
-    out->n_smem_nodes = ctx->n_smem_nodes;
+    out->n_smem_nodes = 0;  // every node slot is read from global memory
     out->node_bytes = (uint64_t)ctx->n_nodes * 32;
     if (ctx->cfg.storage == FPO_STORAGE_LATENT) {
         out->leaf_record_bytes = 64;  // one FP16 latent of 32 values (the decoder is shared)
@@ -485,7 +476,6 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
     p.nodes = ctx->d_nodes;
     p.root_kind = ctx->root_kind;
     p.depth = ctx->depth;
-    p.n_smem_nodes = ctx->n_smem_nodes;
     p.grid_scale64 = (double)(1u << ctx->depth) / ctx->aabb_size;
     p.grid_scale = (float)p.grid_scale64;
     for (int k = 0; k < 3; ++k) {
@@ -723,7 +713,7 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             mshape = materialise_pipeline_shape(ctx->cfg.storage, ctx->cfg.n1, ctx->cfg.n2, PIPE_MAT_SMEM_BUDGET);
             if (FPO_PIPE_MAT_CTAS > 0) mshape.ctas_per_sm = FPO_PIPE_MAT_CTAS;
         }
-        const long need = (long)PIPE_TRAV_CTAS * (traverse_smem_bytes(ctx->n_smem_nodes, false, PIPE_TRAV_THREADS) + PIPE_STATIC_SMEM + reserved) +
+        const long need = (long)PIPE_TRAV_CTAS * (traverse_smem_bytes(PIPE_TRAV_THREADS) + PIPE_STATIC_SMEM + reserved) +
                           (long)mshape.ctas_per_sm * (mshape.smem_per_cta + PIPE_STATIC_SMEM + reserved);
         // The driver rounds a carveout request up to one of the SM's shared-
         // memory configurations: ask for the smallest one that holds `need`.

@@ -121,7 +121,6 @@ struct TraverseParams {
     const uint32_t *nodes;
     uint32_t root_kind;
     int depth;
-    uint32_t n_smem_nodes;
     float grid_scale;         // 2^D / aabb_size
     float amin[3];
     double grid_scale64, amin64[3];  // the same in FP64 (gradient-check replay)
@@ -150,6 +149,7 @@ struct TraverseParams {
     uint32_t refill_min;      // warp refills its idle lanes once this many are idle (32: whole tiles)
     uint32_t inner_steps;     // steps a lane takes between two refill checks
     int block_threads;        // 128 or 256
+    int rays_per_warp, list_cap; // fused mode: rays of one warp and length of its visit list (set by the launcher)
     int max_ctas_per_sm;      // 0: as many as fit
     int carveout;             // preferred shared-memory carveout in percent (0: the driver's default)
     unsigned long long *stats; // FPO_FLAG_STATS: [steps, leaf visits, rays entering the tree]
@@ -182,7 +182,7 @@ struct CtxView {
     uint32_t *d_status;
     bool half_table;
     bool has_tree;
-    uint32_t n_leaves, n_nodes, root_kind, n_smem_nodes;
+    uint32_t n_leaves, n_nodes, root_kind;
     int depth;
     double aabb_min[3], aabb_size;
     const uint32_t *d_nodes, *d_perm;
@@ -305,7 +305,7 @@ int launch_set_coeffs(const float *src, const uint32_t *perm, float *sig, float 
 int launch_leaf_adam(const LeafAdamParams &p, int sm_count, void *stream);
 int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int sm_count,
                     void *stream);
-int traverse_smem_bytes(uint32_t n_smem_nodes, bool per_ray_basis, int threads);
+int traverse_smem_bytes(int threads);
 bool fused_supported(int n1, int n2);
 
 }  // namespace fpo

@@ -6,8 +6,9 @@
 //  traverse_kernel      persistent ray traversal of the union octree with
 //                       exact ray-leaf segments and empty-space skipping,
 //                       SH colour + sigmoid (Eq. 1) and front-to-back
-//                       compositing with early stop; the IDFT either read
-//                       from the per-frame table or fused per visit.
+//                       compositing with early stop, from the per-frame table.
+//  fused_kernel         the same from the coefficient records, with the IDFT
+//                       per visit (rays with per-ray times), and its adjoint.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -21,15 +22,6 @@
 
 #ifndef FPO_FAST_STEP
 #define FPO_FAST_STEP 1
-#endif
-#ifndef FPO_GENERIC_NODE_LOAD
-#define FPO_GENERIC_NODE_LOAD 1
-#endif
-// Node slots come from global memory (read-only path); 1 keeps the top
-// nodes in shared memory, read through one generic pointer (measured: no gain
-// alone, 1.4% slower per pipelined frame, where the 16 KB per CTA is L1).
-#ifndef FPO_NODE_SMEM
-#define FPO_NODE_SMEM 0
 #endif
 #ifndef FPO_FAST_SIGMOID
 #define FPO_FAST_SIGMOID 1
@@ -95,17 +87,6 @@ __device__ __forceinline__ float sigmoidf_(float x) { return __fdividef(1.0f, 1.
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.0f / (1.0f + __expf(-x)); }
 #endif
 
-// VW floats from a read-only global address aligned to 4 VW bytes.
-template <int VW>
-__device__ __forceinline__ void load_vec(const float *p, float *v);
-
-// The FP32 coefficient records of (n1, n2) take 32-byte loads when both
-// padded strides are multiples of 8 floats: (31, 5) and (21, 5).
-__host__ __device__ constexpr bool fused_ldg256(int n1, int n2)
-{
-    return ((n1 + 3) & ~3) % 8 == 0 && ((27 * n2 + 3) & ~3) % 8 == 0;
-}
-
 // One 32-byte read-only global load (sm_100+ 256-bit vector load); p is
 // 32-byte aligned.
 __device__ __forceinline__ void ldg256(const float *p, float *v)
@@ -113,22 +94,6 @@ __device__ __forceinline__ void ldg256(const float *p, float *v)
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
         : "l"(p));
-}
-
-template <>
-__device__ __forceinline__ void load_vec<8>(const float *p, float *v)
-{
-    ldg256(p, v);
-}
-
-template <>
-__device__ __forceinline__ void load_vec<4>(const float *p, float *v)
-{
-    const float4 w = __ldg(reinterpret_cast<const float4 *>(p));
-    v[0] = w.x;
-    v[1] = w.y;
-    v[2] = w.z;
-    v[3] = w.w;
 }
 
 }  // namespace
@@ -710,10 +675,6 @@ int launch_materialise(const MaterialiseParams &p, int sm_count, void *stream)
 
 namespace {
 
-struct FrameShared {
-    float b[MAX_BASIS];  // Eq. 8 at the shared frame time
-};
-
 // Per-lane state of one ray, kept in registers across the warp's step loop.
 struct RayState {
     float go[3];   // origin in grid units, moved to the cube entry point
@@ -743,8 +704,7 @@ __device__ __forceinline__ void write_result(const TraverseParams &p, const RayS
 // Sets up ray `ray` (camera pixel (px, py) or explicit ray): generation,
 // SH basis, clip against the grid cube.  Returns false when the ray misses
 // the tree (its background result is written at once).
-__device__ bool init_ray_geom(const TraverseParams &p, bool prt, float *s_bray,
-                              int stride, uint32_t *s_stack, RayState &R, uint32_t ray, int px, int py)
+__device__ bool init_ray_geom(const TraverseParams &p, uint32_t *s_stack, RayState &R, uint32_t ray, int px, int py)
 {
     float ox, oy, oz, dx, dy, dz;
     if (p.fr.mode == FPO_RAYS_CAMERA) {
@@ -769,12 +729,6 @@ __device__ bool init_ray_geom(const TraverseParams &p, bool prt, float *s_bray,
         dx *= inv;
         dy *= inv;
         dz *= inv;
-    }
-    if (prt) {
-        // Eq. 8 at this ray's own time, one column of the per-thread table
-        const float u = p.fr.rt[ray] / (float)p.fr.period_T;
-        const int nb = p.n1 > p.n2 ? p.n1 : p.n2;
-        for (int i = 0; i < nb; ++i) s_bray[i * stride] = basis_fp32(i, u);
     }
     sh_basis(dx, dy, dz, R.Y);
     R.C0 = R.C1 = R.C2 = 0.0f;
@@ -820,17 +774,6 @@ __device__ bool init_ray_geom(const TraverseParams &p, bool prt, float *s_bray,
     return true;
 }
 
-// As init_ray_geom; a ray that misses the tree gets its background result.
-template <bool DBG>
-__device__ __forceinline__ bool init_ray(const TraverseParams &p, bool prt,
-                                         float *s_bray, int stride, uint32_t *s_stack, RayState &R,
-                                         uint32_t ray, int px, int py)
-{
-    if (init_ray_geom(p, prt, s_bray, stride, s_stack, R, ray, px, py)) return true;
-    write_result(p, R, DBG);
-    return false;
-}
-
 // The cube holding cell R.P: its kind (ROOT_EMPTY / ROOT_LEAF), leaf index and
 // level.  Descends from the deepest still-valid ancestor in the per-thread
 // stack, updating the stack on the way down.
@@ -839,8 +782,8 @@ struct Cube {
     int lvl;
 };
 
-__device__ __forceinline__ Cube locate(const TraverseParams &p, const uint32_t *__restrict__ s_nodes,
-                                       uint32_t *s_stack, int stride, const int P[3], int lvl_start)
+__device__ __forceinline__ Cube locate(const TraverseParams &p, uint32_t *s_stack, int stride, const int P[3],
+                                       int lvl_start)
 {
     Cube cb;
     cb.leaf = 0;
@@ -856,18 +799,7 @@ __device__ __forceinline__ Cube locate(const TraverseParams &p, const uint32_t *
         const int sh = D - 1 - lvl;
         const uint32_t c = ((P[0] >> sh) & 1) | (((P[1] >> sh) & 1) << 1) | (((P[2] >> sh) & 1) << 2);
         const uint32_t idx = node * 8 + c;
-#if FPO_NODE_SMEM == 0
-        // every node slot from global memory (read-only path)
         const uint32_t sl = __ldg(p.nodes + idx);
-        (void)s_nodes;
-#elif FPO_GENERIC_NODE_LOAD
-        // one generic load from shared (top nodes) or global memory: no branch
-        // between two load paths for lanes at different levels
-        const uint32_t *src = node < p.n_smem_nodes ? s_nodes : p.nodes;
-        const uint32_t sl = src[idx];
-#else
-        const uint32_t sl = node < p.n_smem_nodes ? s_nodes[idx] : __ldg(p.nodes + idx);
-#endif
         ++lvl;
         if (sl == 0u) { cb.kind = ROOT_EMPTY; break; }
         if (sl & LEAF_BIT) { cb.kind = ROOT_LEAF; cb.leaf = sl & ~LEAF_BIT; break; }
@@ -957,9 +889,9 @@ __device__ __forceinline__ void move_to(RayState &R, int D, const int Pn[3], flo
     R.P[2] = Pn[2];
 }
 
-// Table modes of the traversal: the fused per-visit IDFT, or the per-frame
-// table in FP32 (128-byte lines) or FP16 (64-byte lines).
-constexpr int TM_FUSED = 0, TM_TABLE_F32 = 1, TM_TABLE_F16 = 2;
+// Table modes of the traversal: the per-frame table in FP32 (128-byte lines)
+// or FP16 (64-byte lines).
+constexpr int TM_TABLE_F32 = 1, TM_TABLE_F16 = 2;
 
 __device__ __forceinline__ const float4 *table_record(const TraverseParams &p, uint32_t leaf)
 {
@@ -971,12 +903,11 @@ __device__ __forceinline__ const __half *table_record_f16(const TraverseParams &
     return reinterpret_cast<const __half *>(p.table) + (size_t)leaf * TABLE_STRIDE;
 }
 
-// Shades one leaf segment of length delta (Eq. 7 and 9 from the table or
-// fused, Eq. 1 colour, emission-absorption update).  Returns true when the
-// transmittance fell below stop_T.
-template <int TM, bool DBG, int N1, int N2>
-__device__ __forceinline__ bool shade(const TraverseParams &p, const float *bsrc, int bstride,
-                                      RayState &R, uint32_t leaf, float delta)
+// Shades one leaf segment of length delta (Eq. 7 and 9 from the table, Eq. 1
+// colour, emission-absorption update).  Returns true when the transmittance
+// fell below stop_T.
+template <int TM, bool DBG>
+__device__ __forceinline__ bool shade(const TraverseParams &p, RayState &R, uint32_t leaf, float delta)
 {
     float sigma, z[27];
     if constexpr (TM == TM_TABLE_F16) {
@@ -994,7 +925,7 @@ __device__ __forceinline__ bool shade(const TraverseParams &p, const float *bsrc
         sigma = v[0];
 #pragma unroll
         for (int q = 0; q < 27; ++q) z[q] = v[q + 1];
-    } else if constexpr (TM == TM_TABLE_F32) {
+    } else {
         const float4 *rec = table_record(p, leaf);
         float v[32];
 #if FPO_LDG256
@@ -1023,56 +954,6 @@ __device__ __forceinline__ bool shade(const TraverseParams &p, const float *bsrc
         sigma = v[0];
 #pragma unroll
         for (int q = 0; q < 27; ++q) z[q] = v[q + 1];
-    } else {
-        const float4 *sr = p.sig + (size_t)leaf * p.sig_stride4;
-        const float *zr = p.zc + (size_t)leaf * p.z_stride;
-        float bz[N2];
-#pragma unroll
-        for (int i = 0; i < N2; ++i) bz[i] = bsrc[i * bstride];
-#pragma unroll
-        for (int q = 0; q < 27; ++q) z[q] = 0.0f;
-        float acc = 0.0f;
-        if constexpr (FPO_LDG256 && fused_ldg256(N1, N2)) {
-            // 32-byte loads: both record strides are multiples of 8 floats
-#pragma unroll
-            for (int q = 0; q < (N1 + 7) / 8; ++q) {
-                float wv[8];
-                ldg256(reinterpret_cast<const float *>(sr) + 8 * q, wv);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (8 * q + j < N1) acc = fmaf(wv[j], bsrc[(8 * q + j) * bstride], acc);
-            }
-#pragma unroll
-            for (int q = 0; q < (27 * N2 + 7) / 8; ++q) {
-                float wv[8];
-                ldg256(zr + 8 * q, wv);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int e = 8 * q + j;
-                    if (e < 27 * N2) z[e / N2] = fmaf(wv[j], bz[e % N2], z[e / N2]);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < (N1 + 3) / 4; ++q) {
-                const float4 w = __ldg(sr + q);
-                const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (4 * q + j < N1) acc = fmaf(wv[j], bsrc[(4 * q + j) * bstride], acc);
-            }
-#pragma unroll
-            for (int q4 = 0; q4 < (27 * N2 + 3) / 4; ++q4) {
-                const float4 w = __ldg(reinterpret_cast<const float4 *>(zr) + q4);
-                const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int e = 4 * q4 + j;
-                    if (e < 27 * N2) z[e / N2] = fmaf(wv[j], bz[e % N2], z[e / N2]);
-                }
-            }
-        }
-        sigma = fmaxf(acc, 0.0f);
     }
     float col[3];
 #pragma unroll
@@ -1110,29 +991,15 @@ __device__ __forceinline__ bool step_cap(const TraverseParams &p, RayState &R)
     return false;
 }
 
-// Fused mode: the coefficient records of the next leaf (672 B at n1 = 31,
-// n2 = 5) are pulled into L2 by two bulk prefetches while the current leaf is
-// shaded, so its 32-byte loads hit L2 instead of HBM.
-__device__ __forceinline__ void prefetch_records(const TraverseParams &p, uint32_t leaf, int n1, int n2)
-{
-    const float4 *sr = p.sig + (size_t)leaf * p.sig_stride4;
-    const float *zr = p.zc + (size_t)leaf * p.z_stride;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(sr), "r"((uint32_t)(p.sig_stride4 * 16)));
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(zr), "r"((uint32_t)(p.z_stride * 4)));
-    (void)n1;
-    (void)n2;
-}
-
 // One step of the software-pipelined walk: the exit of cube `cb` (which
-// holds R.P), the next cube located and its table record (or coefficient
-// records) prefetched before `cb` is shaded, so the record's latency hides
-// behind the shading arithmetic; then the move.  `cb` becomes the next cube.
+// holds R.P), the next cube located and its table record prefetched before
+// `cb` is shaded, so the record's latency hides behind the shading
+// arithmetic; then the move.  `cb` becomes the next cube.
 // Returns false once the ray is finished (left the grid, early stop, or
 // step cap).
-template <int TM, bool DBG, int N1, int N2>
-__device__ __forceinline__ bool pipelined_step(const TraverseParams &p, const float *bsrc, int bstride,
-                                               const uint32_t *__restrict__ s_nodes, uint32_t *s_stack,
-                                               int stride, RayState &R, Cube &cb)
+template <int TM, bool DBG>
+__device__ __forceinline__ bool pipelined_step(const TraverseParams &p, uint32_t *s_stack, int stride, RayState &R,
+                                               Cube &cb)
 {
     const int D = p.depth, G = 1 << D;
     int m, lo[3], csz;
@@ -1143,57 +1010,43 @@ __device__ __forceinline__ bool pipelined_step(const TraverseParams &p, const fl
     nx.kind = ROOT_EMPTY;
     if (FPO_PREFETCH && inside) {
         const uint32_t diff = (uint32_t)((R.P[0] ^ Pn[0]) | (R.P[1] ^ Pn[1]) | (R.P[2] ^ Pn[2]));
-        nx = locate(p, s_nodes, s_stack, stride, Pn, D - 1 - (31 - __clz(diff)));
+        nx = locate(p, s_stack, stride, Pn, D - 1 - (31 - __clz(diff)));
         if (nx.kind == ROOT_LEAF) {
             if constexpr (TM == TM_TABLE_F32) {
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(table_record(p, nx.leaf)));
                 if (FPO_PREFETCH_SIBLINGS)  // the aligned group of 4 lines holding it (siblings are adjacent)
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], 512;" ::"l"(table_record(p, nx.leaf & ~3u)));
-            } else if constexpr (TM == TM_TABLE_F16) {
+            } else {
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(table_record_f16(p, nx.leaf)));
                 if (FPO_PREFETCH_SIBLINGS)
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], 512;" ::"l"(table_record_f16(p, nx.leaf & ~7u)));
-            } else {
-                prefetch_records(p, nx.leaf, N1, N2);
             }
         }
     }
     if (cb.kind == ROOT_LEAF && tx > R.t)
-        if (shade<TM, DBG, N1, N2>(p, bsrc, bstride, R, cb.leaf, tx - R.t)) return false;
+        if (shade<TM, DBG>(p, R, cb.leaf, tx - R.t)) return false;
     if (!inside) return false;
     move_to(R, D, Pn, tx);
     if (step_cap(p, R)) return false;
     if (FPO_PREFETCH)
         cb = nx;
     else
-        cb = locate(p, s_nodes, s_stack, stride, R.P, R.lvl_start);
+        cb = locate(p, s_stack, stride, R.P, R.lvl_start);
     return true;
 }
 
 // A whole ray (lane-loop schedule).
-template <int TM, bool DBG, int N1, int N2>
-__device__ void trace_ray(const TraverseParams &p, const float *bsrc, int bstride,
-                          const uint32_t *__restrict__ s_nodes, uint32_t *s_stack, int stride,
-                          RayState &R)
+template <int TM, bool DBG>
+__device__ void trace_ray(const TraverseParams &p, uint32_t *s_stack, int stride, RayState &R)
 {
-    Cube cb = locate(p, s_nodes, s_stack, stride, R.P, R.lvl_start);
-    while (pipelined_step<TM, DBG, N1, N2>(p, bsrc, bstride, s_nodes, s_stack, stride, R, cb)) {
+    Cube cb = locate(p, s_stack, stride, R.P, R.lvl_start);
+    while (pipelined_step<TM, DBG>(p, s_stack, stride, R, cb)) {
     }
 }
 
 }  // namespace
 
 namespace {
-
-// CTA prologue: stage the top n_smem_nodes nodes in shared memory, and the
-// frame basis (Eq. 8 at the shared t).
-__device__ void frame_prologue(const TraverseParams &p, uint32_t *s_nodes, FrameShared &fs)
-{
-    const uint4 *src = reinterpret_cast<const uint4 *>(p.nodes);
-    uint4 *dst = reinterpret_cast<uint4 *>(s_nodes);
-    for (uint32_t i = threadIdx.x; i < p.n_smem_nodes * 2; i += blockDim.x) dst[i] = __ldg(src + i);
-    if (threadIdx.x < MAX_BASIS) fs.b[threadIdx.x] = p.fc.b[threadIdx.x];
-}
 
 // Ray k (0..31) of a tile: a camera pixel of a TILE_W x TILE_H block, or an
 // explicit ray.
@@ -1213,6 +1066,20 @@ __device__ __forceinline__ bool tile_ray(const TraverseParams &p, uint32_t tile,
     return ray < p.fr.n_rays;
 }
 
+// The last warp of the grid to finish resets the tile counter for the next
+// launch (every warp has made its final grab before counting itself).
+__device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
+{
+    if (lane == 0) {
+        __threadfence();
+        const uint32_t done = atomicAdd(p.tiles + 1, 1u);
+        if (done == gridDim.x * (blockDim.x / 32) - 1) {
+            atomicExch(p.tiles, 0u);
+            atomicExch(p.tiles + 1, 0u);
+        }
+    }
+}
+
 }  // namespace
 
 // Persistent kernel: a grid of (SM count x resident CTAs) whose warps pull
@@ -1220,38 +1087,20 @@ __device__ __forceinline__ bool tile_ray(const TraverseParams &p, uint32_t tile,
 // atomic counter.  Warp-level ray compaction: every lane holds its own ray;
 // when at least REFILL_MIN lanes are idle, the warp hands them the next rays
 // of its current tile (fetching a new tile when that one is used up), so
-// long rays do not leave most of a warp idle.  Each CTA first stages the top
-// n_smem_nodes nodes of the breadth-first node array and the frame constants
-// in shared memory.  The last CTA to finish resets the counter.
-// Register caps: 64 lets four 256-thread CTAs share an SM in materialised
-// mode (measured fastest of 48..80 on the 3.5M-leaf body at 1080p); the fused
-// per-visit IDFT needs more.
+// long rays do not leave most of a warp idle.  The last CTA to finish resets
+// the counter.  Register cap: 64 lets four 256-thread CTAs share an SM
+// (measured fastest of 48..80 on the 3.5M-leaf body at 1080p).
 #ifndef FPO_TRAV_MAXNREG_MAT
 #define FPO_TRAV_MAXNREG_MAT 64
 #endif
-#ifndef FPO_TRAV_MAXNREG_FUSED
-#define FPO_TRAV_MAXNREG_FUSED 128
-#endif
 
-template <int TM, bool DBG, int N1, int N2, bool COMPACT>
-__global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) traverse_kernel(const __grid_constant__ TraverseParams p)
+template <int TM, bool DBG, bool COMPACT>
+__global__ void __maxnreg__(FPO_TRAV_MAXNREG_MAT) traverse_kernel(const __grid_constant__ TraverseParams p)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ FrameShared fs;
     const int stride = blockDim.x;
-    uint32_t *s_nodes = smem;
-    uint32_t *s_stack = smem + p.n_smem_nodes * 8;
-    float *s_bray = reinterpret_cast<float *>(s_stack + STACK_LEVELS * stride);
-    const bool prt = TM == TM_FUSED && p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
-
-    frame_prologue(p, s_nodes, fs);
-    __syncthreads();
-
     const int lane = threadIdx.x & 31;
-    uint32_t *my_stack = s_stack + threadIdx.x;
-    float *my_b = s_bray + threadIdx.x;
-    const float *bsrc = prt ? my_b : fs.b;
-    const int bstride = prt ? stride : 1;
+    uint32_t *my_stack = smem + threadIdx.x;
 
     auto grab_tile = [&]() -> uint32_t {
         uint32_t tl = 0;
@@ -1276,9 +1125,11 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
             int px = 0, py = 0;
             if (tile_ray(p, tile, (uint32_t)lane, ray, px, py)) {
                 RayState R;
-                if (init_ray<DBG>(p, prt, my_b, stride, my_stack, R, ray, px, py)) {
-                    trace_ray<TM, DBG, N1, N2>(p, bsrc, bstride, s_nodes, my_stack, stride, R);
+                if (init_ray_geom(p, my_stack, R, ray, px, py)) {
+                    trace_ray<TM, DBG>(p, my_stack, stride, R);
                     finish(R);
+                } else {
+                    write_result(p, R, DBG);  // misses the tree: background
                 }
             }
         }
@@ -1306,8 +1157,9 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
                         uint32_t ray;
                         int px = 0, py = 0;
                         if (tile_ray(p, cur_tile, cur_next + rank, ray, px, py)) {
-                            active = init_ray<DBG>(p, prt, my_b, stride, my_stack, R, ray, px, py);
-                            if (active) cb = locate(p, s_nodes, my_stack, stride, R.P, R.lvl_start);
+                            active = init_ray_geom(p, my_stack, R, ray, px, py);
+                            if (active) cb = locate(p, my_stack, stride, R.P, R.lvl_start);
+                            else write_result(p, R, DBG);
                         }
                     }
                     cur_next += take;
@@ -1323,7 +1175,7 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
             if (active) {
 #pragma unroll 1
                 for (uint32_t k = 0; k < p.inner_steps; ++k) {
-                    if (!pipelined_step<TM, DBG, N1, N2>(p, bsrc, bstride, s_nodes, my_stack, stride, R, cb)) {
+                    if (!pipelined_step<TM, DBG>(p, my_stack, stride, R, cb)) {
                         finish(R);
                         active = false;
                         break;
@@ -1332,33 +1184,17 @@ __global__ void __maxnreg__(TM ? FPO_TRAV_MAXNREG_MAT : FPO_TRAV_MAXNREG_FUSED) 
             }
         }
     }
-    // The last warp of the grid to finish resets the tile counter for the
-    // next launch (every warp has made its final grab before counting itself).
-    if (lane == 0) {
-        __threadfence();
-        const uint32_t done = atomicAdd(p.tiles + 1, 1u);
-        if (done == gridDim.x * (blockDim.x / 32) - 1) {
-            atomicExch(p.tiles, 0u);
-            atomicExch(p.tiles + 1, 0u);
-        }
-    }
+    finish_tiles(p, lane);
 }
 
+int traverse_smem_bytes(int threads) { return STACK_LEVELS * threads * 4; }
 
-int traverse_smem_bytes(uint32_t n_smem_nodes, bool per_ray_basis, int threads)
-{
-    return (int)(n_smem_nodes * 32u + STACK_LEVELS * threads * 4u +
-                 (per_ray_basis ? 32u * threads * 4u : 0u));
-}
-
-
-template <int TM, bool DBG, int N1, int N2, bool COMPACT>
+template <int TM, bool DBG, bool COMPACT>
 static int launch_t(const TraverseParams &p, int sm_count, cudaStream_t s)
 {
-    const bool prt = TM == TM_FUSED && p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
     const int threads = p.block_threads;
-    const int smem = traverse_smem_bytes(p.n_smem_nodes, prt, threads);
-    auto k = traverse_kernel<TM, DBG, N1, N2, COMPACT>;
+    const int smem = traverse_smem_bytes(threads);
+    auto k = traverse_kernel<TM, DBG, COMPACT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1378,21 +1214,424 @@ static int launch_t(const TraverseParams &p, int sm_count, cudaStream_t s)
 
 // The compaction schedule (refill_min < 32) or the plain one, each with or
 // without the debug outputs (visit logs, final T, leaf marks, counters).
-template <int TM, int N1, int N2>
+template <int TM>
 static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaStream_t s)
 {
     if (p.refill_min < 32)
-        return debug ? launch_t<TM, true, N1, N2, true>(p, sm_count, s) : launch_t<TM, false, N1, N2, true>(p, sm_count, s);
-    return debug ? launch_t<TM, true, N1, N2, false>(p, sm_count, s) : launch_t<TM, false, N1, N2, false>(p, sm_count, s);
+        return debug ? launch_t<TM, true, true>(p, sm_count, s) : launch_t<TM, false, true>(p, sm_count, s);
+    return debug ? launch_t<TM, true, false>(p, sm_count, s) : launch_t<TM, false, false>(p, sm_count, s);
 }
 
-static int launch_fused(const TraverseParams &p, bool debug, int sm_count, cudaStream_t s)
+// ---------------------------------------------------------------------------
+// Per-visit IDFT (FUSED mode: rays with per-ray times, and frames on request)
+// and its adjoint (Sec. 4.3: back-propagation through the IDFT).
+//
+// A warp owns R rays (lanes 0..R-1) and alternates between four phases, so
+// that the walk, which few lanes of incoherent rays need at the same time, and
+// the work of a visit, which reads and writes whole rows, each have the warp
+// to themselves:
+//   walk       the R lanes step through the tree without shading and append
+//              their leaf segments to the warp's list in shared memory (a
+//              round = the visits of one step), until the list is full or
+//              every ray has left the grid; the records are pulled into L2;
+//   shade      all 32 lanes evaluate the list, FU_UNROLL visits at a time: lane
+//              l takes elements l, l + 32, ... of a visit's record (each load
+//              is one contiguous line), multiplies them by its ray's weights
+//              (Eq. 8 at the ray's time; Y_k(d) IDFT_i(t) for the colours, so
+//              Eq. 7, 9 and the sum of Eq. 1 are one dot product), and four
+//              sums are reduced by halving butterflies that keep all lanes busy;
+//   composite  lane l takes its own visits in order; a ray that falls below
+//              stop_T ignores the rest of its list (at most a list's worth of
+//              visits is evaluated for nothing);
+//   scatter    (adjoint) all 32 lanes add a visit's gradient row with
+//              contiguous 8-byte vector atomics.
+// The one-lane-per-ray form that this replaces read 21 scattered 32-byte
+// pieces per visit in each lane, with the whole warp waiting for the few
+// lanes that were inside a leaf, and left most SMs idle below 38,912 rays.
+//
+// Adjoint: with w_j = T_j alpha_j and C the forward colour (which includes
+// T_end bg), S_j = C - sum_{k<=j} w_k c_k is the colour behind segment j and
+//   dL/dsigma_j = delta_j sum_c g_c (T_{j+1} c_jc - S_jc),
+//   dL/du_jc    = g_c w_j c_jc (1 - c_jc),   u = sum_k z_ck Y_k,
+//   dL/dk_sigma_i += dL/dsigma_j [sigma_raw > 0] IDFT_i(t),
+//   dL/dk_cki     += dL/du_jc Y_k IDFT_i(t).
+// Walk, shade and composite are the same code in both directions, so the
+// adjoint sees the forward's segments and early stop.
+
+constexpr int FU_WARPS = 2;    // warps per CTA (they share nothing but its launch)
+constexpr int FU_UNROLL = 4;   // visits a warp evaluates at a time
+#ifndef FPO_FUSED_MIN_RAYS
+#define FPO_FUSED_MIN_RAYS 2
+#endif
+#ifndef FPO_FUSED_WARPS_PER_SM
+#define FPO_FUSED_WARPS_PER_SM 32
+#endif
+#ifndef FPO_FUSED_LIST
+#define FPO_FUSED_LIST 4
+#endif
+#ifndef FPO_FUSED_REFILL
+#define FPO_FUSED_REFILL 12
+#endif
+#ifndef FPO_FUSED_PREFETCH
+#define FPO_FUSED_PREFETCH 1
+#endif
+constexpr uint32_t FU_REFILL = FPO_FUSED_REFILL;  // idle lanes, of 32, at which a warp takes new rays
+constexpr bool FU_PREFETCH = FPO_FUSED_PREFETCH;
+
+template <int N1, int N2>
+struct FusedSize {
+    static constexpr int NZ = 9 * N2;            // weights shared by the three channels
+    static constexpr int NW = N1 + NZ;           // weights per ray
+    static constexpr int NWP = NW | 1;           // odd row stride: no bank conflicts between rays
+    static constexpr int ZR = (27 * N2 + 31) / 32;
+    static constexpr int NC = N1 + 27 * N2;
+};
+
+// Shared memory of one warp, in 32-bit words (a multiple of 4): the list
+// (visit, result, round mask per entry), the ancestor stacks, the weights.
+__host__ __device__ inline int fused_warp_words(int rays, int cap, int depth, int nwp)
 {
-    // Fused per-visit IDFT: compile-time Fourier sizes (the settings of Tab. 3).
-    if (p.n1 == 31 && p.n2 == 5) return launch_sched<TM_FUSED, 31, 5>(p, debug, sm_count, s);
-    if (p.n1 == 11 && p.n2 == 5) return launch_sched<TM_FUSED, 11, 5>(p, debug, sm_count, s);
-    if (p.n1 == 21 && p.n2 == 5) return launch_sched<TM_FUSED, 21, 5>(p, debug, sm_count, s);
-    if (p.n1 == 31 && p.n2 == 11) return launch_sched<TM_FUSED, 31, 11>(p, debug, sm_count, s);
+    return (9 * cap + rays * (depth + 1) + rays * nwp + 3) & ~3;
+}
+
+template <int N1, int N2, bool ADJ, bool DBG>
+__global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_constant__ BackwardParams q)
+{
+    using S = FusedSize<N1, N2>;
+    extern __shared__ __align__(16) uint32_t smem[];
+    const TraverseParams &p = q.tp;
+    const int lane = threadIdx.x & 31;
+    const int R = p.rays_per_warp, E = p.list_cap;
+    const int D = p.depth, G = 1 << D;
+    uint32_t *mem = smem + (threadIdx.x >> 5) * fused_warp_words(R, E, D, S::NWP);
+    uint4 *ent = reinterpret_cast<uint4 *>(mem);             // leaf, delta, lane, step
+    float *res = reinterpret_cast<float *>(mem + 4 * E);     // [E][4]
+    uint32_t *rounds = mem + 8 * E;
+    uint32_t *stack = rounds + E + (lane < R ? lane : 0);    // stride R
+    float *wt = reinterpret_cast<float *>(rounds + E + R * (D + 1));
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const bool prt = p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
+
+    const uint32_t lanes = R == 32 ? 0xffffffffu : (1u << R) - 1u;  // the lanes that walk
+    const uint32_t n_slots = p.n_tiles * 32u;
+    const uint32_t refill = max(1u, (uint32_t)R * FU_REFILL / 32u);
+    bool more = true;  // the queue has rays left (warp-uniform)
+    bool active = false, walking = false, stopped = false, capped = false;
+    RayState W;
+    uint32_t ray = 0;
+    float g0 = 0.0f, g1 = 0.0f, g2 = 0.0f, Cf0 = 0.0f, Cf1 = 0.0f, Cf2 = 0.0f;
+    Cube cb;
+    cb.kind = ROOT_EMPTY;
+    cb.leaf = 0;
+    cb.lvl = 0;
+
+    for (;;) {
+        // --- refill: idle lanes take the next rays of the queue
+        uint32_t idle = __ballot_sync(0xffffffffu, !active) & lanes, fresh = 0;
+        while (more && ((uint32_t)__popc(idle) >= refill || idle == lanes)) {
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(p.tiles, (uint32_t)__popc(idle));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (base >= n_slots) {
+                more = false;
+                break;
+            }
+            const uint32_t slot = base + __popc(idle & lt_mask);
+            bool ok = false;
+            if (((idle >> lane) & 1u) && slot < n_slots) {
+                int px = 0, py = 0;
+                if (tile_ray(p, slot >> 5, slot & 31u, ray, px, py)) {
+                    ok = init_ray_geom(p, stack, W, ray, px, py);
+                    if (!ok && !ADJ) write_result(p, W, DBG);  // misses the tree: background
+                }
+            }
+            active |= ok;
+            fresh |= __ballot_sync(0xffffffffu, ok);
+            idle = __ballot_sync(0xffffffffu, !active) & lanes;
+        }
+        if (idle == lanes) break;  // (the queue is empty then)
+        if (fresh) {
+            // the new rays' weights: b_i at the ray's time, then Y_k b_i
+            const bool mine = (fresh >> lane) & 1u;
+            float u = 0.0f;
+            if (prt && mine) u = p.fr.rt[ray] / (float)p.fr.period_T;
+            for (uint32_t f = fresh; f; f &= f - 1u) {
+                const int r = __ffs((int)f) - 1;
+                const float ur = __shfl_sync(0xffffffffu, u, r);
+                if (lane < N1) wt[r * S::NWP + lane] = prt ? basis_fp32(lane, ur) : p.fc.b[lane];
+            }
+            __syncwarp();
+            if (mine) {
+                float *w = wt + lane * S::NWP;
+                float b[N2];
+#pragma unroll
+                for (int i = 0; i < N2; ++i) b[i] = w[i];
+#pragma unroll
+                for (int k = 0; k < 9; ++k)
+#pragma unroll
+                    for (int i = 0; i < N2; ++i) w[N1 + k * N2 + i] = W.Y[k] * b[i];
+                if (ADJ) {
+                    g0 = q.dL_drgb[3 * (size_t)ray];
+                    g1 = q.dL_drgb[3 * (size_t)ray + 1];
+                    g2 = q.dL_drgb[3 * (size_t)ray + 2];
+                    Cf0 = q.out_rgb[3 * (size_t)ray];
+                    Cf1 = q.out_rgb[3 * (size_t)ray + 1];
+                    Cf2 = q.out_rgb[3 * (size_t)ray + 2];
+                }
+                walking = true;
+                stopped = capped = false;
+                cb = locate(p, stack, R, W.P, 0);
+            }
+        }
+        {
+            // --- walk
+            uint32_t n = 0, nr = 0, act;
+            do {
+                bool hit = false;
+                uint32_t leaf = 0, step = 0;
+                float delta = 0.0f;
+                if (walking) {
+                    int m, lo[3], csz;
+                    const float tx = cube_exit(W, D, cb.lvl, m, lo, csz);
+                    hit = cb.kind == ROOT_LEAF && tx > W.t;
+                    leaf = cb.leaf;
+                    delta = tx - W.t;
+                    step = W.steps;
+                    int Pn[3];
+                    walking = next_cell(W, G, m, lo, csz, tx, Pn);
+                    if (walking) {
+                        move_to(W, D, Pn, tx);
+                        if (++W.steps > p.max_steps) {
+                            capped = true;
+                            walking = false;
+                        } else {
+                            cb = locate(p, stack, R, W.P, W.lvl_start);
+                        }
+                    }
+                }
+                const uint32_t mask = __ballot_sync(0xffffffffu, hit);
+                if (mask) {
+                    if (hit) ent[n + __popc(mask & lt_mask)] = make_uint4(leaf, __float_as_uint(delta), (uint32_t)lane, step);
+                    if (lane == 0) rounds[nr] = mask;
+                    ++nr;
+                    n += __popc(mask);
+                }
+                act = __ballot_sync(0xffffffffu, walking);
+            } while (act && n + (uint32_t)R <= (uint32_t)E && !(more && (uint32_t)__popc(lanes & ~act) >= refill));
+            __syncwarp();
+            if (FU_PREFETCH) {
+                // every line of the list's records into L2, one line a lane
+                const uint32_t sb = (uint32_t)p.sig_stride4 * 16u, zb = (uint32_t)p.z_stride * 4u;
+                constexpr uint32_t LN = 1 + (27 * N2 * 4 + 127) / 128;
+                for (uint32_t e = lane; e < n * LN; e += 32) {
+                    const uint32_t v = e / LN, l = e % LN;
+                    const uint32_t lf = ent[v].x;
+                    const char *a = l == 0 ? reinterpret_cast<const char *>(p.sig) + (size_t)lf * sb
+                                           : reinterpret_cast<const char *>(p.zc) + (size_t)lf * zb + (l - 1) * 128u;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+                }
+            }
+
+            // --- shade
+            for (uint32_t v0 = 0; v0 < n; v0 += FU_UNROLL) {
+                float part[FU_UNROLL][4];
+                uint32_t ray_lane[FU_UNROLL];
+                float zv[FU_UNROLL][S::ZR], sv[FU_UNROLL];
+#pragma unroll
+                for (int a = 0; a < FU_UNROLL; ++a) {
+                    const uint4 en = ent[min(v0 + a, n - 1)];
+                    ray_lane[a] = en.z;
+                    const float *sr = reinterpret_cast<const float *>(p.sig + (size_t)en.x * p.sig_stride4);
+                    const float *zr = p.zc + (size_t)en.x * p.z_stride;
+                    sv[a] = lane < N1 ? __ldg(sr + lane) : 0.0f;
+#pragma unroll
+                    for (int r = 0; r < S::ZR; ++r) zv[a][r] = 32 * r + lane < 27 * N2 ? __ldg(zr + 32 * r + lane) : 0.0f;
+                }
+#pragma unroll
+                for (int a = 0; a < FU_UNROLL; ++a) {
+                    const float *w = wt + ray_lane[a] * S::NWP;
+                    part[a][0] = lane < N1 ? sv[a] * w[lane] : 0.0f;
+                    part[a][1] = part[a][2] = part[a][3] = 0.0f;
+#pragma unroll
+                    for (int r = 0; r < S::ZR; ++r) {
+                        const int j = 32 * r + lane;  // element of the SH record: channel j / NZ, weight j % NZ
+                        const float x = w[N1 + j % S::NZ];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            // (compile-time where the 32 elements lie in one channel)
+                            if (32 * r >= c * S::NZ && 32 * r + 31 < (c + 1) * S::NZ) part[a][1 + c] = fmaf(zv[a][r], x, part[a][1 + c]);
+                            else if (32 * r + 31 >= c * S::NZ && 32 * r < (c + 1) * S::NZ && j >= c * S::NZ && j < (c + 1) * S::NZ)
+                                part[a][1 + c] = fmaf(zv[a][r], x, part[a][1 + c]);
+                        }
+                    }
+                }
+                // 16 sums over 32 lanes: each butterfly step halves the values a
+                // lane still carries; lane (b4 b3 b2 b1 b0) ends with value 2 b4 + b3
+                // of visit 2 b2 + b1
+                const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+                float s1[FU_UNROLL];
+#pragma unroll
+                for (int a = 0; a < FU_UNROLL; ++a) {
+                    float k0 = b4 ? part[a][2] : part[a][0], k1 = b4 ? part[a][3] : part[a][1];
+                    k0 += __shfl_xor_sync(0xffffffffu, b4 ? part[a][0] : part[a][2], 16);
+                    k1 += __shfl_xor_sync(0xffffffffu, b4 ? part[a][1] : part[a][3], 16);
+                    s1[a] = (b3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8);
+                }
+                float s2[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)  // visit 2 b2 + h
+                    s2[h] = (b2 ? s1[2 + h] : s1[h]) + __shfl_xor_sync(0xffffffffu, b2 ? s1[h] : s1[2 + h], 4);
+                float s = (b1 ? s2[1] : s2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? s2[0] : s2[1], 2);
+                s += __shfl_xor_sync(0xffffffffu, s, 1);
+                const int val = (b4 ? 2 : 0) + (b3 ? 1 : 0);
+                const uint32_t at = v0 + (b2 ? 2 : 0) + (b1 ? 1 : 0);
+                if (!(lane & 1) && at < n) {
+                    float o;
+                    if (val == 0) {
+                        // e^{-sigma delta}, with the sign bit set where sigma_raw > 0
+                        // (the adjoint's mask of max(0, sigma_raw))
+                        o = __expf(-fmaxf(s, 0.0f) * __uint_as_float(ent[at].y));
+                        if (s > 0.0f) o = -o;
+                    } else {
+                        o = sigmoidf_(s);
+                    }
+                    res[4 * at + val] = o;
+                }
+            }
+            __syncwarp();
+
+            // --- composite
+            uint32_t base = 0;
+            for (uint32_t r = 0; r < nr; ++r) {
+                const uint32_t mask = rounds[r];
+                const uint32_t at = base + __popc(mask & lt_mask);
+                base += __popc(mask);
+                if (!((mask >> lane) & 1u)) continue;
+                if (stopped) {
+                    if (ADJ) ent[at].x = 0xffffffffu;
+                    continue;
+                }
+                const float4 f = reinterpret_cast<const float4 *>(res)[at];
+                const float e = fabsf(f.x);
+                const float w = W.T * (1.0f - e);
+                W.C0 = fmaf(w, f.y, W.C0);
+                W.C1 = fmaf(w, f.z, W.C1);
+                W.C2 = fmaf(w, f.w, W.C2);
+                W.T *= e;
+                if (ADJ) {
+                    const float delta = __uint_as_float(ent[at].y);
+                    const float gs = delta * (g0 * (W.T * f.y - (Cf0 - W.C0)) + g1 * (W.T * f.z - (Cf1 - W.C1)) +
+                                              g2 * (W.T * f.w - (Cf2 - W.C2)));
+                    reinterpret_cast<float4 *>(res)[at] =
+                        make_float4(__float_as_int(f.x) < 0 ? gs : 0.0f, g0 * w * f.y * (1.0f - f.y),
+                                    g1 * w * f.z * (1.0f - f.z), g2 * w * f.w * (1.0f - f.w));
+                }
+                if (DBG) {
+                    const uint32_t leaf = ent[at].x;
+                    if (p.flags & FPO_FLAG_RECORD_VISITS) {
+                        if (W.n_visits < p.visit_cap)
+                            p.visit_log[(size_t)ray * p.visit_cap + W.n_visits] = p.perm[leaf];
+                        else
+                            atomicOr(p.status, STATUS_VISIT_OVERFLOW);
+                    }
+                    if (p.flags & FPO_FLAG_MARK_LEAVES) p.leaf_mark[p.perm[leaf]] = 1;
+                }
+                ++W.n_visits;
+                if (W.T < p.stop_T) {
+                    stopped = true;
+                    walking = false;
+                    W.steps = ent[at].w;  // the steps up to the stop, not those walked ahead
+                }
+            }
+            __syncwarp();
+
+            // --- scatter
+            if (ADJ) {
+                for (uint32_t v = lane; v < n; v += 32) {  // leaf -> row of the gradient
+                    if (ent[v].x == 0xffffffffu) continue;
+                    const uint32_t id = p.perm[ent[v].x];
+                    ent[v].x = id;
+                    if (q.leaf_mark) q.leaf_mark[id] = 1;
+                }
+                __syncwarp();
+#pragma unroll 2
+                for (uint32_t v = 0; v < n; ++v) {
+                    const uint4 en = ent[v];
+                    if (en.x == 0xffffffffu) continue;
+                    const float *w = wt + en.z * S::NWP;
+                    float *row = q.dL_dcoeffs + (size_t)en.x * S::NC;
+#pragma unroll
+                    for (int r = 0; r < (S::NC + 63) / 64; ++r) {
+                        const int el = 64 * r + 2 * lane;
+                        auto gval = [&](int k) {  // element k of the canonical row
+                            const int j = k - N1;
+                            return j < 0 ? res[4 * v] * w[k] : res[4 * v + 1 + j / S::NZ] * w[N1 + j % S::NZ];
+                        };
+                        if (el < S::NC) atomicAdd(reinterpret_cast<float2 *>(row + el), make_float2(gval(el), gval(el + 1)));
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        if (active && !walking) {
+            if (capped && !stopped) atomicOr(p.status, STATUS_TRAVERSAL_LIMIT);
+            if (!ADJ) {
+                write_result(p, W, DBG);
+                if (DBG && (p.flags & FPO_FLAG_STATS)) {
+                    atomicAdd(p.stats, (unsigned long long)W.steps + 1ull);
+                    atomicAdd(p.stats + 1, (unsigned long long)W.n_visits);
+                    atomicAdd(p.stats + 2, 1ull);
+                }
+            }
+            active = false;
+        }
+        __syncwarp();  // the next rays overwrite the weights and stacks
+    }
+    finish_tiles(p, lane);
+}
+
+// Rays per warp and list length.  Few rays: fewer of them per warp, so that
+// every SM gets several warps (a warp's time is that of its longest ray
+// either way, and the shading lanes are all busy for any R).
+static void fused_shape(uint32_t tiles32, int sm_count, int *rays, int *cap)
+{
+    const uint64_t n = (uint64_t)tiles32 * 32;
+    int r = 32;
+    while (r > FPO_FUSED_MIN_RAYS && n < (uint64_t)sm_count * FPO_FUSED_WARPS_PER_SM * r) r >>= 1;
+    *rays = r;
+    *cap = r * FPO_FUSED_LIST < 64 ? 64 : r * FPO_FUSED_LIST;
+}
+
+template <int N1, int N2, bool ADJ, bool DBG>
+static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
+{
+    TraverseParams &p = q.tp;
+    fused_shape(p.n_tiles, sm_count, &p.rays_per_warp, &p.list_cap);
+    const int threads = 32 * FU_WARPS;
+    const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, p.depth, FusedSize<N1, N2>::NWP);
+    auto k = fused_kernel<N1, N2, ADJ, DBG>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return (int)e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
+    if (e != cudaSuccess) return (int)e;
+    if (per_sm < 1) per_sm = 1;
+    uint64_t blocks = (uint64_t)sm_count * per_sm;
+    const uint64_t need = ((uint64_t)p.n_tiles * 32u / (uint32_t)p.rays_per_warp + FU_WARPS - 1) / FU_WARPS;
+    if (need < blocks) blocks = need ? need : 1;
+    k<<<(unsigned)blocks, threads, smem, s>>>(q);
+    return (int)cudaGetLastError();
+}
+
+// Compile-time Fourier sizes (the settings of Tab. 3).
+template <bool ADJ, bool DBG>
+static int launch_fused(const BackwardParams &q, int sm_count, cudaStream_t s)
+{
+    const int n1 = q.tp.n1, n2 = q.tp.n2;
+    if (n1 == 31 && n2 == 5) return launch_fused_t<31, 5, ADJ, DBG>(q, sm_count, s);
+    if (n1 == 11 && n2 == 5) return launch_fused_t<11, 5, ADJ, DBG>(q, sm_count, s);
+    if (n1 == 21 && n2 == 5) return launch_fused_t<21, 5, ADJ, DBG>(q, sm_count, s);
+    if (n1 == 31 && n2 == 11) return launch_fused_t<31, 11, ADJ, DBG>(q, sm_count, s);
     return -1;
 }
 
@@ -1407,207 +1646,11 @@ int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int 
 {
     cudaStream_t s = (cudaStream_t)stream;
     if (materialised)
-        return p.half_table ? launch_sched<TM_TABLE_F16, 0, 0>(p, debug, sm_count, s)
-                            : launch_sched<TM_TABLE_F32, 0, 0>(p, debug, sm_count, s);
-    return launch_fused(p, debug, sm_count, s);
-}
-
-
-// ---------------------------------------------------------------------------
-// Adjoint of the render (Sec. 4.3: back-propagation through the IDFT).
-//
-// Each ray is replayed front to back with the fused per-visit IDFT (the same
-// stepping and arithmetic as the fused forward, so the same segments and the
-// same early stop), recomputing the transmittance instead of storing
-// samples.  With w_j = T_j alpha_j and C the forward colour (which includes
-// T_end bg), S_j = C - sum_{k<=j} w_k c_k is the colour behind segment j and
-//   dL/dsigma_j = delta_j sum_c g_c (T_{j+1} c_jc - S_jc),
-//   dL/du_jc    = g_c w_j c_jc (1 - c_jc),   u = sum_k z_ck Y_k,
-//   dL/dk_sigma_i += dL/dsigma_j [sigma_raw > 0] IDFT_i(t),
-//   dL/dk_cki     += dL/du_jc Y_k IDFT_i(t),
-// accumulated with 16-byte vector atomics (one 8-byte atomic at an unaligned
-// end) into the canonical gradient row of the leaf's upload id.
-
-template <int N1, int N2>
-__device__ void backward_ray(const BackwardParams &q, const float *bsrc, int bstride,
-                             const uint32_t *__restrict__ s_nodes, uint32_t *s_stack, int stride,
-                             RayState &R)
-{
-    constexpr int NC = N1 + 27 * N2;
-    static_assert(NC % 2 == 0, "gradient rows are written in pairs");
-    const TraverseParams &p = q.tp;
-    const int D = p.depth, G = 1 << D;
-    const float g0 = q.dL_drgb[3 * (size_t)R.ray], g1 = q.dL_drgb[3 * (size_t)R.ray + 1],
-                g2 = q.dL_drgb[3 * (size_t)R.ray + 2];
-    const float Cf0 = q.out_rgb[3 * (size_t)R.ray], Cf1 = q.out_rgb[3 * (size_t)R.ray + 1],
-                Cf2 = q.out_rgb[3 * (size_t)R.ray + 2];
-    float P0 = 0.0f, P1 = 0.0f, P2 = 0.0f;  // sum_{k<=j} w_k c_k
-    float bz[N2];  // the density basis stays in shared memory (bsrc)
-#pragma unroll
-    for (int i = 0; i < N2; ++i) bz[i] = bsrc[i * bstride];
-    Cube cb = locate(p, s_nodes, s_stack, stride, R.P, R.lvl_start);
-    for (;;) {
-        int m, lo[3], csz;
-        const float tx = cube_exit(R, D, cb.lvl, m, lo, csz);
-        // as in the forward: locate the next cube and prefetch its records
-        // before this one is processed
-        int Pn[3];
-        const bool inside = next_cell(R, G, m, lo, csz, tx, Pn);
-        Cube nx;
-        nx.kind = ROOT_EMPTY;
-        if (FPO_PREFETCH && inside) {
-            const uint32_t diff = (uint32_t)((R.P[0] ^ Pn[0]) | (R.P[1] ^ Pn[1]) | (R.P[2] ^ Pn[2]));
-            nx = locate(p, s_nodes, s_stack, stride, Pn, D - 1 - (31 - __clz(diff)));
-            if (nx.kind == ROOT_LEAF) prefetch_records(p, nx.leaf, N1, N2);
-        }
-        if (cb.kind == ROOT_LEAF && tx > R.t) {
-            const float delta = tx - R.t;
-            const float *sr = reinterpret_cast<const float *>(p.sig + (size_t)cb.leaf * p.sig_stride4);
-            const float *zr = p.zc + (size_t)cb.leaf * p.z_stride;
-            constexpr int VW = (FPO_LDG256 && fused_ldg256(N1, N2)) ? 8 : 4;  // floats per load
-            float sraw = 0.0f;
-#pragma unroll
-            for (int k4 = 0; k4 < (N1 + VW - 1) / VW; ++k4) {
-                float wv[VW];
-                load_vec<VW>(sr + VW * k4, wv);
-#pragma unroll
-                for (int j = 0; j < VW; ++j)
-                    if (VW * k4 + j < N1) sraw = fmaf(wv[j], bsrc[(VW * k4 + j) * bstride], sraw);
-            }
-            const float sigma = fmaxf(sraw, 0.0f);
-            float z[27];
-#pragma unroll
-            for (int k = 0; k < 27; ++k) z[k] = 0.0f;
-#pragma unroll
-            for (int k4 = 0; k4 < (27 * N2 + VW - 1) / VW; ++k4) {
-                float wv[VW];
-                load_vec<VW>(zr + VW * k4, wv);
-#pragma unroll
-                for (int j = 0; j < VW; ++j) {
-                    const int e = VW * k4 + j;
-                    if (e < 27 * N2) z[e / N2] = fmaf(wv[j], bz[e % N2], z[e / N2]);
-                }
-            }
-            float col[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                float u = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) u = fmaf(z[9 * c + k], R.Y[k], u);
-                col[c] = sigmoidf_(u);
-            }
-            const float e = __expf(-sigma * delta);
-            const float w = R.T * (1.0f - e);
-            const float Tn = R.T * e;
-            P0 = fmaf(w, col[0], P0);
-            P1 = fmaf(w, col[1], P1);
-            P2 = fmaf(w, col[2], P2);
-            const float gs = delta * (g0 * (Tn * col[0] - (Cf0 - P0)) + g1 * (Tn * col[1] - (Cf1 - P1)) +
-                                      g2 * (Tn * col[2] - (Cf2 - P2)));
-            const float dsr = sraw > 0.0f ? gs : 0.0f;
-            const float gu[3] = {g0 * w * col[0] * (1.0f - col[0]), g1 * w * col[1] * (1.0f - col[1]),
-                                 g2 * w * col[2] * (1.0f - col[2])};
-            const uint32_t id = p.perm[cb.leaf];
-            float *row = q.dL_dcoeffs + (size_t)id * NC;
-            if (q.leaf_mark) q.leaf_mark[id] = 1;
-            // dL/dk for element el of the row (compile-time el)
-            auto gval = [&](int el) -> float {
-                if (el < N1) return dsr * bsrc[el * bstride];
-                const int j = el - N1, c = j / (9 * N2), k = (j / N2) % 9, i = j % N2;
-                return gu[c] * R.Y[k] * bz[i];
-            };
-            // 16-byte vector atomics; a row that starts 8 bytes past a 16-byte
-            // boundary (NC = 2 mod 4, odd id) opens with one 8-byte atomic
-            if (NC % 4 == 0 || (id & 1u) == 0u) {
-#pragma unroll
-                for (int e4 = 0; e4 < NC / 4; ++e4)
-                    atomicAdd(reinterpret_cast<float4 *>(row) + e4,
-                              make_float4(gval(4 * e4), gval(4 * e4 + 1), gval(4 * e4 + 2), gval(4 * e4 + 3)));
-                if constexpr (NC % 4 == 2)
-                    atomicAdd(reinterpret_cast<float2 *>(row + NC - 2), make_float2(gval(NC - 2), gval(NC - 1)));
-            } else {
-                atomicAdd(reinterpret_cast<float2 *>(row), make_float2(gval(0), gval(1)));
-#pragma unroll
-                for (int e4 = 0; e4 < NC / 4; ++e4)
-                    atomicAdd(reinterpret_cast<float4 *>(row + 2) + e4,
-                              make_float4(gval(2 + 4 * e4), gval(3 + 4 * e4), gval(4 + 4 * e4), gval(5 + 4 * e4)));
-            }
-            R.T = Tn;
-            if (R.T < p.stop_T) return;
-        }
-        if (!inside) return;
-        move_to(R, D, Pn, tx);
-        if (step_cap(p, R)) return;
-        if (FPO_PREFETCH)
-            cb = nx;
-        else
-            cb = locate(p, s_nodes, s_stack, stride, R.P, R.lvl_start);
-    }
-}
-
-template <int N1, int N2>
-__global__ void __maxnreg__(128) backward_kernel(const __grid_constant__ BackwardParams q)
-{
-    extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ FrameShared fs;
-    const TraverseParams &p = q.tp;
-    const int stride = blockDim.x;
-    uint32_t *s_nodes = smem;
-    uint32_t *s_stack = smem + p.n_smem_nodes * 8;
-    float *s_bray = reinterpret_cast<float *>(s_stack + STACK_LEVELS * stride);
-    const bool prt = p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
-    frame_prologue(p, s_nodes, fs);
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    uint32_t *my_stack = s_stack + threadIdx.x;
-    float *my_b = s_bray + threadIdx.x;
-    const float *bsrc = prt ? my_b : fs.b;
-    const int bstride = prt ? stride : 1;
-    for (;;) {
-        uint32_t tile = 0;
-        if (lane == 0) tile = atomicAdd(p.tiles, 1u);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
-        if (tile >= p.n_tiles) break;
-        uint32_t ray;
-        int px = 0, py = 0;
-        if (!tile_ray(p, tile, (uint32_t)lane, ray, px, py)) continue;
-        RayState R;
-        if (!init_ray_geom(p, prt, my_b, stride, my_stack, R, ray, px, py)) continue;
-        backward_ray<N1, N2>(q, bsrc, bstride, s_nodes, my_stack, stride, R);
-    }
-    if (lane == 0) {
-        __threadfence();
-        const uint32_t done = atomicAdd(p.tiles + 1, 1u);
-        if (done == gridDim.x * (blockDim.x / 32) - 1) {
-            atomicExch(p.tiles, 0u);
-            atomicExch(p.tiles + 1, 0u);
-        }
-    }
-}
-
-template <int N1, int N2>
-static int launch_b(const BackwardParams &q, int sm_count, cudaStream_t s)
-{
-    const TraverseParams &p = q.tp;
-    const bool prt = p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
-    const int threads = 256;
-    const int smem = traverse_smem_bytes(p.n_smem_nodes, prt, threads);
-    auto k = backward_kernel<N1, N2>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 p.carveout > 0 ? p.carveout : (int)cudaSharedmemCarveoutDefault);
-    if (e != cudaSuccess) return (int)e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
-    if (e != cudaSuccess) return (int)e;
-    if (per_sm < 1) per_sm = 1;
-    if (p.max_ctas_per_sm > 0 && per_sm > p.max_ctas_per_sm) per_sm = p.max_ctas_per_sm;
-    uint64_t blocks = (uint64_t)sm_count * per_sm;
-    const uint64_t need = (p.n_tiles + (threads / 32) - 1) / (threads / 32);
-    if (need < blocks) blocks = need ? need : 1;
-    k<<<(unsigned)blocks, threads, smem, s>>>(q);
-    return (int)cudaGetLastError();
+        return p.half_table ? launch_sched<TM_TABLE_F16>(p, debug, sm_count, s)
+                            : launch_sched<TM_TABLE_F32>(p, debug, sm_count, s);
+    BackwardParams q{};
+    q.tp = p;
+    return debug ? launch_fused<false, true>(q, sm_count, s) : launch_fused<false, false>(q, sm_count, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1704,7 +1747,7 @@ __device__ __forceinline__ double segment64(const Ray64 &r, const int lo[3], int
 // pass 1 accumulates the gradients with C from pass 0.
 template <int N1, int N2>
 __device__ void replay_fp64(const BackwardParams &q, RayState R, const Ray64 &r, int pass, double C[3],
-                            const uint32_t *__restrict__ s_nodes, uint32_t *s_stack, int stride)
+                            uint32_t *s_stack, int stride)
 {
     constexpr int NC = N1 + 27 * N2;
     const TraverseParams &p = q.tp;
@@ -1714,7 +1757,7 @@ __device__ void replay_fp64(const BackwardParams &q, RayState R, const Ray64 &r,
         for (int c = 0; c < 3; ++c) g[c] = (double)q.dL_drgb[3 * (size_t)R.ray + c];
     double T = 1.0, P[3] = {0.0, 0.0, 0.0};
     for (;;) {
-        const Cube cb = locate(p, s_nodes, s_stack, stride, R.P, R.lvl_start);
+        const Cube cb = locate(p, s_stack, stride, R.P, R.lvl_start);
         int m, lo[3], csz;
         const float tx = cube_exit(R, D, cb.lvl, m, lo, csz);
         if (cb.kind == ROOT_LEAF && tx > R.t) {
@@ -1766,16 +1809,10 @@ template <int N1, int N2>
 __global__ void __launch_bounds__(128) backward_fp64_kernel(const __grid_constant__ BackwardParams q)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ FrameShared fs;
     const TraverseParams &p = q.tp;
     const int stride = blockDim.x;
-    uint32_t *s_nodes = smem;
-    uint32_t *s_stack = smem + p.n_smem_nodes * 8;
-    float *s_bray = reinterpret_cast<float *>(s_stack + STACK_LEVELS * stride);
-    frame_prologue(p, s_nodes, fs);
-    __syncthreads();
     const int lane = threadIdx.x & 31;
-    uint32_t *my_stack = s_stack + threadIdx.x;
+    uint32_t *my_stack = smem + threadIdx.x;
     for (;;) {
         uint32_t tile = 0;
         if (lane == 0) tile = atomicAdd(p.tiles, 1u);
@@ -1786,21 +1823,14 @@ __global__ void __launch_bounds__(128) backward_fp64_kernel(const __grid_constan
         if (!tile_ray(p, tile, (uint32_t)lane, ray, px, py)) continue;
         RayState R0;
         // the FP32 ray as the forward sets it up (it decides the stepping)
-        if (!init_ray_geom(p, false, s_bray + threadIdx.x, stride, my_stack, R0, ray, px, py)) continue;
+        if (!init_ray_geom(p, my_stack, R0, ray, px, py)) continue;
         Ray64 r;
         ray64_setup(p, ray, px, py, r);
         double C[3];
-        replay_fp64<N1, N2>(q, R0, r, 0, C, s_nodes, my_stack, stride);
-        replay_fp64<N1, N2>(q, R0, r, 1, C, s_nodes, my_stack, stride);
+        replay_fp64<N1, N2>(q, R0, r, 0, C, my_stack, stride);
+        replay_fp64<N1, N2>(q, R0, r, 1, C, my_stack, stride);
     }
-    if (lane == 0) {
-        __threadfence();
-        const uint32_t done = atomicAdd(p.tiles + 1, 1u);
-        if (done == gridDim.x * (blockDim.x / 32) - 1) {
-            atomicExch(p.tiles, 0u);
-            atomicExch(p.tiles + 1, 0u);
-        }
-    }
+    finish_tiles(p, lane);
 }
 
 template <int N1, int N2>
@@ -1808,7 +1838,7 @@ static int launch_b64(const BackwardParams &q, int sm_count, cudaStream_t s)
 {
     const TraverseParams &p = q.tp;
     const int threads = 128;
-    const int smem = traverse_smem_bytes(p.n_smem_nodes, false, threads);
+    const int smem = traverse_smem_bytes(threads);
     auto k = backward_fp64_kernel<N1, N2>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return (int)e;
@@ -1822,12 +1852,12 @@ static int launch_b64(const BackwardParams &q, int sm_count, cudaStream_t s)
 int launch_backward(const BackwardParams &q, int sm_count, void *stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
-    const TraverseParams &p = q.tp;
-    const bool fp64 = q.dL_dcoeffs64 != nullptr;
-    if (p.n1 == 31 && p.n2 == 5) return fp64 ? launch_b64<31, 5>(q, sm_count, s) : launch_b<31, 5>(q, sm_count, s);
-    if (p.n1 == 11 && p.n2 == 5) return fp64 ? launch_b64<11, 5>(q, sm_count, s) : launch_b<11, 5>(q, sm_count, s);
-    if (p.n1 == 21 && p.n2 == 5) return fp64 ? launch_b64<21, 5>(q, sm_count, s) : launch_b<21, 5>(q, sm_count, s);
-    if (p.n1 == 31 && p.n2 == 11) return fp64 ? launch_b64<31, 11>(q, sm_count, s) : launch_b<31, 11>(q, sm_count, s);
+    if (q.dL_dcoeffs64 == nullptr) return launch_fused<true, false>(q, sm_count, s);
+    const int n1 = q.tp.n1, n2 = q.tp.n2;
+    if (n1 == 31 && n2 == 5) return launch_b64<31, 5>(q, sm_count, s);
+    if (n1 == 11 && n2 == 5) return launch_b64<11, 5>(q, sm_count, s);
+    if (n1 == 21 && n2 == 5) return launch_b64<21, 5>(q, sm_count, s);
+    if (n1 == 31 && n2 == 11) return launch_b64<31, 11>(q, sm_count, s);
     return -1;
 }
 
