@@ -85,7 +85,8 @@ typedef struct {
      * (128 or 256); the number of idle lanes at which a warp refills them
      * with new rays (1..32; 32 refills only a fully idle warp); the number of
      * steps a lane takes between two such checks (default: to the end of its
-     * ray). */
+     * ray).  They apply to the table mode; the fused mode schedules its rays
+     * itself. */
     int32_t traverse_threads;
     int32_t refill_min;
     int32_t inner_steps;

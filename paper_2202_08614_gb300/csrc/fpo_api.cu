@@ -112,6 +112,7 @@ struct fpo_ctx {
     uint32_t max_depth = 0;
     double aabb_min[3] = {0, 0, 0}, aabb_size = 1.0;
     uint32_t *d_nodes = nullptr;
+    uint32_t *d_top = nullptr, *d_bricks = nullptr;  // brick index, or NULL
     uint32_t *d_perm = nullptr;
     void *d_sig = nullptr;    // density records (storage precision)
     void *d_z = nullptr;      // SH records (storage precision)
@@ -136,6 +137,8 @@ struct fpo_ctx {
     void free_tree()
     {
         dfree(d_nodes);
+        dfree(d_top);
+        dfree(d_bricks);
         dfree(d_perm);
         dfree(d_sig);
         dfree(d_z);
@@ -313,6 +316,8 @@ int fpo_upload_tree(fpo_ctx *ctx, const fpo_tree_desc *tree)
         return FPO_OK;
     };
     if ((st = up((void **)&ctx->d_nodes, pk.nodes.data(), pk.nodes.size() * 4, "nodes")) ||
+        (st = up((void **)&ctx->d_top, pk.top.data(), pk.top.size() * 4, "top blocks")) ||
+        (st = up((void **)&ctx->d_bricks, pk.bricks.data(), pk.bricks.size() * 4, "bricks")) ||
         (st = up((void **)&ctx->d_perm, pk.perm.data(), pk.perm.size() * 4, "perm")) ||
         (st = up((void **)&ctx->d_sig, sig.data(), sig.size(), "sigma records")) ||
         (st = up((void **)&ctx->d_z, zc.data(), zc.size(), "SH records")) ||
@@ -474,6 +479,9 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
     p.fr.rt = rays->t_per_ray;
     frame_consts(p.fr, ctx->cfg.n1 > ctx->cfg.n2 ? ctx->cfg.n1 : ctx->cfg.n2, p.fc);
     p.nodes = ctx->d_nodes;
+    p.top = reinterpret_cast<const uint4 *>(ctx->d_top);
+    p.bricks = reinterpret_cast<const uint4 *>(ctx->d_bricks);
+    p.top_bits = ctx->depth - 4;
     p.root_kind = ctx->root_kind;
     p.depth = ctx->depth;
     p.grid_scale64 = (double)(1u << ctx->depth) / ctx->aabb_size;
@@ -713,7 +721,7 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             mshape = materialise_pipeline_shape(ctx->cfg.storage, ctx->cfg.n1, ctx->cfg.n2, PIPE_MAT_SMEM_BUDGET);
             if (FPO_PIPE_MAT_CTAS > 0) mshape.ctas_per_sm = FPO_PIPE_MAT_CTAS;
         }
-        const long need = (long)PIPE_TRAV_CTAS * (traverse_smem_bytes(PIPE_TRAV_THREADS) + PIPE_STATIC_SMEM + reserved) +
+        const long need = (long)PIPE_TRAV_CTAS * (traverse_smem_bytes(ctx->d_top != nullptr, PIPE_TRAV_THREADS) + PIPE_STATIC_SMEM + reserved) +
                           (long)mshape.ctas_per_sm * (mshape.smem_per_cta + PIPE_STATIC_SMEM + reserved);
         // The driver rounds a carveout request up to one of the SM's shared-
         // memory configurations: ask for the smallest one that holds `need`.

@@ -25,6 +25,20 @@ constexpr uint32_t LEAF_BIT = 0x80000000u;
 constexpr uint32_t ROOT_EMPTY = 0, ROOT_LEAF = 1, ROOT_NODE = 2;
 constexpr int MAX_DEPTH = 12;
 
+// Brick index, for trees whose leaves are all finest cells (every union octree
+// of fully divided frames), 4 <= depth <= 11: the finest grid as 4x4x4 bricks,
+// grouped 4x4x4 again into 16^3-cell blocks.  Bit x + 4y + 16z of a 64-bit mask
+// stands for child (x, y, z).  Both records are 16 bytes:
+//   top[block], a dense grid of blocks, x fastest: {mask of its non-empty
+//     bricks (low, high), index of the first of them, side of the octree's
+//     largest empty cube around it if the mask is 0};
+//   bricks[i], in the order of the mask bits: {mask of its leaves (low, high),
+//     first leaf, 0}.
+// A brick's leaves are numbered in the order of its mask bits.  The cubes found
+// in it (leaf, empty 1, 2, 4, 8, 16, ...) are the octree's.  The 3.5M-leaf body
+// takes 0.5 + 1 MB, its node array 17 MB.
+constexpr int BRICK_MIN_DEPTH = 4, BRICK_MAX_DEPTH = 11;
+
 // Leaf records.  FP32 storage: a density record of SIG_STRIDE(n1) floats
 // (n1 rounded up to a multiple of 4, 128 bytes for n1 = 31) and an SH record
 // of Z_STRIDE(n2) floats (27 n2 rounded up to a multiple of 4), both arrays
@@ -83,6 +97,7 @@ struct PackedTree {
     int depth = 0;                 // grid depth D: finest cell = 1 / 2^D of the cube
     std::vector<uint32_t> nodes;   // [n_nodes * 8]
     std::vector<uint32_t> perm;    // internal leaf index -> upload index
+    std::vector<uint32_t> top, bricks;  // brick index, 4 words per entry (empty: none)
 };
 
 // Validates a tree description (and packs it when `out` is non-null).
@@ -119,6 +134,8 @@ struct TraverseParams {
     FrameConsts fc;
     // tree
     const uint32_t *nodes;
+    const uint4 *top, *bricks; // brick index (nullptr: leaves at several depths, or a very shallow or deep tree)
+    int top_bits;              // log2 of the top grid's cells a side
     uint32_t root_kind;
     int depth;
     float grid_scale;         // 2^D / aabb_size
@@ -305,7 +322,7 @@ int launch_set_coeffs(const float *src, const uint32_t *perm, float *sig, float 
 int launch_leaf_adam(const LeafAdamParams &p, int sm_count, void *stream);
 int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int sm_count,
                     void *stream);
-int traverse_smem_bytes(int threads);
+int traverse_smem_bytes(bool brick, int threads);
 bool fused_supported(int n1, int n2);
 
 }  // namespace fpo

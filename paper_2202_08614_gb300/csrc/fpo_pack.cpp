@@ -31,6 +31,73 @@ std::string fmt(const char *f, long long a, long long b = 0, long long c = 0)
     return buf;
 }
 
+// The brick index of a tree whose leaves are all at depth D.  The leaves come
+// in Morton order (breadth-first order is that, here): those of a brick are
+// contiguous, and are renumbered into the order of the brick's mask bits, in
+// the permutation and in the nodes.
+void build_bricks(const fpo_tree_desc *tree, int D, PackedTree *out)
+{
+    const uint32_t n = (uint32_t)out->perm.size();
+    const int tb = D - 4;
+    const size_t T = (size_t)1 << tb;
+    out->top.assign(T * T * T * 4, 0u);
+    std::vector<uint32_t> perm(n), renum(n);
+    struct Brick { uint32_t m[2], base; };
+    Brick found[64];  // the bricks of the current block, by mask bit
+    auto set = [](uint32_t m[2], uint32_t b) { m[b >> 5] |= 1u << (b & 31u); };
+    auto has = [](const uint32_t m[2], uint32_t b) { return (m[b >> 5] >> (b & 31u)) & 1u; };
+    auto cell = [&](uint32_t i, int k) { return tree->leaf_xyz[3 * (size_t)out->perm[i] + k]; };
+    uint32_t i = 0;
+    while (i < n) {  // a block of 16^3 cells
+        const uint32_t bx = cell(i, 0) >> 4, by = cell(i, 1) >> 4, bz = cell(i, 2) >> 4;
+        uint32_t bmask[2] = {0, 0};
+        while (i < n && cell(i, 0) >> 4 == bx && cell(i, 1) >> 4 == by && cell(i, 2) >> 4 == bz) {  // a brick
+            const uint32_t x = cell(i, 0) >> 2, y = cell(i, 1) >> 2, z = cell(i, 2) >> 2;
+            Brick b = {{0, 0}, i};
+            uint32_t order[64];
+            for (; i < n && cell(i, 0) >> 2 == x && cell(i, 1) >> 2 == y && cell(i, 2) >> 2 == z; ++i) {
+                const uint32_t bit = (cell(i, 0) & 3u) | ((cell(i, 1) & 3u) << 2) | ((cell(i, 2) & 3u) << 4);
+                set(b.m, bit);
+                order[bit] = i;
+            }
+            uint32_t at = b.base;
+            for (uint32_t bit = 0; bit < 64; ++bit)
+                if (has(b.m, bit)) {
+                    renum[order[bit]] = at;
+                    perm[at++] = out->perm[order[bit]];
+                }
+            const uint32_t j = (x & 3u) | ((y & 3u) << 2) | ((z & 3u) << 4);
+            set(bmask, j);
+            found[j] = b;
+        }
+        uint32_t *t = &out->top[(((size_t)bz * T + by) * T + bx) * 4];
+        t[0] = bmask[0];
+        t[1] = bmask[1];
+        t[2] = (uint32_t)(out->bricks.size() / 4);
+        for (uint32_t j = 0; j < 64; ++j)
+            if (has(bmask, j)) out->bricks.insert(out->bricks.end(), {found[j].m[0], found[j].m[1], found[j].base, 0u});
+    }
+    // empty blocks: the side of the octree's empty cube that holds them
+    for (size_t c = 0; c < T * T * T; ++c) {
+        uint32_t *t = &out->top[c * 4];
+        if (t[0] | t[1]) continue;
+        const uint32_t x = (uint32_t)(c % T), y = (uint32_t)(c / T % T), z = (uint32_t)(c / T / T);
+        uint32_t node = 0;
+        for (int l = 0; l < tb; ++l) {
+            const int sh = tb - 1 - l;
+            const uint32_t o = ((x >> sh) & 1u) | (((y >> sh) & 1u) << 1) | (((z >> sh) & 1u) << 2);
+            node = out->nodes[(size_t)node * 8 + o];
+            if (node == 0) {
+                t[3] = 1u << (D - l - 1);
+                break;
+            }
+        }
+    }
+    for (uint32_t &s : out->nodes)
+        if (s & LEAF_BIT) s = LEAF_BIT | renum[s & ~LEAF_BIT];
+    out->perm.swap(perm);
+}
+
 }  // namespace
 
 int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out, std::string *err)
@@ -147,6 +214,9 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
             out->nodes[qi * 8 + c] = slot;
         }
     }
+    bool uniform = dmax >= BRICK_MIN_DEPTH && dmax <= BRICK_MAX_DEPTH;
+    for (uint32_t j = 0; j < n && uniform; ++j) uniform = tree->leaf_depth[j] == dmax;
+    if (uniform) build_bricks(tree, dmax, out);
     return FPO_OK;
 }
 
