@@ -440,41 +440,53 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
 // loss against target coefficients (plus an optional extra dL/dy), and the
 // back-propagation to every weight, bias and latent, with BF16 operands (A
 // and B of each MMA both BF16; FP32's exponent range, so no loss scaling)
-// and FP32 accumulation in TMEM.  One warpgroup per CTA and one CTA per SM
-// (all 512 TMEM columns); thread t owns row t of a 128-leaf tile and TMEM
-// lane t.  Per tile, nine GEMMs (M = 128, no-swizzle K-major operands):
-//   Z1 = [X 1] W1'^T,  Z2 = [H1 1] W2'^T,  Y = [H2 1] W3'^T       (forward)
+// and FP32 accumulation in TMEM.  One 256-thread CTA per SM (all 512 TMEM
+// columns); threads t and t + 128 own row t of a 128-leaf tile, TMEM lane t,
+// and half of each layer's columns.  Per tile, nine GEMMs (M = 128):
+//   Z1 = X W1^T,  Z2 = H1 W2^T,  Y = H2 W3^T                       (forward)
 //   dH2 = dY W3,  dH1 = d2 W2,  dX = d1 W1                        (data)
-//   G3 += [H2^T; 1] dY,  G2 += [H1^T; 1] d2,  G1 += [X^T; 1] d1    (weights)
-// H = relu(Z) in BF16, d2 = dH2 [Z2 > 0], d1 = dH1 [Z1 > 0], dY = 2 cw (Y -
-// target) + extra.  The weight gradients accumulate in TMEM over all of the
-// CTA's tiles, transposed (lane = input feature, column = output feature);
-// the ones row of each transposed activation makes lane 64 (32 for layer 1)
-// the bias gradient.  The transposed operands (activations and gradients
-// with the tile's rows as K) are written by the epilogues next to the
-// row-major ones.  The M = 128 A operands of the weight GEMMs hold only
-// 40 or 72 meaningful rows; the rest of each descriptor's extent reads
+//   G3 += [H2 1]^T dY,  G2 += [H1 1]^T d2,  G1 += [X 1]^T d1       (weights)
+// H = relu(Z + b) in BF16 (the biases are added in FP32), d2 = dH2 [Z2 > 0],
+// d1 = dH1 [Z1 > 0], dY = 2 cw (Y - target) + extra.  The weight gradients
+// accumulate in TMEM over all of the CTA's tiles, transposed (lane = input
+// feature, column = output feature); the ones column after each activation's
+// features makes lane 64 (32 for layer 1) the bias gradient.
+//
+// Every matrix is in shared memory once, row-major in 8 x 16-byte core
+// matrices: the GEMMs that sum over features read it K-major, those that sum
+// over the tile's rows (the weight gradients) or over output features (the
+// data gradients' weights) read the same core matrices MN-major through the
+// descriptor's transpose bits.  (Writing transposed copies from the
+// epilogues, 2 bytes at a time, took most of a tile's time, and left no
+// room for what follows.)  The target rows, gathered by leaf, arrive by
+// asynchronous copies, a row by contiguous 8-byte pieces, while the tile
+// before is back-propagated.  The M = 128 A operands of the weight GEMMs hold
+// 40 or 72 meaningful features; the rest of each descriptor's extent reads
 // whatever lies after them in shared memory, which lands only in TMEM lanes
 // that are never read.
+// What bounds it: the chain of six dependent MMA rounds with their epilogues.
 namespace {
 
-constexpr int TG_K1 = 48, TG_K2 = 80, TG_NC = 176, TG_KR = 128;
-constexpr int TGO_W1 = 0;                          // [64][48]   W1 | b1 (B of Z1)
-constexpr int TGO_W2 = TGO_W1 + 64 * TG_K1 * 2;    // [64][80]   W2 | b2 (B of Z2)
-constexpr int TGO_W3 = TGO_W2 + 64 * TG_K2 * 2;    // [176][80]  W3 | b3 (B of Y)
-constexpr int TGO_W3T = TGO_W3 + TG_NC * TG_K2 * 2;  // [64][176] W3^T (B of dH2)
-constexpr int TGO_W2T = TGO_W3T + 64 * TG_NC * 2;  // [64][64]   W2^T (B of dH1)
-constexpr int TGO_W1T = TGO_W2T + 64 * 64 * 2;     // [32][64]   W1^T (B of dX)
-constexpr int TGO_XT = TGO_W1T + 32 * 64 * 2;      // [40][128]  [X^T; 1] (A of G1)
-constexpr int TGO_H1T = TGO_XT + 40 * TG_KR * 2;   // [72][128]  [H1^T; 1] (A of G2)
-constexpr int TGO_H2T = TGO_H1T + 72 * TG_KR * 2;  // [72][128]  [H2^T; 1] (A of G3)
-constexpr int TGO_A = TGO_H2T + 72 * TG_KR * 2;    // the tile's A operand: [X 1], [H1 1], [H2 1], dY, d2, d1
-constexpr int TGO_B = TGO_A + 128 * TG_NC * 2;     // the weight GEMMs' B operand: dY^T, d2^T, d1^T
-constexpr int TG_SMEM = TGO_B + TG_NC * TG_KR * 2;
-static_assert(TGO_XT + 128 * TG_KR * 2 <= TG_SMEM && TGO_H2T + 128 * TG_KR * 2 <= TG_SMEM,
-              "the weight GEMMs' A descriptors stay inside the CTA's shared memory");
+constexpr int TG_THREADS = 256, TG_NC = 176;
+constexpr int TG_KX = 40, TG_KH = 72;              // features and the ones column, in 8-wide chunks
+constexpr int TGO_W1 = 0;                          // [64][32]   W1
+constexpr int TGO_W2 = TGO_W1 + 64 * 32 * 2;       // [64][64]   W2
+constexpr int TGO_W3 = TGO_W2 + 64 * 64 * 2;       // [176][64]  W3
+constexpr int TGO_X = TGO_W3 + TG_NC * 64 * 2;     // [128][40]  [X 1]
+constexpr int TGO_H1 = TGO_X + 128 * TG_KX * 2;    // [128][72]  [H1 1]
+constexpr int TGO_H2 = TGO_H1 + 128 * TG_KH * 2;   // [128][72]  [H2 1]
+constexpr int TGO_DY = TGO_H2 + 128 * TG_KH * 2;   // [128][176] dY, then [128][64] d2, then d1
+constexpr int TGO_T = TGO_DY + 128 * TG_NC * 2;    // [128][stride] FP32 target rows
+constexpr int TG_TSTRIDE = TG_NC + 2;              // floats; target_stride(nc) at most
+constexpr int TGO_B = TGO_T + 128 * TG_TSTRIDE * 4;  // b1[64] b2[64] b3[176] cw[176]
+constexpr int TG_SMEM = TGO_B + (64 + 64 + 2 * TG_NC) * 4;
+static_assert(TG_SMEM <= 227 * 1024 - 1024, "one CTA per SM");
 // TMEM columns: per-tile scratch (Z1, Z2, Y, dH2, dH1, dX) and the weight gradients
 constexpr uint32_t TC_SCR = 0, TC_G3 = 192, TC_G2 = 384, TC_G1 = 448, TC_COLS = 512;
+
+// Row stride of the target tile: even (8-byte copies) and 2 mod 4, so that the
+// 8-byte reads of 16 consecutive rows hit 16 different bank pairs.
+__host__ __device__ constexpr int target_stride(int nc) { return nc + (6 - nc % 4) % 4; }
 
 struct DecoderGradTcParams {
     fpo_mlp w, g;
@@ -493,24 +505,36 @@ __device__ __forceinline__ uint32_t idesc_bf16(int M, int N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D[128 x N] (+)= A[128 x K] B[N x K]^T, BF16; acc0: accumulate from the first K slice on.
-__device__ __forceinline__ void gemm_bf16(uint32_t d_tmem, uint32_t a_saddr, uint32_t b_saddr, int K, int N,
-                                          uint32_t acc0)
+// An operand as the MMAs of one GEMM read it: start address, byte strides
+// between 8-element groups along K (per 16-wide MMA step: two groups) and
+// along M or N, and whether M or N is the contiguous direction.
+struct Operand {
+    uint32_t addr, k8, mn8;
+    bool mn_major;
+};
+// A row-major matrix in core matrices with `cols` columns: summed over its
+// columns (K-major), or over its rows (MN-major).
+__device__ __forceinline__ Operand over_cols(uint32_t addr, int cols) { return {addr, 128u, (uint32_t)cols * 16u, false}; }
+__device__ __forceinline__ Operand over_rows(uint32_t addr, int cols) { return {addr, (uint32_t)cols * 16u, 128u, true}; }
+
+// D[128 x N] (+)= A B^T over K, BF16; acc0: accumulate from the first K slice on.
+// No-swizzle descriptors: K-major, LBO = K group stride, SBO = row group stride;
+// MN-major, LBO = K group stride, SBO = M/N group stride.
+__device__ __forceinline__ void gemm_bf16(uint32_t d_tmem, Operand a, Operand b, int K, int N, uint32_t acc0)
 {
-    const uint32_t idesc = idesc_bf16(128, N);
-    const uint32_t sbo = (uint32_t)(K / 8) * 128u;
+    const uint32_t idesc = idesc_bf16(128, N) | (a.mn_major ? 1u << 15 : 0u) | (b.mn_major ? 1u << 16 : 0u);
 #pragma unroll 1
-    for (int s = 0; s < K / 16; ++s) {
-        const uint64_t a = smem_desc(a_saddr + 256u * s, 128u, sbo);
-        const uint64_t b = smem_desc(b_saddr + 256u * s, 128u, sbo);
-        mma_f16(d_tmem, a, b, idesc, s > 0 ? 1u : acc0);
-    }
+    for (int s = 0; s < K / 16; ++s)
+        mma_f16(d_tmem, smem_desc(a.addr + 2u * s * a.k8, a.k8, a.mn8), smem_desc(b.addr + 2u * s * b.k8, b.k8, b.mn8), idesc,
+                s > 0 ? 1u : acc0);
 }
 
-__device__ __forceinline__ void put1_bf(unsigned char *base, int row, int k, int K, float v)
+__device__ __forceinline__ void cp_async(void *dst, const void *src, bool pair)
 {
-    *reinterpret_cast<__nv_bfloat16 *>(base + core_off(row, k, K)) = __float2bfloat16_rn(v);
+    if (pair) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ptx::smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // 8 consecutive values of row `row` (K-chunk j) as BF16.
 __device__ __forceinline__ void put8_bf(unsigned char *base, int row, int j, int K, const float *v)
@@ -524,20 +548,13 @@ __device__ __forceinline__ void put8_bf(unsigned char *base, int row, int j, int
     *reinterpret_cast<uint4 *>(base + core_off(row, 8 * j, K)) = make_uint4(h[0], h[1], h[2], h[3]);
 }
 
-// K-chunk j of row `row` = {hi(b), lo(b), 0 x 6} in BF16 (hi + lo carries b
-// to about 16 bits), or {c, c, 0 x 6}: the constant columns of an A operand.
-__device__ __forceinline__ void put_pair_bf(unsigned char *base, int row, int j, int K, float a, float b)
+// K-chunk j of row `row` = {c, 0 x 7} in BF16: the ones column of an activation.
+__device__ __forceinline__ void put_one_bf(unsigned char *base, int row, int j, int K, float c)
 {
-    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(c, 0.0f);
     *reinterpret_cast<uint4 *>(base + core_off(row, 8 * j, K)) =
         make_uint4(*reinterpret_cast<const uint32_t *>(&p), 0u, 0u, 0u);
 }
-__device__ __forceinline__ void put_bias_bf(unsigned char *base, int row, int j, int K, float b)
-{
-    const float hi = __bfloat162float(__float2bfloat16_rn(b));
-    put_pair_bf(base, row, j, K, hi, b - hi);
-}
-
 // Rows owned by the lanes of a warp (lane r: row offset off_r, validity ok_r)
 // moved in coalesced pieces through a per-warp shared tile of H rows x 33
 // floats: for each row, the 32 lanes move 32 consecutive floats (columns col0
@@ -600,15 +617,43 @@ __device__ __forceinline__ void warp_store_rows(const float v[32], float *base_l
 
 }  // namespace
 
-__global__ void __launch_bounds__(128, 1) decoder_grad_tc_kernel(const __grid_constant__ DecoderGradTcParams p)
+__global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __grid_constant__ DecoderGradTcParams p)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ uint64_t s_bar, s_never;
     __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
     __shared__ double s_loss;
-    const int t = threadIdx.x, warp = t >> 5;
-    const int nc = p.nc;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int m = t & 127, half = t >> 7;  // row of the tile, and which half of the columns
+    const int nc = p.nc, ts = target_stride(nc);
+    const bool pair = (nc & 1) == 0 && (reinterpret_cast<uintptr_t>(p.targets) & 7u) == 0;
+    float *s_t = reinterpret_cast<float *>(sm + TGO_T);
+    float *s_b1 = reinterpret_cast<float *>(sm + TGO_B), *s_b2 = s_b1 + 64, *s_b3 = s_b2 + 64, *s_cw = s_b3 + TG_NC;
+    const uint32_t n_tiles = (p.batch + 127) / 128;
+
+    // Warp w moves rows 16 w .. 16 w + 15 of a tile: the target rows by
+    // asynchronous copies, the latents into registers (lane = feature).
+    float xr[16];
+    auto load_rows = [&](uint32_t tile) {
+        const uint32_t r0 = tile * 128 + (uint32_t)warp * 16;
+        const uint32_t mine = lane < 16 && tile < n_tiles && r0 + lane < p.batch ? p.rows[r0 + lane] : 0u;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const size_t row = __shfl_sync(0xffffffffu, mine, i);
+            xr[i] = 0.0f;
+            if (tile >= n_tiles || r0 + i >= p.batch) continue;
+            xr[i] = p.latents[row * 32 + lane];
+            const float *src = p.targets + row * nc;
+            float *dst = s_t + (warp * 16 + i) * ts;
+            if (pair) {
+                for (int c = 2 * lane; c < nc; c += 64) cp_async(dst + c, src + c, true);
+            } else {
+                for (int c = lane; c < nc; c += 32) cp_async(dst + c, src + c, false);
+            }
+        }
+    };
+    load_rows(blockIdx.x);
     if (t == 0) {
         s_fail = 0;
         s_loss = 0.0;
@@ -622,42 +667,21 @@ __global__ void __launch_bounds__(128, 1) decoder_grad_tc_kernel(const __grid_co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // --- weights as BF16 B operands, once per CTA
-    for (int q = t; q < 64 * (TG_K1 / 8); q += 128) {
-        const int n = q / (TG_K1 / 8), j = q % (TG_K1 / 8);
-        if (j < 4) put8_bf(sm + TGO_W1, n, j, TG_K1, p.w.w1 + n * 32 + 8 * j);
-        else if (j == 4) put_bias_bf(sm + TGO_W1, n, j, TG_K1, p.w.b1[n]);
-        else put_pair_bf(sm + TGO_W1, n, j, TG_K1, 0.0f, 0.0f);
+    // --- weights as BF16 operands and FP32 biases, once per CTA
+    for (int q = t; q < 64 * 4; q += TG_THREADS) put8_bf(sm + TGO_W1, q >> 2, q & 3, 32, p.w.w1 + q * 8);
+    for (int q = t; q < 64 * 8; q += TG_THREADS) put8_bf(sm + TGO_W2, q >> 3, q & 7, 64, p.w.w2 + q * 8);
+    for (int q = t; q < TG_NC * 8; q += TG_THREADS) {
+        const int n = q >> 3, j = q & 7;
+        const float zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        put8_bf(sm + TGO_W3, n, j, 64, n < nc ? p.w.w3 + q * 8 : zero);
     }
-    for (int q = t; q < 64 * (TG_K2 / 8); q += 128) {
-        const int n = q / (TG_K2 / 8), j = q % (TG_K2 / 8);
-        if (j < 8) put8_bf(sm + TGO_W2, n, j, TG_K2, p.w.w2 + n * 64 + 8 * j);
-        else if (j == 8) put_bias_bf(sm + TGO_W2, n, j, TG_K2, p.w.b2[n]);
-        else put_pair_bf(sm + TGO_W2, n, j, TG_K2, 0.0f, 0.0f);
+    if (t < 64) {
+        s_b1[t] = p.w.b1[t];
+        s_b2[t] = p.w.b2[t];
     }
-    for (int q = t; q < TG_NC * (TG_K2 / 8); q += 128) {
-        const int n = q / (TG_K2 / 8), j = q % (TG_K2 / 8);
-        if (n >= nc || j == 9) put_pair_bf(sm + TGO_W3, n, j, TG_K2, 0.0f, 0.0f);
-        else if (j < 8) put8_bf(sm + TGO_W3, n, j, TG_K2, p.w.w3 + n * 64 + 8 * j);
-        else put_bias_bf(sm + TGO_W3, n, j, TG_K2, p.w.b3[n]);
-    }
-    for (int q = t; q < 64 * TG_NC; q += 128) {  // W3^T[k][j] = W3[j][k]
-        const int k = q / TG_NC, j = q % TG_NC;
-        put1_bf(sm + TGO_W3T, k, j, TG_NC, j < nc ? p.w.w3[j * 64 + k] : 0.0f);
-    }
-    for (int q = t; q < 64 * 64; q += 128) {  // W2^T[k][o] = W2[o][k]
-        const int k = q >> 6, o = q & 63;
-        put1_bf(sm + TGO_W2T, k, o, 64, p.w.w2[o * 64 + k]);
-    }
-    for (int q = t; q < 32 * 64; q += 128) {  // W1^T[k][o] = W1[o][k]
-        const int k = q >> 6, o = q & 63;
-        put1_bf(sm + TGO_W1T, k, o, 64, p.w.w1[o * 32 + k]);
-    }
-    // the transposed activations' rows past the ones row, inside their allocation
-    for (int q = t; q < 7 * TG_KR; q += 128) {
-        put1_bf(sm + TGO_XT, 33 + q / TG_KR, q % TG_KR, TG_KR, 0.0f);
-        put1_bf(sm + TGO_H1T, 65 + q / TG_KR, q % TG_KR, TG_KR, 0.0f);
-        put1_bf(sm + TGO_H2T, 65 + q / TG_KR, q % TG_KR, TG_KR, 0.0f);
+    for (int q = t; q < TG_NC; q += TG_THREADS) {
+        s_b3[q] = q < nc ? p.w.b3[q] : 0.0f;
+        s_cw[q] = q < nc ? p.coef_weight[q] : 0.0f;
     }
     fence_async_smem();
     fence_before();
@@ -665,7 +689,7 @@ __global__ void __launch_bounds__(128, 1) decoder_grad_tc_kernel(const __grid_co
     fence_after();
 
     const uint32_t tm = s_tmem;
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;  // this warp's lane quarter
+    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;  // this warp's lane quarter
     const uint32_t sa = ptx::smem_u32(sm);
     uint32_t phase = 0;
     bool first_wait = p.test_timeout != 0;
@@ -685,204 +709,184 @@ __global__ void __launch_bounds__(128, 1) decoder_grad_tc_kernel(const __grid_co
         phase ^= 1u;
         return true;
     };
-    const uint32_t n_tiles = (p.batch + 127) / 128;
+    // H = relu(Z + b) of this thread's 32 columns into `dst`; returns the mask of Z + b > 0
+    auto relu_half = [&](unsigned char *dst, const float *b) -> uint32_t {
+        float v[32];
+        tmem_ld32(tm + lane_off + TC_SCR + 32 * half, v);
+        uint32_t mask = 0;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            v[e] += b[32 * half + e];
+            if (v[e] > 0.0f) mask |= 1u << e;
+            v[e] = fmaxf(v[e], 0.0f);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) put8_bf(dst, m, 4 * half + c, TG_KH, v + 8 * c);
+        return mask;
+    };
+    // d = dH [mask] of this thread's 32 columns (over dY, or over the layer's before)
+    auto masked_half = [&](uint32_t mask) {
+        float v[32];
+        tmem_ld32(tm + lane_off + TC_SCR + 32 * half, v);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = (mask >> e) & 1u ? v[e] : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_DY, m, 4 * half + c, 64, v + 8 * c);
+    };
     float lsum = 0.0f;
     uint32_t acc_w = 0;  // the weight gradients accumulate from the CTA's second tile on
     for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const uint32_t r0 = tile * 128;
-        const bool valid = r0 + (uint32_t)t < p.batch;
-        const size_t row = valid ? p.rows[r0 + t] : 0;
+        const bool valid = r0 + (uint32_t)m < p.batch;
         const float one = valid ? 1.0f : 0.0f;
-        // X: [x 1] (A of Z1) and [X^T; 1] (A of G1)
-        {
-            float x[32];
+        // (the previous tile's last MMAs, which read X, H1 and d1, are done)
 #pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = valid ? p.latents[row * 32 + k] : 0.0f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) put8_bf(sm + TGO_A, t, j, TG_K1, x + 8 * j);
-            put_pair_bf(sm + TGO_A, t, 4, TG_K1, one, one);
-            put_pair_bf(sm + TGO_A, t, 5, TG_K1, 0.0f, 0.0f);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) put1_bf(sm + TGO_XT, k, t, TG_KR, x[k]);
-            put1_bf(sm + TGO_XT, 32, t, TG_KR, one);
+        for (int i = 0; i < 16; ++i)
+            *reinterpret_cast<__nv_bfloat16 *>(sm + TGO_X + core_off(warp * 16 + i, lane, TG_KX)) = __float2bfloat16_rn(xr[i]);
+        if (half == 0) put_one_bf(sm + TGO_X, m, 4, TG_KX, one);
+        else {
+            put_one_bf(sm + TGO_H1, m, 8, TG_KH, one);
+            put_one_bf(sm + TGO_H2, m, 8, TG_KH, one);
         }
         hand_off();
         if (t == 0) {
             fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W1, TG_K1, 64, 0);
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_X, TG_KX), over_cols(sa + TGO_W1, 32), 32, 64, 0);
             mma_commit(&s_bar);
         }
         if (!wait_mmas()) break;
-        // H1 = relu(Z1): [H1 1] (A of Z2), [H1^T; 1] (A of G2), the mask of Z1 > 0
-        uint32_t m1[2], m2[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR + 32 * h, v);
-            m1[h] = 0;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                if (v[e] > 0.0f) m1[h] |= 1u << e;
-                v[e] = fmaxf(v[e], 0.0f);
-                put1_bf(sm + TGO_H1T, 32 * h + e, t, TG_KR, v[e]);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_A, t, 4 * h + c, TG_K2, v + 8 * c);
-        }
-        put_pair_bf(sm + TGO_A, t, 8, TG_K2, one, one);
-        put_pair_bf(sm + TGO_A, t, 9, TG_K2, 0.0f, 0.0f);
-        put1_bf(sm + TGO_H1T, 64, t, TG_KR, one);
+        const uint32_t m1 = relu_half(sm + TGO_H1, s_b1);
         hand_off();
         if (t == 0) {
             fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W2, TG_K2, 64, 0);
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_H1, TG_KH), over_cols(sa + TGO_W2, 64), 64, 64, 0);
             mma_commit(&s_bar);
         }
         if (!wait_mmas()) break;
-        // H2 = relu(Z2) in place of H1 (Z2 is done with it)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR + 32 * h, v);
-            m2[h] = 0;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                if (v[e] > 0.0f) m2[h] |= 1u << e;
-                v[e] = fmaxf(v[e], 0.0f);
-                put1_bf(sm + TGO_H2T, 32 * h + e, t, TG_KR, v[e]);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_A, t, 4 * h + c, TG_K2, v + 8 * c);
-        }
-        put1_bf(sm + TGO_H2T, 64, t, TG_KR, one);
+        const uint32_t m2 = relu_half(sm + TGO_H2, s_b2);
+        cp_async_wait();  // this thread's copies of the tile's targets (all threads': the barrier below)
         hand_off();
         if (t == 0) {
             fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W3, TG_K2, TG_NC, 0);
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_H2, TG_KH), over_cols(sa + TGO_W3, 64), 64, TG_NC, 0);
             mma_commit(&s_bar);
         }
         if (!wait_mmas()) break;
-        // dY = 2 cw (Y - target) + extra: dY (A of dH2, over the H2 it replaces) and dY^T (B of G3)
+        // dY = 2 cw (Y - target) + extra
+        const float *trow = s_t + m * ts;
+        const float *xrow = p.extra_dy && valid ? p.extra_dy + (size_t)p.rows[r0 + m] * nc : nullptr;
 #pragma unroll 1
-        for (int c = 0; c < TG_NC / 32 + 1; ++c) {
+        for (int c = 3 * half; c < 3 * half + 3; ++c) {
             float v[32];
             tmem_ld32(tm + lane_off + TC_SCR + 32 * c, v);  // columns 176..191: unused scratch
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
+            for (int e = 0; e < 32; e += 2) {
                 const int j = 32 * c + e;
-                float d = 0.0f;
-                if (valid && j < nc) {
-                    const float err = v[e] - p.targets[row * nc + j];
-                    const float cw = p.coef_weight[j];
-                    lsum = fmaf(cw * err, err, lsum);
-                    d = 2.0f * cw * err;
-                    if (p.extra_dy) d += p.extra_dy[row * nc + j];
+                float2 tv = make_float2(0.0f, 0.0f), bb = tv, cw = tv;
+                if (j < nc) {  // (an odd nc ends inside a pair: cw is 0 there)
+                    tv = *reinterpret_cast<const float2 *>(trow + j);
+                    bb = *reinterpret_cast<const float2 *>(s_b3 + j);
+                    cw = *reinterpret_cast<const float2 *>(s_cw + j);
                 }
-                v[e] = d;
-                if (j < TG_NC) put1_bf(sm + TGO_B, j, t, TG_KR, d);
+                const float tq[2] = {tv.x, tv.y}, bq[2] = {bb.x, bb.y}, cq[2] = {cw.x, cw.y};
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    float d = 0.0f;
+                    if (valid && j + k < nc) {
+                        const float err = v[e + k] + bq[k] - tq[k];
+                        lsum = fmaf(cq[k] * err, err, lsum);
+                        d = 2.0f * cq[k] * err;
+                        if (xrow) d += xrow[j + k];
+                    }
+                    v[e + k] = d;
+                }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (4 * c + q < TG_NC / 8) put8_bf(sm + TGO_A, t, 4 * c + q, TG_NC, v + 8 * q);
+                if (4 * c + q < TG_NC / 8) put8_bf(sm + TGO_DY, m, 4 * c + q, TG_NC, v + 8 * q);
         }
         hand_off();
         if (t == 0) {
             fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W3T, TG_NC, 64, 0);
-            gemm_bf16(tm + TC_G3, sa + TGO_H2T, sa + TGO_B, TG_KR, TG_NC, acc_w);
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, TG_NC), over_rows(sa + TGO_W3, 64), TG_NC, 64, 0);
+            gemm_bf16(tm + TC_G3, over_rows(sa + TGO_H2, TG_KH), over_rows(sa + TGO_DY, TG_NC), 128, TG_NC, acc_w);
+            mma_commit(&s_bar);
+        }
+        load_rows(tile + gridDim.x);  // the target tile is free: in flight from here on
+        if (!wait_mmas()) break;
+        masked_half(m2);
+        hand_off();
+        if (t == 0) {
+            fence_after();
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, 64), over_rows(sa + TGO_W2, 64), 64, 64, 0);
+            gemm_bf16(tm + TC_G2, over_rows(sa + TGO_H1, TG_KH), over_rows(sa + TGO_DY, 64), 128, 64, acc_w);
             mma_commit(&s_bar);
         }
         if (!wait_mmas()) break;
-        // d2 = dH2 [Z2 > 0]: A of dH1 (over dY) and d2^T (B of G2, over dY^T)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR + 32 * h, v);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                v[e] = (m2[h] >> e) & 1u ? v[e] : 0.0f;
-                put1_bf(sm + TGO_B, 32 * h + e, t, TG_KR, v[e]);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_A, t, 4 * h + c, 64, v + 8 * c);
-        }
+        masked_half(m1);
         hand_off();
         if (t == 0) {
             fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W2T, 64, 64, 0);
-            gemm_bf16(tm + TC_G2, sa + TGO_H1T, sa + TGO_B, TG_KR, 64, acc_w);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        // d1 = dH1 [Z1 > 0]: A of dX and d1^T (B of G1)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR + 32 * h, v);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                v[e] = (m1[h] >> e) & 1u ? v[e] : 0.0f;
-                put1_bf(sm + TGO_B, 32 * h + e, t, TG_KR, v[e]);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_A, t, 4 * h + c, 64, v + 8 * c);
-        }
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, sa + TGO_A, sa + TGO_W1T, 64, 32, 0);
-            gemm_bf16(tm + TC_G1, sa + TGO_XT, sa + TGO_B, TG_KR, 64, acc_w);
+            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, 64), over_rows(sa + TGO_W1, 32), 64, 32, 0);
+            gemm_bf16(tm + TC_G1, over_rows(sa + TGO_X, TG_KX), over_rows(sa + TGO_DY, 64), 128, 64, acc_w);
             mma_commit(&s_bar);
         }
         if (!wait_mmas()) break;
         // dL/d(latent) of the tile's rows
-        {
+        if (half == 0) {
             float v[32];
             tmem_ld32(tm + lane_off + TC_SCR, v);
-            if (valid) {  // (scalar stores: the caller's array needs only float alignment)
+            if (valid) {
+                float *dst = p.dlatents + (size_t)(r0 + m) * 32;
+                if ((reinterpret_cast<uintptr_t>(p.dlatents) & 15u) == 0) {
 #pragma unroll
-                for (int k = 0; k < 32; ++k) p.dlatents[(size_t)(r0 + t) * 32 + k] = v[k];
+                    for (int k = 0; k < 8; ++k)
+                        reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                } else {  // (the caller's array needs only float alignment)
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) dst[k] = v[k];
+                }
             }
         }
         fence_before();  // TMEM reads done before the next tile's MMAs
         acc_w = 1;
     }
+    cp_async_wait();
     if (!s_fail) {
         // the weight gradients: lane k of G3 / G2 / G1 is input feature k, lane
         // 64 (32 for G1) the bias; column j / o the output feature
 #pragma unroll 1
-        for (int c = 0; c < TG_NC / 32 + 1; ++c) {
+        for (int c = 3 * half; c < 3 * half + 3; ++c) {
             float v[32];
             tmem_ld32(tm + lane_off + TC_G3 + 32 * c, v);  // columns past 175 belong to G3's padding
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
                 const int j = 32 * c + e;
                 if (j >= nc) continue;
-                if (t < 64) atomicAdd(p.g.w3 + j * 64 + t, v[e]);
-                else if (t == 64) atomicAdd(p.g.b3 + j, v[e]);
+                if (m < 64) atomicAdd(p.g.w3 + j * 64 + m, v[e]);
+                else if (m == 64) atomicAdd(p.g.b3 + j, v[e]);
             }
         }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        {
             float v[32];
-            tmem_ld32(tm + lane_off + TC_G2 + 32 * h, v);
+            tmem_ld32(tm + lane_off + TC_G2 + 32 * half, v);
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
-                const int o = 32 * h + e;
-                if (t < 64) atomicAdd(p.g.w2 + o * 64 + t, v[e]);
-                else if (t == 64) atomicAdd(p.g.b2 + o, v[e]);
+                const int o = 32 * half + e;
+                if (m < 64) atomicAdd(p.g.w2 + o * 64 + m, v[e]);
+                else if (m == 64) atomicAdd(p.g.b2 + o, v[e]);
             }
-            tmem_ld32(tm + lane_off + TC_G1 + 32 * h, v);
+            tmem_ld32(tm + lane_off + TC_G1 + 32 * half, v);
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
-                const int o = 32 * h + e;
-                if (t < 32) atomicAdd(p.g.w1 + o * 32 + t, v[e]);
-                else if (t == 32) atomicAdd(p.g.b1 + o, v[e]);
+                const int o = 32 * half + e;
+                if (m < 32) atomicAdd(p.g.w1 + o * 32 + m, v[e]);
+                else if (m == 32) atomicAdd(p.g.b1 + o, v[e]);
             }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-        if ((t & 31) == 0) atomicAdd(&s_loss, (double)lsum);
+        if (lane == 0) atomicAdd(&s_loss, (double)lsum);
     } else if (t == 0) {
         // the commit whose wait gave up: wait for it once more (bounded)
         // before TMEM is freed
@@ -1242,7 +1246,7 @@ extern "C" int fpo_decoder_grad_tc(const fpo_mlp *w, int32_t n1, int32_t n2, uin
     if (e != cudaSuccess) return set_last_error(FPO_ERR_CUDA, cudaGetErrorString(e));
     const uint32_t n_tiles = (batch + 127) / 128;
     const uint32_t blocks = n_tiles < (uint32_t)sms ? n_tiles : (uint32_t)sms;
-    decoder_grad_tc_kernel<<<blocks, 128, smem, (cudaStream_t)cuda_stream>>>(p);
+    decoder_grad_tc_kernel<<<blocks, TG_THREADS, smem, (cudaStream_t)cuda_stream>>>(p);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_last_error(FPO_ERR_CUDA, cudaGetErrorString(e));
     return FPO_OK;
