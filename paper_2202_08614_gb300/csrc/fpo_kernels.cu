@@ -1258,12 +1258,11 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 //              their leaf segments to the warp's list in shared memory (a
 //              round = the visits of one step), until the list is full or
 //              every ray has left the grid; the records are pulled into L2;
-//   shade      all 32 lanes evaluate the list, FU_UNROLL visits at a time: lane
-//              l takes elements l, l + 32, ... of a visit's record (each load
-//              is one contiguous line), multiplies them by its ray's weights
-//              (Eq. 8 at the ray's time; Y_k(d) IDFT_i(t) for the colours, so
-//              Eq. 7, 9 and the sum of Eq. 1 are one dot product), and four
-//              sums are reduced by halving butterflies that keep all lanes busy;
+//   shade      all 32 lanes evaluate the list, 8 visits at a time: four lanes
+//              share a visit's record in 64-byte pieces and multiply it by its
+//              ray's weights (Eq. 8 at the ray's time; Y_k(d) IDFT_i(t) for the
+//              colours, so that Eq. 7, 9 and the sum of Eq. 1 are one dot
+//              product over the record as it is stored);
 //   composite  lane l takes its own visits in order; a ray that falls below
 //              stop_T ignores the rest of its list (at most a list's worth of
 //              visits is evaluated for nothing);
@@ -1283,7 +1282,10 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 // adjoint sees the forward's segments and early stop.
 
 constexpr int FU_WARPS = 2;    // warps per CTA (they share nothing but its launch)
-constexpr int FU_UNROLL = 4;   // visits a warp evaluates at a time
+constexpr int FU_GROUP = 8;    // visits a warp evaluates at a time, 4 lanes each
+#ifndef FPO_FUSED_MAXNREG
+#define FPO_FUSED_MAXNREG 128
+#endif
 #ifndef FPO_FUSED_MIN_RAYS
 #define FPO_FUSED_MIN_RAYS 2
 #endif
@@ -1304,22 +1306,23 @@ constexpr bool FU_PREFETCH = FPO_FUSED_PREFETCH;
 
 template <int N1, int N2>
 struct FusedSize {
-    static constexpr int NZ = 9 * N2;            // weights shared by the three channels
-    static constexpr int NW = N1 + NZ;           // weights per ray
-    static constexpr int NWP = NW | 1;           // odd row stride: no bank conflicts between rays
-    static constexpr int ZR = (27 * N2 + 31) / 32;
+    static constexpr int SC = (N1 + 3) / 4, ZC = (27 * N2 + 3) / 4;    // 16-byte pieces of a record's two parts
+    static constexpr int SI = (SC + 3) / 4, ZI = (ZC + 3) / 4;         // ... of each of a visit's four lanes
+    static constexpr int NZ = 9 * N2;                                  // elements of a channel
+    static constexpr int WROW = 4 * (SC + ZC);                         // weights of a ray, in record order
     static constexpr int NC = N1 + 27 * N2;
+    static_assert(NC % 2 == 0, "gradient rows start at a multiple of 8 bytes");
 };
 
 // Shared memory of one warp, in 32-bit words (a multiple of 4): the list
-// (visit, result, round mask per entry), the ancestor stacks, the weights.
-__host__ __device__ inline int fused_warp_words(int rays, int cap, int stack_levels, int nwp)
+// (visit, result, round mask per entry), the weights, the ancestor stacks.
+__host__ __device__ inline int fused_warp_words(int rays, int cap, int stack_levels, int wrow)
 {
-    return (9 * cap + rays * stack_levels + rays * nwp + 3) & ~3;
+    return (9 * cap + rays * stack_levels + rays * wrow + 3) & ~3;
 }
 
 template <int N1, int N2, bool ADJ, bool DBG, bool BRICK>
-__global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_constant__ BackwardParams q)
+__global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constant__ BackwardParams q)
 {
     using S = FusedSize<N1, N2>;
     extern __shared__ __align__(16) uint32_t smem[];
@@ -1328,12 +1331,12 @@ __global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_const
     const int R = p.rays_per_warp, E = p.list_cap;
     const int G = 1 << p.depth;
     const int levels = BRICK ? 0 : p.depth + 1;  // of the ancestor stacks
-    uint32_t *mem = smem + (threadIdx.x >> 5) * fused_warp_words(R, E, levels, S::NWP);
+    uint32_t *mem = smem + (threadIdx.x >> 5) * fused_warp_words(R, E, levels, S::WROW);
     uint4 *ent = reinterpret_cast<uint4 *>(mem);             // leaf, delta, lane, step
     float *res = reinterpret_cast<float *>(mem + 4 * E);     // [E][4]
-    uint32_t *rounds = mem + 8 * E;
+    float *wt = reinterpret_cast<float *>(mem + 8 * E);      // [R][WROW]
+    uint32_t *rounds = mem + 8 * E + R * S::WROW;
     uint32_t *stack = BRICK ? nullptr : rounds + E + (lane < R ? lane : 0);  // stride R
-    float *wt = reinterpret_cast<float *>(rounds + E + R * levels);
     const uint32_t lt_mask = (1u << lane) - 1u;
     const bool prt = p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
 
@@ -1383,18 +1386,24 @@ __global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_const
             for (uint32_t f = fresh; f; f &= f - 1u) {
                 const int r = __ffs((int)f) - 1;
                 const float ur = __shfl_sync(0xffffffffu, u, r);
-                if (lane < N1) wt[r * S::NWP + lane] = prt ? basis_fp32(lane, ur) : p.fc.b[lane];
+                float yk = 0.0f;  // lane k < 9: Y_k
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float y = __shfl_sync(0xffffffffu, W.Y[k], r);
+                    yk = lane == k ? y : yk;
+                }
+                const float b = lane < N1 ? (prt ? basis_fp32(lane, ur) : p.fc.b[lane]) : 0.0f;
+                float *w = wt + r * S::WROW;
+                if (lane < 4 * S::SC) w[lane] = b;
+                w += 4 * S::SC;
+#pragma unroll
+                for (int h = 0; h < (S::ZC * 4 + 31) / 32; ++h) {
+                    const int e = 32 * h + lane, el = e % S::NZ;
+                    const float x = __shfl_sync(0xffffffffu, yk, el / N2) * __shfl_sync(0xffffffffu, b, el % N2);
+                    if (e < 4 * S::ZC) w[e] = e < 27 * N2 ? x : 0.0f;
+                }
             }
-            __syncwarp();
             if (mine) {
-                float *w = wt + lane * S::NWP;
-                float b[N2];
-#pragma unroll
-                for (int i = 0; i < N2; ++i) b[i] = w[i];
-#pragma unroll
-                for (int k = 0; k < 9; ++k)
-#pragma unroll
-                    for (int i = 0; i < N2; ++i) w[N1 + k * N2 + i] = W.Y[k] * b[i];
                 if (ADJ) {
                     g0 = q.dL_drgb[3 * (size_t)ray];
                     g1 = q.dL_drgb[3 * (size_t)ray + 1];
@@ -1456,73 +1465,65 @@ __global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_const
                                            : reinterpret_cast<const char *>(p.zc) + (size_t)lf * zb + (l - 1) * 128u;
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
                 }
+                if (ADJ) {  // and those of the gradient rows, which the reductions then find there
+                    constexpr uint32_t GN = (S::NC * 4 + 127) / 128;
+                    for (uint32_t e = lane; e < n * GN; e += 32)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(
+                                         q.dL_dcoeffs + (size_t)p.perm[ent[e / GN].x] * S::NC) + e % GN * 128u));
+                }
             }
 
             // --- shade
-            for (uint32_t v0 = 0; v0 < n; v0 += FU_UNROLL) {
-                float part[FU_UNROLL][4];
-                uint32_t ray_lane[FU_UNROLL];
-                float zv[FU_UNROLL][S::ZR], sv[FU_UNROLL];
+            for (uint32_t v0 = 0; v0 < n; v0 += FU_GROUP) {
+                const uint32_t at = v0 + ((uint32_t)lane >> 2);
+                const int l = lane & 3;
+                const uint4 en = ent[min(at, n - 1)];
+                const float4 *sr = p.sig + (size_t)en.x * p.sig_stride4 + l;
+                const float4 *zr = reinterpret_cast<const float4 *>(p.zc + (size_t)en.x * p.z_stride) + l;
+                const float4 *w = reinterpret_cast<const float4 *>(wt + en.z * S::WROW) + l;
+                float4 sv[S::SI], zv[S::ZI];
+                const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-                for (int a = 0; a < FU_UNROLL; ++a) {
-                    const uint4 en = ent[min(v0 + a, n - 1)];
-                    ray_lane[a] = en.z;
-                    const float *sr = reinterpret_cast<const float *>(p.sig + (size_t)en.x * p.sig_stride4);
-                    const float *zr = p.zc + (size_t)en.x * p.z_stride;
-                    sv[a] = lane < N1 ? __ldg(sr + lane) : 0.0f;
+                for (int i = 0; i < S::SI; ++i) sv[i] = 4 * i + 3 < S::SC || 4 * i + l < S::SC ? __ldg(sr + 4 * i) : zero;
 #pragma unroll
-                    for (int r = 0; r < S::ZR; ++r) zv[a][r] = 32 * r + lane < 27 * N2 ? __ldg(zr + 32 * r + lane) : 0.0f;
+                for (int i = 0; i < S::ZI; ++i) zv[i] = 4 * i + 3 < S::ZC || 4 * i + l < S::ZC ? __ldg(zr + 4 * i) : zero;
+                float part[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // sigma_raw, u_0, u_1, u_2: this lane's share
+#pragma unroll
+                for (int i = 0; i < S::SI; ++i) {
+                    const float4 wv = 4 * i + 3 < S::SC || 4 * i + l < S::SC ? w[4 * i] : zero;
+                    part[0] = fmaf(sv[i].x, wv.x, part[0]);
+                    part[0] = fmaf(sv[i].y, wv.y, part[0]);
+                    part[0] = fmaf(sv[i].z, wv.z, part[0]);
+                    part[0] = fmaf(sv[i].w, wv.w, part[0]);
                 }
 #pragma unroll
-                for (int a = 0; a < FU_UNROLL; ++a) {
-                    const float *w = wt + ray_lane[a] * S::NWP;
-                    part[a][0] = lane < N1 ? sv[a] * w[lane] : 0.0f;
-                    part[a][1] = part[a][2] = part[a][3] = 0.0f;
+                for (int i = 0; i < S::ZI; ++i) {
+                    const float4 wv = 4 * i + 3 < S::ZC || 4 * i + l < S::ZC ? w[S::SC + 4 * i] : zero;
+                    const float x[4] = {zv[i].x, zv[i].y, zv[i].z, zv[i].w}, y[4] = {wv.x, wv.y, wv.z, wv.w};
+                    const int c = 16 * i / S::NZ;  // channel of the group's first element
+                    const bool one = 16 * i + 15 < (c + 1) * S::NZ || c == 2;  // ... and of all 16
 #pragma unroll
-                    for (int r = 0; r < S::ZR; ++r) {
-                        const int j = 32 * r + lane;  // element of the SH record: channel j / NZ, weight j % NZ
-                        const float x = w[N1 + j % S::NZ];
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            // (compile-time where the 32 elements lie in one channel)
-                            if (32 * r >= c * S::NZ && 32 * r + 31 < (c + 1) * S::NZ) part[a][1 + c] = fmaf(zv[a][r], x, part[a][1 + c]);
-                            else if (32 * r + 31 >= c * S::NZ && 32 * r < (c + 1) * S::NZ && j >= c * S::NZ && j < (c + 1) * S::NZ)
-                                part[a][1 + c] = fmaf(zv[a][r], x, part[a][1 + c]);
-                        }
+                    for (int e = 0; e < 4; ++e) {
+                        if (one || 16 * i + 4 * l + e < (c + 1) * S::NZ) part[1 + c] = fmaf(x[e], y[e], part[1 + c]);
+                        else part[c < 2 ? 2 + c : 3] = fmaf(x[e], y[e], part[c < 2 ? 2 + c : 3]);
                     }
                 }
-                // 16 sums over 32 lanes: each butterfly step halves the values a
-                // lane still carries; lane (b4 b3 b2 b1 b0) ends with value 2 b4 + b3
-                // of visit 2 b2 + b1
-                const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-                float s1[FU_UNROLL];
-#pragma unroll
-                for (int a = 0; a < FU_UNROLL; ++a) {
-                    float k0 = b4 ? part[a][2] : part[a][0], k1 = b4 ? part[a][3] : part[a][1];
-                    k0 += __shfl_xor_sync(0xffffffffu, b4 ? part[a][0] : part[a][2], 16);
-                    k1 += __shfl_xor_sync(0xffffffffu, b4 ? part[a][1] : part[a][3], 16);
-                    s1[a] = (b3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8);
+                // four sums over four lanes; lane l ends with sum l
+                const bool b1 = l & 2, b0 = l & 1;
+                float k0 = b1 ? part[2] : part[0], k1 = b1 ? part[3] : part[1];
+                k0 += __shfl_xor_sync(0xffffffffu, b1 ? part[0] : part[2], 2);
+                k1 += __shfl_xor_sync(0xffffffffu, b1 ? part[1] : part[3], 2);
+                const float s = (b0 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b0 ? k0 : k1, 1);
+                float o;
+                if (l == 0) {
+                    // e^{-sigma delta}, with the sign bit set where sigma_raw > 0
+                    // (the adjoint's mask of max(0, sigma_raw))
+                    o = __expf(-fmaxf(s, 0.0f) * __uint_as_float(en.y));
+                    if (s > 0.0f) o = -o;
+                } else {
+                    o = sigmoidf_(s);
                 }
-                float s2[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h)  // visit 2 b2 + h
-                    s2[h] = (b2 ? s1[2 + h] : s1[h]) + __shfl_xor_sync(0xffffffffu, b2 ? s1[h] : s1[2 + h], 4);
-                float s = (b1 ? s2[1] : s2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? s2[0] : s2[1], 2);
-                s += __shfl_xor_sync(0xffffffffu, s, 1);
-                const int val = (b4 ? 2 : 0) + (b3 ? 1 : 0);
-                const uint32_t at = v0 + (b2 ? 2 : 0) + (b1 ? 1 : 0);
-                if (!(lane & 1) && at < n) {
-                    float o;
-                    if (val == 0) {
-                        // e^{-sigma delta}, with the sign bit set where sigma_raw > 0
-                        // (the adjoint's mask of max(0, sigma_raw))
-                        o = __expf(-fmaxf(s, 0.0f) * __uint_as_float(ent[at].y));
-                        if (s > 0.0f) o = -o;
-                    } else {
-                        o = sigmoidf_(s);
-                    }
-                    res[4 * at + val] = o;
-                }
+                if (at < n) res[4 * at + l] = o;
             }
             __syncwarp();
 
@@ -1584,14 +1585,14 @@ __global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_const
                 for (uint32_t v = 0; v < n; ++v) {
                     const uint4 en = ent[v];
                     if (en.x == 0xffffffffu) continue;
-                    const float *w = wt + en.z * S::NWP;
+                    const float *w = wt + en.z * S::WROW;
                     float *row = q.dL_dcoeffs + (size_t)en.x * S::NC;
 #pragma unroll
                     for (int r = 0; r < (S::NC + 63) / 64; ++r) {
                         const int el = 64 * r + 2 * lane;
                         auto gval = [&](int k) {  // element k of the canonical row
                             const int j = k - N1;
-                            return j < 0 ? res[4 * v] * w[k] : res[4 * v + 1 + j / S::NZ] * w[N1 + j % S::NZ];
+                            return j < 0 ? res[4 * v] * w[k] : res[4 * v + 1 + j / S::NZ] * w[4 * S::SC + j];
                         };
                         if (el < S::NC) atomicAdd(reinterpret_cast<float2 *>(row + el), make_float2(gval(el), gval(el + 1)));
                     }
@@ -1619,11 +1620,11 @@ __global__ void __launch_bounds__(32 * FU_WARPS) fused_kernel(const __grid_const
 // Rays per warp and list length.  Few rays: fewer of them per warp, so that
 // every SM gets several warps (a warp's time is that of its longest ray
 // either way, and the shading lanes are all busy for any R).
-static void fused_shape(uint32_t tiles32, int sm_count, int *rays, int *cap)
+static void fused_shape(uint32_t tiles32, int sm_count, int warps_per_sm, int *rays, int *cap)
 {
     const uint64_t n = (uint64_t)tiles32 * 32;
-    int r = 32;
-    while (r > FPO_FUSED_MIN_RAYS && n < (uint64_t)sm_count * FPO_FUSED_WARPS_PER_SM * r) r >>= 1;
+    int r = 16;
+    while (r > FPO_FUSED_MIN_RAYS && n < (uint64_t)sm_count * warps_per_sm * r) r >>= 1;
     *rays = r;
     *cap = r * FPO_FUSED_LIST < 64 ? 64 : r * FPO_FUSED_LIST;
 }
@@ -1632,9 +1633,9 @@ template <int N1, int N2, bool ADJ, bool DBG, bool BRICK>
 static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
 {
     TraverseParams &p = q.tp;
-    fused_shape(p.n_tiles, sm_count, &p.rays_per_warp, &p.list_cap);
+    fused_shape(p.n_tiles, sm_count, ADJ ? 2 * FPO_FUSED_WARPS_PER_SM : FPO_FUSED_WARPS_PER_SM, &p.rays_per_warp, &p.list_cap);
     const int threads = 32 * FU_WARPS;
-    const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, BRICK ? 0 : p.depth + 1, FusedSize<N1, N2>::NWP);
+    const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, BRICK ? 0 : p.depth + 1, FusedSize<N1, N2>::WROW);
     auto k = fused_kernel<N1, N2, ADJ, DBG, BRICK>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return (int)e;
