@@ -31,51 +31,86 @@ std::string fmt(const char *f, long long a, long long b = 0, long long c = 0)
     return buf;
 }
 
-// The brick index of a tree whose leaves are all at depth D.  The leaves come
-// in Morton order (breadth-first order is that, here): those of a brick are
-// contiguous, and are renumbered into the order of the brick's mask bits, in
-// the permutation and in the nodes.
-void build_bricks(const fpo_tree_desc *tree, int D, PackedTree *out)
+// Packs a tree whose leaves are all at depth D (BRICK_MIN_DEPTH <= D <=
+// BRICK_MAX_DEPTH): the breadth-first nodes and the brick index, from the
+// sorted Morton codes alone.  Breadth-first order is Morton order, level by
+// level; the leaves of a brick are then put into the order of its mask bits.
+// key[i].first >> shift: code of the i-th leaf, key[i].second: its upload index.
+void pack_uniform(const std::vector<std::pair<uint64_t, uint32_t>> &key, int shift, int D, PackedTree *out)
 {
-    const uint32_t n = (uint32_t)out->perm.size();
+    const uint32_t n = (uint32_t)key.size();
+    auto code = [&](uint32_t i) { return key[i].first >> shift; };
+    uint8_t lin[64];  // x + 4y + 16z of a cell's Morton index in its brick
+    for (uint32_t m = 0; m < 64; ++m)
+        lin[m] = (uint8_t)((m & 1u) | ((m >> 2) & 2u) | (((m >> 1) & 1u) << 2) | (((m >> 4) & 1u) << 3) |
+                           (((m >> 2) & 1u) << 4) | ((m >> 5) << 5));
+    auto below = [](uint64_t mask, uint32_t bit) { return (uint32_t)__builtin_popcountll(mask & ((1ull << bit) - 1ull)); };
     const int tb = D - 4;
     const size_t T = (size_t)1 << tb;
     out->top.assign(T * T * T * 4, 0u);
-    std::vector<uint32_t> perm(n), renum(n);
-    struct Brick { uint32_t m[2], base; };
-    Brick found[64];  // the bricks of the current block, by mask bit
-    auto set = [](uint32_t m[2], uint32_t b) { m[b >> 5] |= 1u << (b & 31u); };
-    auto has = [](const uint32_t m[2], uint32_t b) { return (m[b >> 5] >> (b & 31u)) & 1u; };
-    auto cell = [&](uint32_t i, int k) { return tree->leaf_xyz[3 * (size_t)out->perm[i] + k]; };
-    uint32_t i = 0;
-    while (i < n) {  // a block of 16^3 cells
-        const uint32_t bx = cell(i, 0) >> 4, by = cell(i, 1) >> 4, bz = cell(i, 2) >> 4;
-        uint32_t bmask[2] = {0, 0};
-        while (i < n && cell(i, 0) >> 4 == bx && cell(i, 1) >> 4 == by && cell(i, 2) >> 4 == bz) {  // a brick
-            const uint32_t x = cell(i, 0) >> 2, y = cell(i, 1) >> 2, z = cell(i, 2) >> 2;
-            Brick b = {{0, 0}, i};
-            uint32_t order[64];
-            for (; i < n && cell(i, 0) >> 2 == x && cell(i, 1) >> 2 == y && cell(i, 2) >> 2 == z; ++i) {
-                const uint32_t bit = (cell(i, 0) & 3u) | ((cell(i, 1) & 3u) << 2) | ((cell(i, 2) & 3u) << 4);
-                set(b.m, bit);
-                order[bit] = i;
-            }
-            uint32_t at = b.base;
-            for (uint32_t bit = 0; bit < 64; ++bit)
-                if (has(b.m, bit)) {
-                    renum[order[bit]] = at;
-                    perm[at++] = out->perm[order[bit]];
+    out->perm.resize(n);
+    // level D - 1: parents of leaves; the leaves' numbers and the bricks
+    std::vector<std::vector<uint32_t>> slots(D);       // [level][8 x nodes], child numbers within the next level
+    std::vector<uint64_t> pre;                         // the nodes' codes at the current level
+    slots[D - 1].reserve((size_t)n * 2 + 8);
+    pre.reserve(n / 4 + 1);
+    struct Brick { uint64_t mask; uint32_t base; };
+    Brick found[64];
+    for (uint32_t i = 0; i < n;) {  // a block of 16^3 cells
+        const uint64_t block = code(i) >> 12;
+        uint64_t bmask = 0;
+        while (i < n && code(i) >> 12 == block) {  // a brick
+            const uint64_t brick = code(i) >> 6;
+            Brick b = {0, i};
+            uint32_t e = i;
+            for (; e < n && code(e) >> 6 == brick; ++e) b.mask |= 1ull << lin[code(e) & 63u];
+            for (; i < e; ++i) {
+                const uint32_t leaf = b.base + below(b.mask, lin[code(i) & 63u]);
+                out->perm[leaf] = key[i].second;
+                const uint64_t node = code(i) >> 3;
+                if (pre.empty() || pre.back() != node) {
+                    pre.push_back(node);
+                    slots[D - 1].resize(slots[D - 1].size() + 8, 0u);
                 }
-            const uint32_t j = (x & 3u) | ((y & 3u) << 2) | ((z & 3u) << 4);
-            set(bmask, j);
+                slots[D - 1][slots[D - 1].size() - 8 + (code(i) & 7u)] = LEAF_BIT | leaf;
+            }
+            const uint32_t j = lin[brick & 63u];
+            bmask |= 1ull << j;
             found[j] = b;
         }
-        uint32_t *t = &out->top[(((size_t)bz * T + by) * T + bx) * 4];
-        t[0] = bmask[0];
-        t[1] = bmask[1];
+        uint32_t x = 0, y = 0, z = 0;
+        for (int k = 0; k < tb; ++k) {
+            x |= (uint32_t)((block >> (3 * k)) & 1u) << k;
+            y |= (uint32_t)((block >> (3 * k + 1)) & 1u) << k;
+            z |= (uint32_t)((block >> (3 * k + 2)) & 1u) << k;
+        }
+        uint32_t *t = &out->top[(((size_t)z * T + y) * T + x) * 4];
+        t[0] = (uint32_t)bmask;
+        t[1] = (uint32_t)(bmask >> 32);
         t[2] = (uint32_t)(out->bricks.size() / 4);
-        for (uint32_t j = 0; j < 64; ++j)
-            if (has(bmask, j)) out->bricks.insert(out->bricks.end(), {found[j].m[0], found[j].m[1], found[j].base, 0u});
+        for (uint64_t m = bmask; m; m &= m - 1) {
+            const Brick &b = found[__builtin_ctzll(m)];
+            out->bricks.insert(out->bricks.end(), {(uint32_t)b.mask, (uint32_t)(b.mask >> 32), b.base, 0u});
+        }
+    }
+    for (int l = D - 2; l >= 0; --l) {
+        std::vector<uint64_t> up;
+        for (uint32_t i = 0; i < pre.size(); ++i) {
+            if (up.empty() || up.back() != pre[i] >> 3) {
+                up.push_back(pre[i] >> 3);
+                slots[l].resize(slots[l].size() + 8, 0u);
+            }
+            slots[l][slots[l].size() - 8 + (pre[i] & 7u)] = i + 1;  // (0 stays: empty)
+        }
+        pre.swap(up);
+    }
+    size_t total = 0;
+    for (const auto &s : slots) total += s.size();
+    out->nodes.reserve(total);
+    uint32_t next = 0;  // first node of the level after
+    for (int l = 0; l < D; ++l) {
+        next += (uint32_t)(slots[l].size() / 8);
+        for (const uint32_t c : slots[l]) out->nodes.push_back(c == 0u || (c & LEAF_BIT) ? c : next + c - 1);
     }
     // empty blocks: the side of the octree's empty cube that holds them
     for (size_t c = 0; c < T * T * T; ++c) {
@@ -93,9 +128,6 @@ void build_bricks(const fpo_tree_desc *tree, int D, PackedTree *out)
             }
         }
     }
-    for (uint32_t &s : out->nodes)
-        if (s & LEAF_BIT) s = LEAF_BIT | renum[s & ~LEAF_BIT];
-    out->perm.swap(perm);
 }
 
 }  // namespace
@@ -143,7 +175,7 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
         const int s = M - d;
         iv[j] = {interleave3(x << s, y << s, z << s), j};
     }
-    std::sort(iv.begin(), iv.end());
+    if (!std::is_sorted(iv.begin(), iv.end())) std::sort(iv.begin(), iv.end());
     for (uint32_t i = 0; i + 1 < n; ++i) {
         const uint32_t j = iv[i].second;
         const uint64_t len = 1ull << (3 * (M - (int)tree->leaf_depth[j]));
@@ -165,6 +197,12 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
         return FPO_OK;
     }
     out->root_kind = ROOT_NODE;
+    bool uniform = dmax >= BRICK_MIN_DEPTH && dmax <= BRICK_MAX_DEPTH;
+    for (uint32_t j = 0; j < n && uniform; ++j) uniform = tree->leaf_depth[j] == dmax;
+    if (uniform) {
+        pack_uniform(iv, 3 * (M - dmax), dmax, out);
+        return FPO_OK;
+    }
 
     // Temporary pointer tree: child >= 0 node, -1 empty, <= -2 leaf -(2 + id).
     struct TNode { int32_t c[8]; };
@@ -214,9 +252,6 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
             out->nodes[qi * 8 + c] = slot;
         }
     }
-    bool uniform = dmax >= BRICK_MIN_DEPTH && dmax <= BRICK_MAX_DEPTH;
-    for (uint32_t j = 0; j < n && uniform; ++j) uniform = tree->leaf_depth[j] == dmax;
-    if (uniform) build_bricks(tree, dmax, out);
     return FPO_OK;
 }
 
