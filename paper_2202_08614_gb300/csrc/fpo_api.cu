@@ -404,7 +404,7 @@ int check_render_opts(const fpo_ctx *ctx, const fpo_frame_opts *opts, uint64_t n
 
 // cos(pi x) and sin(pi x), exact at multiples of 1/2: x is reduced exactly to
 // [-1, 1] and then to a quarter period.
-static double cospi_h(double x, bool sine)
+double cospi_h(double x, bool sine)
 {
     x = std::remainder(x, 2.0);
     const double q = std::nearbyint(2.0 * x);

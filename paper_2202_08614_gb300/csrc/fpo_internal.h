@@ -126,6 +126,8 @@ struct FrameConsts {
     float f[3], r[3], u[3], eye[3];  // camera: forward, right, up, eye
     float sx_scale, sy_scale;        // tan(fov / 2) times the aspect ratio, and plain
 };
+// cos(pi x), or sin(pi x) with `sine`, on the host.
+double cospi_h(double x, bool sine);
 // Eq. 8 at time t for i < n into b (32 values, zero from n on).
 void time_basis(double t, double period_T, int n, float b[32]);
 

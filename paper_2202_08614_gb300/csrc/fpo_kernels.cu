@@ -1960,20 +1960,31 @@ int launch_set_coeffs(const float *src, const uint32_t *perm, float *sig, float 
 // takes at frames t = 1..T (the unified per-frame octrees).  One thread per
 // output coefficient (leaf, j): coalesced stores; the threads of one series
 // read the same per-frame value (L1 broadcast).  The DFT weights
-// (w_i / T) {cos, sin}, w_0 = 1, w_i = 2, come from FP64 into shared memory.
+// (w_i / T) {cos, sin}, w_0 = 1, w_i = 2, of coefficient i at frame t depend on
+// (h t) mod T only (harmonic h = i / 2 rounded up): the T distinct values are
+// computed on the host in FP64 and passed as kernel parameters.  (Every CTA
+// evaluating its 32 T weights in FP64 took a tenth of the launch.)
 
 constexpr int DFT_MAX_T = 256;
 
+struct DftWeights {
+    float c[DFT_MAX_T], s[DFT_MAX_T], w0;  // (2 / T) cos, sin(2 pi k / T); 1 / T
+};
+__device__ __forceinline__ float dft_weight(const DftWeights &W, int i, int t, int T)
+{
+    if (i == 0) return W.w0;
+    const int k = ((i + 1) / 2 * t) % T;
+    return (i & 1) ? W.s[k] : W.c[k];
+}
+
 __global__ void __launch_bounds__(256) dft_kernel(const float *__restrict__ values, float *__restrict__ coeffs,
-                                                  uint32_t n_leaves, int n1, int n2, int T)
+                                                  uint32_t n_leaves, int n1, int n2, int T,
+                                                  const __grid_constant__ DftWeights W)
 {
     __shared__ float s_w[32 * DFT_MAX_T];
     const int nb = n1 > n2 ? n1 : n2;
     for (int q = threadIdx.x; q < nb * T; q += blockDim.x) {
-        const int i = q / T, t = q % T + 1;
-        const double u = (double)t / (double)T;
-        const double w = (i == 0 ? 1.0 : 2.0) / (double)T;
-        s_w[q] = (float)(w * ((i & 1) ? sinpi((double)(i + 1) * u) : cospi((double)i * u)));
+        s_w[q] = dft_weight(W, q / T, q % T + 1, T);
     }
     __syncthreads();
     const int nc = n1 + 27 * n2;
@@ -2003,7 +2014,8 @@ __global__ void __launch_bounds__(256) dft_kernel(const float *__restrict__ valu
 constexpr int DFT_TILE = 32, DFT_TC = 8, DFT_XPAD = 29, DFT_N2 = 5;
 
 __global__ void __launch_bounds__(256) dft_tile_kernel(const float *__restrict__ values, float *__restrict__ coeffs,
-                                                       uint32_t n_leaves, int n1, int T)
+                                                       uint32_t n_leaves, int n1, int T,
+                                                       const __grid_constant__ DftWeights W)
 {
     extern __shared__ __align__(16) float dft_smem[];
     float *s_w = dft_smem;                          // [T][32]: weight of coefficient i at frame t
@@ -2012,9 +2024,7 @@ __global__ void __launch_bounds__(256) dft_tile_kernel(const float *__restrict__
     float *s_out = s_x + DFT_TC * DFT_TILE * DFT_XPAD;  // [32 leaves][nc]
     for (int q = threadIdx.x; q < 32 * T; q += blockDim.x) {
         const int t = q / 32, i = q % 32, nb = n1 > DFT_N2 ? n1 : DFT_N2;
-        const double u = (double)(t + 1) / (double)T;
-        const double w = (i == 0 ? 1.0 : 2.0) / (double)T;
-        s_w[q] = i < nb ? (float)(w * ((i & 1) ? sinpi((double)(i + 1) * u) : cospi((double)i * u))) : 0.0f;
+        s_w[q] = i < nb ? dft_weight(W, i, t + 1, T) : 0.0f;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int ser[4];
@@ -2129,7 +2139,8 @@ constexpr int DFT_FRAME_FLOATS = DFT_TILE * 28;  // one frame of a tile
 
 __global__ void __launch_bounds__(DFTB_THREADS) dft_bulk_kernel(const float *__restrict__ values,
                                                                 float *__restrict__ coeffs, uint32_t n_leaves,
-                                                                int n1, int T, uint32_t *status, bool test_timeout)
+                                                                int n1, int T, uint32_t *status, bool test_timeout,
+                                                                const __grid_constant__ DftWeights W)
 {
     extern __shared__ __align__(128) float dftb_smem[];
     __shared__ uint64_t bars[DFTB_STAGES];
@@ -2165,9 +2176,7 @@ __global__ void __launch_bounds__(DFTB_THREADS) dft_bulk_kernel(const float *__r
     }
     for (int q = threadIdx.x; q < 32 * T; q += blockDim.x) {
         const int t = q / 32, i = q % 32, nb = n1 > DFT_N2 ? n1 : DFT_N2;
-        const double u = (double)(t + 1) / (double)T;
-        const double w = (i == 0 ? 1.0 : 2.0) / (double)T;
-        s_w[q] = i < nb ? (float)(w * ((i & 1) ? sinpi((double)(i + 1) * u) : cospi((double)i * u))) : 0.0f;
+        s_w[q] = i < nb ? dft_weight(W, i, t + 1, T) : 0.0f;
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2270,6 +2279,12 @@ int launch_dft(const float *values, float *coeffs, uint32_t n_leaves, int n1, in
                bool test_timeout, int sm_count, void *stream)
 {
     if (n_leaves == 0) return (int)cudaSuccess;
+    DftWeights W;
+    W.w0 = (float)(1.0 / T);
+    for (int k = 0; k < DFT_MAX_T; ++k) {
+        W.c[k] = k < T ? (float)(2.0 / T * cospi_h(2.0 * k / T, false)) : 0.0f;
+        W.s[k] = k < T ? (float)(2.0 / T * cospi_h(2.0 * k / T, true)) : 0.0f;
+    }
     // bulk copies need a 16-byte aligned base (every frame row of a tile
     // starts a multiple of 112 bytes further); other bases take the tile kernel
     if (n2 == DFT_N2 && n1 <= 32 && (reinterpret_cast<uintptr_t>(values) & 15u) == 0) {
@@ -2286,7 +2301,7 @@ int launch_dft(const float *values, float *coeffs, uint32_t n_leaves, int n1, in
         uint64_t blocks = (uint64_t)sm_count * per_sm;
         if (blocks > n_tiles) blocks = n_tiles;
         dft_bulk_kernel<<<(unsigned)blocks, DFTB_THREADS, smem, (cudaStream_t)stream>>>(values, coeffs, n_leaves, n1, T,
-                                                                                         status, test_timeout);
+                                                                                         status, test_timeout, W);
         return (int)cudaGetLastError();
     }
     if (n2 == DFT_N2 && n1 <= 32) {
@@ -2301,13 +2316,13 @@ int launch_dft(const float *values, float *coeffs, uint32_t n_leaves, int n1, in
         const uint64_t n_tiles = (n_leaves + DFT_TILE - 1) / DFT_TILE;
         uint64_t blocks = (uint64_t)sm_count * per_sm;
         if (blocks > n_tiles) blocks = n_tiles;
-        dft_tile_kernel<<<(unsigned)blocks, 256, smem, (cudaStream_t)stream>>>(values, coeffs, n_leaves, n1, T);
+        dft_tile_kernel<<<(unsigned)blocks, 256, smem, (cudaStream_t)stream>>>(values, coeffs, n_leaves, n1, T, W);
         return (int)cudaGetLastError();
     }
     const uint64_t total = (uint64_t)n_leaves * (n1 + 27 * n2);
     uint64_t blocks = (total + 255) / 256;
     if (blocks > (uint64_t)sm_count * 32) blocks = (uint64_t)sm_count * 32;
-    dft_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(values, coeffs, n_leaves, n1, n2, T);
+    dft_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(values, coeffs, n_leaves, n1, n2, T, W);
     return (int)cudaGetLastError();
 }
 
