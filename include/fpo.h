@@ -461,6 +461,20 @@ int fpo_adam(float *param, const float *grad, float *m, float *v, uint64_t n, co
              uint32_t dim, float lr, float beta1, float beta2, float eps, uint32_t step,
              void *cuda_stream);
 
+/* fpo_adam on up to 8 arrays in one launch (a model's weight arrays and the
+ * batch's latent rows), each with its learning rate; the gradient is first
+ * multiplied by grad_scale, and written back scaled unless that is 1.  The
+ * arrays of two parts must not overlap.  Errors: INVALID_ARG, CUDA. */
+typedef struct {
+    float *param, *grad, *m, *v;
+    uint64_t n;
+    const uint32_t *rows; /* as for fpo_adam: NULL, or device [n / dim] */
+    uint32_t dim;
+    float lr, grad_scale;
+} fpo_adam_part;
+int fpo_adam_parts(const fpo_adam_part *parts, uint32_t n_parts, float beta1, float beta2, float eps, uint32_t step,
+                   void *cuda_stream);
+
 /* LATENT storage: gives the uploaded tree its per-leaf latents (device FP16
  * [n_leaves][32], upload order) and decoder (device arrays, copied into the
  * context).  fpo_render then decodes the per-frame table with

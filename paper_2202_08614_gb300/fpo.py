@@ -35,7 +35,8 @@ EXPORTS = ["fpo_create", "fpo_validate_tree", "fpo_upload_tree", "fpo_render",
            "fpo_last_error", "fpo_version", "fpo_render_noalloc", "fpo_set_coeffs",
            "fpo_dft_leaves", "fpo_union_trees", "fpo_latent_table", "fpo_decoder_grad",
            "fpo_adam", "fpo_set_latents", "fpo_render_frames", "fpo_adam_leaves",
-           "fpo_decoder_forward", "fpo_set_coeffs_from_decoder", "fpo_fma_peak", "fpo_decoder_grad_tc"]
+           "fpo_decoder_forward", "fpo_set_coeffs_from_decoder", "fpo_fma_peak", "fpo_decoder_grad_tc",
+           "fpo_adam_parts"]
 
 
 class FPOError(RuntimeError):
@@ -86,6 +87,12 @@ class Mlp(C.Structure):
                 ("w3", C.c_void_p), ("b3", C.c_void_p)]
 
 
+class AdamPart(C.Structure):
+    _fields_ = [("param", C.c_void_p), ("grad", C.c_void_p), ("m", C.c_void_p), ("v", C.c_void_p),
+                ("n", C.c_uint64), ("rows", C.c_void_p), ("dim", C.c_uint32), ("lr", C.c_float),
+                ("grad_scale", C.c_float)]
+
+
 class TreeInfo(C.Structure):
     _fields_ = [("n_leaves", C.c_uint32), ("n_nodes", C.c_uint32), ("max_depth", C.c_uint32),
                 ("n_smem_nodes", C.c_uint32), ("node_bytes", C.c_uint64),
@@ -123,6 +130,8 @@ def lib():
         L.fpo_fma_peak.argtypes = [C.c_uint32, C.c_uint32, C.c_uint32, P, C.POINTER(C.c_double), P]
         L.fpo_adam.argtypes = [P, P, P, P, C.c_uint64, P, C.c_uint32, C.c_float, C.c_float,
                                C.c_float, C.c_float, C.c_uint32, P]
+        L.fpo_adam_parts.argtypes = [C.POINTER(AdamPart), C.c_uint32, C.c_float, C.c_float, C.c_float,
+                                     C.c_uint32, P]
         L.fpo_set_latents.argtypes = [P, P, C.POINTER(Decoder), P]
         L.fpo_render_frames.argtypes = [P, P, C.c_uint32, C.POINTER(FrameOpts), P, P, P]
         L.fpo_adam_leaves.argtypes = [P, P, P, P, P, P, C.c_float, C.c_float, C.c_float, C.c_float,

@@ -42,7 +42,13 @@ class LatentModel:
         }
         self.m = {k: torch.zeros_like(v) for k, v in self.p.items()}
         self.v = {k: torch.zeros_like(v) for k, v in self.p.items()}
-        self.g = {k: torch.zeros_like(v) for k, v in self.p.items() if k != "lat"}
+        # the weight gradients are views of one array, cleared and scaled as one
+        self._g = torch.zeros(sum(v.numel() for k, v in self.p.items() if k != "lat"), device=device)
+        self.g, at = {}, 0
+        for k, v in self.p.items():
+            if k != "lat":
+                self.g[k] = self._g[at:at + v.numel()].view_as(v)
+                at += v.numel()
         self.step_count = 0
 
     def state_dict(self):
@@ -84,8 +90,7 @@ class LatentModel:
         import torch
 
         if not accumulate:
-            for t in self.g.values():
-                t.zero_()
+            self._g.zero_()
         b = rows.shape[0]
         dl = torch.empty((b, 32), device=rows.device)
         loss = torch.zeros(1, dtype=torch.float64, device=rows.device)
@@ -118,13 +123,17 @@ class LatentModel:
                                                 C.c_void_p(fpo._stream_handle(stream))))
         return out
 
-    def _adam(self, key, grad, lr, rows=None, dim=0, stream=None):
-        p, m, v = self.p[key], self.m[key], self.v[key]
-        n = grad.numel()
-        fpo.check(fpo.lib().fpo_adam(
-            C.c_void_p(p.data_ptr()), C.c_void_p(grad.data_ptr()), C.c_void_p(m.data_ptr()),
-            C.c_void_p(v.data_ptr()), n, C.c_void_p(rows.data_ptr() if rows is not None else None),
-            dim, lr, 0.9, 0.999, 1e-8, self.step_count, C.c_void_p(fpo._stream_handle(stream))))
+    def _adam(self, parts, stream=None):
+        """One Adam launch; parts: (key, gradient, learning rate, gradient scale, rows or None)."""
+        arr = (fpo.AdamPart * len(parts))()
+        for a, (key, grad, lr, scale, rows) in zip(arr, parts):
+            p = self.p[key]
+            a.param, a.grad, a.m, a.v = p.data_ptr(), grad.data_ptr(), self.m[key].data_ptr(), self.v[key].data_ptr()
+            a.n, a.lr, a.grad_scale = grad.numel(), lr, scale
+            if rows is not None:
+                a.rows, a.dim = rows.data_ptr(), p.shape[1]
+        fpo.check(fpo.lib().fpo_adam_parts(arr, len(parts), 0.9, 0.999, 1e-8, self.step_count,
+                                           C.c_void_p(fpo._stream_handle(stream))))
 
     def step(self, rows, targets, coef_weight, lr_w=1e-3, lr_lat=1e-2, pixel=None):
         """One Adam step on the batch `rows` (mean weighted L2 to `targets`).
@@ -133,21 +142,19 @@ class LatentModel:
         by leaf, [n, nc], already a mean over rays), added to the gradients."""
         dl, loss = self.grad(rows, targets, coef_weight)
         self.step_count += 1
-        scale = 1.0 / rows.shape[0]
-        for k in self.g:
-            self.g[k].mul_(scale)
-        dl.mul_(scale)
+        scale = w_scale = 1.0 / rows.shape[0]
         dl_px = None
         if pixel is not None:
             rows_px, dy = pixel
             if rows_px.shape[0]:
+                self._g.mul_(scale)  # the pixel term's gradients are a mean already
+                w_scale = 1.0
                 dl_px, _ = self.grad(rows_px, targets, self._zero_weight(targets.device), extra_dy=dy,
                                      accumulate=True)
-        for k in ("w1", "b1", "w2", "b2", "w3", "b3"):
-            self._adam(k, self.g[k], lr_w)
-        self._adam("lat", dl, lr_lat, rows=rows, dim=32)
+        self._adam([(k, self.g[k], lr_w, w_scale, None) for k in ("w1", "b1", "w2", "b2", "w3", "b3")] +
+                   [("lat", dl, lr_lat, scale, rows)])
         if dl_px is not None:
-            self._adam("lat", dl_px, lr_lat, rows=pixel[0], dim=32)
+            self._adam([("lat", dl_px, lr_lat, 1.0, pixel[0])])
         return loss
 
     def _zero_weight(self, device):
