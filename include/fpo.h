@@ -170,7 +170,15 @@ enum {
      * fpo_set_coeffs_from_decoder take it too, each as it documents.) */
     FPO_FLAG_TEST_DEVICE_TIMEOUT = 64,
     /* fpo_set_coeffs_from_decoder: decode on the tensor cores. */
-    FPO_FLAG_TENSOR_CORES = 128
+    FPO_FLAG_TENSOR_CORES = 128,
+    /* fpo_render_backward (FP32): keep the gradient in the context, as a list
+     * of leaf visits, for the next fpo_adam_leaves, instead of adding every
+     * visit's n1 + 27 n2 values to dL_dcoeffs.  Visits that do not fit the
+     * list are added to dL_dcoeffs and their leaves marked as usual (so both
+     * arrays are still needed, and FPO_FLAG_MARK_LEAVES with them): pass the
+     * same two arrays to fpo_adam_leaves.  A list that fpo_adam_leaves has
+     * not consumed is dropped by fpo_upload_tree and fpo_set_coeffs. */
+    FPO_FLAG_DEFER_GRADIENT = 256
 };
 
 /* Per-call options.  bg: background colour added with the final
@@ -263,7 +271,12 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * Of the debug flags only FPO_FLAG_MARK_LEAVES is honoured: it sets
  * leaf_mark[id] = 1 for every leaf the replay visits (the rows that receive
  * gradient), which fpo_adam_leaves consumes; the others are ignored.
- * FPO_FLAG_FP64_GRADCHECK selects the FP64 replay (see the flag).
+ * FPO_FLAG_FP64_GRADCHECK selects the FP64 replay, FPO_FLAG_DEFER_GRADIENT
+ * leaves the gradient to the next fpo_adam_leaves (see the flags).
+ * Batches of up to 262,144 rays keep their visits in a workspace of the
+ * context (grown on the first larger batch outside a stream capture, at most
+ * 0.4 GB) and add them to dL_dcoeffs in a second, evenly divided pass; other
+ * calls, and visits beyond the workspace, add them from the replay.
  * Errors: INVALID_ARG, NO_TREE, UNSUPPORTED, CUDA. */
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
                         const float *out_rgb, const float *dL_drgb, float *dL_dcoeffs,
@@ -301,7 +314,8 @@ int fpo_set_coeffs(fpo_ctx *ctx, const float *coeffs, void *cuda_stream);
  * on the leaves a batch visited: Adam (Kingma & Ba; lr, beta1, beta2, eps,
  * step >= 1 for the bias corrections 1 - beta^step) on every row of param
  * whose leaf_mark is non-zero, using the gradient row of grad (as
- * accumulated by fpo_render_backward with FPO_FLAG_MARK_LEAVES), with the
+ * accumulated by fpo_render_backward with FPO_FLAG_MARK_LEAVES), or that a
+ * FPO_FLAG_DEFER_GRADIENT call since the last step visited (their sums), with the
  * moment rows m and v (zero before the first step).  Rows without a mark are
  * left alone, as in a sparse-gradient Adam.  For each updated leaf the new
  * coefficients also go into the context's FP32 records (what fpo_set_coeffs

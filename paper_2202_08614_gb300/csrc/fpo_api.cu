@@ -96,6 +96,11 @@ constexpr int DEFAULT_TRAVERSE_THREADS = 256;
 constexpr uint32_t DEFAULT_REFILL_MIN = 32;
 constexpr uint32_t DEFAULT_INNER_STEPS = 0xffffffffu;  // a lane runs its ray to the end
 
+// Visit list of an adjoint call: batches of up to VL_MAX_RAYS rays, room for
+// VL_PER_RAY visits a ray (the 3.5M-leaf body: 15 on average), counter words.
+constexpr uint32_t VL_MAX_RAYS = 1u << 18, VL_PER_RAY = 32;
+constexpr int VL_COUNT = 24;
+
 }  // namespace
 
 struct fpo_ctx {
@@ -132,10 +137,30 @@ struct fpo_ctx {
     size_t ptable_leaves[PIPE_MAX] = {};
     cudaStream_t aux = nullptr;           // IDFT passes / decodes
     cudaStream_t trav[PIPE_MAX] = {};     // slots 1.. : their traversal streams
+    // visits of an adjoint call (VisitList), grown by ensure_visit_list
+    uint2 *d_vl_id = nullptr;
+    float4 *d_vl_val = nullptr;
+    uint32_t *d_vl_next = nullptr, *d_vl_head = nullptr;
+    float *d_vl_w = nullptr;
+    uint32_t vl_cap = 0, vl_rays = 0;   // entries; rays with room for weights
+    uint32_t vl_used = 0;               // rays whose visits await fpo_adam_leaves
     cudaEvent_t ev_entry = nullptr, ev_mat[PIPE_MAX] = {}, ev_trav[PIPE_MAX] = {};
+
+    void free_visit_list()
+    {
+        dfree(d_vl_id);
+        dfree(d_vl_val);
+        dfree(d_vl_next);
+        dfree(d_vl_w);
+        vl_cap = vl_rays = 0;
+    }
 
     void free_tree()
     {
+        free_visit_list();
+        dfree(d_vl_head);
+        vl_used = 0;
+        if (d_status) cudaMemset(d_status + VL_COUNT, 0, 2 * sizeof(uint32_t));
         dfree(d_nodes);
         dfree(d_top);
         dfree(d_bricks);
@@ -787,6 +812,79 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
     return FPO_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The context's visit list for an adjoint call over n_rays rays.  It stays
+// empty (cap 0: the replay adds its rows itself) for large batches, when the
+// workspace would have to grow during a stream capture or while it holds
+// deferred visits, or when there is no memory for it.
+VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
+{
+    VisitList L{};
+    if (n_rays > VL_MAX_RAYS || (c->vl_used && !defer)) return L;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return L;
+    }
+    const bool may_alloc = cap == cudaStreamCaptureStatusNone;
+    const uint32_t n = (uint32_t)n_rays;
+    if (c->vl_used + n > c->vl_rays) {
+        if (c->vl_used || !may_alloc) return L;
+        c->free_visit_list();
+        uint32_t room = 4096;  // rays, in powers of two
+        while (room < n) room *= 2;
+        const size_t e = (size_t)room * VL_PER_RAY, nw = (size_t)c->cfg.n1 + 9 * (size_t)c->cfg.n2;
+        cudaError_t err = cudaMalloc((void **)&c->d_vl_id, e * sizeof(uint2));
+        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_val, e * sizeof(float4));
+        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_next, e * sizeof(uint32_t));
+        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_w, (size_t)room * nw * sizeof(float));
+        if (err != cudaSuccess) {
+            cudaGetLastError();
+            c->free_visit_list();
+            return L;
+        }
+        c->vl_cap = (uint32_t)e;
+        c->vl_rays = room;
+    }
+    if (defer && !c->d_vl_head) {
+        if (!may_alloc || cudaMalloc((void **)&c->d_vl_head, (size_t)c->n_leaves * 4) != cudaSuccess) {
+            cudaGetLastError();
+            return L;
+        }
+        if (cudaMemsetAsync(c->d_vl_head, 0xff, (size_t)c->n_leaves * 4, s) != cudaSuccess) {
+            cudaGetLastError();
+            dfree(c->d_vl_head);
+            return L;
+        }
+    }
+    L.cap = c->vl_cap;
+    L.count = c->d_status + VL_COUNT;
+    L.id = c->d_vl_id;
+    L.val = c->d_vl_val;
+    L.head = defer ? c->d_vl_head : nullptr;
+    L.next = c->d_vl_next;
+    L.w = c->d_vl_w;
+    L.ray_base = c->vl_used;
+    return L;
+}
+
+// Deferred visits that no fpo_adam_leaves has taken are forgotten.
+cudaError_t drop_visits(fpo_ctx *c, cudaStream_t s)
+{
+    if (!c->vl_used) return cudaSuccess;
+    c->vl_used = 0;
+    cudaError_t e = cudaMemsetAsync(c->d_vl_head, 0xff, (size_t)c->n_leaves * 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status + VL_COUNT, 0, 2 * sizeof(uint32_t), s);
+    return e;
+}
+
+}  // namespace
+
+extern "C" {
+
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
                         const float *out_rgb, const float *dL_drgb, float *dL_dcoeffs,
                         void *cuda_stream)
@@ -811,6 +909,9 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
     const bool mark = (opts->flags & FPO_FLAG_MARK_LEAVES) != 0;
     if (mark && !opts->leaf_mark) return fail(FPO_ERR_INVALID_ARG, "FPO_FLAG_MARK_LEAVES needs leaf_mark");
+    const bool defer = (opts->flags & FPO_FLAG_DEFER_GRADIENT) != 0;
+    if (defer && (fp64 || !mark))
+        return fail(FPO_ERR_INVALID_ARG, "FPO_FLAG_DEFER_GRADIENT needs FPO_FLAG_MARK_LEAVES and the FP32 adjoint");
     fpo_frame_opts o = *opts;
     o.flags = 0;  // the other debug outputs belong to the forward
     BackwardParams q{};
@@ -820,8 +921,15 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     q.dL_dcoeffs = fp64 ? nullptr : dL_dcoeffs;
     q.dL_dcoeffs64 = fp64 ? reinterpret_cast<double *>(dL_dcoeffs) : nullptr;
     q.leaf_mark = mark ? opts->leaf_mark : nullptr;
-    const int ce = launch_backward(q, ctx->sm_count, cuda_stream);
+    if (!fp64) q.list = visit_list(ctx, n_rays, defer, (cudaStream_t)cuda_stream);
+    int ce = launch_backward(q, ctx->sm_count, cuda_stream);
     if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
+    if (q.list.cap && defer) {
+        ctx->vl_used += (uint32_t)n_rays;
+    } else if (q.list.cap) {
+        ce = launch_grad_scatter(q, ctx->sm_count, cuda_stream);
+        if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "gradient scatter launch");
+    }
     return FPO_OK;
 }
 
@@ -869,6 +977,8 @@ int fpo_set_coeffs(fpo_ctx *ctx, const float *coeffs, void *cuda_stream)
     ctx->table_ok = false;  // the coefficients change
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
+    const cudaError_t de = drop_visits(ctx, (cudaStream_t)cuda_stream);
+    if (de != cudaSuccess) return cuda_fail(de, "visit list reset");
     const int ce = launch_set_coeffs(coeffs, ctx->d_perm, static_cast<float *>(ctx->d_sig),
                                      static_cast<float *>(ctx->d_z), ctx->n_leaves, ctx->cfg.n1,
                                      ctx->cfg.n2, ctx->sm_count, cuda_stream);
@@ -939,8 +1049,18 @@ int fpo_adam_leaves(fpo_ctx *ctx, float *param, float *grad, float *m, float *v,
     p.eps = eps;
     p.bc1 = (float)(1.0 - std::pow((double)beta1, (double)step));
     p.bc2 = (float)(1.0 - std::pow((double)beta2, (double)step));
+    if (ctx->vl_used) {
+        p.list.cap = ctx->vl_cap;
+        p.list.count = ctx->d_status + VL_COUNT;
+        p.list.id = ctx->d_vl_id;
+        p.list.val = ctx->d_vl_val;
+        p.list.head = ctx->d_vl_head;
+        p.list.next = ctx->d_vl_next;
+        p.list.w = ctx->d_vl_w;
+    }
     const int ce = launch_leaf_adam(p, ctx->sm_count, cuda_stream);
     if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "adam_leaves launch");
+    ctx->vl_used = 0;
     return FPO_OK;
 }
 

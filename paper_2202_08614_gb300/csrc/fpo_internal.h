@@ -283,7 +283,21 @@ int launch_decode_records_tc(const fpo_mlp &w, int n1, int n2, uint32_t n, const
 int launch_adam(const fpo_adam_part *parts, uint32_t n_parts, float b1, float b2, float eps, uint32_t step, int sm_count,
                 void *stream);
 
+// Visits of an adjoint call, kept for a second pass (a workspace of the
+// context): what a visit adds to the gradient row of its leaf is the outer
+// product of 4 numbers (dL/dsigma_raw and dL/du_c) and its ray's weights.
+struct VisitList {
+    uint32_t cap;             // entries; 0: no list
+    uint32_t *count;          // [0] entries appended (may exceed cap), [1] finished warps of the pass over them
+    uint2 *id;                // upload leaf id, ray (ray_base + index in the call)
+    float4 *val;
+    uint32_t *head, *next;    // deferred gradients: per leaf, its last entry and the one before each; else nullptr
+    float *w;                 // [rays][n1 + 9 n2]: IDFT_i(t), then Y_k(d) IDFT_i(t)
+    uint32_t ray_base;
+};
+
 struct BackwardParams {
+    VisitList list;
     TraverseParams tp;          // rays, tree and options as for the fused forward
     const float *out_rgb;       // forward colour [rays][3]
     const float *dL_drgb;       // [rays][3]
@@ -303,6 +317,7 @@ struct LeafAdamParams {
     uint32_t n_leaves;
     int n1, n2, sig_stride, z_stride;
     float lr, beta1, beta2, eps, bc1, bc2;  // bc = 1 - beta^step
+    VisitList list;               // the deferred gradient (cap 0: none)
 };
 
 // Launchers (return cudaError_t as int).
@@ -317,6 +332,8 @@ struct MatShape {
 MatShape materialise_pipeline_shape(int storage, int n1, int n2, int smem_budget);
 int materialise_smem_bytes(const MaterialiseParams &p);  // dynamic shared memory of one CTA
 int launch_backward(const BackwardParams &q, int sm_count, void *stream);
+// Adds the list's visits to q.dL_dcoeffs and empties it.
+int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream);
 int launch_dft(const float *values, float *coeffs, uint32_t n_leaves, int n1, int n2, int T, uint32_t *status,
                bool test_timeout, int sm_count, void *stream);
 int launch_set_coeffs(const float *src, const uint32_t *perm, float *sig, float *zc, uint32_t n_leaves,

@@ -1266,8 +1266,12 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 //   composite  lane l takes its own visits in order; a ray that falls below
 //              stop_T ignores the rest of its list (at most a list's worth of
 //              visits is evaluated for nothing);
-//   scatter    (adjoint) all 32 lanes add a visit's gradient row with
-//              contiguous 8-byte vector atomics.
+//   scatter    (adjoint) the visits go to a list in global memory, from which
+//              grad_scatter_kernel or the leaf Adam takes them; without one, or
+//              when it is full, all 32 lanes add a visit's gradient row with
+//              contiguous 8-byte vector atomics (a row a visit: added from
+//              here, the rows of the rays that run longest came last and
+//              alone).
 // The one-lane-per-ray form that this replaces read 21 scattered 32-byte
 // pieces per visit in each lane, with the whole warp waiting for the few
 // lanes that were inside a leaf, and left most SMs idle below 38,912 rays.
@@ -1386,6 +1390,7 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
             for (uint32_t f = fresh; f; f &= f - 1u) {
                 const int r = __ffs((int)f) - 1;
                 const float ur = __shfl_sync(0xffffffffu, u, r);
+                const uint32_t rr = ADJ ? __shfl_sync(0xffffffffu, ray, r) : 0u;
                 float yk = 0.0f;  // lane k < 9: Y_k
 #pragma unroll
                 for (int k = 0; k < 9; ++k) {
@@ -1401,7 +1406,9 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
                     const int e = 32 * h + lane, el = e % S::NZ;
                     const float x = __shfl_sync(0xffffffffu, yk, el / N2) * __shfl_sync(0xffffffffu, b, el % N2);
                     if (e < 4 * S::ZC) w[e] = e < 27 * N2 ? x : 0.0f;
+                    if (ADJ && q.list.cap && e < S::NZ) q.list.w[(size_t)(q.list.ray_base + rr) * (N1 + S::NZ) + N1 + e] = x;
                 }
+                if (ADJ && q.list.cap && lane < N1) q.list.w[(size_t)(q.list.ray_base + rr) * (N1 + S::NZ) + lane] = b;
             }
             if (mine) {
                 if (ADJ) {
@@ -1464,12 +1471,6 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
                     const char *a = l == 0 ? reinterpret_cast<const char *>(p.sig) + (size_t)lf * sb
                                            : reinterpret_cast<const char *>(p.zc) + (size_t)lf * zb + (l - 1) * 128u;
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-                }
-                if (ADJ) {  // and those of the gradient rows, which the reductions then find there
-                    constexpr uint32_t GN = (S::NC * 4 + 127) / 128;
-                    for (uint32_t e = lane; e < n * GN; e += 32)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(
-                                         q.dL_dcoeffs + (size_t)p.perm[ent[e / GN].x] * S::NC) + e % GN * 128u));
                 }
             }
 
@@ -1574,15 +1575,33 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
 
             // --- scatter
             if (ADJ) {
-                for (uint32_t v = lane; v < n; v += 32) {  // leaf -> row of the gradient
-                    if (ent[v].x == 0xffffffffu) continue;
-                    const uint32_t id = p.perm[ent[v].x];
-                    ent[v].x = id;
-                    if (q.leaf_mark) q.leaf_mark[id] = 1;
+                // into the list (a leaf's row from here on is its upload id); what
+                // does not fit is added here
+                bool here = false;
+                for (uint32_t v0 = 0; v0 < n; v0 += 32) {
+                    const uint32_t v = v0 + (uint32_t)lane;
+                    const uint4 en = v < n ? ent[v] : make_uint4(0xffffffffu, 0u, 0u, 0u);
+                    const bool ok = en.x != 0xffffffffu;
+                    const uint32_t mask = __ballot_sync(0xffffffffu, ok);
+                    const uint32_t rr = __shfl_sync(0xffffffffu, ray, (int)en.z);
+                    const uint32_t id = ok ? p.perm[en.x] : 0xffffffffu;
+                    uint32_t at = 0xffffffffu;
+                    if (q.list.cap && mask) {
+                        if (lane == 0) at = atomicAdd(q.list.count, (uint32_t)__popc(mask));
+                        at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & lt_mask);
+                    }
+                    const bool listed = ok && at < q.list.cap;
+                    if (listed) {
+                        q.list.id[at] = make_uint2(id, q.list.ray_base + rr);
+                        q.list.val[at] = reinterpret_cast<const float4 *>(res)[v];
+                        if (q.list.head) q.list.next[at] = atomicExch(q.list.head + id, at);
+                    }
+                    if (v < n) ent[v].x = listed ? 0xffffffffu : id;
+                    if (ok && q.leaf_mark && !(listed && q.list.head)) q.leaf_mark[id] = 1;
+                    here |= __any_sync(0xffffffffu, ok && !listed);
                 }
                 __syncwarp();
-#pragma unroll 2
-                for (uint32_t v = 0; v < n; ++v) {
+                for (uint32_t v = 0; here && v < n; ++v) {
                     const uint4 en = ent[v];
                     if (en.x == 0xffffffffu) continue;
                     const float *w = wt + en.z * S::WROW;
@@ -1882,6 +1901,72 @@ static int launch_b64(const BackwardParams &q, int sm_count, cudaStream_t s)
     if (need < blocks) blocks = need ? need : 1;
     k<<<(unsigned)blocks, threads, smem, s>>>(q);
     return (int)cudaGetLastError();
+}
+
+// The gradient rows of the list's visits into dL_dcoeffs: a warp takes 32
+// entries at a time, a row by contiguous 8-byte vector atomics.  Bound by the
+// random read-modify-write of the rows in DRAM (1M rows of a 2.3 GB array:
+// 0.31 ms with any coalesced form of atomic, plain read-add-write included).
+template <int N1, int N2>
+__global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list, float *grad)
+{
+    constexpr int NZ = 9 * N2, NC = N1 + 27 * N2, RN = (NC + 63) / 64;
+    const int lane = threadIdx.x & 31;
+    const uint32_t n = min(*list.count, list.cap);
+    const uint32_t warps = gridDim.x * blockDim.x / 32;
+    // the weight and value index of this lane's elements
+    int wi[2 * RN], ci[2 * RN];
+#pragma unroll
+    for (int r = 0; r < RN; ++r)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = min(64 * r + 2 * lane + h, NC - 1), j = k - N1;
+            wi[2 * r + h] = j < 0 ? k : N1 + j % NZ;
+            ci[2 * r + h] = j < 0 ? 0 : 1 + j / NZ;
+        }
+    for (uint32_t v0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * 32; v0 < n; v0 += warps * 32) {
+        const uint32_t v = v0 + (uint32_t)lane;
+        const uint2 id = v < n ? list.id[v] : make_uint2(0u, 0u);
+        const float4 val = v < n ? list.val[v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const int m = (int)min(32u, n - v0);
+#pragma unroll 2
+        for (int i = 0; i < m; ++i) {
+            float *row = grad + (size_t)__shfl_sync(0xffffffffu, id.x, i) * NC;
+            const float *w = list.w + (size_t)__shfl_sync(0xffffffffu, id.y, i) * (N1 + NZ);
+            const float c0 = __shfl_sync(0xffffffffu, val.x, i), c1 = __shfl_sync(0xffffffffu, val.y, i),
+                        c2 = __shfl_sync(0xffffffffu, val.z, i), c3 = __shfl_sync(0xffffffffu, val.w, i);
+            auto gval = [&](int q) {
+                const float c = ci[q] == 0 ? c0 : (ci[q] == 1 ? c1 : (ci[q] == 2 ? c2 : c3));
+                return c * __ldg(w + wi[q]);
+            };
+#pragma unroll
+            for (int r = 0; r < RN; ++r)
+                if (64 * r + 2 * lane < NC)
+                    atomicAdd(reinterpret_cast<float2 *>(row + 64 * r + 2 * lane), make_float2(gval(2 * r), gval(2 * r + 1)));
+        }
+    }
+    // the last warp empties the list
+    if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(list.count + 1, 1u) == warps - 1) {
+            atomicExch(list.count, 0u);
+            atomicExch(list.count + 1, 0u);
+        }
+    }
+}
+
+int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream)
+{
+    const int n1 = q.tp.n1, n2 = q.tp.n2;
+    auto go = [&](auto kern) {
+        kern<<<(unsigned)sm_count * 4u, 256, 0, (cudaStream_t)stream>>>(q.list, q.dL_dcoeffs);
+        return (int)cudaGetLastError();
+    };
+    if (n1 == 31 && n2 == 5) return go(grad_scatter_kernel<31, 5>);
+    if (n1 == 11 && n2 == 5) return go(grad_scatter_kernel<11, 5>);
+    if (n1 == 21 && n2 == 5) return go(grad_scatter_kernel<21, 5>);
+    if (n1 == 31 && n2 == 11) return go(grad_scatter_kernel<31, 11>);
+    return -1;
 }
 
 int launch_backward(const BackwardParams &q, int sm_count, void *stream)

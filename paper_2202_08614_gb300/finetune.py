@@ -4,11 +4,12 @@ pixel error of Eq. 13 over rays drawn from the training views and frames.
 One step on a batch of explicit rays with per-ray frame times:
   forward   fpo_render (per-visit IDFT, since every ray has its own t),
   loss      mean over rays of the squared RGB error, dL/drgb = 2 (rgb - y) / B,
-  adjoint   fpo_render_backward into a dense gradient buffer, marking the
-            leaves it touches,
-  update    fpo_adam_leaves: Adam on the marked rows only, written straight
-            into the renderer's FP32 records; the gradient rows and marks are
-            reset in the same pass.
+  adjoint   fpo_render_backward, which leaves the gradient in the renderer as a
+            list of leaf visits (and takes the dense gradient buffer and the
+            marks for visits beyond the list),
+  update    fpo_adam_leaves: Adam on the visited leaves' rows only, written
+            straight into the renderer's FP32 records; lists, gradient rows and
+            marks are reset in the same pass.
 Nothing in a step waits for the host.  Rows the batch did not visit keep their
 moments (a sparse-gradient Adam): with a 3.5M-leaf tree a batch of 65,536
 rays touches a small fraction of the rows, and a dense update would move all
@@ -107,7 +108,7 @@ class FineTuner:
         dl = diff * (2.0 / max(1, rgb.shape[0]))
         rec(1)
         self.r.render_backward(rgb, dl, self.grad, rays_o=rays_o, rays_d=rays_d, t_per_ray=t, bg=self.bg,
-                               stop_T=self.stop_T, leaf_mark=self.mark)
+                               stop_T=self.stop_T, leaf_mark=self.mark, defer=True)
         rec(2)
         self.steps += 1
         self.r.adam_leaves(self.param, self.grad, self.m, self.v, self.mark, self.steps, lr=self.lr,

@@ -27,7 +27,7 @@ IDFT = {"auto": 0, "fused": 1, "materialise": 2}
 TABLE = {"auto": 0, "f32": 1, "f16": 2}
 RAYS_CAMERA, RAYS_EXPLICIT = 0, 1
 FLAG_RECORD_VISITS, FLAG_OUT_T, FLAG_MARK_LEAVES, FLAG_STATS, FLAG_REUSE_TABLE = 1, 2, 4, 8, 16
-FLAG_FP64_GRADCHECK, FLAG_TEST_DEVICE_TIMEOUT, FLAG_TENSOR_CORES = 32, 64, 128
+FLAG_FP64_GRADCHECK, FLAG_TEST_DEVICE_TIMEOUT, FLAG_TENSOR_CORES, FLAG_DEFER_GRADIENT = 32, 64, 128, 256
 
 # Every symbol include/fpo.h declares.
 EXPORTS = ["fpo_create", "fpo_validate_tree", "fpo_upload_tree", "fpo_render",
@@ -416,10 +416,12 @@ class Renderer:
 
     def render_backward(self, out_rgb, dL_drgb, dL_dcoeffs, camera=None, t=0.0, rays_o=None,
                         rays_d=None, t_per_ray=None, bg=(1.0, 1.0, 1.0), stop_T=1e-4, leaf_mark=None,
-                        stream=None, fp64=False):
+                        stream=None, fp64=False, defer=False):
         """Accumulates dL/d(coefficients) [n_leaves, n1 + 27 n2] (canonical) into
         dL_dcoeffs; sets leaf_mark[id] = 1 (uint8 CUDA tensor) for visited leaves.
-        fp64: the gradient-check replay (dL_dcoeffs is then a float64 tensor)."""
+        fp64: the gradient-check replay (dL_dcoeffs is then a float64 tensor).
+        defer: leave the gradient to the next adam_leaves with the same arrays
+        (FPO_FLAG_DEFER_GRADIENT; needs leaf_mark)."""
         import torch
 
         r, keep, n = self._rays(camera, t, rays_o, rays_d, t_per_ray)
@@ -435,6 +437,8 @@ class Renderer:
         if leaf_mark is not None:
             flags |= FLAG_MARK_LEAVES
             opts.leaf_mark = leaf_mark.data_ptr()
+        if defer:
+            flags |= FLAG_DEFER_GRADIENT
         opts.flags = flags
         g = dL_drgb.contiguous()
         o = out_rgb.contiguous()

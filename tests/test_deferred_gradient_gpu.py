@@ -1,0 +1,116 @@
+"""Gradients as visit lists: the second pass of fpo_render_backward and the
+deferred form that fpo_adam_leaves takes, against the replay that adds every
+row itself (large batches take it) and against each other."""
+
+import numpy as np
+import pytest
+
+from paper_2202_08614_gb300 import fpo, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def _rays(n, seed):
+    rng = np.random.default_rng(seed)
+    o = torch.as_tensor(rng.uniform(-0.6, 1.6, (n, 3)), dtype=torch.float32, device="cuda")
+    d = torch.as_tensor(rng.uniform(0.2, 0.8, (n, 3)), dtype=torch.float32, device="cuda") - o
+    t = torch.as_tensor(rng.uniform(0, 60, n), dtype=torch.float32, device="cuda")
+    g = torch.as_tensor(rng.normal(size=(n, 3)), dtype=torch.float32, device="cuda")
+    return o, d, t, g
+
+
+def _close(a, b):
+    # FP32 sums of at most 4000 visits of a leaf in another order: each within
+    # 4000 * 2^-24 = 2.4e-4 of its sum of |terms| in the worst case, and within
+    # a few sqrt(4000) * 2^-24 = 4e-6 of it as a random walk; terms of both
+    # signs make that sum up to about ten times the largest element
+    assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max())
+
+
+@pytest.mark.parametrize("n1,n2", [(31, 5), (11, 5), (21, 5), (31, 11)])
+@pytest.mark.parametrize("deep", [False, True])
+def test_list_pass_equals_the_replays_own_adds(n1, n2, deep):
+    # with 270,000 more rays of zero gradient the batch is beyond the list's
+    # 2^18 rays, and the replay adds the rows of the 300
+    tree = synth.random_tree(11, max_depth=5, n1=n1, n2=n2) if deep else synth.shell_tree(3, 5, n1, n2)
+    r = fpo.Renderer(n1=n1, n2=n2, idft_mode="fused")
+    r.upload(tree)
+    o, d, t, g = _rays(300, n1 + n2)
+    rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    one = torch.zeros(tree.coeffs.shape, device="cuda")
+    mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+    r.render_backward(rgb, g, one, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark)
+    many, mark2 = torch.zeros_like(one), torch.zeros_like(mark)
+    rep = lambda x: x.repeat(901, *([1] * (x.dim() - 1))).contiguous()
+    g2 = torch.zeros((300 * 901, 3), device="cuda")
+    g2[:300] = g
+    r.render_backward(rep(rgb), g2, many, rays_o=rep(o), rays_d=rep(d), t_per_ray=rep(t), leaf_mark=mark2)
+    r.status()
+    r.close()
+    assert float(one.abs().max()) > 0 and torch.equal(mark, mark2)
+    _close(many, one)
+
+
+def _step(defer, calls, overflow=False):
+    tree = synth.shell_tree(7)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    p = torch.as_tensor(tree.coeffs, device="cuda")
+    p, m, v, grad = p.clone(), torch.full_like(p, 1e-3), torch.full_like(p, 1e-4), torch.zeros_like(p)
+    mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+    if overflow:  # the list keeps the room of its first batch: 4096 rays, 32 visits each
+        o, d, t, g = _rays(8, 1)
+        rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+        r.render_backward(rgb, g * 0, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=defer)
+    for k in range(calls):
+        o, d, t, g = _rays(4000, 20 + k)
+        rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+        r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=defer)
+    r.adam_leaves(p, grad, m, v, mark, 5)
+    rows = (p != torch.as_tensor(tree.coeffs, device="cuda")).any(1)
+    img = r.render(camera=synth.shell_camera(64, 48), t=9.0)["rgb"].clone()
+    r.set_coeffs(p)
+    img2 = r.render(camera=synth.shell_camera(64, 48), t=9.0)["rgb"]
+    r.status()
+    r.close()
+    assert not grad.any() and not mark.any() and torch.equal(img, img2)
+    return p, m, v, rows
+
+
+# one batch; several on one list; one that does not fit beside another (its rows go to grad)
+@pytest.mark.parametrize("calls,overflow", [(1, False), (3, False), (1, True)])
+def test_deferred_step_equals_the_dense_one(calls, overflow):
+    a, b = _step(False, calls, overflow), _step(True, calls, overflow)
+    assert torch.equal(a[3], b[3]) and int(a[3].sum()) > 1000
+    for x, y in zip(a[:3], b[:3]):
+        _close(x, y)
+
+
+def test_set_coeffs_drops_a_pending_list():
+    tree = synth.shell_tree(7)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    p = torch.as_tensor(tree.coeffs, device="cuda").clone()
+    m, v, grad = torch.zeros_like(p), torch.zeros_like(p), torch.zeros_like(p)
+    mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+    o, d, t, g = _rays(500, 3)
+    rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=True)
+    r.set_coeffs(p)
+    r.adam_leaves(p, grad, m, v, mark, 1)
+    r.status()
+    assert not m.any() and torch.equal(p, torch.as_tensor(tree.coeffs, device="cuda"))
+    with pytest.raises(fpo.FPOError):  # needs the marks
+        r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t, defer=True)
+    r.close()
