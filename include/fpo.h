@@ -241,17 +241,18 @@ int fpo_render(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
  * handles (NULL entries allowed); event k is recorded once frame k's pixels
  * are written (on the stream that traversed it), so a caller can read frame
  * k back while later frames render.  The result equals n_frames calls of
- * fpo_render.  In the table mode the work is pipelined over four slots:
- * frame k uses slot k mod 4, with its own table (the context keeps four:
- * 4 x n_leaves x 128 bytes, 64 for an FP16 table), traversal stream (slot 0:
- * cuda_stream; the others internal) and tile counter; the tables of the
+ * fpo_render.  In the table mode the work is pipelined over slots, four of
+ * them with an FP32 table and six with an FP16 table: frame k uses slot
+ * k mod 4 (6), with its own table (the context keeps as many as calls have
+ * used: up to 4 x n_leaves x 128 or 6 x n_leaves x 64 bytes), traversal
+ * stream (slot 0: cuda_stream; the others internal) and tile counter; the tables of the
  * next frames are computed on another internal stream while earlier frames
  * are traversed (frames that all share one t, bit-equal, take a single
  * table pass), and consecutive traversals may overlap (the call orders
  * all of it after cuda_stream's previous work and before everything
  * enqueued on cuda_stream after the call).  Both kernels
- * share every SM: the call picks their launch shapes itself (two 384-thread
- * traversal CTAs and one or two IDFT CTAs per SM, or for LATENT storage one
+ * share every SM: the call picks their launch shapes itself (768 traversal
+ * threads and one or two IDFT CTAs per SM, or for LATENT storage one
  * 256-thread decoder CTA, with a shared-memory carveout that holds them
  * all), whatever traverse_threads says.  Errors: as fpo_render. */
 int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,

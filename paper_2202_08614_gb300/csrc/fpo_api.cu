@@ -58,12 +58,26 @@ void dfree(T *&p)
 }
 
 // Launch shapes of the frame pipeline (fpo_render_frames).  The traversal of
-// frame k and the IDFT pass of frame k + 1 share every SM: two 384-thread
-// traversal CTAs (64 registers a thread) leave a quarter of the register file
-// to the IDFT pass (materialise_pipeline_shape: one 128-thread CTA of the
+// frame k and the IDFT pass of frame k + 1 share every SM: 768 traversal
+// threads (64 registers each) leave a quarter of the register file to the
+// IDFT pass (materialise_pipeline_shape: one 128-thread CTA of the
 // thread-per-leaf form, or two 256-thread CTAs of the warp-cooperative form),
 // whose stage rings are capped so that all CTAs' shared memory fits one
-// carveout.
+// carveout.  With the FP16 table the passes are short, and what counts is how
+// soon the next traversal's warps take the places of the last ones: CTAs of
+// two warps, and six tables in flight (BF16 frames 407 -> 381 us, latent
+// 790 -> 766, FP8 views 231 -> 200; 128 threads 384 / 773 / 201, depth 8 the
+// same).  The FP32-table frames, 5.09 ms for eight, gain from neither (5.16
+// with CTAs of 64, 5.08 at depth 6).
+#ifndef FPO_PIPE_TRAV_THREADS_F16
+#define FPO_PIPE_TRAV_THREADS_F16 64
+#endif
+#ifndef FPO_PIPE_TRAV_CTAS_F16
+#define FPO_PIPE_TRAV_CTAS_F16 12
+#endif
+#ifndef FPO_PIPE_DEPTH_F16
+#define FPO_PIPE_DEPTH_F16 6
+#endif
 #ifndef FPO_PIPE_TRAV_THREADS
 #define FPO_PIPE_TRAV_THREADS 384
 #endif
@@ -74,13 +88,13 @@ void dfree(T *&p)
 #define FPO_PIPE_MAT_CTAS 0  // IDFT-pass CTAs per SM in the pipeline (0: materialise_pipeline_shape's choice)
 #endif
 #ifndef FPO_PIPE_DEPTH
-// Tables (and traversal streams) in flight in fpo_render_frames.  Measured
-// (FP32 / BF16 1080p frames, ms): depth 2 0.675 / 0.516, 3 0.656 / 0.486,
-// 4 0.639 / 0.457, 5 0.653 / 0.480, 6 0.648 / 0.465, 8 0.649 / 0.469.
+// Tables (and traversal streams) in flight in fpo_render_frames, FP32 table.
 #define FPO_PIPE_DEPTH 4
 #endif
 constexpr int PIPE_MAX = 8;
-static_assert(FPO_PIPE_DEPTH >= 2 && FPO_PIPE_DEPTH <= PIPE_MAX, "pipeline depth");
+static_assert(FPO_PIPE_DEPTH >= 2 && FPO_PIPE_DEPTH <= PIPE_MAX && FPO_PIPE_DEPTH_F16 >= 2 && FPO_PIPE_DEPTH_F16 <= PIPE_MAX,
+              "pipeline depth");
+static_assert(1 + 2 * PIPE_MAX <= 24, "tile counters stay below the visit list's status words");
 #ifndef FPO_PIPE_SLOT_STREAMS
 #define FPO_PIPE_SLOT_STREAMS 1  // each pipeline slot's traversals on its own stream (0: all on the caller's)
 #endif
@@ -545,6 +559,7 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
     }
     p.max_steps = ctx->cfg.max_steps > 0 ? (uint32_t)ctx->cfg.max_steps : 3u * (1u << ctx->depth) + 16u;
     p.block_threads = ctx->cfg.traverse_threads ? ctx->cfg.traverse_threads : DEFAULT_TRAVERSE_THREADS;
+    p.few_tiles_split = ctx->cfg.traverse_threads == 0;
     p.refill_min = ctx->cfg.refill_min ? (uint32_t)ctx->cfg.refill_min : DEFAULT_REFILL_MIN;
     p.inner_steps = ctx->cfg.inner_steps ? (uint32_t)ctx->cfg.inner_steps : DEFAULT_INNER_STEPS;
     p.stats = reinterpret_cast<unsigned long long *>(opts->stats);
@@ -706,7 +721,17 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
     cudaError_t e = cudaSuccess;
-    for (int b = 0; b < FPO_PIPE_DEPTH; ++b) {
+    // Views of one frame time (every t bit-equal): one table pass, and every
+    // traversal of the call reads that table (nothing rewrites it before the
+    // call's end, after which the caller's stream has waited for them all).
+    bool one_t = n_frames > 1;
+    for (uint32_t k = 1; k < n_frames && one_t; ++k)
+        one_t = memcmp(&frames[k].t, &frames[0].t, sizeof(double)) == 0;
+    const int depth = ctx->half_table ? FPO_PIPE_DEPTH_F16 : FPO_PIPE_DEPTH;
+    const int slots = n_frames < (uint32_t)depth ? (int)n_frames : depth;  // in use by this call
+    const int trav_threads = ctx->half_table ? FPO_PIPE_TRAV_THREADS_F16 : PIPE_TRAV_THREADS;
+    const int trav_ctas = ctx->half_table ? FPO_PIPE_TRAV_CTAS_F16 : PIPE_TRAV_CTAS;
+    for (int b = 0; b < (one_t ? 1 : slots); ++b) {
         float *&tb = b ? ctx->d_ptable[b] : ctx->d_table;
         size_t &tl = b ? ctx->ptable_leaves[b] : ctx->table_leaves;
         if (tl < ctx->n_leaves) {
@@ -716,11 +741,11 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             tl = ctx->n_leaves;
         }
     }
-    if (!ctx->aux || !ctx->trav[FPO_PIPE_DEPTH - 1] || !ctx->ev_trav[FPO_PIPE_DEPTH - 1]) {
+    if (!ctx->aux || !ctx->trav[depth - 1] || !ctx->ev_trav[depth - 1]) {
         // created once; a failed attempt is retried whole
         if (!ctx->aux) e = cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking);
         if (e == cudaSuccess && !ctx->ev_entry) e = cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming);
-        for (int b = 0; b < FPO_PIPE_DEPTH && e == cudaSuccess; ++b) {
+        for (int b = 0; b < depth && e == cudaSuccess; ++b) {
             if (b && !ctx->trav[b]) e = cudaStreamCreateWithFlags(&ctx->trav[b], cudaStreamNonBlocking);
             if (e == cudaSuccess && !ctx->ev_mat[b]) e = cudaEventCreateWithFlags(&ctx->ev_mat[b], cudaEventDisableTiming);
             if (e == cudaSuccess && !ctx->ev_trav[b]) e = cudaEventCreateWithFlags(&ctx->ev_trav[b], cudaEventDisableTiming);
@@ -746,7 +771,7 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             mshape = materialise_pipeline_shape(ctx->cfg.storage, ctx->cfg.n1, ctx->cfg.n2, PIPE_MAT_SMEM_BUDGET);
             if (FPO_PIPE_MAT_CTAS > 0) mshape.ctas_per_sm = FPO_PIPE_MAT_CTAS;
         }
-        const long need = (long)PIPE_TRAV_CTAS * (traverse_smem_bytes(ctx->d_top != nullptr, PIPE_TRAV_THREADS) + PIPE_STATIC_SMEM + reserved) +
+        const long need = (long)trav_ctas * (traverse_smem_bytes(ctx->d_top != nullptr, trav_threads) + PIPE_STATIC_SMEM + reserved) +
                           (long)mshape.ctas_per_sm * (mshape.smem_per_cta + PIPE_STATIC_SMEM + reserved);
         // The driver rounds a carveout request up to one of the SM's shared-
         // memory configurations: ask for the smallest one that holds `need`.
@@ -768,21 +793,15 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
     // waits for every slot's last traversal at the end.
     if ((e = cudaEventRecord(ctx->ev_entry, s)) != cudaSuccess || (e = cudaStreamWaitEvent(ctx->aux, ctx->ev_entry, 0)) != cudaSuccess)
         return cuda_fail(e, "stream ordering");
-    for (int b = 1; b < FPO_PIPE_DEPTH; ++b)
+    for (int b = 1; b < slots; ++b)
         if ((e = cudaStreamWaitEvent(ctx->trav[b], ctx->ev_entry, 0)) != cudaSuccess) return cuda_fail(e, "stream ordering");
-    // Views of one frame time (every t bit-equal): one table pass, and every
-    // traversal of the call reads that table (nothing rewrites it before the
-    // call's end, after which the caller's stream has waited for them all).
-    bool one_t = n_frames > 1;
-    for (uint32_t k = 1; k < n_frames && one_t; ++k)
-        one_t = memcmp(&frames[k].t, &frames[0].t, sizeof(double)) == 0;
     for (uint32_t k = 0; k < n_frames; ++k) {
-        const int b = (int)(k % FPO_PIPE_DEPTH);
+        const int b = (int)(k % (uint32_t)depth);
         float *tbl = one_t ? ctx->d_table : (b ? ctx->d_ptable[b] : ctx->d_table);
         cudaStream_t ts = FPO_PIPE_SLOT_STREAMS && b ? ctx->trav[b] : s;
         int ce = cudaSuccess;
         if (!one_t || k == 0) {
-            if (k >= FPO_PIPE_DEPTH && (e = cudaStreamWaitEvent(ctx->aux, ctx->ev_trav[b], 0)) != cudaSuccess)
+            if (k >= (uint32_t)depth && (e = cudaStreamWaitEvent(ctx->aux, ctx->ev_trav[b], 0)) != cudaSuccess)
                 return cuda_fail(e, "wait");
             ce = overlap ? launch_table_pass(ctx, frames[k].t, tbl, mshape.ctas_per_sm, ctx->aux, mshape.stages, carveout, false)
                          : launch_table_pass(ctx, frames[k].t, tbl, 0, ctx->aux, 0, 0, false);
@@ -796,8 +815,8 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
         p.table = reinterpret_cast<const float4 *>(tbl);
         p.tiles = ctx->d_status + 1 + (FPO_PIPE_SLOT_STREAMS ? 2 * b : 0);  // this slot's tile counter and finished warps
         if (overlap) {
-            p.block_threads = PIPE_TRAV_THREADS;
-            p.max_ctas_per_sm = PIPE_TRAV_CTAS;
+            p.block_threads = trav_threads;
+            p.max_ctas_per_sm = trav_ctas;
             p.carveout = carveout;
         }
         ce = launch_traverse(p, true, false, ctx->sm_count, ts);
@@ -807,7 +826,7 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             return cuda_fail(e, "cudaEventRecord(frame_done)");
     }
     // everything above is ordered before the caller's later work
-    for (uint32_t b = 1; b < FPO_PIPE_DEPTH && b < n_frames; ++b)
+    for (int b = 1; b < slots; ++b)
         if ((e = cudaStreamWaitEvent(s, ctx->ev_trav[b], 0)) != cudaSuccess) return cuda_fail(e, "stream ordering");
     return FPO_OK;
 }

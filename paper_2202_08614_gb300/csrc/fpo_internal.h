@@ -168,6 +168,7 @@ struct TraverseParams {
     uint32_t refill_min;      // warp refills its idle lanes once this many are idle (32: whole tiles)
     uint32_t inner_steps;     // steps a lane takes between two refill checks
     int block_threads;        // 128 or 256
+    int few_tiles_split;      // 1: smaller CTAs when there are few tiles (block_threads is not the user's choice)
     int rays_per_warp, list_cap; // fused mode: rays of one warp and length of its visit list (set by the launcher)
     int max_ctas_per_sm;      // 0: as many as fit
     int carveout;             // preferred shared-memory carveout in percent (0: the driver's default)

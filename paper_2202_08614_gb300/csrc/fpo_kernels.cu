@@ -872,6 +872,10 @@ __device__ __forceinline__ float cube_exit(const RayState &R, int csz, int &m, i
     return tx;
 }
 
+// floor(x) as an integer for |x| < 2^22 (below 0 it comes out negative): one
+// FMA-pipe and one ALU operation, where the conversion has a quarter of the rate.
+__device__ __forceinline__ int small_floor(float x) { return __float_as_int(__fadd_rd(x, 8388608.0f)) - 0x4B000000; }
+
 // Next cell after leaving the cube through axis m at distance tx.  Along m:
 // the adjacent cube; along the other axes: the cell holding the exit point,
 // clamped to this cube's extent and never moving backwards, so every step
@@ -897,10 +901,10 @@ __device__ __forceinline__ bool next_cell(const RayState &R, int G, int m, const
                 Pn[a] = R.pos[a] ? lo[a] + csz : lo[a] - 1;
                 inside = (unsigned)Pn[a] < (unsigned)G;
             } else {
-                int q = (int)floorf(fmaf(tx, R.gd[a], R.go[a]));
-                q = min(max(q, lo[a]), lo[a] + csz - 1);
-                if (R.gd[a] > 0.0f) q = max(q, R.P[a]);
-                else if (R.gd[a] < 0.0f) q = min(q, R.P[a]);
+                // between this cube's near and far side as the ray goes along the
+                // axis, never behind R.P (a ray parallel to the axis stays)
+                const int q0 = small_floor(fmaf(tx, R.gd[a], R.go[a]));
+                const int q = min(max(q0, R.pos[a] ? R.P[a] : lo[a]), R.pos[a] ? lo[a] + csz - 1 : R.P[a]);
                 Pn[a] = q;
             }
         }
@@ -1110,14 +1114,20 @@ __device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
 // when at least REFILL_MIN lanes are idle, the warp hands them the next rays
 // of its current tile (fetching a new tile when that one is used up), so
 // long rays do not leave most of a warp idle.  The last CTA to finish resets
-// the counter.  Register cap: 64 lets four 256-thread CTAs share an SM
-// (measured fastest of 48..80 on the 3.5M-leaf body at 1080p).
+// the counter.  Register cap: 64 in the frame pipeline, where the IDFT pass
+// takes a quarter of the register file (eight 1080p FP32 frames: 5.09 ms at
+// 64, 5.12 at 72, 5.52 at 56, 5.54 at 48); alone, the FP32-table walk
+// gains more from the 72 registers it wants than from a fourth CTA (826 ->
+// 801 us a frame, 38.7 -> 34.6 us a 128x128 frame).
 #ifndef FPO_TRAV_MAXNREG_MAT
 #define FPO_TRAV_MAXNREG_MAT 64
 #endif
 
-template <int TM, bool DBG, bool COMPACT, bool BRICK>
-__global__ void __maxnreg__(FPO_TRAV_MAXNREG_MAT) traverse_kernel(const __grid_constant__ TraverseParams p)
+#ifndef FPO_TRAV_MAXNREG_ALONE
+#define FPO_TRAV_MAXNREG_ALONE 80
+#endif
+template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS>
+__global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ TraverseParams p)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int stride = blockDim.x;
@@ -1211,12 +1221,20 @@ __global__ void __maxnreg__(FPO_TRAV_MAXNREG_MAT) traverse_kernel(const __grid_c
 
 int traverse_smem_bytes(bool brick, int threads) { return brick ? 0 : STACK_LEVELS * threads * 4; }
 
-template <int TM, bool DBG, bool COMPACT, bool BRICK>
+template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS>
 static int launch_t(const TraverseParams &p, int sm_count, cudaStream_t s)
 {
+    // Few tiles: one-warp CTAs, all resident at once, so that the hardware
+    // deals them out evenly (64 CTAs of 8 warps put the 512 tiles of a 128x128
+    // frame on 64 of the 152 SMs).
+    auto k = traverse_kernel<TM, DBG, COMPACT, BRICK, REGS>;
+    if (p.few_tiles_split && p.n_tiles < 32u * (uint32_t)sm_count) {
+        // (within the default shared memory: nothing to set or to ask for)
+        k<<<p.n_tiles ? p.n_tiles : 1u, 32, traverse_smem_bytes(BRICK, 32), s>>>(p);
+        return (int)cudaGetLastError();
+    }
     const int threads = p.block_threads;
     const int smem = traverse_smem_bytes(BRICK, threads);
-    auto k = traverse_kernel<TM, DBG, COMPACT, BRICK>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1239,11 +1257,16 @@ static int launch_t(const TraverseParams &p, int sm_count, cudaStream_t s)
 template <int TM>
 static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaStream_t s)
 {
+    constexpr int R = FPO_TRAV_MAXNREG_MAT;
     if (p.refill_min < 32)  // (a tuning option: the octree descent serves every tree)
-        return debug ? launch_t<TM, true, true, false>(p, sm_count, s) : launch_t<TM, false, true, false>(p, sm_count, s);
-    if (p.top)
-        return debug ? launch_t<TM, true, false, true>(p, sm_count, s) : launch_t<TM, false, false, true>(p, sm_count, s);
-    return debug ? launch_t<TM, true, false, false>(p, sm_count, s) : launch_t<TM, false, false, false>(p, sm_count, s);
+        return debug ? launch_t<TM, true, true, false, R>(p, sm_count, s) : launch_t<TM, false, true, false, R>(p, sm_count, s);
+    if (p.top) {
+        if (TM == TM_TABLE_F32 && p.max_ctas_per_sm == 0)
+            return debug ? launch_t<TM, true, false, true, FPO_TRAV_MAXNREG_ALONE>(p, sm_count, s)
+                         : launch_t<TM, false, false, true, FPO_TRAV_MAXNREG_ALONE>(p, sm_count, s);
+        return debug ? launch_t<TM, true, false, true, R>(p, sm_count, s) : launch_t<TM, false, false, true, R>(p, sm_count, s);
+    }
+    return debug ? launch_t<TM, true, false, false, R>(p, sm_count, s) : launch_t<TM, false, false, false, R>(p, sm_count, s);
 }
 
 // ---------------------------------------------------------------------------
