@@ -555,66 +555,6 @@ __device__ __forceinline__ void put_one_bf(unsigned char *base, int row, int j, 
     *reinterpret_cast<uint4 *>(base + core_off(row, 8 * j, K)) =
         make_uint4(*reinterpret_cast<const uint32_t *>(&p), 0u, 0u, 0u);
 }
-// Rows owned by the lanes of a warp (lane r: row offset off_r, validity ok_r)
-// moved in coalesced pieces through a per-warp shared tile of H rows x 33
-// floats: for each row, the 32 lanes move 32 consecutive floats (columns col0
-// + lane, those below ncols), and the tile turns them into each lane's own
-// 32 values (H = 32: one pass; H = 16: two passes of half the rows).
-template <int H>
-__device__ __forceinline__ void warp_load_rows(float v[32], const float *__restrict__ base, size_t off, bool ok,
-                                               int col0, int ncols, float *tile)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int h = 0; h < 32 / H; ++h) {
-#pragma unroll 4
-        for (int i = 0; i < H; ++i) {
-            const int r = H * h + i;
-            const size_t o = __shfl_sync(0xffffffffu, off, r);
-            const bool k = __shfl_sync(0xffffffffu, ok, r);
-            const int c = col0 + lane;
-            tile[i * 33 + lane] = k && c < ncols ? base[o + c] : 0.0f;
-        }
-        __syncwarp();
-        if ((lane / H) == h) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) v[e] = tile[(lane - H * h) * 33 + e];
-        }
-        __syncwarp();
-    }
-}
-
-// The inverse: each lane's 32 values of its row to columns col0 + e (those
-// below ncols) of its row, where a column j goes to base_lo[off_lo + j] for
-// j < split and to base_hi[off_hi + j - split] otherwise (H as above).
-template <int H>
-__device__ __forceinline__ void warp_store_rows(const float v[32], float *base_lo, size_t off_lo, float *base_hi,
-                                                size_t off_hi, int split, bool ok, int col0, int ncols, float *tile)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int h = 0; h < 32 / H; ++h) {
-        if ((lane / H) == h) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) tile[(lane - H * h) * 33 + e] = v[e];
-        }
-        __syncwarp();
-#pragma unroll 4
-        for (int i = 0; i < H; ++i) {
-            const int r = H * h + i;
-            const size_t olo = __shfl_sync(0xffffffffu, off_lo, r), ohi = __shfl_sync(0xffffffffu, off_hi, r);
-            const bool k = __shfl_sync(0xffffffffu, ok, r);
-            const int c = col0 + lane;
-            if (k && c < ncols) {
-                const float x = tile[i * 33 + lane];
-                if (c < split) base_lo[olo + c] = x;
-                else base_hi[ohi + c - split] = x;
-            }
-        }
-        __syncwarp();
-    }
-}
-
 }  // namespace
 
 __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __grid_constant__ DecoderGradTcParams p)
@@ -907,22 +847,56 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
 // rounded to BF16 and then FP16, FP16 hidden activations, biases as FP16
 // hi/lo pairs, FP32 accumulation) but the last layer unfolded (all
 // n1 + 27 n2 coefficients): what the pixel loss of the decoder's training
-// renders.  DR_GROUPS independent warpgroup pipelines per CTA, one CTA per SM,
-// each with 96 TMEM columns (Z1 and Z2 in the first 64; the last layer in two
-// halves, columns 0..95 and 96..175 of Y, each in the 96) and one
-// shared-memory region for its tile's A operands; the next tile's latents
-// are gathered while the last layer runs.  Tile rows are records: row
-// i gathers latent perm[i] and writes record i (density values at stride ss,
-// SH values at stride zs).
+// renders.  Eight independent warpgroup pipelines per CTA, one CTA per SM,
+// each with 64 TMEM columns (Z1, then Z2, then the last layer in three windows
+// of 64 columns that overlap by 8) and one shared-memory region for its
+// tile's A operands.  Tile rows are records: thread i gathers latent
+// perm[i] and writes record i, 32 bytes of it at a time straight from its
+// TMEM lane (a piece of 8 SH values never crosses a window, and 8 values
+// start on 32 bytes where the record's stride allows it).  Turning the rows
+// through shared memory to write them coalesced took most of the time, and
+// the memory of four more pipelines: 438k leaves 266 -> 103 us.
 namespace {
-constexpr int DR_GROUPS = 4, DR_NC = 176, DR_COLS = 96, DR_NH0 = 96, DR_NH1 = DR_NC - DR_NH0;
+constexpr int DR_GROUPS = 8, DR_NC = 176, DR_COLS = 64, DR_WINDOWS = 3, DR_STEP = 56;
+static_assert((DR_WINDOWS - 1) * DR_STEP + DR_COLS == DR_NC, "the windows cover the last layer");
 constexpr int DRO_W1 = 0;                        // [64][48]  W1 | b1
 constexpr int DRO_W2 = DRO_W1 + 64 * K1 * 2;     // [64][80]  W2 | b2
 constexpr int DRO_W3 = DRO_W2 + 64 * K2 * 2;     // [176][80] W3 | b3
 constexpr int DRO_A = DRO_W3 + DR_NC * K2 * 2;   // per group: [128][80] (X, then H1, then H2)
 constexpr int DR_GROUP_BYTES = 128 * K2 * 2;
-constexpr int DRO_ROWS = DRO_A + DR_GROUPS * DR_GROUP_BYTES;  // per warp: 32 x 33 floats
-constexpr int DR_SMEM = DRO_ROWS + DR_GROUPS * 4 * 32 * 33 * 4;
+constexpr int DR_SMEM = DRO_A + DR_GROUPS * DR_GROUP_BYTES;
+
+// Four pieces of 8 consecutive columns of this thread's TMEM lane; waits for them.
+__device__ __forceinline__ void tmem_ld8x4(const uint32_t a[4], float v[32])
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3])
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ float tmem_ld1(uint32_t a)
+{
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=r"(r) : "r"(a) : "memory");
+    return __uint_as_float(r);
+}
+
+// 8 floats to a 32-byte aligned global address.
+__device__ __forceinline__ void stg256(float *p, const float *v)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
 
 struct DecodeTcParams {
     fpo_mlp w;                  // FP32 master weights
@@ -1010,7 +984,6 @@ __global__ void __launch_bounds__(128 * DR_GROUPS, 1) decode_records_tc_kernel(c
     const uint32_t tmem = s_tmem + (uint32_t)DR_COLS * (uint32_t)group;
     const uint32_t my_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     unsigned char *ga = sm + DRO_A + group * DR_GROUP_BYTES;
-    float *rows_tile = reinterpret_cast<float *>(sm + DRO_ROWS) + warp * 32 * 33;
     const uint32_t sa_a = ptx::smem_u32(ga), sa_w1 = ptx::smem_u32(sm + DRO_W1), sa_w2 = ptx::smem_u32(sm + DRO_W2),
                    sa_w3 = ptx::smem_u32(sm + DRO_W3);
     uint32_t phase = 0;
@@ -1045,25 +1018,29 @@ __global__ void __launch_bounds__(128 * DR_GROUPS, 1) decode_records_tc_kernel(c
     };
     const uint32_t n_tiles = (p.n + 127) / 128;
     const uint32_t first = blockIdx.x * DR_GROUPS + group, step = gridDim.x * DR_GROUPS;
-    // this thread's row of a tile: the gathered FP32 latent (all zero past the end)
-    auto gather = [&](uint32_t tile, float x[32]) {
-        const uint32_t rec = tile * 128 + (uint32_t)m;
-        const bool ok = tile < n_tiles && rec < p.n;
-        const size_t src = ok ? p.perm[rec] : 0;
-        warp_load_rows<32>(x, p.latents, src * 32, ok, 0, 32, rows_tile);
-    };
-    float xn[32];
-    gather(first, xn);
+    const bool lat16 = (reinterpret_cast<uintptr_t>(p.latents) & 15u) == 0;
+    const int zpieces = (p.zs + 7) / 8, nz = nc - p.n1;
+    const int whole = min(zpieces, (DR_NC - p.n1) / 8);  // pieces that end inside the layer
     for (uint32_t tile = first; tile < n_tiles; tile += step) {
         const uint32_t rec = tile * 128 + (uint32_t)m;
         const bool valid = rec < p.n;
         {
+            // this thread's row: the gathered FP32 latent (all zero past the end)
+            const float *src = p.latents + (valid ? (size_t)p.perm[rec] : 0) * 32;
             __half2 hx = __float2half2_rn(0.0f);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {  // FP16 latents, as the inference decoder holds them
-                put8(ga, m, j, K1, xn + 8 * j);
+                float x[8];
+                if (valid && lat16) {
+                    const float4 lo = __ldg(reinterpret_cast<const float4 *>(src) + 2 * j), hi = __ldg(reinterpret_cast<const float4 *>(src) + 2 * j + 1);
+                    x[0] = lo.x, x[1] = lo.y, x[2] = lo.z, x[3] = lo.w, x[4] = hi.x, x[5] = hi.y, x[6] = hi.z, x[7] = hi.w;
+                } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) hx = __hmax2(hx, __float2half2_rn(fabsf(xn[8 * j + e])));
+                    for (int e = 0; e < 8; ++e) x[e] = valid ? __ldg(src + 8 * j + e) : 0.0f;
+                }
+                put8(ga, m, j, K1, x);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) hx = __hmax2(hx, __float2half2_rn(fabsf(x[e])));
             }
             hmax = __hmax2(hmax, hx);
             put_bias_chunk(ga, m, 4, K1, 0.0f, true);
@@ -1090,23 +1067,66 @@ __global__ void __launch_bounds__(128 * DR_GROUPS, 1) decode_records_tc_kernel(c
             for (int c = 0; c < 4; ++c) put8_relu(ga, m, 4 * h + c, K2, v + 8 * c, hmax);
         }
         hand_off();
-        // Y -> record `rec` in two halves: columns < n1 to the density record,
-        // the rest to the SH record; the next tile's latents are gathered
-        // while the first half's MMAs run
+        // Y -> record `rec`, window by window: the density record from the
+        // first, and the pieces of 8 SH values that each window holds whole
         bool ok = true;
+        int k = 0;
 #pragma unroll 1
-        for (int half = 0; half < 2 && ok; ++half) {
-            const int n_cols = half ? DR_NH1 : DR_NH0, col0 = half ? DR_NH0 : 0;
-            issue_layer(sa_w3 + (uint32_t)core_off(col0, 0, K2), K2, n_cols);
-            if (half == 0) gather(tile + step, xn);
+        for (int win = 0; win < DR_WINDOWS; ++win) {
+            const int col0 = DR_STEP * win;
+            issue_layer(sa_w3 + (uint32_t)core_off(col0, 0, K2), K2, DR_COLS);
             if (!(ok = wait_layer())) break;
-#pragma unroll 1
-            for (int c = 0; c < DR_NH0 / 32; ++c) {
+            if (win == 0) {
                 float v[32];
-                tmem_ld32(my_lane + 32 * c, v);  // columns past n_cols: the group's unused scratch
-                warp_store_rows<32>(v, p.sig, (size_t)rec * p.ss, p.zc, (size_t)rec * p.zs, p.n1, valid,
-                                    col0 + 32 * c, col0 + n_cols < nc ? col0 + n_cols : nc, rows_tile);
+                tmem_ld32(my_lane, v);
+                if (valid) {
+                    float *dst = p.sig + (size_t)rec * p.ss;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        if (4 * q < p.ss)
+                            *reinterpret_cast<float4 *>(dst + 4 * q) =
+                                make_float4(4 * q < p.n1 ? v[4 * q] : 0.0f, 4 * q + 1 < p.n1 ? v[4 * q + 1] : 0.0f,
+                                            4 * q + 2 < p.n1 ? v[4 * q + 2] : 0.0f, 4 * q + 3 < p.n1 ? v[4 * q + 3] : 0.0f);
+                }
             }
+            // 8 values of SH piece q (elements past 27 n2 are padding: zero)
+            auto put_piece = [&](int q, float *v) {
+                if (!valid) return;
+                float *dst = p.zc + (size_t)rec * p.zs + 8 * q;
+                if (8 * q + 8 > nz) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = 8 * q + e < nz ? v[e] : 0.0f;
+                }
+                if ((p.zs & 7) == 0) {
+                    stg256(dst, v);
+                } else {
+                    *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                    if (8 * q + 4 < p.zs) *reinterpret_cast<float4 *>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+                }
+            };
+            const int k_end = win == DR_WINDOWS - 1 ? whole : min(whole, (col0 + DR_COLS - 8 - p.n1) / 8 + 1);
+#pragma unroll 1
+            for (; k < k_end; k += 4) {
+                float v[32];
+                uint32_t a[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = my_lane + (uint32_t)(p.n1 + 8 * (k + q < k_end ? k + q : k) - col0);
+                tmem_ld8x4(a, v);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (k + q < k_end) put_piece(k + q, v + 8 * q);
+            }
+            if (win == DR_WINDOWS - 1 && whole < zpieces) {
+                // the last piece ends past the layer: only the columns there are
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int c = p.n1 + 8 * whole + e;
+                    v[e] = c < nc ? tmem_ld1(my_lane + (uint32_t)(c - col0)) : 0.0f;
+                }
+                put_piece(whole, v);
+            }
+            k = k_end;
             fence_before();  // TMEM reads done before the group's next MMAs
             group_sync(group);
         }
