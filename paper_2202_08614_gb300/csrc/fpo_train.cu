@@ -23,25 +23,78 @@ namespace fpo {
 namespace {
 
 // Tiles of TG_ROWS leaves; thread (tr, tc) = (tid >> 4, tid & 15) owns rows
-// 4 tr .. 4 tr + 3 and the outputs tc + 16 j of each activation layer, and the
-// weight-gradient entries (tc + 16 j, tr + 16 i) of each layer, summed in
-// registers over all of its CTA's tiles.  Weights are kept as [out][in] rows
-// padded to in + 1 floats, activations as [row][feature] rows padded the same
-// way: a warp then reads 16 consecutive words or a broadcast whichever index
-// it varies, so no shared-memory read has a bank conflict.
+// 4 tr .. 4 tr + 3 in the products over a tile: with the outputs tc + 16 j of
+// each layer going forward, with the features 4 tc .. 4 tc + 3 going back; and
+// the weight-gradient entries (output 4 tc + 64 q + e, feature 4 tr + i) of
+// each layer, summed in registers over all of its CTA's tiles.  Weights are
+// kept as [out][in] rows and activations as [row][feature] rows, both padded
+// to 4 mod 32 floats: every operand is then read 16 bytes at a time (4 reads
+// for 44 to 64 FMAs, where single words took 15 for 44) in the fewest
+// wavefronts, whichever index a warp varies.  8,191 leaves: 65 -> 52 us.
 constexpr int TG_THREADS = 256;
 constexpr int TG_ROWS = 64;   // leaves per tile
 constexpr int TG_MAXC = 176;  // n1 + 27 n2 <= 176 (31 + 135 = 166)
 constexpr int TG_J = TG_MAXC / 16;
-constexpr int S1 = 33, S2 = 65, SY = TG_MAXC + 1;  // padded row strides
+constexpr int S1 = 36, S2 = 68, SY = TG_MAXC + 4;  // padded row strides
 
-struct GradSmem {
+struct alignas(16) GradSmem {
     float w1[64 * S1], w2[64 * S2], w3[TG_MAXC * S2], b1[64], b2[64], b3[TG_MAXC];
     float x[TG_ROWS * S1], h1[TG_ROWS * S2], h2[TG_ROWS * S2], dy[TG_ROWS * SY];
     float d2[TG_ROWS * S2], d1[TG_ROWS * S2];
     uint32_t row[TG_ROWS];
     double loss;
 };
+
+__device__ __forceinline__ void lds4(const float *p, float v[4])
+{
+    const float4 q = *reinterpret_cast<const float4 *>(p);
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+    v[3] = q.w;
+}
+
+// a[i][j] += sum_k x[4 tr + i][k] w[tc + 16 j][k], k < K in order.
+template <int K, int J, int S>
+__device__ __forceinline__ void product_forward(float a[4][J], const float *x, const float *w, int tr, int tc)
+{
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float xv[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) lds4(x + (4 * tr + i) * S + k, xv[i]);
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            float wv[4];
+            lds4(w + (tc + 16 * j) * S + k, wv);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[i][j] = fmaf(xv[i][e], wv[e], a[i][j]);
+        }
+    }
+}
+
+// a[i][f] += sum_c d[4 tr + i][c] w[c][4 tc + f], c < C (a multiple of 4) in order.
+template <int SD, int SW>
+__device__ __forceinline__ void product_back(float a[4][4], const float *d, const float *w, int C, int tr, int tc)
+{
+#pragma unroll 2
+    for (int c = 0; c < C; c += 4) {
+        float dv[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) lds4(d + (4 * tr + i) * SD + c, dv[i]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float wv[4];
+            lds4(w + (c + e) * SW + 4 * tc, wv);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) a[i][f] = fmaf(dv[i][e], wv[f], a[i][f]);
+        }
+    }
+}
 
 }  // namespace
 
@@ -61,9 +114,9 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
     for (int i = tid; i < TG_MAXC; i += TG_THREADS) S.b3[i] = i < nc ? p.w.b3[i] : 0.0f;
     if (tid == 0) S.loss = 0.0;
 
-    float g3[TG_J][4], g2[4][4], g1[4][2], gb = 0.0f, gb2 = 0.0f, gb1 = 0.0f, lsum = 0.0f;
+    float g3[12][4], g2[4][4], g1[4][2], gb = 0.0f, gb2 = 0.0f, gb1 = 0.0f, lsum = 0.0f;
 #pragma unroll
-    for (int j = 0; j < TG_J; ++j)
+    for (int j = 0; j < 12; ++j)
 #pragma unroll
         for (int i = 0; i < 4; ++i) g3[j][i] = 0.0f;
 #pragma unroll
@@ -92,18 +145,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) a[i][j] = S.b1[tc + 16 * j];
-#pragma unroll 4
-            for (int k = 0; k < 32; ++k) {
-                float xv[4], wv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = S.x[(4 * tr + i) * S1 + k];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) wv[j] = S.w1[(tc + 16 * j) * S1 + k];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a[i][j] = fmaf(xv[i], wv[j], a[i][j]);
-            }
+            product_forward<32, 4, S1>(a, S.x, S.w1, tr, tc);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -117,18 +159,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) a[i][j] = S.b2[tc + 16 * j];
-#pragma unroll 4
-            for (int k = 0; k < 64; ++k) {
-                float xv[4], wv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = S.h1[(4 * tr + i) * S2 + k];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) wv[j] = S.w2[(tc + 16 * j) * S2 + k];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a[i][j] = fmaf(xv[i], wv[j], a[i][j]);
-            }
+            product_forward<64, 4, S2>(a, S.h1, S.w2, tr, tc);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -142,18 +173,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < TG_J; ++j) a[i][j] = S.b3[tc + 16 * j];
-#pragma unroll 2
-            for (int k = 0; k < 64; ++k) {
-                float xv[4], wv[TG_J];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) xv[i] = S.h2[(4 * tr + i) * S2 + k];
-#pragma unroll
-                for (int j = 0; j < TG_J; ++j) wv[j] = S.w3[(tc + 16 * j) * S2 + k];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < TG_J; ++j) a[i][j] = fmaf(xv[i], wv[j], a[i][j]);
-            }
+            product_forward<64, TG_J, S2>(a, S.h2, S.w3, tr, tc);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = 4 * tr + i;
@@ -181,36 +201,29 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) a[i][j] = 0.0f;
-#pragma unroll 2
-            for (int c = 0; c < nc; ++c) {
-                float dv[4], wv[4];
+            // (the columns from nc to TG_MAXC of dy and the rows of W3 there are zero)
+            product_back<SY, S2>(a, S.dy, S.w3, (nc + 3) & ~3, tr, tc);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) dv[i] = S.dy[(4 * tr + i) * SY + c];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) wv[j] = S.w3[c * S2 + tc + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a[i][j] = fmaf(dv[i], wv[j], a[i][j]);
+            for (int i = 0; i < 4; ++i) {
+                const int o = (4 * tr + i) * S2 + 4 * tc;
+                float h[4];
+                lds4(S.h2 + o, h);
+                *reinterpret_cast<float4 *>(S.d2 + o) = make_float4(h[0] > 0.0f ? a[i][0] : 0.0f, h[1] > 0.0f ? a[i][1] : 0.0f,
+                                                                    h[2] > 0.0f ? a[i][2] : 0.0f, h[3] > 0.0f ? a[i][3] : 0.0f);
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int o = (4 * tr + i) * S2 + tc + 16 * j;
-                    S.d2[o] = S.h2[o] > 0.0f ? a[i][j] : 0.0f;
-                }
 #pragma unroll 2
             for (int r = 0; r < nr; ++r) {
-                float dv[TG_J], hv[4];
+                float hv[4];
+                lds4(S.h2 + r * S2 + 4 * tr, hv);
 #pragma unroll
-                for (int j = 0; j < TG_J; ++j) dv[j] = S.dy[r * SY + tc + 16 * j];
+                for (int q = 0; q < 3; ++q) {
+                    float dv[4];
+                    lds4(S.dy + r * SY + (q < 2 || tc < 12 ? 4 * tc + 64 * q : 0), dv);  // (176 = 2 x 64 + 4 x 12 outputs)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) hv[i] = S.h2[r * S2 + tr + 16 * i];
+                    for (int e = 0; e < 4; ++e)
 #pragma unroll
-                for (int j = 0; j < TG_J; ++j)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) g3[j][i] = fmaf(dv[j], hv[i], g3[j][i]);
+                        for (int i = 0; i < 4; ++i) g3[4 * q + e][i] = fmaf(dv[e], hv[i], g3[4 * q + e][i]);
+                }
             }
             if (tid < nc)
                 for (int r = 0; r < nr; ++r) gb += S.dy[r * SY + tid];
@@ -223,36 +236,24 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) a[i][j] = 0.0f;
-#pragma unroll 4
-            for (int o = 0; o < 64; ++o) {
-                float dv[4], wv[4];
+            product_back<S2, S2>(a, S.d2, S.w2, 64, tr, tc);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) dv[i] = S.d2[(4 * tr + i) * S2 + o];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) wv[j] = S.w2[o * S2 + tc + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a[i][j] = fmaf(dv[i], wv[j], a[i][j]);
+            for (int i = 0; i < 4; ++i) {
+                const int o = (4 * tr + i) * S2 + 4 * tc;
+                float h[4];
+                lds4(S.h1 + o, h);
+                *reinterpret_cast<float4 *>(S.d1 + o) = make_float4(h[0] > 0.0f ? a[i][0] : 0.0f, h[1] > 0.0f ? a[i][1] : 0.0f,
+                                                                    h[2] > 0.0f ? a[i][2] : 0.0f, h[3] > 0.0f ? a[i][3] : 0.0f);
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int o = (4 * tr + i) * S2 + tc + 16 * j;
-                    S.d1[o] = S.h1[o] > 0.0f ? a[i][j] : 0.0f;
-                }
 #pragma unroll 4
             for (int r = 0; r < nr; ++r) {
                 float dv[4], hv[4];
+                lds4(S.d2 + r * S2 + 4 * tc, dv);
+                lds4(S.h1 + r * S2 + 4 * tr, hv);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) dv[j] = S.d2[r * S2 + tc + 16 * j];
+                for (int e = 0; e < 4; ++e)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) hv[i] = S.h1[r * S2 + tr + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) g2[j][i] = fmaf(dv[j], hv[i], g2[j][i]);
+                    for (int i = 0; i < 4; ++i) g2[e][i] = fmaf(dv[e], hv[i], g2[e][i]);
             }
             if (tid < 64)
                 for (int r = 0; r < nr; ++r) gb2 += S.d2[r * S2 + tid];
@@ -263,57 +264,65 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_kernel(const __gri
             float a[4][2];
 #pragma unroll
             for (int i = 0; i < 4; ++i) a[i][0] = a[i][1] = 0.0f;
-#pragma unroll 4
-            for (int o = 0; o < 64; ++o) {
-                float dv[4], wv[2];
+#pragma unroll 2
+            for (int o = 0; o < 64; o += 4) {  // features 2 tc, 2 tc + 1
+                float dv[4][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) dv[i] = S.d1[(4 * tr + i) * S2 + o];
+                for (int i = 0; i < 4; ++i) lds4(S.d1 + (4 * tr + i) * S2 + o, dv[i]);
 #pragma unroll
-                for (int j = 0; j < 2; ++j) wv[j] = S.w1[o * S1 + tc + 16 * j];
+                for (int e = 0; e < 4; ++e) {
+                    const float2 wv = *reinterpret_cast<const float2 *>(S.w1 + (o + e) * S1 + 2 * tc);
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) a[i][j] = fmaf(dv[i], wv[j], a[i][j]);
+                    for (int i = 0; i < 4; ++i) {
+                        a[i][0] = fmaf(dv[i][e], wv.x, a[i][0]);
+                        a[i][1] = fmaf(dv[i][e], wv.y, a[i][1]);
+                    }
+                }
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = 4 * tr + i;
                 if (r < nr) {
-                    p.dlatents[(size_t)(r0 + r) * 32 + tc] = a[i][0];
-                    p.dlatents[(size_t)(r0 + r) * 32 + tc + 16] = a[i][1];
+                    p.dlatents[(size_t)(r0 + r) * 32 + 2 * tc] = a[i][0];
+                    p.dlatents[(size_t)(r0 + r) * 32 + 2 * tc + 1] = a[i][1];
                 }
             }
 #pragma unroll 4
             for (int r = 0; r < nr; ++r) {
-                float dv[4], xv[2];
+                float dv[4];
+                lds4(S.d1 + r * S2 + 4 * tc, dv);
+                const float2 xv = *reinterpret_cast<const float2 *>(S.x + r * S1 + 2 * tr);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) dv[j] = S.d1[r * S2 + tc + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 2; ++i) xv[i] = S.x[r * S1 + tr + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) g1[j][i] = fmaf(dv[j], xv[i], g1[j][i]);
+                for (int e = 0; e < 4; ++e) {
+                    g1[e][0] = fmaf(dv[e], xv.x, g1[e][0]);
+                    g1[e][1] = fmaf(dv[e], xv.y, g1[e][1]);
+                }
             }
             if (tid < 64)
                 for (int r = 0; r < nr; ++r) gb1 += S.d1[r * S2 + tid];
         }
     }
     // this CTA's sums into the global gradients
+    const bool a16 = ((reinterpret_cast<uintptr_t>(p.g.w3) | reinterpret_cast<uintptr_t>(p.g.w2)) & 15u) == 0;
+    auto add4 = [&](float *dst, const float *v) {
+        if (a16) {
+            atomicAdd(reinterpret_cast<float4 *>(dst), make_float4(v[0], v[1], v[2], v[3]));
+        } else {
 #pragma unroll
-    for (int j = 0; j < TG_J; ++j)
-        if (tc + 16 * j < nc) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) atomicAdd(p.g.w3 + (tc + 16 * j) * 64 + tr + 16 * i, g3[j][i]);
+            for (int i = 0; i < 4; ++i) atomicAdd(dst + i, v[i]);
         }
+    };
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int q = 0; q < 3; ++q)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) atomicAdd(p.g.w2 + (tc + 16 * j) * 64 + tr + 16 * i, g2[j][i]);
+        for (int e = 0; e < 4; ++e)
+            if ((q < 2 || tc < 12) && 4 * tc + 64 * q + e < nc) add4(p.g.w3 + (4 * tc + 64 * q + e) * 64 + 4 * tr, g3[4 * q + e]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int e = 0; e < 4; ++e) add4(p.g.w2 + (4 * tc + e) * 64 + 4 * tr, g2[e]);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) atomicAdd(p.g.w1 + (tc + 16 * j) * 32 + tr + 16 * i, g1[j][i]);
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) atomicAdd(p.g.w1 + (4 * tc + e) * 32 + 2 * tr + i, g1[e][i]);
     if (tid < nc) atomicAdd(p.g.b3 + tid, gb);
     if (tid < 64) {
         atomicAdd(p.g.b2 + tid, gb2);
