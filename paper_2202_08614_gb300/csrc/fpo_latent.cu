@@ -440,9 +440,10 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
 // loss against target coefficients (plus an optional extra dL/dy), and the
 // back-propagation to every weight, bias and latent, with BF16 operands (A
 // and B of each MMA both BF16; FP32's exponent range, so no loss scaling)
-// and FP32 accumulation in TMEM.  One 256-thread CTA per SM (all 512 TMEM
-// columns); threads t and t + 128 own row t of a 128-leaf tile, TMEM lane t,
-// and half of each layer's columns.  Per tile, nine GEMMs (M = 128):
+// and FP32 accumulation in TMEM.  One CTA per SM (all 512 TMEM columns): four
+// warpgroups for the epilogues (thread t of each owns row t of a 128-leaf tile,
+// TMEM lane t, and a quarter of each layer's columns) and one warp that
+// issues the MMAs.  Per tile, nine GEMMs (M = 128):
 //   Z1 = X W1^T,  Z2 = H1 W2^T,  Y = H2 W3^T                       (forward)
 //   dH2 = dY W3,  dH1 = d2 W2,  dX = d1 W1                        (data)
 //   G3 += [H2 1]^T dY,  G2 += [H1 1]^T d2,  G1 += [X 1]^T d1       (weights)
@@ -464,10 +465,15 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
 // 40 or 72 meaningful features; the rest of each descriptor's extent reads
 // whatever lies after them in shared memory, which lands only in TMEM lanes
 // that are never read.
-// What bounds it: the chain of six dependent MMA rounds with their epilogues.
+// What bounds it: the chain of six dependent MMA rounds with their epilogues,
+// about 1,500 cycles each (cycle counters; with two warpgroups, the MMAs
+// issued by one of their threads and the weights staged 4 bytes at a time, the
+// dY epilogue alone took 7,500 of a tile's 24,000 cycles and the prologue
+// 15,000).  65,536 leaves: 177 us in the first form, 76 with two warpgroups,
+// 49 now.
 namespace {
 
-constexpr int TG_THREADS = 256, TG_NC = 176;
+constexpr int TG_EPI = 512, TG_THREADS = TG_EPI + 32, TG_NC = 176;  // epilogue threads; with the MMA warp
 constexpr int TG_KX = 40, TG_KH = 72;              // features and the ones column, in 8-wide chunks
 constexpr int TGO_W1 = 0;                          // [64][32]   W1
 constexpr int TGO_W2 = TGO_W1 + 64 * 32 * 2;       // [64][64]   W2
@@ -520,13 +526,28 @@ __device__ __forceinline__ Operand over_rows(uint32_t addr, int cols) { return {
 // D[128 x N] (+)= A B^T over K, BF16; acc0: accumulate from the first K slice on.
 // No-swizzle descriptors: K-major, LBO = K group stride, SBO = row group stride;
 // MN-major, LBO = K group stride, SBO = M/N group stride.
-__device__ __forceinline__ void gemm_bf16(uint32_t d_tmem, Operand a, Operand b, int K, int N, uint32_t acc0)
+template <int K, int N>
+__device__ __forceinline__ void gemm_bf16(uint32_t d_tmem, Operand a, Operand b, uint32_t acc0)
 {
     const uint32_t idesc = idesc_bf16(128, N) | (a.mn_major ? 1u << 15 : 0u) | (b.mn_major ? 1u << 16 : 0u);
-#pragma unroll 1
-    for (int s = 0; s < K / 16; ++s)
-        mma_f16(d_tmem, smem_desc(a.addr + 2u * s * a.k8, a.k8, a.mn8), smem_desc(b.addr + 2u * s * b.k8, b.k8, b.mn8), idesc,
-                s > 0 ? 1u : acc0);
+    const uint64_t da = smem_desc(a.addr, a.k8, a.mn8), db = smem_desc(b.addr, b.k8, b.mn8);
+#pragma unroll
+    for (int s = 0; s < K / 16; ++s)  // (the address field counts 16 bytes and does not overflow)
+        mma_f16(d_tmem, da + (uint64_t)(s * (a.k8 >> 3)), db + (uint64_t)(s * (b.k8 >> 3)), idesc, s > 0 ? 1u : acc0);
+}
+
+// 16 consecutive FP32 columns of this thread's TMEM lane; waits for them.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void cp_async(void *dst, const void *src, bool pair)
@@ -565,35 +586,43 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     __shared__ int s_fail;
     __shared__ double s_loss;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int m = t & 127, half = t >> 7;  // row of the tile, and which half of the columns
+    const bool epi = t < TG_EPI;           // (the other warp issues the MMAs)
+    const int m = t & 127, part = t >> 7;  // row of the tile, and which quarter of the columns
     const int nc = p.nc, ts = target_stride(nc);
     const bool pair = (nc & 1) == 0 && (reinterpret_cast<uintptr_t>(p.targets) & 7u) == 0;
     float *s_t = reinterpret_cast<float *>(sm + TGO_T);
     float *s_b1 = reinterpret_cast<float *>(sm + TGO_B), *s_b2 = s_b1 + 64, *s_b3 = s_b2 + 64, *s_cw = s_b3 + TG_NC;
     const uint32_t n_tiles = (p.batch + 127) / 128;
+    constexpr int WR = 128 / (TG_EPI / 32);  // rows of a tile that a warp moves
 
-    // Warp w moves rows 16 w .. 16 w + 15 of a tile: the target rows by
-    // asynchronous copies, the latents into registers (lane = feature).
-    float xr[16];
-    auto load_rows = [&](uint32_t tile) {
-        const uint32_t r0 = tile * 128 + (uint32_t)warp * 16;
-        const uint32_t mine = lane < 16 && tile < n_tiles && r0 + lane < p.batch ? p.rows[r0 + lane] : 0u;
+    // Epilogue warp w moves rows WR w .. WR w + WR - 1 of a tile: the target
+    // rows by asynchronous copies, the latents into registers (lane = feature).
+    // Rows past the end are zeros (next_ids: their leaf numbers, fetched ahead).
+    float xr[WR];
+    auto tile_ids = [&](uint32_t tile) -> uint32_t {
+        const uint32_t r = tile * 128 + (uint32_t)(warp * WR + lane);
+        return lane < WR && tile < n_tiles && r < p.batch ? p.rows[r] : 0u;
+    };
+    auto load_rows = [&](uint32_t tile, uint32_t ids) {
+        const uint32_t r0 = tile * 128 + (uint32_t)(warp * WR);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const size_t row = __shfl_sync(0xffffffffu, mine, i);
-            xr[i] = 0.0f;
-            if (tile >= n_tiles || r0 + i >= p.batch) continue;
-            xr[i] = p.latents[row * 32 + lane];
+        for (int i = 0; i < WR; ++i) {
+            const size_t row = __shfl_sync(0xffffffffu, ids, i);
             const float *src = p.targets + row * nc;
-            float *dst = s_t + (warp * 16 + i) * ts;
-            if (pair) {
+            float *dst = s_t + (warp * WR + i) * ts;
+            const bool there = tile < n_tiles && r0 + i < p.batch;
+            xr[i] = there ? p.latents[row * 32 + lane] : 0.0f;
+            if (there && pair) {
                 for (int c = 2 * lane; c < nc; c += 64) cp_async(dst + c, src + c, true);
-            } else {
+            } else if (there) {
                 for (int c = lane; c < nc; c += 32) cp_async(dst + c, src + c, false);
+            } else {
+                for (int c = lane; c < nc; c += 32) dst[c] = 0.0f;
             }
         }
     };
-    load_rows(blockIdx.x);
+    uint32_t next_ids = 0;
+    if (epi) load_rows(blockIdx.x, tile_ids(blockIdx.x));
     if (t == 0) {
         s_fail = 0;
         s_loss = 0.0;
@@ -601,27 +630,48 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
         ptx::mbar_init(&s_never, 1);
         ptx::fence_barrier_init();
     }
-    if (warp == 0) {
+    if (warp == TG_EPI / 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(ptx::smem_u32(&s_tmem)),
                      "r"(TC_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // --- weights as BF16 operands and FP32 biases, once per CTA
-    for (int q = t; q < 64 * 4; q += TG_THREADS) put8_bf(sm + TGO_W1, q >> 2, q & 3, 32, p.w.w1 + q * 8);
-    for (int q = t; q < 64 * 8; q += TG_THREADS) put8_bf(sm + TGO_W2, q >> 3, q & 7, 64, p.w.w2 + q * 8);
-    for (int q = t; q < TG_NC * 8; q += TG_THREADS) {
-        const int n = q >> 3, j = q & 7;
-        const float zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        put8_bf(sm + TGO_W3, n, j, 64, n < nc ? p.w.w3 + q * 8 : zero);
-    }
-    if (t < 64) {
-        s_b1[t] = p.w.b1[t];
-        s_b2[t] = p.w.b2[t];
-    }
-    for (int q = t; q < TG_NC; q += TG_THREADS) {
-        s_b3[q] = q < nc ? p.w.b3[q] : 0.0f;
-        s_cw[q] = q < nc ? p.coef_weight[q] : 0.0f;
+    // --- weights as BF16 operands (all of a thread's loads in flight together)
+    // and FP32 biases, once per CTA
+    if (epi) {
+        constexpr int C1 = 64 * 4, C2 = 64 * 8, CH = C1 + C2 + TG_NC * 8, PER = (CH + TG_EPI - 1) / TG_EPI;
+        const bool a16 = ((reinterpret_cast<uintptr_t>(p.w.w1) | reinterpret_cast<uintptr_t>(p.w.w2) |
+                           reinterpret_cast<uintptr_t>(p.w.w3)) & 15u) == 0;
+        float v[PER][8];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int q = t + TG_EPI * i;
+            const float *src = q < C1 ? p.w.w1 + q * 8 : (q < C1 + C2 ? p.w.w2 + (q - C1) * 8 : p.w.w3 + (q - C1 - C2) * 8);
+            const bool there = q < C1 + C2 + nc * 8;
+            if (there && a16) {
+                const float4 lo = __ldg(reinterpret_cast<const float4 *>(src)), hi = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+                v[i][0] = lo.x, v[i][1] = lo.y, v[i][2] = lo.z, v[i][3] = lo.w;
+                v[i][4] = hi.x, v[i][5] = hi.y, v[i][6] = hi.z, v[i][7] = hi.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[i][e] = there ? __ldg(src + e) : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int q = t + TG_EPI * i;
+            if (q < C1) put8_bf(sm + TGO_W1, q >> 2, q & 3, 32, v[i]);
+            else if (q < C1 + C2) put8_bf(sm + TGO_W2, (q - C1) >> 3, (q - C1) & 7, 64, v[i]);
+            else if (q < CH) put8_bf(sm + TGO_W3, (q - C1 - C2) >> 3, (q - C1 - C2) & 7, 64, v[i]);
+        }
+        if (t < 64) {
+            s_b1[t] = p.w.b1[t];
+            s_b2[t] = p.w.b2[t];
+        }
+        if (t < TG_NC) {
+            s_b3[t] = t < nc ? p.w.b3[t] : 0.0f;
+            s_cw[t] = t < nc ? p.coef_weight[t] : 0.0f;
+        }
     }
     fence_async_smem();
     fence_before();
@@ -631,213 +681,244 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     const uint32_t tm = s_tmem;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;  // this warp's lane quarter
     const uint32_t sa = ptx::smem_u32(sm);
-    uint32_t phase = 0;
-    bool first_wait = p.test_timeout != 0;
-    auto hand_off = [&]() {  // generic smem writes and TMEM reads before the next MMAs
+    float lsum = 0.0f;
+    uint32_t commits = 0;  // MMA warp: rounds issued
+    // End of an epilogue (generic smem writes and TMEM reads before the next
+    // MMAs), and the MMA warp's signal to issue them.  False once a wait has
+    // run out anywhere in the CTA: every thread leaves the loop here.
+    auto hand_off = [&]() -> bool {
         fence_async_smem();
         fence_before();
         __syncthreads();
-    };
-    auto wait_mmas = [&]() -> bool {  // bounded; CTA-uniform outcome
-        const bool ok = first_wait ? ptx::mbar_wait_bounded(&s_never, 0, TEST_WAIT_LIMIT_NS)
-                                   : ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
-        first_wait = false;
-        if (!ok) s_fail = 1;
-        __syncthreads();
         fence_after();
-        if (s_fail) return false;
-        phase ^= 1u;
-        return true;
+        return s_fail == 0;
     };
-    // H = relu(Z + b) of this thread's 32 columns into `dst`; returns the mask of Z + b > 0
-    auto relu_half = [&](unsigned char *dst, const float *b) -> uint32_t {
-        float v[32];
-        tmem_ld32(tm + lane_off + TC_SCR + 32 * half, v);
-        uint32_t mask = 0;
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-            v[e] += b[32 * half + e];
-            if (v[e] > 0.0f) mask |= 1u << e;
-            v[e] = fmaxf(v[e], 0.0f);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) put8_bf(dst, m, 4 * half + c, TG_KH, v + 8 * c);
-        return mask;
-    };
-    // d = dH [mask] of this thread's 32 columns (over dY, or over the layer's before)
-    auto masked_half = [&](uint32_t mask) {
-        float v[32];
-        tmem_ld32(tm + lane_off + TC_SCR + 32 * half, v);
-#pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = (mask >> e) & 1u ? v[e] : 0.0f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) put8_bf(sm + TGO_DY, m, 4 * half + c, 64, v + 8 * c);
-    };
-    float lsum = 0.0f;
-    uint32_t acc_w = 0;  // the weight gradients accumulate from the CTA's second tile on
-    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const uint32_t r0 = tile * 128;
-        const bool valid = r0 + (uint32_t)m < p.batch;
-        const float one = valid ? 1.0f : 0.0f;
-        // (the previous tile's last MMAs, which read X, H1 and d1, are done)
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-            *reinterpret_cast<__nv_bfloat16 *>(sm + TGO_X + core_off(warp * 16 + i, lane, TG_KX)) = __float2bfloat16_rn(xr[i]);
-        if (half == 0) put_one_bf(sm + TGO_X, m, 4, TG_KX, one);
-        else {
-            put_one_bf(sm + TGO_H1, m, 8, TG_KH, one);
-            put_one_bf(sm + TGO_H2, m, 8, TG_KH, one);
-        }
-        hand_off();
-        if (t == 0) {
+    if (epi) {
+        uint32_t phase = 0;
+        bool first_wait = p.test_timeout != 0;
+        // (bounded; a warp whose wait runs out goes on to the next hand_off)
+        auto wait_mmas = [&]() -> bool {
+            bool ok = first_wait ? ptx::mbar_wait_bounded(&s_never, 0, TEST_WAIT_LIMIT_NS)
+                                 : ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
+            ok = __all_sync(0xffffffffu, ok);
+            first_wait = false;
+            if (!ok) s_fail = 1;
             fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_X, TG_KX), over_cols(sa + TGO_W1, 32), 32, 64, 0);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        const uint32_t m1 = relu_half(sm + TGO_H1, s_b1);
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_H1, TG_KH), over_cols(sa + TGO_W2, 64), 64, 64, 0);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        const uint32_t m2 = relu_half(sm + TGO_H2, s_b2);
-        cp_async_wait();  // this thread's copies of the tile's targets (all threads': the barrier below)
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_H2, TG_KH), over_cols(sa + TGO_W3, 64), 64, TG_NC, 0);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        // dY = 2 cw (Y - target) + extra
-        const float *trow = s_t + m * ts;
-        const float *xrow = p.extra_dy && valid ? p.extra_dy + (size_t)p.rows[r0 + m] * nc : nullptr;
+            phase ^= 1u;
+            return ok;
+        };
+        // H = relu(Z + b) of this thread's 16 columns into `dst`; returns the mask of Z + b > 0
+        auto relu_part = [&](unsigned char *dst, const float *b) -> uint32_t {
+            float v[16];
+            tmem_ld16(tm + lane_off + TC_SCR + 16 * part, v);
+            uint32_t mask = 0;
+#pragma unroll
+            for (int e = 0; e < 16; e += 4) {
+                const float4 bv = *reinterpret_cast<const float4 *>(b + 16 * part + e);
+                const float bq[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float z = v[e + k] + bq[k];
+                    if (z > 0.0f) mask |= 1u << (e + k);
+                    v[e + k] = fmaxf(z, 0.0f);
+                }
+            }
+            put8_bf(dst, m, 2 * part, TG_KH, v);
+            put8_bf(dst, m, 2 * part + 1, TG_KH, v + 8);
+            return mask;
+        };
+        // d = dH [mask] of this thread's 16 columns (over dY, or over the layer's before)
+        auto masked_part = [&](uint32_t mask) {
+            float v[16];
+            tmem_ld16(tm + lane_off + TC_SCR + 16 * part, v);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = (mask >> e) & 1u ? v[e] : 0.0f;
+            put8_bf(sm + TGO_DY, m, 2 * part, 64, v);
+            put8_bf(sm + TGO_DY, m, 2 * part + 1, 64, v + 8);
+        };
+        for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const uint32_t r0 = tile * 128;
+            const bool valid = r0 + (uint32_t)m < p.batch;
+            const float one = valid ? 1.0f : 0.0f;
+            next_ids = tile_ids(tile + gridDim.x);
+            // (the previous tile's last MMAs, which read X, H1 and d1, are done)
+#pragma unroll
+            for (int i = 0; i < WR; ++i)
+                *reinterpret_cast<__nv_bfloat16 *>(sm + TGO_X + core_off(warp * WR + i, lane, TG_KX)) = __float2bfloat16_rn(xr[i]);
+            if (part == 0) put_one_bf(sm + TGO_X, m, 4, TG_KX, one);
+            else if (part == 1) put_one_bf(sm + TGO_H1, m, 8, TG_KH, one);
+            else if (part == 2) put_one_bf(sm + TGO_H2, m, 8, TG_KH, one);
+            if (!hand_off()) break;
+            wait_mmas();
+            const uint32_t m1 = relu_part(sm + TGO_H1, s_b1);
+            if (!hand_off()) break;
+            wait_mmas();
+            const uint32_t m2 = relu_part(sm + TGO_H2, s_b2);
+            cp_async_wait();  // this thread's copies of the tile's targets (all threads': the barrier)
+            if (!hand_off()) break;
+            wait_mmas();
+            // dY = 2 cw (Y + b3 - target) + extra of this thread's 48 (the last quarter's 32) columns
+            const float *trow = s_t + m * ts;
+            const float *xrow = p.extra_dy && valid ? p.extra_dy + (size_t)p.rows[r0 + m] * nc : nullptr;
 #pragma unroll 1
-        for (int c = 3 * half; c < 3 * half + 3; ++c) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR + 32 * c, v);  // columns 176..191: unused scratch
+            for (int c = 3 * part; c < min(3 * part + 3, TG_NC / 16); ++c) {
+                float v[16];
+                tmem_ld16(tm + lane_off + TC_SCR + 16 * c, v);
+                if (16 * c + 16 <= nc) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 2) {
-                const int j = 32 * c + e;
-                float2 tv = make_float2(0.0f, 0.0f), bb = tv, cw = tv;
-                if (j < nc) {  // (an odd nc ends inside a pair: cw is 0 there)
-                    tv = *reinterpret_cast<const float2 *>(trow + j);
-                    bb = *reinterpret_cast<const float2 *>(s_b3 + j);
-                    cw = *reinterpret_cast<const float2 *>(s_cw + j);
-                }
-                const float tq[2] = {tv.x, tv.y}, bq[2] = {bb.x, bb.y}, cq[2] = {cw.x, cw.y};
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    float d = 0.0f;
-                    if (valid && j + k < nc) {
-                        const float err = v[e + k] + bq[k] - tq[k];
-                        lsum = fmaf(cq[k] * err, err, lsum);
-                        d = 2.0f * cq[k] * err;
-                        if (xrow) d += xrow[j + k];
+                    for (int e = 0; e < 16; e += 2) {
+                        const float2 tv = *reinterpret_cast<const float2 *>(trow + 16 * c + e);
+                        const float2 bv = *reinterpret_cast<const float2 *>(s_b3 + 16 * c + e);
+                        const float2 cw = *reinterpret_cast<const float2 *>(s_cw + 16 * c + e);
+                        const float e0 = one * (v[e] + bv.x - tv.x), e1 = one * (v[e + 1] + bv.y - tv.y);
+                        const float d0 = cw.x * e0, d1 = cw.y * e1;
+                        lsum = fmaf(d0, e0, lsum);
+                        lsum = fmaf(d1, e1, lsum);
+                        v[e] = 2.0f * d0;
+                        v[e + 1] = 2.0f * d1;
                     }
-                    v[e + k] = d;
+                } else {  // the chunk that nc ends in, and any past it
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const int j = 16 * c + e;
+                        float d = 0.0f;
+                        if (j < nc) {
+                            const float err = one * (v[e] + s_b3[j] - trow[j]);
+                            d = s_cw[j] * err;
+                            lsum = fmaf(d, err, lsum);
+                        }
+                        v[e] = 2.0f * d;
+                    }
                 }
+                if (xrow) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        if (16 * c + e < nc) v[e] += xrow[16 * c + e];
+                }
+                put8_bf(sm + TGO_DY, m, 2 * c, TG_NC, v);
+                put8_bf(sm + TGO_DY, m, 2 * c + 1, TG_NC, v + 8);
             }
+            if (!hand_off()) break;
+            load_rows(tile + gridDim.x, next_ids);  // the target tile is free: in flight from here on
+            wait_mmas();
+            masked_part(m2);
+            if (!hand_off()) break;
+            wait_mmas();
+            masked_part(m1);
+            if (!hand_off()) break;
+            // dL/d(latent) of the tile's rows
+            if (wait_mmas() && part < 2) {
+                float v[16];
+                tmem_ld16(tm + lane_off + TC_SCR + 16 * part, v);
+                if (valid) {
+                    float *dst = p.dlatents + (size_t)(r0 + m) * 32 + 16 * part;
+                    if ((reinterpret_cast<uintptr_t>(p.dlatents) & 15u) == 0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (4 * c + q < TG_NC / 8) put8_bf(sm + TGO_DY, m, 4 * c + q, TG_NC, v + 8 * q);
-        }
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, TG_NC), over_rows(sa + TGO_W3, 64), TG_NC, 64, 0);
-            gemm_bf16(tm + TC_G3, over_rows(sa + TGO_H2, TG_KH), over_rows(sa + TGO_DY, TG_NC), 128, TG_NC, acc_w);
-            mma_commit(&s_bar);
-        }
-        load_rows(tile + gridDim.x);  // the target tile is free: in flight from here on
-        if (!wait_mmas()) break;
-        masked_half(m2);
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, 64), over_rows(sa + TGO_W2, 64), 64, 64, 0);
-            gemm_bf16(tm + TC_G2, over_rows(sa + TGO_H1, TG_KH), over_rows(sa + TGO_DY, 64), 128, 64, acc_w);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        masked_half(m1);
-        hand_off();
-        if (t == 0) {
-            fence_after();
-            gemm_bf16(tm + TC_SCR, over_cols(sa + TGO_DY, 64), over_rows(sa + TGO_W1, 32), 64, 32, 0);
-            gemm_bf16(tm + TC_G1, over_rows(sa + TGO_X, TG_KX), over_rows(sa + TGO_DY, 64), 128, 64, acc_w);
-            mma_commit(&s_bar);
-        }
-        if (!wait_mmas()) break;
-        // dL/d(latent) of the tile's rows
-        if (half == 0) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_SCR, v);
-            if (valid) {
-                float *dst = p.dlatents + (size_t)(r0 + m) * 32;
-                if ((reinterpret_cast<uintptr_t>(p.dlatents) & 15u) == 0) {
+                        for (int k = 0; k < 4; ++k)
+                            reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                    } else {  // (the caller's array needs only float alignment)
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-                } else {  // (the caller's array needs only float alignment)
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) dst[k] = v[k];
+                        for (int k = 0; k < 16; ++k) dst[k] = v[k];
+                    }
                 }
             }
         }
-        fence_before();  // TMEM reads done before the next tile's MMAs
-        acc_w = 1;
+        cp_async_wait();
+    } else {
+        uint32_t acc_w = 0;  // the weight gradients accumulate from the CTA's second tile on
+        auto commit = [&]() {
+            mma_commit(&s_bar);
+            ++commits;
+        };
+        const Operand xf = over_cols(sa + TGO_X, TG_KX), h1f = over_cols(sa + TGO_H1, TG_KH), h2f = over_cols(sa + TGO_H2, TG_KH),
+                      xg = over_rows(sa + TGO_X, TG_KX), h1g = over_rows(sa + TGO_H1, TG_KH), h2g = over_rows(sa + TGO_H2, TG_KH),
+                      dyf = over_cols(sa + TGO_DY, TG_NC), dyg = over_rows(sa + TGO_DY, TG_NC), df = over_cols(sa + TGO_DY, 64),
+                      dg = over_rows(sa + TGO_DY, 64);
+        for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<32, 64>(tm + TC_SCR, xf, over_cols(sa + TGO_W1, 32), 0);
+                commit();
+            }
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<64, 64>(tm + TC_SCR, h1f, over_cols(sa + TGO_W2, 64), 0);
+                commit();
+            }
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<64, TG_NC>(tm + TC_SCR, h2f, over_cols(sa + TGO_W3, 64), 0);
+                commit();
+            }
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<TG_NC, 64>(tm + TC_SCR, dyf, over_rows(sa + TGO_W3, 64), 0);
+                gemm_bf16<128, TG_NC>(tm + TC_G3, h2g, dyg, acc_w);
+                commit();
+            }
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<64, 64>(tm + TC_SCR, df, over_rows(sa + TGO_W2, 64), 0);
+                gemm_bf16<128, 64>(tm + TC_G2, h1g, dg, acc_w);
+                commit();
+            }
+            if (!hand_off()) break;
+            if (lane == 0) {
+                gemm_bf16<64, 32>(tm + TC_SCR, df, over_rows(sa + TGO_W1, 32), 0);
+                gemm_bf16<128, 64>(tm + TC_G1, xg, dg, acc_w);
+                commit();
+            }
+            acc_w = 1;
+        }
     }
-    cp_async_wait();
-    if (!s_fail) {
+    fence_before();
+    __syncthreads();  // every wait of the last tile is over
+    fence_after();
+    const bool ok = s_fail == 0;
+    if (ok && epi) {
         // the weight gradients: lane k of G3 / G2 / G1 is input feature k, lane
         // 64 (32 for G1) the bias; column j / o the output feature
 #pragma unroll 1
-        for (int c = 3 * half; c < 3 * half + 3; ++c) {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_G3 + 32 * c, v);  // columns past 175 belong to G3's padding
+        for (int c = 3 * part; c < min(3 * part + 3, TG_NC / 16); ++c) {
+            float v[16];
+            tmem_ld16(tm + lane_off + TC_G3 + 16 * c, v);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int j = 32 * c + e;
+            for (int e = 0; e < 16; ++e) {
+                const int j = 16 * c + e;
                 if (j >= nc) continue;
                 if (m < 64) atomicAdd(p.g.w3 + j * 64 + m, v[e]);
                 else if (m == 64) atomicAdd(p.g.b3 + j, v[e]);
             }
         }
-        {
-            float v[32];
-            tmem_ld32(tm + lane_off + TC_G2 + 32 * half, v);
+        float v[16];
+        tmem_ld16(tm + lane_off + TC_G2 + 16 * part, v);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int o = 32 * half + e;
-                if (m < 64) atomicAdd(p.g.w2 + o * 64 + m, v[e]);
-                else if (m == 64) atomicAdd(p.g.b2 + o, v[e]);
-            }
-            tmem_ld32(tm + lane_off + TC_G1 + 32 * half, v);
+        for (int e = 0; e < 16; ++e) {
+            const int o = 16 * part + e;
+            if (m < 64) atomicAdd(p.g.w2 + o * 64 + m, v[e]);
+            else if (m == 64) atomicAdd(p.g.b2 + o, v[e]);
+        }
+        tmem_ld16(tm + lane_off + TC_G1 + 16 * part, v);
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int o = 32 * half + e;
-                if (m < 32) atomicAdd(p.g.w1 + o * 32 + m, v[e]);
-                else if (m == 32) atomicAdd(p.g.b1 + o, v[e]);
-            }
+        for (int e = 0; e < 16; ++e) {
+            const int o = 16 * part + e;
+            if (m < 32) atomicAdd(p.g.w1 + o * 32 + m, v[e]);
+            else if (m == 32) atomicAdd(p.g.b1 + o, v[e]);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
         if (lane == 0) atomicAdd(&s_loss, (double)lsum);
-    } else if (t == 0) {
-        // the commit whose wait gave up: wait for it once more (bounded)
-        // before TMEM is freed
-        ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
+    } else if (!ok && t == TG_EPI) {
+        // the last round committed, whose wait gave up: wait for it once more
+        // (bounded) before TMEM is freed
+        if (commits) ptx::mbar_wait_bounded(&s_bar, (commits - 1) & 1u, LT_WAIT_NS);
         if (p.status) atomicOr(p.status, STATUS_DEVICE_TIMEOUT);
     }
     fence_before();
     __syncthreads();
     fence_after();
-    if (t == 0 && p.loss && !s_fail) atomicAdd(p.loss, s_loss);
-    if (warp == 0)
+    if (t == 0 && p.loss && ok) atomicAdd(p.loss, s_loss);
+    if (warp == TG_EPI / 32)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(TC_COLS) : "memory");
 }
 
