@@ -227,14 +227,35 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // 8 consecutive BF16 weights as FP32, in one 16-byte load where the arrays allow it
+    const bool a16 = ((reinterpret_cast<uintptr_t>(p.w1) | reinterpret_cast<uintptr_t>(p.w2) | reinterpret_cast<uintptr_t>(p.w3)) & 15u) == 0;
+    auto load8 = [&](const uint16_t *src, float v[8]) {
+        uint32_t u[4];
+        if (a16) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(src));
+            u[0] = w.x, u[1] = w.y, u[2] = w.z, u[3] = w.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) u[e] = (uint32_t)__ldg(src + 2 * e) | ((uint32_t)__ldg(src + 2 * e + 1) << 16);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            v[2 * e] = __uint_as_float(u[e] << 16);
+            v[2 * e + 1] = __uint_as_float(u[e] & 0xffff0000u);
+        }
+    };
+    auto in_range = [&](const float v[8]) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (!(fabsf(v[e]) <= F16_MAX)) s_range = 1;
+    };
+#pragma unroll 2
     for (int q = tid; q < 64 * (K1 / 8); q += LT_THREADS) {  // W1 | b1: 64 rows x 6 chunks
         const int n = q / (K1 / 8), j = q % (K1 / 8);
         if (j < 4) {
             float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = __bfloat162float(__ushort_as_bfloat16(p.w1[n * 32 + 8 * j + e]));
-            for (int e = 0; e < 8; ++e)
-                if (!(fabsf(v[e]) <= F16_MAX)) s_range = 1;
+            load8(p.w1 + n * 32 + 8 * j, v);
+            in_range(v);
             put8(lt_smem + OFF_W1, n, j, K1, v);
         } else if (j == 4) {
             if (!(fabsf(p.b1[n]) <= F16_MAX)) s_range = 1;
@@ -243,14 +264,13 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
             put_zero_chunk(lt_smem + OFF_W1, n, j, K1);
         }
     }
+#pragma unroll 3
     for (int q = tid; q < 64 * (K2 / 8); q += LT_THREADS) {  // W2 | b2: 64 rows x 10 chunks
         const int n = q / (K2 / 8), j = q % (K2 / 8);
         if (j < 8) {
             float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = __bfloat162float(__ushort_as_bfloat16(p.w2[n * 64 + 8 * j + e]));
-            for (int e = 0; e < 8; ++e)
-                if (!(fabsf(v[e]) <= F16_MAX)) s_range = 1;
+            load8(p.w2 + n * 64 + 8 * j, v);
+            in_range(v);
             put8(lt_smem + OFF_W2, n, j, K2, v);
         } else if (j == 8) {
             if (!(fabsf(p.b2[n]) <= F16_MAX)) s_range = 1;
@@ -261,18 +281,22 @@ __global__ void __launch_bounds__(128 * G, 8 / G) latent_table_kernel(const __gr
     }
     __syncthreads();  // s_basis ready
     // W3'(t): row 0 = sum_i b_i W3[i], row 1 + q = sum_i b_i W3[n1 + q n2 + i],
-    // rows 28..31 = 0.  One output element per thread and pass: the loads of a
-    // row are coalesced over h and independent of each other (unrolled), so
-    // the prologue costs a few memory latencies, not one per term.
-    for (int q = tid; q < 32 * 64; q += LT_THREADS) {
-        const int r = q >> 6, h = q & 63;
+    // rows 28..31 = 0.  Eight output elements per thread: 16-byte loads,
+    // independent of each other, so the fold costs a few memory latencies
+    // (element by element it took most of the prologue).
+    for (int q = tid; q < 32 * 8; q += LT_THREADS) {
+        const int r = q >> 3, c = q & 7;
         const int row0 = r == 0 ? 0 : p.n1 + (r - 1) * p.n2, terms = r == 0 ? p.n1 : (r <= 27 ? p.n2 : 0);
-        float acc = 0.0f;
-#pragma unroll 8
-        for (int i = 0; i < terms; ++i)
-            acc = fmaf(s_basis[i], __bfloat162float(__ushort_as_bfloat16(p.w3[(row0 + i) * 64 + h])), acc);
-        if (!(fabsf(acc) <= F16_MAX)) s_range = 1;
-        *reinterpret_cast<__half *>(lt_smem + OFF_W3 + core_off(r, h, K2)) = __float2half_rn(acc);
+        float acc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 5
+        for (int i = 0; i < terms; ++i) {
+            float v[8];
+            load8(p.w3 + (row0 + i) * 64 + 8 * c, v);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(s_basis[i], v[e], acc[e]);
+        }
+        in_range(acc);
+        put8(lt_smem + OFF_W3, r, c, K2, acc);
     }
     if (tid < 32) {
         const int row0 = tid == 0 ? 0 : p.n1 + (tid - 1) * p.n2, terms = tid == 0 ? p.n1 : (tid <= 27 ? p.n2 : 0);
