@@ -374,6 +374,16 @@ int fpo_union_trees(uint32_t n_frames, const fpo_frame_tree *frames, uint32_t ma
                     uint32_t *n_union, uint8_t *union_depth, uint32_t *union_xyz,
                     float *union_values, uint32_t capacity);
 
+/* Training rays of the pinhole model above, from drawn indices: ray i is pixel
+ * pixel[i] (row * width + column) of camera cam[i] at frame frame[i] (device
+ * int64 [n]); basis: device [n_cams][12], each camera's eye, forward, right
+ * and up vectors.  o, d (unit directions): device [n][3]; t: device [n].
+ * Each value is rounded after every operation, as an elementwise framework
+ * does it.  Errors: INVALID_ARG, CUDA. */
+int fpo_camera_ray_batch(const float *basis, const int64_t *cam, const int64_t *pixel, const int64_t *frame, uint32_t n,
+                         uint32_t width, uint32_t height, double fov_y_deg, float *o, float *d, float *t,
+                         void *cuda_stream);
+
 /* A latent decoder: per leaf a 32-dim FP16 latent, decoded by a shared MLP
  * 32 -> 64 -> 64 -> n1 + 27*n2 with ReLU after the first two layers (the
  * learned stand-in for the per-leaf coefficients of Sec. 4.1; the paper's own

@@ -46,15 +46,15 @@ def camera_ray_batch(cams, n, gen, n_frames=60, basis=None):
 
     B = camera_basis(cams) if basis is None else basis
     W, H = cams[0].width, cams[0].height
-    th = np.tan(np.radians(cams[0].fov_y_deg) / 2)
     v = torch.randint(0, len(cams), (n,), device="cuda", generator=gen)
     p = torch.randint(0, W * H, (n,), device="cuda", generator=gen)
-    t = torch.randint(0, n_frames, (n,), device="cuda", generator=gen).float()
-    sx = ((2 * ((p % W).float() + 0.5) / W - 1) * th * W / H)[:, None]
-    sy = ((1 - 2 * ((p // W).float() + 0.5) / H) * th)[:, None]
-    b = B[v]
-    d = b[:, 3:6] + sx * b[:, 6:9] + sy * b[:, 9:12]
-    return b[:, 0:3].contiguous(), (d / d.norm(dim=1, keepdim=True)).contiguous(), t
+    f = torch.randint(0, n_frames, (n,), device="cuda", generator=gen)
+    B = B.contiguous()
+    o, d, t = (torch.empty(s, device="cuda") for s in ((n, 3), (n, 3), (n,)))
+    ptr = lambda x: x.data_ptr() if n else None
+    fpo.check(fpo.lib().fpo_camera_ray_batch(B.data_ptr(), ptr(v), ptr(p), ptr(f), n, W, H, float(cams[0].fov_y_deg),
+                                             ptr(o), ptr(d), ptr(t), fpo._stream_handle(None)))
+    return o, d, t
 
 
 class FineTuner:

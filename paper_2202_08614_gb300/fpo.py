@@ -36,7 +36,7 @@ EXPORTS = ["fpo_create", "fpo_validate_tree", "fpo_upload_tree", "fpo_render",
            "fpo_dft_leaves", "fpo_union_trees", "fpo_latent_table", "fpo_decoder_grad",
            "fpo_adam", "fpo_set_latents", "fpo_render_frames", "fpo_adam_leaves",
            "fpo_decoder_forward", "fpo_set_coeffs_from_decoder", "fpo_fma_peak", "fpo_decoder_grad_tc",
-           "fpo_adam_parts"]
+           "fpo_adam_parts", "fpo_camera_ray_batch"]
 
 
 class FPOError(RuntimeError):
@@ -130,6 +130,7 @@ def lib():
         L.fpo_fma_peak.argtypes = [C.c_uint32, C.c_uint32, C.c_uint32, P, C.POINTER(C.c_double), P]
         L.fpo_adam.argtypes = [P, P, P, P, C.c_uint64, P, C.c_uint32, C.c_float, C.c_float,
                                C.c_float, C.c_float, C.c_uint32, P]
+        L.fpo_camera_ray_batch.argtypes = [P, P, P, P, C.c_uint32, C.c_uint32, C.c_uint32, C.c_double, P, P, P, P]
         L.fpo_adam_parts.argtypes = [C.POINTER(AdamPart), C.c_uint32, C.c_float, C.c_float, C.c_float,
                                      C.c_uint32, P]
         L.fpo_set_latents.argtypes = [P, P, C.POINTER(Decoder), P]
