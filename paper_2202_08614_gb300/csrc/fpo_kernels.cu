@@ -29,13 +29,6 @@
 #ifndef FPO_LDG256
 #define FPO_LDG256 1
 #endif
-#ifndef FPO_MAT_HALF_WARP
-// FP32 records, n2 = 5, FP32 table: half (1) or a quarter (2) of a warp per
-// leaf; 3: a quarter in the frame pipeline (fewer instructions beside the
-// traversal: 0.676 against 0.689 ms per 1080p frame) and a half alone (0.417
-// against 0.427 ms).  All forms sum in the same order.
-#define FPO_MAT_HALF_WARP 3
-#endif
 namespace fpo {
 namespace {
 
@@ -113,8 +106,22 @@ __device__ __forceinline__ float stored(const unsigned char *rec, int i)
     else return static_cast<float>(reinterpret_cast<const __nv_fp8_e4m3 *>(rec)[i]);
 }
 
-template <int N2, int ST>
-__global__ void __launch_bounds__(MAT_THREADS, 8) materialise_kernel(const __grid_constant__ MaterialiseParams p)
+// How a warp takes the chunk's leaves:
+//   MF_WARP     one leaf at a time, a lane per output (any storage and sizes);
+//   MF_WARP2    the same, two leaves in flight (FP32 records with n2 = 5 and
+//               the FP32 table, a frame alone, where the pass itself is the
+//               bound and registers are free: 799 us a 1080p frame, one leaf
+//               807, four 816, halves of a warp per leaf 831, quarters 820;
+//               copies of 64 instead of 100 KB in flight a CTA 839, 110 KB 817);
+//   MF_QUARTER  four leaves, a quarter of the warp each (the same records in
+//               the frame pipeline, where the traversal beside it feels the
+//               pass's instructions: eight frames in 4.72 ms, halves 5.08).
+// Each is an instantiation of its own: two forms in one kernel took the
+// pipelined frames to 5.14 ms.  All sum in the same order.
+constexpr int MF_WARP = 0, MF_WARP2 = 1, MF_QUARTER = 2;
+
+template <int N2, int ST, int FORM>
+__global__ void __launch_bounds__(MAT_THREADS, FORM == MF_WARP2 ? 2 : 8) materialise_kernel(const __grid_constant__ MaterialiseParams p)
 {
     extern __shared__ __align__(128) unsigned char mat_smem[];
     __shared__ uint64_t bars[MAT_MAX_STAGES];
@@ -161,20 +168,16 @@ __global__ void __launch_bounds__(MAT_THREADS, 8) materialise_kernel(const __gri
 
     const int warp = tid >> 5, lane = tid & 31;
     const float b_lane = lane < nb ? s_b[lane] : 0.0f;
-    const float b_lo = (lane & 15) < nb ? s_b[lane & 15] : 0.0f;              // half-warp form
-    const float b_hi = (lane & 15) + 16 < nb ? s_b[(lane & 15) + 16] : 0.0f;
-    float bq[4];                                                             // quarter-warp form
+    float bq[4];  // quarter-warp form
 #pragma unroll
     for (int k = 0; k < 4; ++k) bq[k] = (lane & 7) + 8 * k < nb ? s_b[(lane & 7) + 8 * k] : 0.0f;
     float bz[N2 > 0 ? N2 : 1];
 #pragma unroll
     for (int i = 0; i < (N2 > 0 ? N2 : 1); ++i) bz[i] = s_b[i];
     uint32_t it = 0;
-    for (;; ++it) {
-        const uint32_t c = blockIdx.x + it * gridDim.x;
-        if (c >= n_chunks) break;
-        const int s = (int)(it % (uint32_t)S);
-        const uint32_t parity = (it / (uint32_t)S) & 1u;
+    int s = 0;  // stage it mod S, and the parity of its it / S-th filling
+    uint32_t parity = 0;
+    for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x, ++it, parity ^= s + 1 == S, s = s + 1 == S ? 0 : s + 1) {
         // (the failure-path test makes the first wait run out; the drain below
         // still waits for every copy in flight)
         const bool ok = p.test_timeout && it == 0 ? ptx::mbar_wait_bounded(&never, 0, TEST_WAIT_LIMIT_NS)
@@ -187,132 +190,73 @@ __global__ void __launch_bounds__(MAT_THREADS, 8) materialise_kernel(const __gri
         const unsigned char *stage_sig = mat_smem + (size_t)s * stage_bytes;
         const unsigned char *stage_z = stage_sig + sig_bytes;
         const float *stage_scale = reinterpret_cast<const float *>(stage_z + z_bytes);
-        if constexpr ((FPO_MAT_HALF_WARP == 2 || FPO_MAT_HALF_WARP == 3) && N2 == 5 && ST == FPO_STORAGE_F32) {
-            if (!p.half_table && (FPO_MAT_HALF_WARP == 2 || p.pipeline)) {
-                // A quarter warp (8 lanes) per leaf, four leaves per pass:
-                // lane ql forms the products of i = ql, ql + 8, ql + 16,
-                // ql + 24 and sums them as the full warp's butterfly does
-                // ((i, i + 16), then + (i + 8, i + 24)), then xor 4, 2, 1 within
-                // the quarter; it forms z_{ql + 8k}, k = 0..3, and stores
-                // row[ql + 8k].
-                const int qw = lane >> 3, ql = lane & 7;
-                for (int l0 = 4 * warp; l0 < m; l0 += 4 * (MAT_THREADS / 32)) {
-                    const int l = l0 + qw;
-                    const bool valid = l < m;
-                    const float *sg = reinterpret_cast<const float *>(stage_sig + (valid ? l : l0) * rec_sig);
-                    const float *zz = reinterpret_cast<const float *>(stage_z + (valid ? l : l0) * rec_z);
-                    float pr[4];
+        if constexpr (FORM == MF_QUARTER) {
+            // A quarter warp (8 lanes) per leaf, the chunk's 32 leaves in one
+            // pass: lane ql forms the products of i = ql, ql + 8, ql + 16,
+            // ql + 24 and sums them as the full warp's butterfly does
+            // ((i, i + 16), then + (i + 8, i + 24)), then xor 4, 2, 1 within
+            // the quarter; it forms and stores row[ql + 8k], k = 0..3:
+            // sigma, or z_{ql + 8k - 1} from where it is stored.
+            static_assert(MAT_CHUNK == 4 * (MAT_THREADS / 32), "one pass");
+            const int l = 4 * warp + (lane >> 3), ql = lane & 7;
+            if (4 * warp < m) {  // (warp-uniform; leaves past m: the stage's old contents, not stored)
+                const float *sg = reinterpret_cast<const float *>(stage_sig + l * rec_sig);
+                const float *zz = reinterpret_cast<const float *>(stage_z + l * rec_z) + (ql - 1) * 5;
+                float pr[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) pr[k] = ql + 8 * k < p.n1 ? __fmul_rn(sg[ql + 8 * k], bq[k]) : 0.0f;
-                    float part = __fadd_rn(__fadd_rn(pr[0], pr[2]), __fadd_rn(pr[1], pr[3]));
+                for (int k = 0; k < 4; ++k) pr[k] = ql + 8 * k < p.n1 ? __fmul_rn(sg[ql + 8 * k], bq[k]) : 0.0f;
+                float part = __fadd_rn(__fadd_rn(pr[0], pr[2]), __fadd_rn(pr[1], pr[3]));
 #pragma unroll
-                    for (int o = 4; o >= 1; o >>= 1) part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, o));
-                    float zq[4];
+                for (int o = 4; o >= 1; o >>= 1) part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, o));
+                float o[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        zq[k] = 0.0f;
-                        if (ql + 8 * k < 27) {
+                for (int k = 0; k < 4; ++k) {
+                    o[k] = 0.0f;
+                    if (k == 3 ? ql < 4 : k > 0 || ql > 0) {
 #pragma unroll
-                            for (int i = 0; i < 5; ++i) zq[k] = fmaf(zz[(ql + 8 * k) * 5 + i], bz[i], zq[k]);
-                        }
-                    }
-                    float o[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        // row[ql + 8k] = z[ql + 8k - 1]: lane ql - 1's zq[k], or lane 7's zq[k - 1] for ql = 0
-                        const float up = __shfl_up_sync(0xffffffffu, zq[k], 1, 8);
-                        const float from7 = __shfl_sync(0xffffffffu, zq[k > 0 ? k - 1 : 0], 7, 8);
-                        const int j = ql + 8 * k;
-                        o[k] = ql == 0 ? (k == 0 ? fmaxf(part, 0.0f) : from7) : (j <= 27 ? up : 0.0f);
-                    }
-                    if (valid) {
-                        float *row = p.table + ((size_t)first + l) * TABLE_STRIDE;
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) row[ql + 8 * k] = o[k];
+                        for (int i = 0; i < 5; ++i) o[k] = fmaf(zz[40 * k + i], bz[i], o[k]);
+                    } else if (k == 0) {
+                        o[k] = fmaxf(part, 0.0f);
                     }
                 }
-                __syncthreads();  // every thread is done with stage s
-                if (tid == 0) {
-                    const uint32_t c2 = c + (uint32_t)S * gridDim.x;
-                    if (c2 < n_chunks) issue(c2, s);
-                }
-                continue;
+                float *row = p.table + ((size_t)first + l) * TABLE_STRIDE + ql;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (l < m) row[8 * k] = o[k];
             }
-        }
-        if constexpr ((FPO_MAT_HALF_WARP == 1 || FPO_MAT_HALF_WARP == 3) && N2 == 5 && ST == FPO_STORAGE_F32) {
-            if (!p.half_table) {
-                // Half a warp per leaf, two leaves per pass: lane sl of a half
-                // forms k_sl b_sl + k_{sl+16} b_{sl+16} (the first step of the
-                // full warp's butterfly) and the butterfly continues within the
-                // half, so the density sums in the same order; z_{sl} and
-                // z_{sl+16} are the same sequential sums.  Each lane stores
-                // row[sl] and row[sl + 16].
-                const int hw = lane >> 4, sl = lane & 15;
-                for (int l0 = 2 * warp; l0 < m; l0 += 2 * (MAT_THREADS / 32)) {
-                    const int l = l0 + hw;
-                    const bool valid = l < m;
-                    const float *sg = reinterpret_cast<const float *>(stage_sig + (valid ? l : l0) * rec_sig);
-                    const float *zz = reinterpret_cast<const float *>(stage_z + (valid ? l : l0) * rec_z);
-                    const float p1 = sl < p.n1 ? __fmul_rn(sg[sl], b_lo) : 0.0f;
-                    const float p2 = sl + 16 < p.n1 ? __fmul_rn(sg[sl + 16], b_hi) : 0.0f;
-                    float part = __fadd_rn(p1, p2);
+        } else {
+            // One warp per leaf: lane i < n1 forms k_sigma_i b_i and a butterfly
+            // sums the density; lanes 0..26 form z_{lane}(t) from n2 consecutive
+            // elements.  Lane j then stores output j.
+            constexpr int UN = FORM == MF_WARP2 ? 2 : 1;
+#pragma unroll UN
+            for (int l = warp; l < m; l += MAT_THREADS / 32) {
+                const unsigned char *sg = stage_sig + l * rec_sig;
+                const unsigned char *zz = stage_z + l * rec_z;
+                float part = lane < p.n1 ? stored<ST>(sg, lane) * b_lane : 0.0f;
 #pragma unroll
-                    for (int o = 8; o >= 1; o >>= 1) part = __fadd_rn(part, __shfl_xor_sync(0xffffffffu, part, o));
-                    float za = 0.0f, zb = 0.0f;
+                for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+                float v = 0.0f;
+                if (lane < 27) {
+                    if constexpr (N2 > 0) {
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) za = fmaf(zz[sl * 5 + i], bz[i], za);
-                    if (sl < 11) {
-#pragma unroll
-                        for (int i = 0; i < 5; ++i) zb = fmaf(zz[(sl + 16) * 5 + i], bz[i], zb);
-                    }
-                    const float za_prev = __shfl_up_sync(0xffffffffu, za, 1, 16);
-                    const float zb_prev = __shfl_up_sync(0xffffffffu, zb, 1, 16);
-                    const float za_15 = __shfl_sync(0xffffffffu, za, 15, 16);
-                    const float o1 = sl == 0 ? fmaxf(part, 0.0f) : za_prev;
-                    const float o2 = sl == 0 ? za_15 : (sl + 16 <= 27 ? zb_prev : 0.0f);
-                    if (valid) {
-                        float *row = p.table + ((size_t)first + l) * TABLE_STRIDE;
-                        row[sl] = o1;
-                        row[sl + 16] = o2;
+                        for (int i = 0; i < N2; ++i) v = fmaf(stored<ST>(zz, lane * N2 + i), bz[i], v);
+                    } else {
+                        for (int i = 0; i < p.n2; ++i) v = fmaf(stored<ST>(zz, lane * p.n2 + i), s_b[i], v);
                     }
                 }
-                __syncthreads();  // every thread is done with stage s
-                if (tid == 0) {
-                    const uint32_t c2 = c + (uint32_t)S * gridDim.x;
-                    if (c2 < n_chunks) issue(c2, s);
+                if (SCALED) {
+                    const float sc = stage_scale[l];
+                    part *= sc;
+                    v *= sc;
                 }
-                continue;
+                const float zprev = __shfl_up_sync(0xffffffffu, v, 1);
+                const float outv = lane == 0 ? fmaxf(part, 0.0f) : (lane <= 27 ? zprev : 0.0f);
+                if (p.half_table)
+                    reinterpret_cast<__half *>(p.table)[((size_t)first + l) * TABLE_STRIDE + lane] = __float2half_rn(outv);
+                else
+                    p.table[((size_t)first + l) * TABLE_STRIDE + lane] = outv;
             }
-        }
-        // One warp per leaf: lane i < n1 forms k_sigma_i b_i and a butterfly
-        // sums the density; lanes 0..26 form z_{lane}(t) from n2 consecutive
-        // elements.  Lane j then stores output j.
-        for (int l = warp; l < m; l += MAT_THREADS / 32) {
-            const unsigned char *sg = stage_sig + l * rec_sig;
-            const unsigned char *zz = stage_z + l * rec_z;
-            float part = lane < p.n1 ? stored<ST>(sg, lane) * b_lane : 0.0f;
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            float v = 0.0f;
-            if (lane < 27) {
-                if constexpr (N2 > 0) {
-#pragma unroll
-                    for (int i = 0; i < N2; ++i) v = fmaf(stored<ST>(zz, lane * N2 + i), bz[i], v);
-                } else {
-                    for (int i = 0; i < p.n2; ++i) v = fmaf(stored<ST>(zz, lane * p.n2 + i), s_b[i], v);
-                }
-            }
-            if (SCALED) {
-                const float sc = stage_scale[l];
-                part *= sc;
-                v *= sc;
-            }
-            const float zprev = __shfl_up_sync(0xffffffffu, v, 1);
-            const float outv = lane == 0 ? fmaxf(part, 0.0f) : (lane <= 27 ? zprev : 0.0f);
-            if (p.half_table)
-                reinterpret_cast<__half *>(p.table)[((size_t)first + l) * TABLE_STRIDE + lane] = __float2half_rn(outv);
-            else
-                p.table[((size_t)first + l) * TABLE_STRIDE + lane] = outv;
         }
         __syncthreads();  // every thread is done with stage s
         if (tid == 0) {
@@ -431,11 +375,9 @@ __global__ void __launch_bounds__(CH, ST == FPO_STORAGE_F32 ? 4 : 1) materialise
 #pragma unroll
     for (int i = 0; i < ML_N2; ++i) bz[i] = s_b[i];
     uint32_t it = 0;
-    for (;; ++it) {
-        const uint32_t c = blockIdx.x + it * gridDim.x;
-        if (c >= n_chunks) break;
-        const int s = (int)(it % (uint32_t)S);
-        const uint32_t parity = (it / (uint32_t)S) & 1u;
+    int s = 0;  // stage it mod S, and the parity of its it / S-th filling
+    uint32_t parity = 0;
+    for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x, ++it, parity ^= s + 1 == S, s = s + 1 == S ? 0 : s + 1) {
         // (the failure-path test makes the first wait run out; the drain below
         // still waits for every copy in flight)
         const bool ok = p.test_timeout && it == 0 ? ptx::mbar_wait_bounded(&never, 0, TEST_WAIT_LIMIT_NS)
@@ -617,10 +559,10 @@ template <int N2>
 static void *pick_materialise(int storage)
 {
     switch (storage) {
-    case FPO_STORAGE_BF16: return (void *)materialise_kernel<N2, FPO_STORAGE_BF16>;
-    case FPO_STORAGE_F16: return (void *)materialise_kernel<N2, FPO_STORAGE_F16>;
-    case FPO_STORAGE_FP8_E4M3: return (void *)materialise_kernel<N2, FPO_STORAGE_FP8_E4M3>;
-    default: return (void *)materialise_kernel<N2, FPO_STORAGE_F32>;
+    case FPO_STORAGE_BF16: return (void *)materialise_kernel<N2, FPO_STORAGE_BF16, MF_WARP>;
+    case FPO_STORAGE_F16: return (void *)materialise_kernel<N2, FPO_STORAGE_F16, MF_WARP>;
+    case FPO_STORAGE_FP8_E4M3: return (void *)materialise_kernel<N2, FPO_STORAGE_FP8_E4M3, MF_WARP>;
+    default: return (void *)materialise_kernel<N2, FPO_STORAGE_F32, MF_WARP>;
     }
 }
 
@@ -637,6 +579,9 @@ int launch_materialise(const MaterialiseParams &p, int sm_count, void *stream)
     const void *kern;
     if (lf)
         kern = lc == ML_CHUNK ? pick_leaf<ML_CHUNK>(p.storage) : pick_leaf<ML_CHUNK_PIPE>(p.storage);
+    else if (p.n2 == 5 && p.storage == FPO_STORAGE_F32 && !p.half_table)
+        kern = p.pipeline ? (const void *)materialise_kernel<5, FPO_STORAGE_F32, MF_QUARTER>
+                          : (const void *)materialise_kernel<5, FPO_STORAGE_F32, MF_WARP2>;
     else
         kern = p.n2 == 5 ? pick_materialise<5>(p.storage)
                          : (p.n2 == 11 ? pick_materialise<11>(p.storage) : pick_materialise<0>(p.storage));
