@@ -1268,7 +1268,7 @@ constexpr int FU_GROUP = 8;    // visits a warp evaluates at a time, 4 lanes eac
 #define FPO_FUSED_LIST 4
 #endif
 #ifndef FPO_FUSED_REFILL
-#define FPO_FUSED_REFILL 12
+#define FPO_FUSED_REFILL 16
 #endif
 #ifndef FPO_FUSED_PREFETCH
 #define FPO_FUSED_PREFETCH 1
@@ -1606,12 +1606,15 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
 
 // Rays per warp and list length.  Few rays: fewer of them per warp, so that
 // every SM gets several warps (a warp's time is that of its longest ray
-// either way, and the shading lanes are all busy for any R).
-static void fused_shape(uint32_t tiles32, int sm_count, int warps_per_sm, int *rays, int *cap)
+// either way, and the shading lanes are all busy for any R).  The same for
+// both directions: now that the adjoint only lists its visits it has the
+// forward's work (a fine-tuning step of 65,536 rays took 1.85 ms with twice
+// the warps in the adjoint and new rays at 12 idle lanes, 1.79 as it is now).
+static void fused_shape(uint32_t tiles32, int sm_count, int *rays, int *cap)
 {
     const uint64_t n = (uint64_t)tiles32 * 32;
     int r = 16;
-    while (r > FPO_FUSED_MIN_RAYS && n < (uint64_t)sm_count * warps_per_sm * r) r >>= 1;
+    while (r > FPO_FUSED_MIN_RAYS && n < (uint64_t)sm_count * FPO_FUSED_WARPS_PER_SM * r) r >>= 1;
     *rays = r;
     *cap = r * FPO_FUSED_LIST < 64 ? 64 : r * FPO_FUSED_LIST;
 }
@@ -1620,7 +1623,7 @@ template <int N1, int N2, bool ADJ, bool DBG, bool BRICK>
 static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
 {
     TraverseParams &p = q.tp;
-    fused_shape(p.n_tiles, sm_count, ADJ ? 2 * FPO_FUSED_WARPS_PER_SM : FPO_FUSED_WARPS_PER_SM, &p.rays_per_warp, &p.list_cap);
+    fused_shape(p.n_tiles, sm_count, &p.rays_per_warp, &p.list_cap);
     const int threads = 32 * FU_WARPS;
     const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, BRICK ? 0 : p.depth + 1, FusedSize<N1, N2>::WROW);
     auto k = fused_kernel<N1, N2, ADJ, DBG, BRICK>;
