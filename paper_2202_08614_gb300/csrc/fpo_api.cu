@@ -162,10 +162,10 @@ struct fpo_ctx {
 
     void free_visit_list()
     {
-        dfree(d_vl_id);
         dfree(d_vl_val);
-        dfree(d_vl_next);
-        dfree(d_vl_w);
+        d_vl_id = nullptr;
+        d_vl_next = nullptr;
+        d_vl_w = nullptr;
         vl_cap = vl_rays = 0;
     }
 
@@ -856,15 +856,16 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
         uint32_t room = 4096;  // rays, in powers of two
         while (room < n) room *= 2;
         const size_t e = (size_t)room * VL_PER_RAY, nw = (size_t)c->cfg.n1 + 9 * (size_t)c->cfg.n2;
-        cudaError_t err = cudaMalloc((void **)&c->d_vl_id, e * sizeof(uint2));
-        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_val, e * sizeof(float4));
-        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_next, e * sizeof(uint32_t));
-        if (err == cudaSuccess) err = cudaMalloc((void **)&c->d_vl_w, (size_t)room * nw * sizeof(float));
-        if (err != cudaSuccess) {
+        // one block (four allocations took 0.2 ms of a context's first adjoint)
+        if (cudaMalloc((void **)&c->d_vl_val, e * (sizeof(float4) + sizeof(uint2) + sizeof(uint32_t)) +
+                                                  (size_t)room * nw * sizeof(float)) != cudaSuccess) {
             cudaGetLastError();
-            c->free_visit_list();
+            c->d_vl_val = nullptr;
             return L;
         }
+        c->d_vl_id = reinterpret_cast<uint2 *>(c->d_vl_val + e);
+        c->d_vl_next = reinterpret_cast<uint32_t *>(c->d_vl_id + e);
+        c->d_vl_w = reinterpret_cast<float *>(c->d_vl_next + e);
         c->vl_cap = (uint32_t)e;
         c->vl_rays = room;
     }
