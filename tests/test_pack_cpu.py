@@ -11,7 +11,7 @@ SRC = os.path.join(ROOT, "paper_2202_08614_gb300", "csrc")
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def pack_check(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("pack") / "pack_check")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", SRC,
@@ -22,7 +22,7 @@ def checker(tmp_path_factory):
 
 # the smallest and the deepest grid of the index, and a tree coarser than its max_depth
 @pytest.mark.parametrize("depth,max_depth", [(4, 4), (5, 5), (6, 12), (8, 9), (11, 11), (11, 12)])
-def test_brick_index_matches_the_octree(checker, depth, max_depth):
+def test_brick_index_matches_the_octree(pack_check, depth, max_depth):
     for seed in range(3):
-        out = subprocess.run([checker, str(depth), str(max_depth), str(seed)], capture_output=True, text=True, check=True)
+        out = subprocess.run([pack_check, str(depth), str(max_depth), str(seed)], capture_output=True, text=True, check=True)
         assert int(out.stdout) == 0
