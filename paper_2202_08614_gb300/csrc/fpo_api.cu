@@ -67,8 +67,8 @@ void dfree(T *&p)
 // soon the next traversal's warps take the places of the last ones: CTAs of
 // two warps, and six tables in flight (BF16 frames 407 -> 381 us, latent
 // 790 -> 766, FP8 views 231 -> 200; 128 threads 384 / 773 / 201, depth 8 the
-// same).  The FP32-table frames, 5.09 ms for eight, gain from neither (5.16
-// with CTAs of 64, 5.08 at depth 6).
+// same).  The FP32-table frames, 4.72 ms for eight, gain from neither (4.87
+// with CTAs of 64, 4.72 at depth 6).
 #ifndef FPO_PIPE_TRAV_THREADS_F16
 #define FPO_PIPE_TRAV_THREADS_F16 64
 #endif

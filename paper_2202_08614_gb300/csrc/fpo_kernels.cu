@@ -1060,8 +1060,8 @@ __device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
 // of its current tile (fetching a new tile when that one is used up), so
 // long rays do not leave most of a warp idle.  The last CTA to finish resets
 // the counter.  Register cap: 64 in the frame pipeline, where the IDFT pass
-// takes a quarter of the register file (eight 1080p FP32 frames: 5.09 ms at
-// 64, 5.12 at 72, 5.52 at 56, 5.54 at 48); alone, the FP32-table walk
+// takes a quarter of the register file (eight 1080p FP32 frames, before the
+// pass's present forms: 5.09 ms at 64, 5.12 at 72, 5.52 at 56, 5.54 at 48); alone, the FP32-table walk
 // gains more from the 72 registers it wants than from a fourth CTA (826 ->
 // 801 us a frame, 38.7 -> 34.6 us a 128x128 frame).
 #ifndef FPO_TRAV_MAXNREG_MAT
@@ -1874,10 +1874,13 @@ static int launch_b64(const BackwardParams &q, int sm_count, cudaStream_t s)
     return (int)cudaGetLastError();
 }
 
-// The gradient rows of the list's visits into dL_dcoeffs: a warp takes 32
-// entries at a time, a row by contiguous 8-byte vector atomics.  Bound by the
-// random read-modify-write of the rows in DRAM (1M rows of a 2.3 GB array:
-// 0.31 ms with any coalesced form of atomic, plain read-add-write included).
+// The gradient rows of the list's visits into dL_dcoeffs: a warp takes up to
+// 32 entries at a time, a row by contiguous 8-byte vector atomics.  Bound by
+// the random read-modify-write of the rows in DRAM (1M rows of a 2.3 GB array:
+// 0.31 ms with any coalesced form of atomic, plain read-add-write included),
+// and for a short list by a warp's chain of entries: it is shared out over all
+// warps, at least 4 entries each (8,192 rays: 43 us with 32 each, 28 now;
+// 4,095: 29 and 11; 2 and 8 at least the same within 2 us).
 template <int N1, int N2>
 __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list, float *grad)
 {
@@ -1895,11 +1898,12 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list,
             wi[2 * r + h] = j < 0 ? k : N1 + j % NZ;
             ci[2 * r + h] = j < 0 ? 0 : 1 + j / NZ;
         }
-    for (uint32_t v0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * 32; v0 < n; v0 += warps * 32) {
+    const uint32_t per = min(32u, max(4u, (n + warps - 1) / warps));
+    for (uint32_t v0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * per; v0 < n; v0 += warps * per) {
         const uint32_t v = v0 + (uint32_t)lane;
-        const uint2 id = v < n ? list.id[v] : make_uint2(0u, 0u);
-        const float4 val = v < n ? list.val[v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        const int m = (int)min(32u, n - v0);
+        const int m = (int)min(per, n - v0);
+        const uint2 id = lane < m ? list.id[v] : make_uint2(0u, 0u);
+        const float4 val = lane < m ? list.val[v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll 2
         for (int i = 0; i < m; ++i) {
             float *row = grad + (size_t)__shfl_sync(0xffffffffu, id.x, i) * NC;

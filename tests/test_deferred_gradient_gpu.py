@@ -62,6 +62,29 @@ def test_list_pass_equals_the_replays_own_adds(n1, n2, deep):
     _close(many, one)
 
 
+@pytest.mark.parametrize("parts", [20000, 40, 7])
+def test_list_pass_at_every_share_of_a_warp(parts):
+    # 20,000 rays' visits give a warp 32 entries at a time; those of 1, 500 or
+    # 2858 rays fewer, down to the least, and leave most warps without any
+    tree = synth.shell_tree(4)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    n = 20000
+    o, d, t, g = _rays(n, 5)
+    rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    whole, cut = (torch.zeros(tree.coeffs.shape, device="cuda") for _ in range(2))
+    r.render_backward(rgb, g, whole, rays_o=o, rays_d=d, t_per_ray=t)
+    step = -(-n // parts)
+    for i in range(0, n, step):
+        k = slice(i, min(i + step, n))
+        r.render_backward(rgb[k].contiguous(), g[k].contiguous(), cut, rays_o=o[k].contiguous(),
+                          rays_d=d[k].contiguous(), t_per_ray=t[k].contiguous())
+    r.status()
+    r.close()
+    assert float(whole.abs().max()) > 0
+    _close(cut, whole)
+
+
 def _step(defer, calls, overflow=False):
     tree = synth.shell_tree(7)
     r = fpo.Renderer(idft_mode="fused")
