@@ -177,7 +177,10 @@ enum {
      * list are added to dL_dcoeffs and their leaves marked as usual (so both
      * arrays are still needed, and FPO_FLAG_MARK_LEAVES with them): pass the
      * same two arrays to fpo_adam_leaves.  A list that fpo_adam_leaves has
-     * not consumed is dropped by fpo_upload_tree and fpo_set_coeffs. */
+     * not consumed is dropped by fpo_upload_tree and fpo_set_coeffs.  A call
+     * under stream capture makes no list (every visit goes to dL_dcoeffs and
+     * the marks), and while a list waits fpo_adam_leaves and fpo_set_coeffs
+     * are refused under capture (INVALID_ARG). */
     FPO_FLAG_DEFER_GRADIENT = 256
 };
 
@@ -275,9 +278,10 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * FPO_FLAG_FP64_GRADCHECK selects the FP64 replay, FPO_FLAG_DEFER_GRADIENT
  * leaves the gradient to the next fpo_adam_leaves (see the flags).
  * Batches of up to 262,144 rays keep their visits in a workspace of the
- * context (grown on the first larger batch outside a stream capture, at most
- * 0.4 GB) and add them to dL_dcoeffs in a second, evenly divided pass; other
- * calls, and visits beyond the workspace, add them from the replay.
+ * context (grown on the first larger batch, at most 0.4 GB) and add them to
+ * dL_dcoeffs in a second, evenly divided pass; other calls, calls under stream
+ * capture (a graph holds nothing of the workspace), and visits beyond it add
+ * them from the replay.
  * Errors: INVALID_ARG, NO_TREE, UNSUPPORTED, CUDA. */
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
                         const float *out_rgb, const float *dL_drgb, float *dL_dcoeffs,

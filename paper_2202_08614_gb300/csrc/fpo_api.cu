@@ -835,23 +835,28 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
 
 namespace {
 
+// Whether work on s goes into a graph (a stream that cannot be asked counts as such).
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // The context's visit list for an adjoint call over n_rays rays.  It stays
 // empty (cap 0: the replay adds its rows itself) for large batches, when the
-// workspace would have to grow during a stream capture or while it holds
-// deferred visits, or when there is no memory for it.
+// workspace would have to grow while it holds deferred visits, when there is
+// no memory for it, and during a stream capture: a graph that held the list
+// would write to freed memory once the list has grown, and its replays would
+// mix their visits with those that wait here.
 VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
 {
     VisitList L{};
-    if (n_rays > VL_MAX_RAYS || (c->vl_used && !defer)) return L;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return L;
-    }
-    const bool may_alloc = cap == cudaStreamCaptureStatusNone;
+    if (n_rays > VL_MAX_RAYS || (c->vl_used && !defer) || capturing(s)) return L;
     const uint32_t n = (uint32_t)n_rays;
     if (c->vl_used + n > c->vl_rays) {
-        if (c->vl_used || !may_alloc) return L;
+        if (c->vl_used) return L;
         c->free_visit_list();
         uint32_t room = 4096;  // rays, in powers of two
         while (room < n) room *= 2;
@@ -870,7 +875,7 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
         c->vl_rays = room;
     }
     if (defer && !c->d_vl_head) {
-        if (!may_alloc || cudaMalloc((void **)&c->d_vl_head, (size_t)c->n_leaves * 4) != cudaSuccess) {
+        if (cudaMalloc((void **)&c->d_vl_head, (size_t)c->n_leaves * 4) != cudaSuccess) {
             cudaGetLastError();
             return L;
         }
@@ -890,6 +895,9 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
     L.ray_base = c->vl_used;
     return L;
 }
+
+// The call that takes or drops deferred visits has to run now, not in a graph.
+constexpr char VISITS_WAIT[] = "deferred visits wait for fpo_adam_leaves: not during a stream capture";
 
 // Deferred visits that no fpo_adam_leaves has taken are forgotten.
 cudaError_t drop_visits(fpo_ctx *c, cudaStream_t s)
@@ -994,9 +1002,10 @@ int fpo_set_coeffs(fpo_ctx *ctx, const float *coeffs, void *cuda_stream)
         return fail(FPO_ERR_UNSUPPORTED, "in-place coefficient updates need FP32 storage");
     if (ctx->n_leaves == 0) return FPO_OK;
     if (!coeffs) return fail(FPO_ERR_INVALID_ARG, "coeffs is NULL");
-    ctx->table_ok = false;  // the coefficients change
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
+    if (ctx->vl_used && capturing((cudaStream_t)cuda_stream)) return fail(FPO_ERR_INVALID_ARG, "%s", VISITS_WAIT);
+    ctx->table_ok = false;  // the coefficients change
     const cudaError_t de = drop_visits(ctx, (cudaStream_t)cuda_stream);
     if (de != cudaSuccess) return cuda_fail(de, "visit list reset");
     const int ce = launch_set_coeffs(coeffs, ctx->d_perm, static_cast<float *>(ctx->d_sig),
@@ -1046,9 +1055,10 @@ int fpo_adam_leaves(fpo_ctx *ctx, float *param, float *grad, float *m, float *v,
     if (step < 1) return fail(FPO_ERR_INVALID_ARG, "step counts from 1");
     if (!(lr >= 0.0f) || !(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) || !(eps > 0.0f))
         return fail(FPO_ERR_INVALID_ARG, "lr >= 0, beta in [0, 1), eps > 0");
-    ctx->table_ok = false;  // the coefficients change
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
+    if (ctx->vl_used && capturing((cudaStream_t)cuda_stream)) return fail(FPO_ERR_INVALID_ARG, "%s", VISITS_WAIT);
+    ctx->table_ok = false;  // the coefficients change
     LeafAdamParams p{};
     p.param = param;
     p.grad = grad;
