@@ -844,6 +844,13 @@ bool capturing(cudaStream_t s)
     return true;
 }
 
+// Lets this thread allocate while some other stream is being captured.
+struct CaptureElsewhere {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CaptureElsewhere() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~CaptureElsewhere() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The context's visit list for an adjoint call over n_rays rays.  It stays
 // empty (cap 0: the replay adds its rows itself) for large batches, when the
 // workspace would have to grow while it holds deferred visits, when there is
@@ -857,6 +864,7 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
     const uint32_t n = (uint32_t)n_rays;
     if (c->vl_used + n > c->vl_rays) {
         if (c->vl_used) return L;
+        const CaptureElsewhere relaxed;
         c->free_visit_list();
         uint32_t room = 4096;  // rays, in powers of two
         while (room < n) room *= 2;
@@ -875,6 +883,7 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
         c->vl_rays = room;
     }
     if (defer && !c->d_vl_head) {
+        const CaptureElsewhere relaxed;
         if (cudaMalloc((void **)&c->d_vl_head, (size_t)c->n_leaves * 4) != cudaSuccess) {
             cudaGetLastError();
             return L;

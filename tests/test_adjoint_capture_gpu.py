@@ -112,3 +112,22 @@ def test_captured_step_replays_and_waiting_visits_are_not_captured():
     r.status()
     r.close()
     assert m.any()
+
+
+def test_first_adjoint_beside_another_streams_capture():
+    # the workspace's allocation does not end a capture under way elsewhere
+    r, p, _ = _setup()
+    a = Batch(r, 300, 5)
+    want, got, x = torch.zeros_like(p), torch.zeros_like(p), torch.zeros(4, device="cuda")
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        x.add_(1.0)
+        a.backward(r, got, stream=side)
+    torch.cuda.synchronize()
+    graph.replay()
+    a.backward(r, want)
+    r.status()
+    r.close()
+    assert float(x[0]) == 1.0
+    _close(got, want)
