@@ -607,7 +607,6 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ uint64_t s_bar, s_never;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail;
     __shared__ double s_loss;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const bool epi = t < TG_EPI;           // (the other warp issues the MMAs)
@@ -648,7 +647,6 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     uint32_t next_ids = 0;
     if (epi) load_rows(blockIdx.x, tile_ids(blockIdx.x));
     if (t == 0) {
-        s_fail = 0;
         s_loss = 0.0;
         ptx::mbar_init(&s_bar, 1);
         ptx::mbar_init(&s_never, 1);
@@ -707,15 +705,19 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     const uint32_t sa = ptx::smem_u32(sm);
     float lsum = 0.0f;
     uint32_t commits = 0;  // MMA warp: rounds issued
+    bool failed = false;   // a wait of this thread's warp ran out
     // End of an epilogue (generic smem writes and TMEM reads before the next
     // MMAs), and the MMA warp's signal to issue them.  False once a wait has
-    // run out anywhere in the CTA: every thread leaves the loop here.
+    // run out anywhere in the CTA: every thread leaves the loop here.  The
+    // barrier itself carries the outcome, the same for every thread; read from
+    // a shared word after it, a slow thread could meet what a fast one's next
+    // wait had left there, and leave alone.
     auto hand_off = [&]() -> bool {
         fence_async_smem();
         fence_before();
-        __syncthreads();
+        const int any = __syncthreads_or(failed);
         fence_after();
-        return s_fail == 0;
+        return any == 0;
     };
     if (epi) {
         uint32_t phase = 0;
@@ -726,7 +728,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
                                  : ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
             ok = __all_sync(0xffffffffu, ok);
             first_wait = false;
-            if (!ok) s_fail = 1;
+            failed |= !ok;
             fence_after();
             phase ^= 1u;
             return ok;
@@ -895,10 +897,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
             acc_w = 1;
         }
     }
-    fence_before();
-    __syncthreads();  // every wait of the last tile is over
-    fence_after();
-    const bool ok = s_fail == 0;
+    const bool ok = hand_off();  // every wait of the last tile is over
     if (ok && epi) {
         // the weight gradients: lane k of G3 / G2 / G1 is input feature k, lane
         // 64 (32 for G1) the bias; column j / o the output feature

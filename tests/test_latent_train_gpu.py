@@ -364,6 +364,29 @@ def test_decoder_grad_tensor_cores_timeout_is_reported():
         assert torch.allclose(m.g[k], ref_g[k], rtol=1e-5, atol=1e-6 * float(ref_g[k].abs().max()))
 
 
+def test_decoder_grad_tensor_cores_timeout_leaves_every_tile():
+    # several tiles a CTA, the first wait of each CTA running out, a hundred
+    # times: all warps leave at the same barrier, and the next call is exact
+    n = b = 152 * 128 * 2 + 77
+    m = LatentModel(n, seed=4, tensor_cores=True)
+    tgt, cw = torch.ones((n, NC), device="cuda"), torch.ones(NC, device="cuda")
+    rows = torch.arange(n, dtype=torch.int32, device="cuda")
+    ref, _ = m.grad(rows, tgt, cw)
+    w, g, dl = m._mlp(m.p), m._mlp(m.g), torch.empty((b, 32), device="cuda")
+    for _ in range(100):
+        fpo.check(fpo.lib().fpo_decoder_grad_tc(
+            C.byref(w), N1, N2, b, C.c_void_p(rows.data_ptr()), C.c_void_p(m.p["lat"].data_ptr()),
+            C.c_void_p(tgt.data_ptr()), C.c_void_p(cw.data_ptr()), None, C.byref(g), C.c_void_p(dl.data_ptr()),
+            None, C.c_void_p(m.status.data_ptr()), fpo.FLAG_TEST_DEVICE_TIMEOUT, None))
+    with pytest.raises(fpo.FPOError) as e:
+        m.check_status()
+    assert e.value.code == -9
+    m.status.zero_()
+    again, _ = m.grad(rows, tgt, cw)
+    m.check_status()
+    assert torch.equal(again, ref)
+
+
 def _f16(a):
     return np.asarray(a, np.float64).astype(np.float16).astype(np.float64)
 
