@@ -175,6 +175,44 @@ struct TraverseParams {
     unsigned long long *stats; // FPO_FLAG_STATS: [steps, leaf visits, rays entering the tree]
 };
 
+// Ray k (0..31) of a tile: a camera pixel of a TILE_W x TILE_H block, or an
+// explicit ray.
+__host__ __device__ __forceinline__ bool tile_ray(const TraverseParams &p, uint32_t tile, uint32_t k, uint32_t &ray,
+                                                  int &px, int &py)
+{
+    if (p.fr.mode == FPO_RAYS_CAMERA) {
+        // row-major tiles: the tiles in flight form one band of rows, whose
+        // table lines stay in L2
+        const uint32_t tx = tile % p.tiles_x, ty = tile / p.tiles_x;
+        px = (int)(tx * TILE_W + k % TILE_W);
+        py = (int)(ty * TILE_H + k / TILE_W);
+        ray = (uint32_t)py * p.fr.width + (uint32_t)px;
+        return px < (int)p.fr.width && py < (int)p.fr.height;
+    }
+    ray = tile * 32 + k;
+    return ray < p.fr.n_rays;
+}
+
+// The queue of the fused mode holds single rays, counted in 32 bits: slot
+// 32 tile + k is ray k of a tile.  Of a camera frame a few pixels wide or high
+// the tiles are mostly empty slots, up to 32 a pixel; when they would pass
+// 2^31 the frame is taken pixel by pixel instead (tiles_x = 0), so that the
+// slots, and what the warps count past them, always fit.
+inline void fused_queue(TraverseParams &p)
+{
+    if (p.fr.mode != FPO_RAYS_CAMERA || p.n_tiles < (1u << 26)) return;
+    p.tiles_x = 0;
+    p.n_tiles = (p.fr.n_rays + 31) / 32;
+}
+__host__ __device__ __forceinline__ bool slot_ray(const TraverseParams &p, uint32_t slot, uint32_t &ray, int &px, int &py)
+{
+    if (p.fr.mode != FPO_RAYS_CAMERA || p.tiles_x) return tile_ray(p, slot >> 5, slot & 31u, ray, px, py);
+    ray = slot;
+    px = (int)(slot % p.fr.width);
+    py = (int)(slot / p.fr.width);
+    return slot < p.fr.n_rays;
+}
+
 struct MaterialiseParams {
     const void *sig;          // [n_leaves] records of sig_stride elements
     const void *zc;           // [n_leaves] records of z_stride elements

@@ -1019,24 +1019,6 @@ __device__ void trace_ray(const TraverseParams &p, uint32_t *s_stack, int stride
 
 namespace {
 
-// Ray k (0..31) of a tile: a camera pixel of a TILE_W x TILE_H block, or an
-// explicit ray.
-__device__ __forceinline__ bool tile_ray(const TraverseParams &p, uint32_t tile, uint32_t k, uint32_t &ray,
-                                         int &px, int &py)
-{
-    if (p.fr.mode == FPO_RAYS_CAMERA) {
-        // row-major tiles: the tiles in flight form one band of rows, whose
-        // table lines stay in L2
-        const uint32_t tx = tile % p.tiles_x, ty = tile / p.tiles_x;
-        px = (int)(tx * TILE_W + k % TILE_W);
-        py = (int)(ty * TILE_H + k / TILE_W);
-        ray = (uint32_t)py * p.fr.width + (uint32_t)px;
-        return px < (int)p.fr.width && py < (int)p.fr.height;
-    }
-    ray = tile * 32 + k;
-    return ray < p.fr.n_rays;
-}
-
 // The last warp of the grid to finish resets the tile counter for the next
 // launch (every warp has made its final grab before counting itself).
 __device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
@@ -1340,7 +1322,7 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
             bool ok = false;
             if (((idle >> lane) & 1u) && slot < n_slots) {
                 int px = 0, py = 0;
-                if (tile_ray(p, slot >> 5, slot & 31u, ray, px, py)) {
+                if (slot_ray(p, slot, ray, px, py)) {
                     ok = init_ray_geom(p, stack, W, ray, px, py);
                     if (!ok && !ADJ) write_result(p, W, DBG);  // misses the tree: background
                 }
@@ -1623,6 +1605,7 @@ template <int N1, int N2, bool ADJ, bool DBG, bool BRICK>
 static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
 {
     TraverseParams &p = q.tp;
+    fused_queue(p);
     fused_shape(p.n_tiles, sm_count, &p.rays_per_warp, &p.list_cap);
     const int threads = 32 * FU_WARPS;
     const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, BRICK ? 0 : p.depth + 1, FusedSize<N1, N2>::WROW);
