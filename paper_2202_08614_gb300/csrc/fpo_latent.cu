@@ -607,6 +607,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ uint64_t s_bar, s_never;
     __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_fail[2];
     __shared__ double s_loss;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const bool epi = t < TG_EPI;           // (the other warp issues the MMAs)
@@ -647,6 +648,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     uint32_t next_ids = 0;
     if (epi) load_rows(blockIdx.x, tile_ids(blockIdx.x));
     if (t == 0) {
+        s_fail[0] = s_fail[1] = 0;
         s_loss = 0.0;
         ptx::mbar_init(&s_bar, 1);
         ptx::mbar_init(&s_never, 1);
@@ -705,33 +707,32 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
     const uint32_t sa = ptx::smem_u32(sm);
     float lsum = 0.0f;
     uint32_t commits = 0;  // MMA warp: rounds issued
-    bool failed = false;   // a wait of this thread's warp ran out
     // End of an epilogue (generic smem writes and TMEM reads before the next
     // MMAs), and the MMA warp's signal to issue them.  False once a wait has
-    // run out anywhere in the CTA: every thread leaves the loop here.  The
-    // barrier itself carries the outcome, the same for every thread; read from
-    // a shared word after it, a slow thread could meet what a fast one's next
-    // wait had left there, and leave alone.
-    auto hand_off = [&]() -> bool {
+    // run out anywhere in the CTA: every thread leaves the loop here.  Hand-offs
+    // take the two words of s_fail by turns (six a tile, so each has its own):
+    // the waits before this one report in s_fail[turn], those after it in the
+    // other, and a slow thread still reads here what the fast ones read.
+    auto hand_off = [&](const int turn) -> bool {
         fence_async_smem();
         fence_before();
-        const int any = __syncthreads_or(failed);
+        __syncthreads();
         fence_after();
-        return any == 0;
+        return s_fail[turn] == 0;
     };
     if (epi) {
         uint32_t phase = 0;
         bool first_wait = p.test_timeout != 0;
         // (bounded; a warp whose wait runs out goes on to the next hand_off)
-        auto wait_mmas = [&]() -> bool {
-            bool ok = first_wait ? ptx::mbar_wait_bounded(&s_never, 0, TEST_WAIT_LIMIT_NS)
-                                 : ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
-            ok = __all_sync(0xffffffffu, ok);
+        auto wait_mmas = [&](const int turn) -> bool {  // turn: of the hand-off after it
+            bool done = first_wait ? ptx::mbar_wait_bounded(&s_never, 0, TEST_WAIT_LIMIT_NS)
+                                   : ptx::mbar_wait_bounded(&s_bar, phase, LT_WAIT_NS);
+            done = __all_sync(0xffffffffu, done);
             first_wait = false;
-            failed |= !ok;
+            if (!done) s_fail[turn] = 1;
             fence_after();
             phase ^= 1u;
-            return ok;
+            return done;
         };
         // H = relu(Z + b) of this thread's 16 columns into `dst`; returns the mask of Z + b > 0
         auto relu_part = [&](unsigned char *dst, const float *b) -> uint32_t {
@@ -774,15 +775,15 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
             if (part == 0) put_one_bf(sm + TGO_X, m, 4, TG_KX, one);
             else if (part == 1) put_one_bf(sm + TGO_H1, m, 8, TG_KH, one);
             else if (part == 2) put_one_bf(sm + TGO_H2, m, 8, TG_KH, one);
-            if (!hand_off()) break;
-            wait_mmas();
+            if (!hand_off(0)) break;
+            wait_mmas(1);
             const uint32_t m1 = relu_part(sm + TGO_H1, s_b1);
-            if (!hand_off()) break;
-            wait_mmas();
+            if (!hand_off(1)) break;
+            wait_mmas(0);
             const uint32_t m2 = relu_part(sm + TGO_H2, s_b2);
             cp_async_wait();  // this thread's copies of the tile's targets (all threads': the barrier)
-            if (!hand_off()) break;
-            wait_mmas();
+            if (!hand_off(0)) break;
+            wait_mmas(1);
             // dY = 2 cw (Y + b3 - target) + extra of this thread's 48 (the last quarter's 32) columns
             const float *trow = s_t + m * ts;
             const float *xrow = p.extra_dy && valid ? p.extra_dy + (size_t)p.rows[r0 + m] * nc : nullptr;
@@ -824,16 +825,16 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
                 put8_bf(sm + TGO_DY, m, 2 * c, TG_NC, v);
                 put8_bf(sm + TGO_DY, m, 2 * c + 1, TG_NC, v + 8);
             }
-            if (!hand_off()) break;
+            if (!hand_off(1)) break;
             load_rows(tile + gridDim.x, next_ids);  // the target tile is free: in flight from here on
-            wait_mmas();
+            wait_mmas(0);
             masked_part(m2);
-            if (!hand_off()) break;
-            wait_mmas();
+            if (!hand_off(0)) break;
+            wait_mmas(1);
             masked_part(m1);
-            if (!hand_off()) break;
+            if (!hand_off(1)) break;
             // dL/d(latent) of the tile's rows
-            if (wait_mmas() && part < 2) {
+            if (wait_mmas(0) && part < 2) {
                 float v[16];
                 tmem_ld16(tm + lane_off + TC_SCR + 16 * part, v);
                 if (valid) {
@@ -861,34 +862,34 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
                       dyf = over_cols(sa + TGO_DY, TG_NC), dyg = over_rows(sa + TGO_DY, TG_NC), df = over_cols(sa + TGO_DY, 64),
                       dg = over_rows(sa + TGO_DY, 64);
         for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            if (!hand_off()) break;
+            if (!hand_off(0)) break;
             if (lane == 0) {
                 gemm_bf16<32, 64>(tm + TC_SCR, xf, over_cols(sa + TGO_W1, 32), 0);
                 commit();
             }
-            if (!hand_off()) break;
+            if (!hand_off(1)) break;
             if (lane == 0) {
                 gemm_bf16<64, 64>(tm + TC_SCR, h1f, over_cols(sa + TGO_W2, 64), 0);
                 commit();
             }
-            if (!hand_off()) break;
+            if (!hand_off(0)) break;
             if (lane == 0) {
                 gemm_bf16<64, TG_NC>(tm + TC_SCR, h2f, over_cols(sa + TGO_W3, 64), 0);
                 commit();
             }
-            if (!hand_off()) break;
+            if (!hand_off(1)) break;
             if (lane == 0) {
                 gemm_bf16<TG_NC, 64>(tm + TC_SCR, dyf, over_rows(sa + TGO_W3, 64), 0);
                 gemm_bf16<128, TG_NC>(tm + TC_G3, h2g, dyg, acc_w);
                 commit();
             }
-            if (!hand_off()) break;
+            if (!hand_off(0)) break;
             if (lane == 0) {
                 gemm_bf16<64, 64>(tm + TC_SCR, df, over_rows(sa + TGO_W2, 64), 0);
                 gemm_bf16<128, 64>(tm + TC_G2, h1g, dg, acc_w);
                 commit();
             }
-            if (!hand_off()) break;
+            if (!hand_off(1)) break;
             if (lane == 0) {
                 gemm_bf16<64, 32>(tm + TC_SCR, df, over_rows(sa + TGO_W1, 32), 0);
                 gemm_bf16<128, 64>(tm + TC_G1, xg, dg, acc_w);
@@ -897,7 +898,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) decoder_grad_tc_kernel(const __
             acc_w = 1;
         }
     }
-    const bool ok = hand_off();  // every wait of the last tile is over
+    hand_off(0);  // every wait of the last tile is over
+    const bool ok = (s_fail[0] | s_fail[1]) == 0;
     if (ok && epi) {
         // the weight gradients: lane k of G3 / G2 / G1 is input feature k, lane
         // 64 (32 for G1) the bias; column j / o the output feature
