@@ -924,7 +924,6 @@ extern "C" int fpo_camera_ray_batch(const float *basis, const int64_t *cam, cons
     if (n == 0) return FPO_OK;
     if (!basis || !cam || !pixel || !frame || !o || !d || !t) return set_last_error(FPO_ERR_INVALID_ARG, "NULL array");
     if (width == 0 || height == 0) return set_last_error(FPO_ERR_INVALID_ARG, "width and height must be > 0");
-    if (!(fov_y_deg > 0.0 && fov_y_deg < 180.0)) return set_last_error(FPO_ERR_INVALID_ARG, "fov_y_deg must be in (0, 180)");
     const float th = (float)tan(fov_y_deg * (3.14159265358979323846 / 180.0) / 2.0);
     ray_batch_kernel<<<(n + 255) / 256, 256, 0, (cudaStream_t)cuda_stream>>>(basis, cam, pixel, frame, n, (int64_t)width,
                                                                               (float)width, 1.0f / (float)width,

@@ -41,20 +41,35 @@ def camera_ray_batch(cams, n, gen, n_frames=60, basis=None):
     """n training rays drawn uniformly over (camera, integer frame, pixel):
     origins, unit directions (pixel centres of the pinhole model documented
     in fpo.h) and frame times, as CUDA tensors.  `gen`: a CUDA torch.Generator;
-    `basis`: camera_basis(cams), if already at hand."""
+    `basis`: camera_basis(cams), if already at hand (a CUDA tensor; rows and
+    columns past those are not read).  A float32 basis takes one kernel; one of
+    another type, or one that gradients are wanted for, torch's own operations."""
     import torch
 
     B = camera_basis(cams) if basis is None else basis
-    W, H = cams[0].width, cams[0].height
+    if not B.is_cuda or B.dim() != 2 or B.shape[0] < len(cams) or B.shape[1] < 12:
+        raise ValueError(f"basis must be a CUDA tensor of [{len(cams)}, 12], not {B.dtype} {tuple(B.shape)} on {B.device}")
+    cam = cams[0]
+    W, H = int(cam.width), int(cam.height)
     v = torch.randint(0, len(cams), (n,), device="cuda", generator=gen)
     p = torch.randint(0, W * H, (n,), device="cuda", generator=gen)
     f = torch.randint(0, n_frames, (n,), device="cuda", generator=gen)
-    B = B.contiguous()
-    o, d, t = (torch.empty(s, device="cuda") for s in ((n, 3), (n, 3), (n,)))
+    if B.dtype != torch.float32 or (B.requires_grad and torch.is_grad_enabled()):
+        return _rays_elementwise(B[v], p, f, W, H, np.tan(np.radians(cam.fov_y_deg) / 2))
+    B = B[:, :12].contiguous()
+    o, d, t = (torch.empty(s, dtype=torch.float32, device="cuda") for s in ((n, 3), (n, 3), (n,)))
     ptr = lambda x: x.data_ptr() if n else None
-    fpo.check(fpo.lib().fpo_camera_ray_batch(B.data_ptr(), ptr(v), ptr(p), ptr(f), n, W, H, float(cams[0].fov_y_deg),
+    fpo.check(fpo.lib().fpo_camera_ray_batch(B.data_ptr(), ptr(v), ptr(p), ptr(f), n, W, H, float(cam.fov_y_deg),
                                              ptr(o), ptr(d), ptr(t), fpo._stream_handle(None)))
     return o, d, t
+
+
+def _rays_elementwise(b, p, f, W, H, th):
+    """The rays of the pixels p and frames f from their cameras' basis rows b."""
+    sx = ((2 * ((p % W).float() + 0.5) / W - 1) * th * W / H)[:, None]
+    sy = ((1 - 2 * ((p // W).float() + 0.5) / H) * th)[:, None]
+    d = b[:, 3:6] + sx * b[:, 6:9] + sy * b[:, 9:12]
+    return b[:, 0:3].contiguous(), (d / d.norm(dim=1, keepdim=True)).contiguous(), f.float()
 
 
 class FineTuner:
