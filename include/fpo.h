@@ -177,9 +177,10 @@ enum {
      * list are added to dL_dcoeffs and their leaves marked as usual (so both
      * arrays are still needed, and FPO_FLAG_MARK_LEAVES with them): pass the
      * same two arrays to fpo_adam_leaves.  A list that fpo_adam_leaves has
-     * not consumed is dropped by fpo_upload_tree and fpo_set_coeffs.  A call
+     * not consumed is dropped by what replaces the coefficients
+     * (fpo_upload_tree, fpo_set_coeffs, fpo_set_coeffs_from_decoder).  A call
      * under stream capture makes no list (every visit goes to dL_dcoeffs and
-     * the marks), and while a list waits fpo_adam_leaves and fpo_set_coeffs
+     * the marks), and while a list waits fpo_adam_leaves and the two setters
      * are refused under capture (INVALID_ARG). */
     FPO_FLAG_DEFER_GRADIENT = 256
 };

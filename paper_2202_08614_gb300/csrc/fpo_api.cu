@@ -1037,9 +1037,12 @@ int fpo_set_coeffs_from_decoder(fpo_ctx *ctx, const fpo_mlp *w, const float *lat
     if (!latents) return fail(FPO_ERR_INVALID_ARG, "latents is NULL");
     if (flags & ~(uint32_t)(FPO_FLAG_TENSOR_CORES | FPO_FLAG_TEST_DEVICE_TIMEOUT))
         return fail(FPO_ERR_INVALID_ARG, "unknown flags");
-    ctx->table_ok = false;  // the coefficients change
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");
+    if (ctx->vl_used && capturing((cudaStream_t)cuda_stream)) return fail(FPO_ERR_INVALID_ARG, "%s", VISITS_WAIT);
+    ctx->table_ok = false;  // the coefficients change
+    const cudaError_t de = drop_visits(ctx, (cudaStream_t)cuda_stream);
+    if (de != cudaSuccess) return cuda_fail(de, "visit list reset");
     const int ce = (flags & FPO_FLAG_TENSOR_CORES)
                        ? launch_decode_records_tc(*w, ctx->cfg.n1, ctx->cfg.n2, ctx->n_leaves, latents, ctx->d_perm,
                                                   static_cast<float *>(ctx->d_sig), static_cast<float *>(ctx->d_z),

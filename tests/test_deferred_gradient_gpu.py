@@ -137,3 +137,24 @@ def test_set_coeffs_drops_a_pending_list():
     with pytest.raises(fpo.FPOError):  # needs the marks
         r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t, defer=True)
     r.close()
+
+
+@pytest.mark.parametrize("tensor_cores", [False, True])
+def test_a_decoder_drops_a_pending_list(tensor_cores):
+    from paper_2202_08614_gb300.latent import LatentModel
+
+    tree = synth.shell_tree(7)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    p = torch.as_tensor(tree.coeffs, device="cuda").clone()
+    m, v, grad = torch.zeros_like(p), torch.zeros_like(p), torch.zeros_like(p)
+    mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+    o, d, t, g = _rays(500, 3)
+    rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=True)
+    model = LatentModel(tree.n_leaves)
+    r.set_coeffs_from_decoder(model._mlp(model.p), model.p["lat"], tensor_cores=tensor_cores)
+    r.adam_leaves(p, grad, m, v, mark, 1)
+    r.status()
+    r.close()
+    assert not m.any() and torch.equal(p, torch.as_tensor(tree.coeffs, device="cuda"))
