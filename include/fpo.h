@@ -174,9 +174,10 @@ enum {
     /* fpo_render_backward (FP32): keep the gradient in the context, as a list
      * of leaf visits, for the next fpo_adam_leaves, instead of adding every
      * visit's n1 + 27 n2 values to dL_dcoeffs.  Visits that do not fit the
-     * list are added to dL_dcoeffs and their leaves marked as usual (so both
-     * arrays are still needed, and FPO_FLAG_MARK_LEAVES with them): pass the
-     * same two arrays to fpo_adam_leaves.  A list that fpo_adam_leaves has
+     * list, and those of a batch of more rays than the tree has leaves, are
+     * added to dL_dcoeffs and their leaves marked as usual (so both arrays are
+     * still needed, and FPO_FLAG_MARK_LEAVES with them): pass the same two
+     * arrays to fpo_adam_leaves.  A list that fpo_adam_leaves has
      * not consumed is dropped by what replaces the coefficients
      * (fpo_upload_tree, fpo_set_coeffs, fpo_set_coeffs_from_decoder).  A call
      * under stream capture makes no list (every visit goes to dL_dcoeffs and

@@ -113,7 +113,7 @@ constexpr uint32_t DEFAULT_INNER_STEPS = 0xffffffffu;  // a lane runs its ray to
 // Visit list of an adjoint call: batches of up to VL_MAX_RAYS rays, room for
 // VL_PER_RAY visits a ray (the 3.5M-leaf body: 15 on average), counter words.
 constexpr uint32_t VL_MAX_RAYS = 1u << 18, VL_PER_RAY = 32;
-constexpr int VL_COUNT = 24;
+constexpr int VL_COUNT = 24, VL_COUNTS = 3;
 
 }  // namespace
 
@@ -151,10 +151,12 @@ struct fpo_ctx {
     size_t ptable_leaves[PIPE_MAX] = {};
     cudaStream_t aux = nullptr;           // IDFT passes / decodes
     cudaStream_t trav[PIPE_MAX] = {};     // slots 1.. : their traversal streams
-    // visits of an adjoint call (VisitList), grown by ensure_visit_list
+    // visits of an adjoint call (VisitList), grown by visit_list
     uint2 *d_vl_id = nullptr;
     float4 *d_vl_val = nullptr;
-    uint32_t *d_vl_next = nullptr, *d_vl_head = nullptr;
+    uint32_t *d_vl_over = nullptr;
+    uint4 *d_vl_slot = nullptr;         // per leaf: its deferred visits' entries, then in the same allocation
+    uint32_t *d_vl_visits = nullptr;    // their number
     float *d_vl_w = nullptr;
     uint32_t vl_cap = 0, vl_rays = 0;   // entries; rays with room for weights
     uint32_t vl_used = 0;               // rays whose visits await fpo_adam_leaves
@@ -164,7 +166,7 @@ struct fpo_ctx {
     {
         dfree(d_vl_val);
         d_vl_id = nullptr;
-        d_vl_next = nullptr;
+        d_vl_over = nullptr;
         d_vl_w = nullptr;
         vl_cap = vl_rays = 0;
     }
@@ -172,9 +174,10 @@ struct fpo_ctx {
     void free_tree()
     {
         free_visit_list();
-        dfree(d_vl_head);
+        dfree(d_vl_slot);
+        d_vl_visits = nullptr;
         vl_used = 0;
-        if (d_status) cudaMemset(d_status + VL_COUNT, 0, 2 * sizeof(uint32_t));
+        if (d_status) cudaMemset(d_status + VL_COUNT, 0, VL_COUNTS * sizeof(uint32_t));
         dfree(d_nodes);
         dfree(d_top);
         dfree(d_bricks);
@@ -851,7 +854,13 @@ struct CaptureElsewhere {
     ~CaptureElsewhere() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-// The context's visit list for an adjoint call over n_rays rays.  It stays
+// The context's visit list for an adjoint call over n_rays rays.  `defer` holds
+// for batches of up to n_leaves rays: with more, a leaf has so many visits that
+// adding them all to the gradient rows now, evenly divided, is the faster way
+// (fine-tuning step, deferred against added now, us: 43,575 leaves, 4,096 rays
+// 206 and 208, 16,384 280 and 284, 65,536 471 and 400; 5,430 leaves, 4,096 rays
+// 190 and 200, 16,384 262 and 210, 65,536 347 and 277; 348,592 leaves, 65,536
+// rays 763 and 849).  The list stays
 // empty (cap 0: the replay adds its rows itself) for large batches, when the
 // workspace would have to grow while it holds deferred visits, when there is
 // no memory for it, and during a stream capture: a graph that held the list
@@ -860,6 +869,7 @@ struct CaptureElsewhere {
 VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
 {
     VisitList L{};
+    defer = defer && n_rays <= c->n_leaves;
     if (n_rays > VL_MAX_RAYS || (c->vl_used && !defer) || capturing(s)) return L;
     const uint32_t n = (uint32_t)n_rays;
     if (c->vl_used + n > c->vl_rays) {
@@ -877,20 +887,23 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
             return L;
         }
         c->d_vl_id = reinterpret_cast<uint2 *>(c->d_vl_val + e);
-        c->d_vl_next = reinterpret_cast<uint32_t *>(c->d_vl_id + e);
-        c->d_vl_w = reinterpret_cast<float *>(c->d_vl_next + e);
+        c->d_vl_over = reinterpret_cast<uint32_t *>(c->d_vl_id + e);
+        c->d_vl_w = reinterpret_cast<float *>(c->d_vl_over + e);
         c->vl_cap = (uint32_t)e;
         c->vl_rays = room;
     }
-    if (defer && !c->d_vl_head) {
+    if (defer && !c->d_vl_slot) {
         const CaptureElsewhere relaxed;
-        if (cudaMalloc((void **)&c->d_vl_head, (size_t)c->n_leaves * 4) != cudaSuccess) {
+        const size_t nl = c->n_leaves;
+        if (cudaMalloc((void **)&c->d_vl_slot, nl * (sizeof(uint4) + sizeof(uint32_t))) != cudaSuccess) {
             cudaGetLastError();
+            c->d_vl_slot = nullptr;
             return L;
         }
-        if (cudaMemsetAsync(c->d_vl_head, 0xff, (size_t)c->n_leaves * 4, s) != cudaSuccess) {
+        c->d_vl_visits = reinterpret_cast<uint32_t *>(c->d_vl_slot + nl);
+        if (cudaMemsetAsync(c->d_vl_visits, 0, nl * sizeof(uint32_t), s) != cudaSuccess) {
             cudaGetLastError();
-            dfree(c->d_vl_head);
+            dfree(c->d_vl_slot);
             return L;
         }
     }
@@ -898,8 +911,9 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
     L.count = c->d_status + VL_COUNT;
     L.id = c->d_vl_id;
     L.val = c->d_vl_val;
-    L.head = defer ? c->d_vl_head : nullptr;
-    L.next = c->d_vl_next;
+    L.over = c->d_vl_over;
+    L.visits = c->d_vl_visits;
+    L.slot = defer ? c->d_vl_slot : nullptr;
     L.w = c->d_vl_w;
     L.ray_base = c->vl_used;
     return L;
@@ -913,8 +927,8 @@ cudaError_t drop_visits(fpo_ctx *c, cudaStream_t s)
 {
     if (!c->vl_used) return cudaSuccess;
     c->vl_used = 0;
-    cudaError_t e = cudaMemsetAsync(c->d_vl_head, 0xff, (size_t)c->n_leaves * 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status + VL_COUNT, 0, 2 * sizeof(uint32_t), s);
+    cudaError_t e = cudaMemsetAsync(c->d_vl_visits, 0, (size_t)c->n_leaves * sizeof(uint32_t), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status + VL_COUNT, 0, VL_COUNTS * sizeof(uint32_t), s);
     return e;
 }
 
@@ -961,7 +975,7 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     if (!fp64) q.list = visit_list(ctx, n_rays, defer, (cudaStream_t)cuda_stream);
     int ce = launch_backward(q, ctx->sm_count, cuda_stream);
     if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
-    if (q.list.cap && defer) {
+    if (q.list.slot) {
         ctx->vl_used += (uint32_t)n_rays;
     } else if (q.list.cap) {
         ce = launch_grad_scatter(q, ctx->sm_count, cuda_stream);
@@ -1096,8 +1110,9 @@ int fpo_adam_leaves(fpo_ctx *ctx, float *param, float *grad, float *m, float *v,
         p.list.count = ctx->d_status + VL_COUNT;
         p.list.id = ctx->d_vl_id;
         p.list.val = ctx->d_vl_val;
-        p.list.head = ctx->d_vl_head;
-        p.list.next = ctx->d_vl_next;
+        p.list.over = ctx->d_vl_over;
+        p.list.visits = ctx->d_vl_visits;
+        p.list.slot = ctx->d_vl_slot;
         p.list.w = ctx->d_vl_w;
     }
     const int ce = launch_leaf_adam(p, ctx->sm_count, cuda_stream);

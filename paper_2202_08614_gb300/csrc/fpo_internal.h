@@ -322,15 +322,26 @@ int launch_decode_records_tc(const fpo_mlp &w, int n1, int n2, uint32_t n, const
 int launch_adam(const fpo_adam_part *parts, uint32_t n_parts, float b1, float b2, float eps, uint32_t step, int sm_count,
                 void *stream);
 
+// Deferred visits that a leaf Adam step sums for one leaf, one after another.
+// A leaf's later ones are added to its gradient row first, evenly divided: a
+// coarse leaf in front of the cameras can have thousands (65,536 rays on 0.3M
+// leaves, one of them 64 cells wide: 6.0 ms a step with the visits of every
+// leaf in one chain, 0.88 now).  Three slots beside the count in one 16-byte
+// word send so many more visits of the 3.5M-leaf body the other way that its
+// step takes 1.93 instead of 1.81 ms.
+constexpr uint32_t VL_SLOTS = 4;
+
 // Visits of an adjoint call, kept for a second pass (a workspace of the
 // context): what a visit adds to the gradient row of its leaf is the outer
 // product of 4 numbers (dL/dsigma_raw and dL/du_c) and its ray's weights.
 struct VisitList {
     uint32_t cap;             // entries; 0: no list
-    uint32_t *count;          // [0] entries appended (may exceed cap), [1] finished warps of the pass over them
+    uint32_t *count;          // [0] entries appended (may exceed cap), [1] finished warps of the pass over them, [2] in `over`
     uint2 *id;                // upload leaf id, ray (ray_base + index in the call)
     float4 *val;
-    uint32_t *head, *next;    // deferred gradients: per leaf, its last entry and the one before each; else nullptr
+    uint32_t *visits;         // deferred gradients: per leaf, its visits so far
+    uint4 *slot;              // ... the entries of the first VL_SLOTS of them (~0: not in the list); else nullptr
+    uint32_t *over;           // ... and the entries of all later ones, any leaf's
     float *w;                 // [rays][n1 + 9 n2]: IDFT_i(t), then Y_k(d) IDFT_i(t)
     uint32_t ray_base;
 };
@@ -373,6 +384,8 @@ int materialise_smem_bytes(const MaterialiseParams &p);  // dynamic shared memor
 int launch_backward(const BackwardParams &q, int sm_count, void *stream);
 // Adds the list's visits to q.dL_dcoeffs and empties it.
 int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream);
+// Adds the visits in list.over to grad and sets their leaves' marks.
+int launch_grad_scatter_over(const VisitList &list, int n1, int n2, float *grad, uint8_t *leaf_mark, int sm_count, void *stream);
 int launch_dft(const float *values, float *coeffs, uint32_t n_leaves, int n1, int n2, int T, uint32_t *status,
                bool test_timeout, int sm_count, void *stream);
 int launch_set_coeffs(const float *src, const uint32_t *perm, float *sig, float *zc, uint32_t n_leaves,

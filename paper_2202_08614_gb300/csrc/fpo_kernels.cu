@@ -1544,10 +1544,21 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
                     if (listed) {
                         q.list.id[at] = make_uint2(id, q.list.ray_base + rr);
                         q.list.val[at] = reinterpret_cast<const float4 *>(res)[v];
-                        if (q.list.head) q.list.next[at] = atomicExch(q.list.head + id, at);
+                    }
+                    if (q.list.slot) {
+                        const uint32_t nth = ok ? atomicAdd(q.list.visits + id, 1u) : 0u;
+                        if (ok && nth < VL_SLOTS) reinterpret_cast<uint32_t *>(q.list.slot + id)[nth] = listed ? at : 0xffffffffu;
+                        const bool over = listed && nth >= VL_SLOTS;
+                        const uint32_t om = __ballot_sync(0xffffffffu, over);
+                        if (om) {  // (entries of the list, so there is room for all)
+                            uint32_t to = 0;
+                            if (lane == 0) to = atomicAdd(q.list.count + 2, (uint32_t)__popc(om));
+                            to = __shfl_sync(0xffffffffu, to, 0) + __popc(om & lt_mask);
+                            if (over) q.list.over[to] = at;
+                        }
                     }
                     if (v < n) ent[v].x = listed ? 0xffffffffu : id;
-                    if (ok && q.leaf_mark && !(listed && q.list.head)) q.leaf_mark[id] = 1;
+                    if (ok && q.leaf_mark && !(listed && q.list.slot)) q.leaf_mark[id] = 1;
                     here |= __any_sync(0xffffffffu, ok && !listed);
                 }
                 __syncwarp();
@@ -1864,12 +1875,14 @@ static int launch_b64(const BackwardParams &q, int sm_count, cudaStream_t s)
 // and for a short list by a warp's chain of entries: it is shared out over all
 // warps, at least 4 entries each (8,192 rays: 43 us with 32 each, 28 now;
 // 4,095: 29 and 11; 2 and 8 at least the same within 2 us).
-template <int N1, int N2>
-__global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list, float *grad)
+// OVER: the entries that list.over names instead, whose leaves get their marks;
+// the leaf Adam step that follows empties the list.
+template <int N1, int N2, bool OVER>
+__global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list, float *grad, uint8_t *leaf_mark)
 {
     constexpr int NZ = 9 * N2, NC = N1 + 27 * N2, RN = (NC + 63) / 64;
     const int lane = threadIdx.x & 31;
-    const uint32_t n = min(*list.count, list.cap);
+    const uint32_t n = min(list.count[OVER ? 2 : 0], list.cap);
     const uint32_t warps = gridDim.x * blockDim.x / 32;
     // the weight and value index of this lane's elements
     int wi[2 * RN], ci[2 * RN];
@@ -1883,10 +1896,11 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list,
         }
     const uint32_t per = min(32u, max(4u, (n + warps - 1) / warps));
     for (uint32_t v0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * per; v0 < n; v0 += warps * per) {
-        const uint32_t v = v0 + (uint32_t)lane;
         const int m = (int)min(per, n - v0);
+        const uint32_t v = OVER ? (lane < m ? list.over[v0 + (uint32_t)lane] : 0u) : v0 + (uint32_t)lane;
         const uint2 id = lane < m ? list.id[v] : make_uint2(0u, 0u);
         const float4 val = lane < m ? list.val[v] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (OVER && lane < m) leaf_mark[id.x] = 1;
 #pragma unroll 2
         for (int i = 0; i < m; ++i) {
             float *row = grad + (size_t)__shfl_sync(0xffffffffu, id.x, i) * NC;
@@ -1904,7 +1918,7 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list,
         }
     }
     // the last warp empties the list
-    if (lane == 0) {
+    if (!OVER && lane == 0) {
         __threadfence();
         if (atomicAdd(list.count + 1, 1u) == warps - 1) {
             atomicExch(list.count, 0u);
@@ -1913,18 +1927,28 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list,
     }
 }
 
-int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream)
+template <bool OVER>
+static int launch_scatter_t(const VisitList &list, int n1, int n2, float *grad, uint8_t *mark, int sm_count, void *stream)
 {
-    const int n1 = q.tp.n1, n2 = q.tp.n2;
     auto go = [&](auto kern) {
-        kern<<<(unsigned)sm_count * 4u, 256, 0, (cudaStream_t)stream>>>(q.list, q.dL_dcoeffs);
+        kern<<<(unsigned)sm_count * 4u, 256, 0, (cudaStream_t)stream>>>(list, grad, mark);
         return (int)cudaGetLastError();
     };
-    if (n1 == 31 && n2 == 5) return go(grad_scatter_kernel<31, 5>);
-    if (n1 == 11 && n2 == 5) return go(grad_scatter_kernel<11, 5>);
-    if (n1 == 21 && n2 == 5) return go(grad_scatter_kernel<21, 5>);
-    if (n1 == 31 && n2 == 11) return go(grad_scatter_kernel<31, 11>);
-    return -1;
+    if (n1 == 31 && n2 == 5) return go(grad_scatter_kernel<31, 5, OVER>);
+    if (n1 == 11 && n2 == 5) return go(grad_scatter_kernel<11, 5, OVER>);
+    if (n1 == 21 && n2 == 5) return go(grad_scatter_kernel<21, 5, OVER>);
+    if (n1 == 31 && n2 == 11) return go(grad_scatter_kernel<31, 11, OVER>);
+    return (int)cudaErrorInvalidValue;  // (the adjoint makes no list for other sizes)
+}
+
+int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream)
+{
+    return launch_scatter_t<false>(q.list, q.tp.n1, q.tp.n2, q.dL_dcoeffs, nullptr, sm_count, stream);
+}
+
+int launch_grad_scatter_over(const VisitList &list, int n1, int n2, float *grad, uint8_t *leaf_mark, int sm_count, void *stream)
+{
+    return launch_scatter_t<true>(list, n1, n2, grad, leaf_mark, sm_count, stream);
 }
 
 int launch_backward(const BackwardParams &q, int sm_count, void *stream)

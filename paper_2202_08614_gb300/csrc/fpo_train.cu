@@ -739,9 +739,10 @@ __global__ void __launch_bounds__(256, 4) leaf_adam_kernel(const __grid_constant
 
 // The same step with the batch's gradient as a list of visits (and, for the
 // leaves with a mark, the rows of grad too): a row's gradient is summed over
-// its leaf's visits in registers, so no gradient row is written, read or
-// cleared: 7 row transfers per updated leaf instead of 9, and none in the
-// adjoint.  Compile-time sizes: those of the adjoint.  A warp has one whole
+// its leaf's first VL_SLOTS visits in registers, so for most leaves no gradient
+// row is written, read or cleared: 7 row transfers per updated leaf instead of
+// 9, and none in the adjoint.  The visits past those are in the rows of grad
+// before this kernel runs (grad_scatter_kernel).  Compile-time sizes: those of the adjoint.  A warp has one whole
 // row in flight, and four CTAs share an SM: 0.97 ms for 0.86M rows of the
 // 3.5M-leaf body (4.1 TB/s of randomly placed rows, what a plain random
 // read-add-write reaches); two rows of 96 elements at three CTAs 1.25 ms.
@@ -756,33 +757,34 @@ __global__ void __launch_bounds__(256, 4) leaf_adam_visits_kernel(const __grid_c
     const VisitList &L = p.list;
     for (uint32_t base = warp * 32; base < p.n_leaves; base += n_warps * 32) {
         const uint32_t i = base + lane;
-        uint32_t id = 0, head = NONE;
+        uint32_t id = 0, visits = 0;
         bool marked = false;
         if (i < p.n_leaves) {
             id = __ldg(p.perm + i);
-            head = L.head[id];
+            visits = min(L.visits[id], VL_SLOTS);
             marked = p.leaf_mark[id] != 0;
         }
-        // every lane fetches its own leaf's last visit: one latency for the warp
-        uint32_t ray = 0, next = NONE;
+        // every lane fetches its own leaf's first visit: one latency for the warp
+        uint4 slot = make_uint4(NONE, NONE, NONE, NONE);
+        if (visits) slot = L.slot[id];
+        uint32_t ray = 0;
         float4 val = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (head != NONE) {
-            ray = L.id[head].y;
-            val = L.val[head];
-            next = L.next[head];
+        if (slot.x != NONE) {
+            ray = L.id[slot.x].y;
+            val = L.val[slot.x];
         }
-        for (uint32_t todo = __ballot_sync(0xffffffffu, marked || head != NONE); todo; todo &= todo - 1) {
+        for (uint32_t todo = __ballot_sync(0xffffffffu, marked || visits); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
             const uint32_t leaf = base + src;
             const size_t at = (size_t)__shfl_sync(0xffffffffu, id, src) * NC;
-            const bool listed = __shfl_sync(0xffffffffu, head, src) != NONE, dense = __shfl_sync(0xffffffffu, marked, src);
-            const uint32_t nx = __shfl_sync(0xffffffffu, next, src);
+            const bool listed = __shfl_sync(0xffffffffu, slot.x, src) != NONE, dense = __shfl_sync(0xffffffffu, marked, src);
+            const uint32_t n = __shfl_sync(0xffffffffu, visits, src);
             const float *w0 = L.w + (size_t)__shfl_sync(0xffffffffu, ray, src) * (N1 + NZ);
             const float4 c = make_float4(__shfl_sync(0xffffffffu, val.x, src), __shfl_sync(0xffffffffu, val.y, src),
                                          __shfl_sync(0xffffffffu, val.z, src), __shfl_sync(0xffffffffu, val.w, src));
             auto pick = [](const float4 &x, int jz) { return jz < 0 ? x.x : (jz < NZ ? x.y : (jz < 2 * NZ ? x.z : x.w)); };
             float g[PER], m[PER], v[PER], w[PER];
-            // every load of the row first, the weights of its last visit among them
+            // every load of the row first, the weights of its first visit among them
 #pragma unroll
             for (int r = 0; r < PER; ++r) {
                 const int j = 32 * r + lane, jz = j - N1;
@@ -796,7 +798,9 @@ __global__ void __launch_bounds__(256, 4) leaf_adam_visits_kernel(const __grid_c
             }
 #pragma unroll
             for (int r = 0; r < PER; ++r) g[r] *= pick(c, 32 * r + lane - N1);
-            for (uint32_t e = nx; e != NONE; e = L.next[e]) {  // the leaf's other visits
+            for (uint32_t k = 1; k < n; ++k) {  // the leaf's other visits
+                const uint32_t e = __shfl_sync(0xffffffffu, k == 1 ? slot.y : (k == 2 ? slot.z : slot.w), src);
+                if (e == NONE) continue;
                 const float *wr = L.w + (size_t)L.id[e].y * (N1 + NZ);
                 const float4 x = L.val[e];
 #pragma unroll
@@ -831,7 +835,7 @@ __global__ void __launch_bounds__(256, 4) leaf_adam_visits_kernel(const __grid_c
             }
         }
         if (marked) p.leaf_mark[id] = 0;
-        if (head != NONE) L.head[id] = NONE;
+        if (visits) L.visits[id] = 0u;
     }
     // the last warp empties the list
     if (lane == 0) {
@@ -839,6 +843,7 @@ __global__ void __launch_bounds__(256, 4) leaf_adam_visits_kernel(const __grid_c
         if (atomicAdd(L.count + 1, 1u) == n_warps - 1) {
             atomicExch(L.count, 0u);
             atomicExch(L.count + 1, 0u);
+            atomicExch(L.count + 2, 0u);
         }
     }
 }
@@ -849,6 +854,8 @@ int launch_leaf_adam(const LeafAdamParams &p, int sm_count, void *stream)
     uint64_t blocks = ((uint64_t)p.n_leaves + 255) / 256;
     if (blocks > (uint64_t)sm_count * 8) blocks = (uint64_t)sm_count * 8;
     if (p.list.cap) {
+        const int ce = launch_grad_scatter_over(p.list, p.n1, p.n2, p.grad, p.leaf_mark, sm_count, stream);
+        if (ce != cudaSuccess) return ce;
         auto go = [&](auto kern) {
             kern<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(p);
             return (int)cudaGetLastError();

@@ -92,7 +92,7 @@ def _step(defer, calls, overflow=False):
     p = torch.as_tensor(tree.coeffs, device="cuda")
     p, m, v, grad = p.clone(), torch.full_like(p, 1e-3), torch.full_like(p, 1e-4), torch.zeros_like(p)
     mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
-    if overflow:  # the list keeps the room of its first batch: 4096 rays, 32 visits each
+    if overflow:  # the list has the room of its first batch: 4096 rays, 32 visits each
         o, d, t, g = _rays(8, 1)
         rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
         r.render_backward(rgb, g * 0, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=defer)
@@ -111,7 +111,8 @@ def _step(defer, calls, overflow=False):
     return p, m, v, rows
 
 
-# one batch; several on one list; one that does not fit beside another (its rows go to grad)
+# one batch; three of which the list has room for the first (the others' rows go to
+# grad); one beside a first, of zero gradient, that sized the list
 @pytest.mark.parametrize("calls,overflow", [(1, False), (3, False), (1, True)])
 def test_deferred_step_equals_the_dense_one(calls, overflow):
     a, b = _step(False, calls, overflow), _step(True, calls, overflow)
@@ -158,3 +159,65 @@ def test_a_decoder_drops_a_pending_list(tensor_cores):
     r.status()
     r.close()
     assert not m.any() and torch.equal(p, torch.as_tensor(tree.coeffs, device="cuda"))
+
+
+def _coarse_tree():
+    """A leaf of an eighth of the cube, in front of 32^3 finest cells."""
+    k = np.arange(32 ** 3)
+    xyz = np.concatenate([[[0, 0, 0]], 32 + np.stack([k % 32, k // 32 % 32, k // 1024], 1)]).astype(np.uint32)
+    depth = np.array([1] + [6] * len(k), np.uint8)
+    c = np.random.default_rng(7).normal(size=(len(depth), 166)).astype(np.float32) * 0.1
+    c[:, 0] = np.where(depth == 1, 0.5, 20.0)
+    return synth.Tree(depth, xyz, c, 6)
+
+
+def _through_both(n, seed):
+    rng = np.random.default_rng(seed)
+    dev = lambda x: torch.as_tensor(x, dtype=torch.float32, device="cuda")
+    o = rng.uniform(-0.6, -0.1, (n, 3))
+    return dev(o), dev(rng.uniform(0.55, 0.75, (n, 3)) - o), dev(rng.uniform(0, 60, n)), dev(rng.normal(size=(n, 3)))
+
+
+def _run(tree, batches, defer, times=None):
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    p0 = torch.as_tensor(tree.coeffs, device="cuda")
+    p, m, v, grad = p0.clone(), torch.full_like(p0, 1e-3), torch.full_like(p0, 1e-4), torch.zeros_like(p0)
+    mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+    rgb = [r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"] for o, d, t, _ in batches]
+    for k in range(1 if times is None else 5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        for (o, d, t, g), y in zip(batches, rgb):
+            r.render_backward(y, g, grad, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=mark, defer=defer)
+        r.adam_leaves(p, grad, m, v, mark, 5)
+        b.record()
+        r.status()
+        assert not grad.any() and not mark.any()
+        if times is not None:
+            times.append(a.elapsed_time(b))
+    r.close()
+    return p, m, v, (p != p0).any(1)
+
+
+# several batches on one list (4096 rays fit), leaves with none to thousands of
+# visits, and more rays than the tree has leaves (the rows go to grad)
+@pytest.mark.parametrize("coarse,sizes", [(False, (1000, 1, 1500)), (False, (40, 40, 40)), (True, (1000, 1500)),
+                                          (True, (20000,)), (False, (6000,)), (False, (2000, 6000))])
+def test_deferred_batches_add_up(coarse, sizes):
+    tree = _coarse_tree() if coarse else synth.shell_tree(7)
+    batches = [(_through_both if coarse else _rays)(n, 50 + i) for i, n in enumerate(sizes)]
+    a, b = _run(tree, batches, False), _run(tree, batches, True)
+    assert torch.equal(a[3], b[3]) and int(a[3].sum()) > 100
+    for x, y in zip(a[:3], b[:3]):
+        _close(x, y)
+
+
+def test_a_coarse_leaf_does_not_hold_up_the_step():
+    # 30,000 visits of one leaf, summed one after another, took twenty times
+    # what the dense step takes
+    tree, batches = _coarse_tree(), [_through_both(30000, 9)]
+    dense, deferred = [], []
+    _run(tree, batches, False, dense)
+    _run(tree, batches, True, deferred)
+    assert min(deferred) <= 3.0 * min(dense)
