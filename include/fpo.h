@@ -280,7 +280,8 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * FPO_FLAG_FP64_GRADCHECK selects the FP64 replay, FPO_FLAG_DEFER_GRADIENT
  * leaves the gradient to the next fpo_adam_leaves (see the flags).
  * Batches of up to 262,144 rays keep their visits in a workspace of the
- * context (grown on the first larger batch, at most 0.4 GB) and add them to
+ * context (up to 4,096 rays 5 MB of what fpo_upload_tree allocates, grown on
+ * the first larger batch, at most 0.4 GB) and add them to
  * dL_dcoeffs in a second, evenly divided pass; other calls, calls under stream
  * capture (a graph holds nothing of the workspace), and visits beyond it add
  * them from the replay.

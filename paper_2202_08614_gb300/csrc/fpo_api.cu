@@ -113,6 +113,11 @@ constexpr uint32_t DEFAULT_INNER_STEPS = 0xffffffffu;  // a lane runs its ray to
 // Visit list of an adjoint call: batches of up to VL_MAX_RAYS rays, room for
 // VL_PER_RAY visits a ray (the 3.5M-leaf body: 15 on average), counter words.
 constexpr uint32_t VL_MAX_RAYS = 1u << 18, VL_PER_RAY = 32;
+// The first VL_BASE_RAYS rays' list shares the allocation of the SH records: an
+// allocation of its own took 130 to 220 us of a context's first adjoint, which
+// for batches of this size and trees of some ten thousand leaves was more than
+// the list had gained.
+constexpr uint32_t VL_BASE_RAYS = 4096;
 constexpr int VL_COUNT = 24, VL_COUNTS = 3;
 
 }  // namespace
@@ -152,6 +157,8 @@ struct fpo_ctx {
     cudaStream_t aux = nullptr;           // IDFT passes / decodes
     cudaStream_t trav[PIPE_MAX] = {};     // slots 1.. : their traversal streams
     // visits of an adjoint call (VisitList), grown by visit_list
+    unsigned char *vl_base = nullptr;   // room for VL_BASE_RAYS behind the SH records
+    unsigned char *d_vl_block = nullptr;  // an allocation for more rays
     uint2 *d_vl_id = nullptr;
     float4 *d_vl_val = nullptr;
     uint32_t *d_vl_over = nullptr;
@@ -162,18 +169,28 @@ struct fpo_ctx {
     uint32_t vl_used = 0;               // rays whose visits await fpo_adam_leaves
     cudaEvent_t ev_entry = nullptr, ev_mat[PIPE_MAX] = {}, ev_trav[PIPE_MAX] = {};
 
-    void free_visit_list()
+    // Bytes of a visit list for `rays` rays, and its arrays in a block of that size.
+    size_t vl_bytes(uint32_t rays) const
     {
-        dfree(d_vl_val);
-        d_vl_id = nullptr;
-        d_vl_over = nullptr;
-        d_vl_w = nullptr;
-        vl_cap = vl_rays = 0;
+        return (size_t)rays * (VL_PER_RAY * (sizeof(float4) + sizeof(uint2) + sizeof(uint32_t)) +
+                               ((size_t)cfg.n1 + 9 * (size_t)cfg.n2) * sizeof(float));
+    }
+    void set_visit_list(unsigned char *block, uint32_t rays)
+    {
+        const size_t e = block ? (size_t)rays * VL_PER_RAY : 0;
+        d_vl_val = reinterpret_cast<float4 *>(block);
+        d_vl_id = reinterpret_cast<uint2 *>(d_vl_val + e);
+        d_vl_over = reinterpret_cast<uint32_t *>(d_vl_id + e);
+        d_vl_w = reinterpret_cast<float *>(d_vl_over + e);
+        vl_cap = (uint32_t)e;
+        vl_rays = block ? rays : 0;
     }
 
     void free_tree()
     {
-        free_visit_list();
+        dfree(d_vl_block);
+        vl_base = nullptr;
+        set_visit_list(nullptr, 0);
         dfree(d_vl_slot);
         d_vl_visits = nullptr;
         vl_used = 0;
@@ -349,23 +366,30 @@ int fpo_upload_tree(fpo_ctx *ctx, const fpo_tree_desc *tree)
     }
     const size_t n_nodes = pk.nodes.size() / 8;
     cudaError_t e = cudaSuccess;
-    auto up = [&](void **dst, const void *src, size_t bytes, const char *what) -> int {
+    auto up = [&](void **dst, const void *src, size_t bytes, const char *what, size_t room = 0) -> int {
         if (bytes == 0) return FPO_OK;
-        e = cudaMalloc(dst, bytes);
+        e = cudaMalloc(dst, bytes + room);
         if (e != cudaSuccess) return cuda_fail(e, what);
         e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(e, what);
         return FPO_OK;
     };
+    // (where an adjoint will want it)
+    const size_t vl_room = storage == FPO_STORAGE_F32 && fused_supported(n1, n2) ? ctx->vl_bytes(VL_BASE_RAYS) : 0;
+    const size_t vl_at = (zc.size() + 255) / 256 * 256;
     if ((st = up((void **)&ctx->d_nodes, pk.nodes.data(), pk.nodes.size() * 4, "nodes")) ||
         (st = up((void **)&ctx->d_top, pk.top.data(), pk.top.size() * 4, "top blocks")) ||
         (st = up((void **)&ctx->d_bricks, pk.bricks.data(), pk.bricks.size() * 4, "bricks")) ||
         (st = up((void **)&ctx->d_perm, pk.perm.data(), pk.perm.size() * 4, "perm")) ||
         (st = up((void **)&ctx->d_sig, sig.data(), sig.size(), "sigma records")) ||
-        (st = up((void **)&ctx->d_z, zc.data(), zc.size(), "SH records")) ||
+        (st = up((void **)&ctx->d_z, zc.data(), zc.size(), "SH records", vl_at - zc.size() + vl_room)) ||
         (st = up((void **)&ctx->d_scale, scale.data(), scale.size() * 4, "FP8 scales"))) {
         ctx->free_tree();
         return st;
+    }
+    if (vl_room && ctx->d_z) {
+        ctx->vl_base = static_cast<unsigned char *>(ctx->d_z) + vl_at;
+        ctx->set_visit_list(ctx->vl_base, VL_BASE_RAYS);
     }
     ctx->n_leaves = tree->n_leaves;
     ctx->n_nodes = (uint32_t)n_nodes;
@@ -875,22 +899,16 @@ VisitList visit_list(fpo_ctx *c, uint64_t n_rays, bool defer, cudaStream_t s)
     if (c->vl_used + n > c->vl_rays) {
         if (c->vl_used) return L;
         const CaptureElsewhere relaxed;
-        c->free_visit_list();
-        uint32_t room = 4096;  // rays, in powers of two
+        dfree(c->d_vl_block);
+        c->set_visit_list(c->vl_base, VL_BASE_RAYS);
+        uint32_t room = VL_BASE_RAYS;  // rays, in powers of two
         while (room < n) room *= 2;
-        const size_t e = (size_t)room * VL_PER_RAY, nw = (size_t)c->cfg.n1 + 9 * (size_t)c->cfg.n2;
-        // one block (four allocations took 0.2 ms of a context's first adjoint)
-        if (cudaMalloc((void **)&c->d_vl_val, e * (sizeof(float4) + sizeof(uint2) + sizeof(uint32_t)) +
-                                                  (size_t)room * nw * sizeof(float)) != cudaSuccess) {
+        if (cudaMalloc((void **)&c->d_vl_block, c->vl_bytes(room)) != cudaSuccess) {
             cudaGetLastError();
-            c->d_vl_val = nullptr;
+            c->d_vl_block = nullptr;
             return L;
         }
-        c->d_vl_id = reinterpret_cast<uint2 *>(c->d_vl_val + e);
-        c->d_vl_over = reinterpret_cast<uint32_t *>(c->d_vl_id + e);
-        c->d_vl_w = reinterpret_cast<float *>(c->d_vl_over + e);
-        c->vl_cap = (uint32_t)e;
-        c->vl_rays = room;
+        c->set_visit_list(c->d_vl_block, room);
     }
     if (defer && !c->d_vl_slot) {
         const CaptureElsewhere relaxed;

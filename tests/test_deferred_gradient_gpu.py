@@ -221,3 +221,37 @@ def test_a_coarse_leaf_does_not_hold_up_the_step():
     _run(tree, batches, False, dense)
     _run(tree, batches, True, deferred)
     assert min(deferred) <= 3.0 * min(dense)
+
+
+def test_a_first_small_adjoint_allocates_nothing():
+    tree = synth.shell_tree(7)
+
+    def grads(n, r):
+        o, d, t, g = _rays(n, 3)
+        rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+        grad = torch.zeros(tree.coeffs.shape, device="cuda")
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        r.render_backward(rgb, g, grad, rays_o=o, rays_d=d, t_per_ray=t)
+        torch.cuda.synchronize()
+        return free - torch.cuda.mem_get_info()[0], grad
+
+    warm = fpo.Renderer(idft_mode="fused")  # (the kernels' code is loaded at their first launch)
+    warm.upload(tree)
+    grads(300, warm)
+    warm.close()
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    used, a = grads(4096, r)
+    assert used == 0
+    more, _ = grads(8192, r)  # a list of its own, and then that one for fewer rays too
+    assert more > 0
+    used, b = grads(4096, r)
+    assert used == 0
+    r.upload(tree)  # back to the first room
+    used, c = grads(4096, r)
+    r.status()
+    r.close()
+    assert used == 0
+    _close(b, a)
+    _close(c, a)
