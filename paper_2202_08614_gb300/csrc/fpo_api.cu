@@ -152,8 +152,8 @@ struct fpo_ctx {
     bool table_ok = false;    // d_table holds the IDFT pass of table_t for the current coefficients
     double table_t = 0.0;
     // slot b of the pipeline: frames b, b + depth, ... (slot 0: d_table, the caller's stream)
-    float *d_ptable[PIPE_MAX] = {};       // slots 1.. : their tables
-    size_t ptable_leaves[PIPE_MAX] = {};
+    float *d_ptables = nullptr;           // the tables of slots 1 .. ptable_slots, one after another
+    int ptable_slots = 0;
     cudaStream_t aux = nullptr;           // IDFT passes / decodes
     cudaStream_t trav[PIPE_MAX] = {};     // slots 1.. : their traversal streams
     // visits of an adjoint call (VisitList), grown by visit_list
@@ -209,10 +209,8 @@ struct fpo_ctx {
         dfree(d_table);
         table_leaves = 0;
         table_ok = false;
-        for (int b = 1; b < PIPE_MAX; ++b) {
-            dfree(d_ptable[b]);
-            ptable_leaves[b] = 0;
-        }
+        dfree(d_ptables);
+        ptable_slots = 0;
         has_tree = false;
     }
 };
@@ -758,21 +756,27 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
     const int slots = n_frames < (uint32_t)depth ? (int)n_frames : depth;  // in use by this call
     const int trav_threads = ctx->half_table ? FPO_PIPE_TRAV_THREADS_F16 : PIPE_TRAV_THREADS;
     const int trav_ctas = ctx->half_table ? FPO_PIPE_TRAV_CTAS_F16 : PIPE_TRAV_CTAS;
-    for (int b = 0; b < (one_t ? 1 : slots); ++b) {
-        float *&tb = b ? ctx->d_ptable[b] : ctx->d_table;
-        size_t &tl = b ? ctx->ptable_leaves[b] : ctx->table_leaves;
-        if (tl < ctx->n_leaves) {
-            dfree(tb);
-            e = cudaMalloc((void **)&tb, table_alloc_bytes(ctx));
-            if (e != cudaSuccess) { tl = 0; return cuda_fail(e, "cudaMalloc(table)"); }
-            tl = ctx->n_leaves;
-        }
+    // Tables, streams and events as this call needs them, the further slots'
+    // tables in one allocation: what a context's first call of a few small
+    // frames spends most of its time on.
+    if (ctx->table_leaves < ctx->n_leaves) {
+        dfree(ctx->d_table);
+        e = cudaMalloc((void **)&ctx->d_table, table_alloc_bytes(ctx));
+        if (e != cudaSuccess) { ctx->table_leaves = 0; return cuda_fail(e, "cudaMalloc(table)"); }
+        ctx->table_leaves = ctx->n_leaves;
     }
-    if (!ctx->aux || !ctx->trav[depth - 1] || !ctx->ev_trav[depth - 1]) {
+    if (!one_t && ctx->ptable_slots < slots - 1) {
+        dfree(ctx->d_ptables);
+        ctx->ptable_slots = 0;
+        e = cudaMalloc((void **)&ctx->d_ptables, (size_t)(slots - 1) * table_alloc_bytes(ctx));
+        if (e != cudaSuccess) { ctx->d_ptables = nullptr; return cuda_fail(e, "cudaMalloc(table)"); }
+        ctx->ptable_slots = slots - 1;
+    }
+    if (!ctx->aux || !ctx->trav[slots - 1] || !ctx->ev_trav[slots - 1]) {
         // created once; a failed attempt is retried whole
         if (!ctx->aux) e = cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking);
         if (e == cudaSuccess && !ctx->ev_entry) e = cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming);
-        for (int b = 0; b < depth && e == cudaSuccess; ++b) {
+        for (int b = 0; b < slots && e == cudaSuccess; ++b) {
             if (b && !ctx->trav[b]) e = cudaStreamCreateWithFlags(&ctx->trav[b], cudaStreamNonBlocking);
             if (e == cudaSuccess && !ctx->ev_mat[b]) e = cudaEventCreateWithFlags(&ctx->ev_mat[b], cudaEventDisableTiming);
             if (e == cudaSuccess && !ctx->ev_trav[b]) e = cudaEventCreateWithFlags(&ctx->ev_trav[b], cudaEventDisableTiming);
@@ -824,7 +828,8 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
         if ((e = cudaStreamWaitEvent(ctx->trav[b], ctx->ev_entry, 0)) != cudaSuccess) return cuda_fail(e, "stream ordering");
     for (uint32_t k = 0; k < n_frames; ++k) {
         const int b = (int)(k % (uint32_t)depth);
-        float *tbl = one_t ? ctx->d_table : (b ? ctx->d_ptable[b] : ctx->d_table);
+        float *tbl = one_t || b == 0 ? ctx->d_table
+                                     : ctx->d_ptables + (size_t)(b - 1) * (table_alloc_bytes(ctx) / sizeof(float));
         cudaStream_t ts = FPO_PIPE_SLOT_STREAMS && b ? ctx->trav[b] : s;
         int ce = cudaSuccess;
         if (!one_t || k == 0) {

@@ -146,3 +146,18 @@ def test_frames_rejects_mixed_sizes():
         assert r.render_frames([], []).shape[0] == 0
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_a_contexts_slots_grow_with_its_calls(storage):
+    tree = synth.shell_tree(5)
+    cams, times = synth.ring_cameras(8, 96, 64), [2.0 + 6.5 * i for i in range(8)]
+    r = fpo.Renderer(storage=storage)
+    r.upload(tree)
+    want = _per_frame(r, cams, times)
+    for n, one_t in ((2, False), (6, True), (3, False), (8, False), (5, False)):
+        got = r.render_frames(cams[:n], [times[0]] * n if one_t else times[:n])
+        ref = _per_frame(r, cams[:n], [times[0]] * n) if one_t else want[:n]
+        r.status()
+        assert torch.equal(got, ref)
+    r.close()
