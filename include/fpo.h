@@ -247,8 +247,8 @@ int fpo_render(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
  * are written (on the stream that traversed it), so a caller can read frame
  * k back while later frames render.  The result equals n_frames calls of
  * fpo_render.  In the table mode the work is pipelined over slots, four of
- * them with an FP32 table and six with an FP16 table: frame k uses slot
- * k mod 4 (6), with its own table (the context keeps as many as calls have
+ * them with an FP32 table and six with an FP16 table (four where six tables
+ * do not fit in memory): frame k uses slot k mod 4 (6), with its own table (the context keeps as many as calls have
  * used: up to 4 x n_leaves x 128 or 6 x n_leaves x 64 bytes), traversal
  * stream (slot 0: cuda_stream; the others internal) and tile counter; the tables of the
  * next frames are computed on another internal stream while earlier frames

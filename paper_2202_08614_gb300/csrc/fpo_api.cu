@@ -154,6 +154,7 @@ struct fpo_ctx {
     // slot b of the pipeline: frames b, b + depth, ... (slot 0: d_table, the caller's stream)
     float *d_ptables = nullptr;           // the tables of slots 1 .. ptable_slots, one after another
     int ptable_slots = 0;
+    int pipe_cap = PIPE_MAX;              // slots that this tree's tables were found to leave memory for
     cudaStream_t aux = nullptr;           // IDFT passes / decodes
     cudaStream_t trav[PIPE_MAX] = {};     // slots 1.. : their traversal streams
     // visits of an adjoint call (VisitList), grown by visit_list
@@ -211,6 +212,7 @@ struct fpo_ctx {
         table_ok = false;
         dfree(d_ptables);
         ptable_slots = 0;
+        pipe_cap = PIPE_MAX;
         has_tree = false;
     }
 };
@@ -752,8 +754,9 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
     bool one_t = n_frames > 1;
     for (uint32_t k = 1; k < n_frames && one_t; ++k)
         one_t = memcmp(&frames[k].t, &frames[0].t, sizeof(double)) == 0;
-    const int depth = ctx->half_table ? FPO_PIPE_DEPTH_F16 : FPO_PIPE_DEPTH;
-    const int slots = n_frames < (uint32_t)depth ? (int)n_frames : depth;  // in use by this call
+    int depth = ctx->half_table ? FPO_PIPE_DEPTH_F16 : FPO_PIPE_DEPTH;
+    if (depth > ctx->pipe_cap) depth = ctx->pipe_cap;
+    int slots = n_frames < (uint32_t)depth ? (int)n_frames : depth;  // in use by this call
     const int trav_threads = ctx->half_table ? FPO_PIPE_TRAV_THREADS_F16 : PIPE_TRAV_THREADS;
     const int trav_ctas = ctx->half_table ? FPO_PIPE_TRAV_CTAS_F16 : PIPE_TRAV_CTAS;
     // Tables, streams and events as this call needs them, the further slots'
@@ -765,12 +768,18 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
         if (e != cudaSuccess) { ctx->table_leaves = 0; return cuda_fail(e, "cudaMalloc(table)"); }
         ctx->table_leaves = ctx->n_leaves;
     }
-    if (!one_t && ctx->ptable_slots < slots - 1) {
+    while (!one_t && ctx->ptable_slots < slots - 1) {
         dfree(ctx->d_ptables);
         ctx->ptable_slots = 0;
         e = cudaMalloc((void **)&ctx->d_ptables, (size_t)(slots - 1) * table_alloc_bytes(ctx));
-        if (e != cudaSuccess) { ctx->d_ptables = nullptr; return cuda_fail(e, "cudaMalloc(table)"); }
-        ctx->ptable_slots = slots - 1;
+        if (e == cudaSuccess) {
+            ctx->ptable_slots = slots - 1;
+        } else {
+            ctx->d_ptables = nullptr;
+            if (e != cudaErrorMemoryAllocation || slots <= FPO_PIPE_DEPTH) return cuda_fail(e, "cudaMalloc(table)");
+            cudaGetLastError();  // a tree so large that six tables do not fit: four
+            slots = depth = ctx->pipe_cap = FPO_PIPE_DEPTH;
+        }
     }
     if (!ctx->aux || !ctx->trav[slots - 1] || !ctx->ev_trav[slots - 1]) {
         // created once; a failed attempt is retried whole

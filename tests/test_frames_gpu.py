@@ -161,3 +161,30 @@ def test_a_contexts_slots_grow_with_its_calls(storage):
         r.status()
         assert torch.equal(got, ref)
     r.close()
+
+
+def test_frames_take_fewer_slots_when_six_tables_do_not_fit():
+    # a 2.6M-leaf tree, FP16 tables of 166 MB; room for three more beside the
+    # first, not for five
+    xyz = synth.shell_leaves(8)
+    n = xyz.shape[0]
+    m = LatentModel(n, seed=3)
+    r = fpo.Renderer(storage="latent")
+    r.upload(synth.Tree(np.full(n, 8, np.uint8), xyz, np.zeros(1, np.float32), 8))
+    r.set_latents(m.p["lat"].half(), *(m.p[k] for k in ("w1", "b1", "w2", "b2", "w3", "b3")))
+    cams, times = synth.ring_cameras(7, 64, 48), [1.5 + 8.0 * i for i in range(7)]
+    want, out = _per_frame(r, cams, times), torch.empty((7, 64 * 48, 3), device="cuda")
+    r.render_frames(cams[:2], times[:2])  # (the kernels' code and two slots' streams)
+    torch.cuda.synchronize()
+    table = n * 64
+    filler = None
+    try:
+        filler = torch.empty(torch.cuda.mem_get_info()[0] - int(3.2 * table), dtype=torch.uint8, device="cuda")
+        for _ in range(2):
+            r.render_frames(cams, times, out=out)
+            r.status()
+            assert torch.equal(out, want)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    r.close()
