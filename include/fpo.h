@@ -211,7 +211,8 @@ typedef struct {
 
 typedef struct {
     uint32_t n_leaves, n_nodes, max_depth, n_smem_nodes;
-    uint64_t node_bytes;      /* device bytes of the node array */
+    uint64_t node_bytes;      /* device bytes of the node array (not of the index beside it that trees of
+                               * finest cells have: 16 a brick of 4^3 cells, and 256 a leaf or 64 KB at most) */
     uint64_t leaf_bytes;      /* device bytes of the stored coefficients (or latents) */
     uint64_t leaf_record_bytes; /* stored bytes per leaf (padded); 64 for LATENT storage */
     uint64_t table_bytes;     /* device bytes of the per-frame IDFT table (0 until used) */

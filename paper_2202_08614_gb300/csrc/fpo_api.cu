@@ -326,7 +326,7 @@ int fpo_upload_tree(fpo_ctx *ctx, const fpo_tree_desc *tree)
     PackedTree pk;
     std::string err;
     const bool latent = ctx->cfg.storage == FPO_STORAGE_LATENT;
-    int st = validate_and_pack(tree, latent ? 0 : ctx->cfg.n1, ctx->cfg.n2, &pk, &err);
+    int st = validate_and_pack(tree, latent ? 0 : ctx->cfg.n1, ctx->cfg.n2, &pk, &err, false);
     if (st != FPO_OK) return fail(st, "%s", err.c_str());
     DeviceGuard g(ctx->cfg.device);
     if (!g.ok) return fail(FPO_ERR_CUDA, "cudaSetDevice failed");

@@ -38,6 +38,17 @@ constexpr int MAX_DEPTH = 12;
 // in it (leaf, empty 1, 2, 4, 8, 16, ...) are the octree's.  The 3.5M-leaf body
 // takes 0.5 + 1 MB, its node array 17 MB.
 constexpr int BRICK_MIN_DEPTH = 4, BRICK_MAX_DEPTH = 11;
+// The top grid is dense, 16 bytes a block: a tree gets the index when that is at
+// most 256 bytes a leaf (the coefficient records take 672 at n1 = 31, n2 = 5), or
+// 64 KB; sparser trees of depth 9 to 11 keep the octree walk.  Blocks a leaf, with
+// n1 = n2 = 1, upload in ms without and with it and an 800x800 frame in us: depth
+// 9, 6.0: 0.47 / 0.80, 126 / 92; 10, 6.0: 3.7 / 6.0, 223 / 156; 11, 6.0: 28 / 51,
+// 507 / 323; 10, 48: 0.56 / 1.4, 125 / 88; 11, 48: 4.3 / 10.9, 212 / 143.  Ten
+// leaves at depth 11 took 22 ms to pack and 33 MB.
+constexpr bool brick_index_fits(uint64_t n_leaves, int depth)
+{
+    return (1ull << (3 * (depth - 4))) <= (n_leaves > 256 ? 16 * n_leaves : 4096);
+}
 
 // Leaf records.  FP32 storage: a density record of SIG_STRIDE(n1) floats
 // (n1 rounded up to a multiple of 4, 128 bytes for n1 = 31) and an SH record
@@ -103,7 +114,8 @@ struct PackedTree {
 // Validates a tree description (and packs it when `out` is non-null).
 // Returns FPO_OK, FPO_ERR_INVALID_ARG or FPO_ERR_BAD_TREE (message in *err).
 int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out,
-                      std::string *err);
+                      std::string *err,
+                      bool any_density = true);
 
 // ---------------------------------------------------------------------------
 // Kernel parameters.

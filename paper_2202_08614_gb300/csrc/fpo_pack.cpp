@@ -112,27 +112,31 @@ void pack_uniform(const std::vector<std::pair<uint64_t, uint32_t>> &key, int shi
         next += (uint32_t)(slots[l].size() / 8);
         for (const uint32_t c : slots[l]) out->nodes.push_back(c == 0u || (c & LEAF_BIT) ? c : next + c - 1);
     }
-    // empty blocks: the side of the octree's empty cube that holds them
-    for (size_t c = 0; c < T * T * T; ++c) {
-        uint32_t *t = &out->top[c * 4];
-        if (t[0] | t[1]) continue;
-        const uint32_t x = (uint32_t)(c % T), y = (uint32_t)(c / T % T), z = (uint32_t)(c / T / T);
-        uint32_t node = 0;
-        for (int l = 0; l < tb; ++l) {
-            const int sh = tb - 1 - l;
-            const uint32_t o = ((x >> sh) & 1u) | (((y >> sh) & 1u) << 1) | (((z >> sh) & 1u) << 2);
-            node = out->nodes[(size_t)node * 8 + o];
-            if (node == 0) {
-                t[3] = 1u << (D - l - 1);
-                break;
+    // empty blocks: the side of the octree's empty cube that holds them, cube by cube
+    struct At { uint32_t node, x, y, z; int l; };
+    std::vector<At> todo;  // nodes of up to 2^tb blocks a side, their first block
+    if (tb > 0) todo.push_back({0, 0, 0, 0, 0});
+    while (!todo.empty()) {
+        const At a = todo.back();
+        todo.pop_back();
+        const uint32_t side = 1u << (tb - a.l - 1);  // of a child, in blocks
+        for (uint32_t o = 0; o < 8; ++o) {
+            const uint32_t x = a.x + (o & 1u) * side, y = a.y + (o >> 1 & 1u) * side, z = a.z + (o >> 2) * side;
+            const uint32_t node = out->nodes[(size_t)a.node * 8 + o];
+            if (node != 0) {
+                if (a.l + 1 < tb) todo.push_back({node, x, y, z, a.l + 1});
+                continue;
             }
+            for (uint32_t w = z; w < z + side; ++w)
+                for (uint32_t v = y; v < y + side; ++v)
+                    for (uint32_t u = x; u < x + side; ++u) out->top[((w * T + v) * T + u) * 4 + 3] = 1u << (D - a.l - 1);
         }
     }
 }
 
 }  // namespace
 
-int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out, std::string *err)
+int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out, std::string *err, bool any_density)
 {
     (void)n2;  // n1 == 0 marks a tree without coefficients (latent storage)
     if (!tree) { *err = "tree description is NULL"; return FPO_ERR_INVALID_ARG; }
@@ -197,7 +201,7 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
         return FPO_OK;
     }
     out->root_kind = ROOT_NODE;
-    bool uniform = dmax >= BRICK_MIN_DEPTH && dmax <= BRICK_MAX_DEPTH;
+    bool uniform = dmax >= BRICK_MIN_DEPTH && dmax <= BRICK_MAX_DEPTH && (any_density || brick_index_fits(n, dmax));
     for (uint32_t j = 0; j < n && uniform; ++j) uniform = tree->leaf_depth[j] == dmax;
     if (uniform) {
         pack_uniform(iv, 3 * (M - dmax), dmax, out);

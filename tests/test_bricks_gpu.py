@@ -21,10 +21,11 @@ def _built():
     __graft_entry__.build()
 
 
-def _uniform_tree(depth, seed, n1=31, n2=5):
+def _uniform_tree(depth, seed, n1=31, n2=5, block=0):
     """Finest cells in clumps of 1, 2, 4 and 8 cells a side and single ones, in
     shuffled upload order: partly filled bricks, bricks in every corner of a
-    block, empty cubes of every size."""
+    block, empty cubes of every size.  block: a full cube of that side besides,
+    for trees with the leaves that the index of a deep grid asks for."""
     rng = np.random.default_rng(seed)
     g = 1 << depth
     cells = {(0, 0, 0), (g - 1, g - 1, g - 1), (g - 1, 0, 0), (0, g - 1, 3)}
@@ -33,15 +34,30 @@ def _uniform_tree(depth, seed, n1=31, n2=5):
             cells |= {(int(lo[0]) + i, int(lo[1]) + j, int(lo[2]) + k)
                       for i in range(s) for j in range(s) for k in range(s) if rng.random() < 0.8}
     xyz = np.array(sorted(cells), np.uint32)
+    if block:
+        lo, k = g // 2 - 7, np.arange(block ** 3)
+        cube = lo + np.stack([k % block, k // block % block, k // block ** 2], 1).astype(np.uint32)
+        xyz = np.concatenate([xyz[((xyz < lo) | (xyz >= lo + block)).any(1)], cube.astype(np.uint32)])
     xyz = xyz[rng.permutation(len(xyz))]
     coeffs = synth.draw_coefficients(rng, len(xyz), n1, n2)
     return synth.Tree(np.full(len(xyz), depth, np.uint8), xyz, coeffs, depth, n1, n2)
 
 
-# 4 and 11: the smallest and the deepest grid the index serves; 3 and 12 walk the octree both times
+# 4: the smallest grid the index serves; 3 and 12, and 9 and 11 with so few leaves, walk the octree both times
 @pytest.mark.parametrize("depth", [3, 4, 5, 6, 9, 11, 12])
 def test_brick_walk_equals_octree_descent(depth):
-    tree = _uniform_tree(depth, 40 + depth)
+    _same_walk(_uniform_tree(depth, 40 + depth), depth)
+
+
+# the leaves that a grid of this depth needs for its index, and no more than a few hundred besides
+@pytest.mark.parametrize("depth,block", [(9, 12), (11, 50)])
+def test_brick_walk_of_deep_grids(depth, block):
+    tree = _uniform_tree(depth, 40 + depth, 1, 1, block + 1)
+    assert tree.n_leaves >= 8 ** (depth - 4) // 16
+    _same_walk(tree, depth, 512, n1=1, n2=1)
+
+
+def _same_walk(tree, depth, cap=128, **sizes):
     rng = np.random.default_rng(depth)
     # rays at the leaves (the grid is mostly empty), axis-parallel ones among them
     n = 4000
@@ -52,9 +68,9 @@ def test_brick_walk_equals_octree_descent(depth):
     d = torch.as_tensor(d, dtype=torch.float32, device="cuda")
     out = []
     for kw in ({}, {"refill_min": 16}):
-        r = fpo.Renderer(**kw)
+        r = fpo.Renderer(**kw, **sizes)
         r.upload(tree)
-        log = r.render(rays_o=o, rays_d=d, t=7.0, visit_cap=128, stop_T=0.0, want_T=True)
+        log = r.render(rays_o=o, rays_d=d, t=7.0, visit_cap=cap, stop_T=0.0, want_T=True)
         rgb = r.render(rays_o=o, rays_d=d, t=7.0, stop_T=0.0)["rgb"]
         r.status()
         out.append((log["visit_count"], log["visit_log"], log["T"], log["rgb"], rgb))
