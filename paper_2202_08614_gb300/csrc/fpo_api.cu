@@ -811,7 +811,8 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
             mshape = materialise_pipeline_shape(ctx->cfg.storage, ctx->cfg.n1, ctx->cfg.n2, PIPE_MAT_SMEM_BUDGET);
             if (FPO_PIPE_MAT_CTAS > 0) mshape.ctas_per_sm = FPO_PIPE_MAT_CTAS;
         }
-        const long need = (long)trav_ctas * (traverse_smem_bytes(ctx->d_top != nullptr, trav_threads) + PIPE_STATIC_SMEM + reserved) +
+        const bool brick = brick_walk(ctx->d_top != nullptr, ctx->cfg.refill_min ? (uint32_t)ctx->cfg.refill_min : DEFAULT_REFILL_MIN);
+        const long need = (long)trav_ctas * (traverse_smem_bytes(brick, trav_threads) + PIPE_STATIC_SMEM + reserved) +
                           (long)mshape.ctas_per_sm * (mshape.smem_per_cta + PIPE_STATIC_SMEM + reserved);
         // The driver rounds a carveout request up to one of the SM's shared-
         // memory configurations: ask for the smallest one that holds `need`.

@@ -406,6 +406,9 @@ int launch_leaf_adam(const LeafAdamParams &p, int sm_count, void *stream);
 int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int sm_count,
                     void *stream);
 int traverse_smem_bytes(bool brick, int threads);
+// Whether the traversal walks the brick index; the compaction schedule
+// (refill_min < 32, a tuning option) walks the octree of every tree.
+constexpr bool brick_walk(bool has_index, uint32_t refill_min) { return has_index && refill_min >= 32; }
 bool fused_supported(int n1, int n2);
 
 }  // namespace fpo

@@ -1185,9 +1185,9 @@ template <int TM>
 static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaStream_t s)
 {
     constexpr int R = FPO_TRAV_MAXNREG_MAT;
-    if (p.refill_min < 32)  // (a tuning option: the octree descent serves every tree)
+    if (p.refill_min < 32)
         return debug ? launch_t<TM, true, true, false, R>(p, sm_count, s) : launch_t<TM, false, true, false, R>(p, sm_count, s);
-    if (p.top) {
+    if (brick_walk(p.top != nullptr, p.refill_min)) {
         if (TM == TM_TABLE_F32 && p.max_ctas_per_sm == 0)
             return debug ? launch_t<TM, true, false, true, FPO_TRAV_MAXNREG_ALONE>(p, sm_count, s)
                          : launch_t<TM, false, false, true, FPO_TRAV_MAXNREG_ALONE>(p, sm_count, s);

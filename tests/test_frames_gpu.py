@@ -188,3 +188,18 @@ def test_frames_take_fewer_slots_when_six_tables_do_not_fit():
         del filler
         torch.cuda.empty_cache()
     r.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_frames_with_the_compaction_schedule(storage):
+    # a tree with the brick index, which this schedule does not walk
+    tree = synth.shell_tree(5)
+    cams, times = synth.ring_cameras(5, 640, 400), [2.0 + 6.5 * i for i in range(5)]
+    r, plain = fpo.Renderer(storage=storage, refill_min=8), fpo.Renderer(storage=storage)
+    r.upload(tree)
+    plain.upload(tree)
+    got = r.render_frames(cams, times)
+    r.status()
+    assert torch.equal(got, plain.render_frames(cams, times))
+    r.close()
+    plain.close()

@@ -1,5 +1,6 @@
-"""The ray queue of the fused mode over camera frames of every shape (host
-code only; the frames of 2^26 tiles and more are a few pixels wide or high)."""
+"""The ray queue of the fused mode over camera frames of every shape, and which
+walk a traversal takes (host code only; the frames of 2^26 tiles and more are a
+few pixels wide or high)."""
 
 import os
 import subprocess
@@ -24,3 +25,16 @@ def queue_check(tmp_path_factory):
 def test_every_pixel_has_one_slot(queue_check, w, h):
     out = subprocess.run([queue_check, str(w), str(h)], capture_output=True, text=True, check=True)
     assert int(out.stdout) == 0
+
+
+def test_the_compaction_schedule_walks_the_octree(tmp_path):
+    # the pipeline's shared-memory estimate asks the rule that the launcher follows
+    src, cuda = tmp_path / "walk.cpp", os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    src.write_text("""#include "fpo_internal.h"
+using fpo::brick_walk;
+static_assert(brick_walk(true, 32) && !brick_walk(true, 31) && !brick_walk(true, 1) && !brick_walk(false, 32), "");
+""")
+    subprocess.run(["g++", "-std=c++17", "-fsyntax-only", "-I", os.path.join(ROOT, "include"), "-I", SRC, "-I",
+                    os.path.join(cuda, "include"), str(src)], check=True)
+    api = open(os.path.join(SRC, "fpo_api.cu")).read()
+    assert "traverse_smem_bytes(brick, trav_threads)" in api and api.count("traverse_smem_bytes(") == 1
