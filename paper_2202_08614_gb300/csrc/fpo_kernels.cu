@@ -1621,16 +1621,22 @@ static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
     const int threads = 32 * FU_WARPS;
     const int smem = FU_WARPS * 4 * fused_warp_words(p.rays_per_warp, p.list_cap, BRICK ? 0 : p.depth + 1, FusedSize<N1, N2>::WROW);
     auto k = fused_kernel<N1, N2, ADJ, DBG, BRICK>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return (int)e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
-    if (e != cudaSuccess) return (int)e;
-    if (per_sm < 1) per_sm = 1;
-    uint64_t blocks = (uint64_t)sm_count * per_sm;
-    const uint64_t need = ((uint64_t)p.n_tiles * 32u / (uint32_t)p.rays_per_warp + FU_WARPS - 1) / FU_WARPS;
-    if (need < blocks) blocks = need ? need : 1;
-    k<<<(unsigned)blocks, threads, smem, s>>>(q);
+    uint64_t need = ((uint64_t)p.n_tiles * 32u / (uint32_t)p.rays_per_warp + FU_WARPS - 1) / FU_WARPS;
+    if (need < 1) need = 1;
+    // A small batch's grid is resident whole (eight CTAs an SM by registers and
+    // by these 24 KB) and asks the driver nothing; what the adjoint's second
+    // launch adds to the host's share of such a call is less than that took.
+    static_assert(FPO_FUSED_MAXNREG * 32 * FU_WARPS * 8 <= 65536, "eight CTAs of registers");
+    if (need > 8u * (uint64_t)sm_count || smem > 24 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return (int)e;
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
+        if (e != cudaSuccess) return (int)e;
+        if (per_sm < 1) per_sm = 1;
+        if (need > (uint64_t)sm_count * per_sm) need = (uint64_t)sm_count * per_sm;
+    }
+    k<<<(unsigned)need, threads, smem, s>>>(q);
     return (int)cudaGetLastError();
 }
 

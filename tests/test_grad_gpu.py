@@ -310,3 +310,26 @@ def test_finetuner_recovers_perturbed_coefficients():
     print(f"held-out loss {l0:.3e} -> {l1:.3e}")
     assert l1 < 0.2 * l0
     assert int(ft.mark.sum()) == 0
+
+
+def test_grids_asked_for_and_not():
+    # rays in batches whose grid (two rays a warp, two warps a CTA) is below, at
+    # and past the eight CTAs an SM that are launched without asking the driver
+    tree = synth.shell_tree(5)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(4)
+    n = 40 * sms * 32
+    o = rng.uniform(-0.6, 1.6, (n, 3))
+    dev = lambda x: torch.as_tensor(x, dtype=torch.float32, device="cuda")
+    o, d, t = dev(o), dev(rng.uniform(0.2, 0.8, (n, 3)) - o), dev(rng.uniform(0, 60, n))
+    whole = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    at = 0
+    for k in (1, 8 * sms * 4 - 32, 8 * sms * 4, 8 * sms * 4 + 1, 16 * sms * 4):
+        s = slice(at, at + k)
+        assert torch.equal(r.render(rays_o=o[s], rays_d=d[s], t_per_ray=t[s])["rgb"], whole[s])
+        at += k
+    assert at <= n
+    r.status()
+    r.close()
