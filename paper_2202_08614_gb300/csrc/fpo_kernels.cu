@@ -1628,7 +1628,8 @@ static int launch_fused_t(BackwardParams q, int sm_count, cudaStream_t s)
     // launch adds to the host's share of such a call is less than that took.
     static_assert(FPO_FUSED_MAXNREG * 32 * FU_WARPS * 8 <= 65536, "eight CTAs of registers");
     if (need > 8u * (uint64_t)sm_count || smem > 24 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // (never below the 48 KB that a launch may use without asking)
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem > 48 * 1024 ? smem : 48 * 1024);
         if (e != cudaSuccess) return (int)e;
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);

@@ -333,3 +333,25 @@ def test_grids_asked_for_and_not():
     assert at <= n
     r.status()
     r.close()
+
+
+def test_a_deeper_tree_after_a_shallow_one():
+    # the ancestor stacks of a deep tree's small batch take more shared memory
+    # than a shallow tree's larger batch, which asks the driver for its own
+    rng = np.random.default_rng(6)
+    dev = lambda x: torch.as_tensor(x, dtype=torch.float32, device="cuda")
+    for depth, n in ((3, 9000), (12, 500)):
+        g = 1 << depth
+        xyz = np.array([[0, 0, 0], [g - 1, g - 1, g - 1], [g // 2, g // 2, g // 2]], np.uint32)
+        tree = synth.Tree(np.full(3, depth, np.uint8), xyz, synth.draw_coefficients(rng, 3), depth)
+        r = fpo.Renderer(idft_mode="fused")
+        r.upload(tree)
+        to = (xyz[rng.integers(0, 3, n)] + rng.uniform(0, 1, (n, 3))) / g
+        d = rng.normal(size=(n, 3))
+        o, d, t = dev(to - d), dev(d), dev(rng.uniform(0, 60, n))
+        out = r.render(rays_o=o, rays_d=d, t_per_ray=t, visit_cap=8)
+        grad = torch.zeros(tree.coeffs.shape, device="cuda")
+        r.render_backward(out["rgb"], torch.ones_like(out["rgb"]), grad, rays_o=o, rays_d=d, t_per_ray=t)
+        r.status()
+        r.close()
+        assert int(out["visit_count"].sum()) > n // 4
