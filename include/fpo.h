@@ -282,10 +282,11 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * leaves the gradient to the next fpo_adam_leaves (see the flags).
  * Batches of up to 262,144 rays keep their visits in a workspace of the
  * context (up to 4,096 rays 5 MB of what fpo_upload_tree allocates, grown on
- * the first larger batch, at most 0.4 GB) and add them to
- * dL_dcoeffs in a second, evenly divided pass; other calls, calls under stream
- * capture (a graph holds nothing of the workspace), and visits beyond it add
- * them from the replay.
+ * the first larger batch, at most 0.4 GB) and add them to dL_dcoeffs in a
+ * second, evenly divided pass.  Larger calls, calls under stream capture (a
+ * graph holds nothing of the workspace), large calls on small trees and whole
+ * images (131,072 rays or more; by one lane a ray, as fpo_render renders
+ * them), and visits beyond the workspace are added from the replay.
  * Errors: INVALID_ARG, NO_TREE, UNSUPPORTED, CUDA. */
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
                         const float *out_rgb, const float *dL_drgb, float *dL_dcoeffs,

@@ -584,6 +584,7 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
         p.tiles_x = 0;
         p.n_tiles = (uint32_t)((n_rays + 31) / 32);
     }
+    p.lanes = lane_per_ray(rays->mode == FPO_RAYS_CAMERA, n_rays, ctx->n_leaves);
     p.max_steps = ctx->cfg.max_steps > 0 ? (uint32_t)ctx->cfg.max_steps : 3u * (1u << ctx->depth) + 16u;
     p.block_threads = ctx->cfg.traverse_threads ? ctx->cfg.traverse_threads : DEFAULT_TRAVERSE_THREADS;
     p.few_tiles_split = ctx->cfg.traverse_threads == 0;
@@ -1005,7 +1006,7 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     q.dL_dcoeffs = fp64 ? nullptr : dL_dcoeffs;
     q.dL_dcoeffs64 = fp64 ? reinterpret_cast<double *>(dL_dcoeffs) : nullptr;
     q.leaf_mark = mark ? opts->leaf_mark : nullptr;
-    if (!fp64) q.list = visit_list(ctx, n_rays, defer, (cudaStream_t)cuda_stream);
+    if (!fp64 && !q.tp.lanes) q.list = visit_list(ctx, n_rays, defer, (cudaStream_t)cuda_stream);
     int ce = launch_backward(q, ctx->sm_count, cuda_stream);
     if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
     if (q.list.slot) {

@@ -16,6 +16,7 @@
 
 #include <cfloat>
 #include <cstdint>
+#include <type_traits>
 
 #include "fpo_internal.h"
 #include "fpo_ptx.cuh"
@@ -871,9 +872,10 @@ __device__ __forceinline__ void move_to(RayState &R, const int Pn[3], float tx)
     R.P[2] = Pn[2];
 }
 
-// Table modes of the traversal: the per-frame table in FP32 (128-byte lines)
-// or FP16 (64-byte lines).
-constexpr int TM_TABLE_F32 = 1, TM_TABLE_F16 = 2;
+// What the traversal shades from: the per-frame table in FP32 (128-byte lines)
+// or FP16 (64-byte lines), or the FP32 coefficient records themselves (camera
+// frames of the fused mode).
+constexpr int TM_RECORDS = 0, TM_TABLE_F32 = 1, TM_TABLE_F16 = 2;
 
 __device__ __forceinline__ const float4 *table_record(const TraverseParams &p, uint32_t leaf)
 {
@@ -885,14 +887,79 @@ __device__ __forceinline__ const __half *table_record_f16(const TraverseParams &
     return reinterpret_cast<const __half *>(p.table) + (size_t)leaf * TABLE_STRIDE;
 }
 
-// Shades one leaf segment of length delta (Eq. 7 and 9 from the table, Eq. 1
-// colour, emission-absorption update).  Returns true when the transmittance
-// fell below stop_T.
-template <int TM, bool DBG>
-__device__ __forceinline__ bool shade(const TraverseParams &p, RayState &R, uint32_t leaf, float delta)
+// VW floats from a read-only global address aligned to 4 VW bytes.
+template <int VW>
+__device__ __forceinline__ void load_vec(const float *p, float *v)
+{
+    if constexpr (VW == 8) {
+        ldg256(p, v);
+    } else {
+        const float4 w = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+    }
+}
+
+// Eq. 8 at a ray's time in shared memory: element i at at[i * stride].
+struct Basis {
+    const float *at;
+    int stride;
+    __device__ __forceinline__ float operator[](int i) const { return at[i * stride]; }
+};
+
+// sigma_raw and z of one leaf at the ray's time (Eq. 7 and 9) from its FP32
+// records, in 32-byte pieces where both records start on 32 bytes.
+template <int N1, int N2>
+__device__ __forceinline__ void record_values(const TraverseParams &p, Basis b, uint32_t leaf, float &sraw, float z[27])
+{
+    float bz[N2];
+#pragma unroll
+    for (int i = 0; i < N2; ++i) bz[i] = b[i];
+    const float *sr = reinterpret_cast<const float *>(p.sig + (size_t)leaf * p.sig_stride4);
+    const float *zr = p.zc + (size_t)leaf * p.z_stride;
+    constexpr int VW = (N1 + 3) / 4 % 2 == 0 && (27 * N2 + 3) / 4 % 2 == 0 ? 8 : 4;
+    sraw = 0.0f;
+#pragma unroll
+    for (int q = 0; q < (N1 + VW - 1) / VW; ++q) {
+        float v[VW];
+        load_vec<VW>(sr + VW * q, v);
+#pragma unroll
+        for (int j = 0; j < VW; ++j)
+            if (VW * q + j < N1) sraw = fmaf(v[j], b[VW * q + j], sraw);
+    }
+#pragma unroll
+    for (int k = 0; k < 27; ++k) z[k] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < (27 * N2 + VW - 1) / VW; ++q) {
+        float v[VW];
+        load_vec<VW>(zr + VW * q, v);
+#pragma unroll
+        for (int j = 0; j < VW; ++j) {
+            const int e = VW * q + j;
+            if (e < 27 * N2) z[e / N2] = fmaf(v[j], bz[e % N2], z[e / N2]);
+        }
+    }
+}
+
+// Both records of a leaf into L2.
+__device__ __forceinline__ void prefetch_records(const TraverseParams &p, uint32_t leaf)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.sig + (size_t)leaf * p.sig_stride4),
+                 "r"((uint32_t)(p.sig_stride4 * 16)));
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.zc + (size_t)leaf * p.z_stride),
+                 "r"((uint32_t)(p.z_stride * 4)));
+}
+
+// Shades one leaf segment of length delta (Eq. 7 and 9 from the table or the
+// records, Eq. 1 colour, emission-absorption update).  Returns true when the
+// transmittance fell below stop_T.
+template <int TM, bool DBG, int N1, int N2>
+__device__ __forceinline__ bool shade(const TraverseParams &p, Basis b, RayState &R, uint32_t leaf, float delta)
 {
     float sigma, z[27];
-    if constexpr (TM == TM_TABLE_F16) {
+    if constexpr (TM == TM_RECORDS) {
+        record_values<N1, N2>(p, b, leaf, sigma, z);
+        sigma = fmaxf(sigma, 0.0f);
+    } else if constexpr (TM == TM_TABLE_F16) {
         // the 64-byte FP16 line: two 32-byte loads, widened to FP32
         const float *hrec = reinterpret_cast<const float *>(table_record_f16(p, leaf));
         float raw[16], v[32];
@@ -979,9 +1046,9 @@ __device__ __forceinline__ bool step_cap(const TraverseParams &p, RayState &R)
 // arithmetic; then the move.  `cb` becomes the next cube.
 // Returns false once the ray is finished (left the grid, early stop, or
 // step cap).
-template <int TM, bool DBG, bool BRICK>
-__device__ __forceinline__ bool pipelined_step(const TraverseParams &p, uint32_t *s_stack, int stride, RayState &R,
-                                               Cube &cb)
+template <int TM, bool DBG, bool BRICK, int N1, int N2>
+__device__ __forceinline__ bool pipelined_step(const TraverseParams &p, Basis b, uint32_t *s_stack, int stride,
+                                               RayState &R, Cube &cb)
 {
     const int G = 1 << p.depth;
     int m, lo[3];
@@ -993,12 +1060,13 @@ __device__ __forceinline__ bool pipelined_step(const TraverseParams &p, uint32_t
     if (inside) {
         nx = locate<BRICK>(p, s_stack, stride, R, Pn, cell_diff(R.P, Pn));
         if (nx.kind == ROOT_LEAF) {
-            if constexpr (TM == TM_TABLE_F32) asm volatile("prefetch.global.L1 [%0];" ::"l"(table_record(p, nx.leaf)));
+            if constexpr (TM == TM_RECORDS) prefetch_records(p, nx.leaf);
+            else if constexpr (TM == TM_TABLE_F32) asm volatile("prefetch.global.L1 [%0];" ::"l"(table_record(p, nx.leaf)));
             else asm volatile("prefetch.global.L1 [%0];" ::"l"(table_record_f16(p, nx.leaf)));
         }
     }
     if (cb.kind == ROOT_LEAF && tx > R.t)
-        if (shade<TM, DBG>(p, R, cb.leaf, tx - R.t)) return false;
+        if (shade<TM, DBG, N1, N2>(p, b, R, cb.leaf, tx - R.t)) return false;
     if (!inside) return false;
     move_to(R, Pn, tx);
     if (step_cap(p, R)) return false;
@@ -1007,17 +1075,36 @@ __device__ __forceinline__ bool pipelined_step(const TraverseParams &p, uint32_t
 }
 
 // A whole ray (lane-loop schedule).
-template <int TM, bool DBG, bool BRICK>
-__device__ void trace_ray(const TraverseParams &p, uint32_t *s_stack, int stride, RayState &R)
+template <int TM, bool DBG, bool BRICK, int N1, int N2>
+__device__ void trace_ray(const TraverseParams &p, Basis b, uint32_t *s_stack, int stride, RayState &R)
 {
     Cube cb = locate<BRICK>(p, s_stack, stride, R, R.P, first_diff(p));
-    while (pipelined_step<TM, DBG, BRICK>(p, s_stack, stride, R, cb)) {
+    while (pipelined_step<TM, DBG, BRICK, N1, N2>(p, b, s_stack, stride, R, cb)) {
     }
 }
 
 }  // namespace
 
 namespace {
+
+// The basis of a lane's rays: of each ray's own time, in a column of the CTA's
+// basis array (set_lane_basis, per ray), or of the call's, once for the CTA.
+__device__ __forceinline__ bool own_times(const TraverseParams &p) { return p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr; }
+__device__ __forceinline__ Basis lane_basis(const TraverseParams &p, uint32_t *mem)
+{
+    float *b = reinterpret_cast<float *>(mem);
+    if (own_times(p)) return {b + threadIdx.x, (int)blockDim.x};
+    if (threadIdx.x < MAX_BASIS) b[threadIdx.x] = p.fc.b[threadIdx.x];
+    __syncthreads();
+    return {b, 1};
+}
+__device__ __forceinline__ void set_lane_basis(const TraverseParams &p, Basis basis, uint32_t ray)
+{
+    if (!own_times(p)) return;
+    const float u = p.fr.rt[ray] / (float)p.fr.period_T;
+    const int nb = p.n1 > p.n2 ? p.n1 : p.n2;
+    for (int i = 0; i < nb; ++i) const_cast<float *>(basis.at)[i * basis.stride] = basis_fp32(i, u);
+}
 
 // The last warp of the grid to finish resets the tile counter for the next
 // launch (every warp has made its final grab before counting itself).
@@ -1053,13 +1140,15 @@ __device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
 #ifndef FPO_TRAV_MAXNREG_ALONE
 #define FPO_TRAV_MAXNREG_ALONE 80
 #endif
-template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS>
+template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS, int N1 = 0, int N2 = 0>
 __global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ TraverseParams p)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int stride = blockDim.x;
     const int lane = threadIdx.x & 31;
     uint32_t *my_stack = BRICK ? nullptr : smem + threadIdx.x;
+    Basis basis = {nullptr, 0};
+    if constexpr (TM == TM_RECORDS) basis = lane_basis(p, smem + (BRICK ? 0 : STACK_LEVELS * stride));
 
     auto grab_tile = [&]() -> uint32_t {
         uint32_t tl = 0;
@@ -1085,7 +1174,8 @@ __global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ Traver
             if (tile_ray(p, tile, (uint32_t)lane, ray, px, py)) {
                 RayState R;
                 if (init_ray_geom(p, my_stack, R, ray, px, py)) {
-                    trace_ray<TM, DBG, BRICK>(p, my_stack, stride, R);
+                    if constexpr (TM == TM_RECORDS) set_lane_basis(p, basis, ray);
+                    trace_ray<TM, DBG, BRICK, N1, N2>(p, basis, my_stack, stride, R);
                     finish(R);
                 } else {
                     write_result(p, R, DBG);  // misses the tree: background
@@ -1134,7 +1224,7 @@ __global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ Traver
             if (active) {
 #pragma unroll 1
                 for (uint32_t k = 0; k < p.inner_steps; ++k) {
-                    if (!pipelined_step<TM, DBG, BRICK>(p, my_stack, stride, R, cb)) {
+                    if (!pipelined_step<TM, DBG, BRICK, N1, N2>(p, basis, my_stack, stride, R, cb)) {
                         finish(R);
                         active = false;
                         break;
@@ -1147,22 +1237,29 @@ __global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ Traver
 }
 
 int traverse_smem_bytes(bool brick, int threads) { return brick ? 0 : STACK_LEVELS * threads * 4; }
+// ... and of the kernels that read the records: the lanes' bases, or the call's
+static int lane_smem_bytes(const TraverseParams &p, int threads)
+{
+    const bool own = p.fr.mode == FPO_RAYS_EXPLICIT && p.fr.rt != nullptr;
+    return traverse_smem_bytes(p.top != nullptr, threads) + MAX_BASIS * 4 * (own ? threads : 1);
+}
 
-template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS>
+template <int TM, bool DBG, bool COMPACT, bool BRICK, int REGS, int N1 = 0, int N2 = 0>
 static int launch_t(const TraverseParams &p, int sm_count, cudaStream_t s)
 {
     // Few tiles: one-warp CTAs, all resident at once, so that the hardware
     // deals them out evenly (64 CTAs of 8 warps put the 512 tiles of a 128x128
     // frame on 64 of the 152 SMs).
-    auto k = traverse_kernel<TM, DBG, COMPACT, BRICK, REGS>;
+    auto k = traverse_kernel<TM, DBG, COMPACT, BRICK, REGS, N1, N2>;
     if (p.few_tiles_split && p.n_tiles < 32u * (uint32_t)sm_count) {
         // (within the default shared memory: nothing to set or to ask for)
-        k<<<p.n_tiles ? p.n_tiles : 1u, 32, traverse_smem_bytes(BRICK, 32), s>>>(p);
+        k<<<p.n_tiles ? p.n_tiles : 1u, 32, TM == TM_RECORDS ? lane_smem_bytes(p, 32) : traverse_smem_bytes(BRICK, 32), s>>>(p);
         return (int)cudaGetLastError();
     }
     const int threads = p.block_threads;
-    const int smem = traverse_smem_bytes(BRICK, threads);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = TM == TM_RECORDS ? lane_smem_bytes(p, threads) : traverse_smem_bytes(BRICK, threads);
+    // (never below the 48 KB that a launch may use without asking)
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem > 48 * 1024 ? smem : 48 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  p.carveout > 0 ? p.carveout : (int)cudaSharedmemCarveoutDefault);
@@ -1197,8 +1294,9 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 }
 
 // ---------------------------------------------------------------------------
-// Per-visit IDFT (FUSED mode: rays with per-ray times, and frames on request)
-// and its adjoint (Sec. 4.3: back-propagation through the IDFT).
+// Per-visit IDFT (FUSED mode: rays with per-ray times, and frames on request;
+// large calls on small trees and whole images take one lane a ray instead, see
+// lane_per_ray) and its adjoint (Sec. 4.3: back-propagation through the IDFT).
 //
 // A warp owns R rays (lanes 0..R-1) and alternates between four phases, so
 // that the walk, which few lanes of incoherent rays need at the same time, and
@@ -1653,6 +1751,163 @@ static int launch_fused_n(const BackwardParams &q, int sm_count, cudaStream_t s)
     return -1;
 }
 
+// A call of the fused mode with one lane a ray (lane_per_ray).  Bound by the
+// records' trips through L1 and by their 166 multiplications a visit, where the
+// warps' way is bound by instructions: it spreads each visit over four lanes
+// also when the 32 rays of a warp read one record.
+constexpr int LANE_REGS = 128;
+template <bool DBG, int N1, int N2>
+static int launch_lane_t(const TraverseParams &p, int sm_count, cudaStream_t s)
+{
+    return p.top ? launch_t<TM_RECORDS, DBG, false, true, LANE_REGS, N1, N2>(p, sm_count, s)
+                 : launch_t<TM_RECORDS, DBG, false, false, LANE_REGS, N1, N2>(p, sm_count, s);
+}
+template <bool DBG>
+static int launch_lane(const TraverseParams &p, int sm_count, cudaStream_t s)
+{
+    if (p.n1 == 31 && p.n2 == 5) return launch_lane_t<DBG, 31, 5>(p, sm_count, s);
+    if (p.n1 == 11 && p.n2 == 5) return launch_lane_t<DBG, 11, 5>(p, sm_count, s);
+    if (p.n1 == 21 && p.n2 == 5) return launch_lane_t<DBG, 21, 5>(p, sm_count, s);
+    if (p.n1 == 31 && p.n2 == 11) return launch_lane_t<DBG, 31, 11>(p, sm_count, s);
+    return -1;
+}
+
+// The adjoint of such a call: each ray is replayed and every visit's gradient
+// row added with 16-byte vector atomics (one 8-byte atomic at an unaligned end).
+// The same stepping and arithmetic as its forward, so the same early stop.
+// 800x800 camera frame, against the warps' adds: 2,252 leaves 511 -> 421 us,
+// 41,929 966 -> 665, 348,592 2695 -> 1952, 3.5M 8344 -> 5726.
+template <int N1, int N2, bool BRICK>
+__device__ void lane_adjoint_ray(const BackwardParams &q, Basis b, uint32_t *s_stack, int stride, RayState &R)
+{
+    constexpr int NC = N1 + 27 * N2;
+    static_assert(NC % 2 == 0, "gradient rows are written in pairs");
+    const TraverseParams &p = q.tp;
+    const int G = 1 << p.depth;
+    const float g0 = q.dL_drgb[3 * (size_t)R.ray], g1 = q.dL_drgb[3 * (size_t)R.ray + 1], g2 = q.dL_drgb[3 * (size_t)R.ray + 2];
+    const float Cf0 = q.out_rgb[3 * (size_t)R.ray], Cf1 = q.out_rgb[3 * (size_t)R.ray + 1], Cf2 = q.out_rgb[3 * (size_t)R.ray + 2];
+    Cube cb = locate<BRICK>(p, s_stack, stride, R, R.P, first_diff(p));
+    for (;;) {
+        int m, lo[3], Pn[3];
+        const float tx = cube_exit(R, cb.csz, m, lo);
+        const bool inside = next_cell(R, G, m, lo, cb.csz, tx, Pn);
+        Cube nx;
+        nx.kind = ROOT_EMPTY;
+        if (inside) {
+            nx = locate<BRICK>(p, s_stack, stride, R, Pn, cell_diff(R.P, Pn));
+            if (nx.kind == ROOT_LEAF) prefetch_records(p, nx.leaf);
+        }
+        if (cb.kind == ROOT_LEAF && tx > R.t) {
+            const float delta = tx - R.t;
+            float sraw, z[27], col[3];
+            record_values<N1, N2>(p, b, cb.leaf, sraw, z);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float u = 0.0f;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) u = fmaf(z[9 * c + k], R.Y[k], u);
+                col[c] = sigmoidf_(u);
+            }
+            const float e = __expf(-fmaxf(sraw, 0.0f) * delta);
+            const float w = R.T * (1.0f - e), Tn = R.T * e;
+            R.C0 = fmaf(w, col[0], R.C0);
+            R.C1 = fmaf(w, col[1], R.C1);
+            R.C2 = fmaf(w, col[2], R.C2);
+            const float gs = delta * (g0 * (Tn * col[0] - (Cf0 - R.C0)) + g1 * (Tn * col[1] - (Cf1 - R.C1)) +
+                                      g2 * (Tn * col[2] - (Cf2 - R.C2)));
+            const float dsr = sraw > 0.0f ? gs : 0.0f;
+            const float gu[3] = {g0 * w * col[0] * (1.0f - col[0]), g1 * w * col[1] * (1.0f - col[1]),
+                                 g2 * w * col[2] * (1.0f - col[2])};
+            const uint32_t id = p.perm[cb.leaf];
+            float *row = q.dL_dcoeffs + (size_t)id * NC;
+            if (q.leaf_mark) q.leaf_mark[id] = 1;
+            auto gval = [&](int el) -> float {  // element el of the row (a constant)
+                if (el < N1) return dsr * b[el];
+                const int j = el - N1, c = j / (9 * N2), k = (j / N2) % 9, i = j % N2;
+                return gu[c] * R.Y[k] * b[i];
+            };
+            // a row that starts 8 bytes past a 16-byte boundary (NC = 2 mod 4,
+            // odd id) opens with one 8-byte atomic
+            if (NC % 4 == 0 || (id & 1u) == 0u) {
+#pragma unroll
+                for (int e4 = 0; e4 < NC / 4; ++e4)
+                    atomicAdd(reinterpret_cast<float4 *>(row) + e4,
+                              make_float4(gval(4 * e4), gval(4 * e4 + 1), gval(4 * e4 + 2), gval(4 * e4 + 3)));
+                if constexpr (NC % 4 == 2)
+                    atomicAdd(reinterpret_cast<float2 *>(row + NC - 2), make_float2(gval(NC - 2), gval(NC - 1)));
+            } else {
+                atomicAdd(reinterpret_cast<float2 *>(row), make_float2(gval(0), gval(1)));
+#pragma unroll
+                for (int e4 = 0; e4 < NC / 4; ++e4)
+                    atomicAdd(reinterpret_cast<float4 *>(row + 2) + e4,
+                              make_float4(gval(2 + 4 * e4), gval(3 + 4 * e4), gval(4 + 4 * e4), gval(5 + 4 * e4)));
+            }
+            R.T = Tn;
+            if (R.T < p.stop_T) return;
+        }
+        if (!inside) return;
+        move_to(R, Pn, tx);
+        if (step_cap(p, R)) return;
+        cb = nx;
+    }
+}
+
+template <int N1, int N2, bool BRICK>
+__global__ void __maxnreg__(LANE_REGS) lane_adjoint_kernel(const __grid_constant__ BackwardParams q)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const TraverseParams &p = q.tp;
+    const int lane = threadIdx.x & 31;
+    uint32_t *my_stack = BRICK ? nullptr : smem + threadIdx.x;
+    const Basis basis = lane_basis(p, smem + (BRICK ? 0 : STACK_LEVELS * blockDim.x));
+    for (;;) {
+        uint32_t tile = 0;
+        if (lane == 0) tile = atomicAdd(p.tiles, 1u);
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+        if (tile >= p.n_tiles) break;
+        uint32_t ray;
+        int px = 0, py = 0;
+        RayState R;
+        if (tile_ray(p, tile, (uint32_t)lane, ray, px, py) && init_ray_geom(p, my_stack, R, ray, px, py)) {
+            set_lane_basis(p, basis, ray);
+            lane_adjoint_ray<N1, N2, BRICK>(q, basis, my_stack, blockDim.x, R);
+        }
+        __syncwarp();
+    }
+    finish_tiles(p, lane);
+}
+
+template <int N1, int N2, bool BRICK>
+static int launch_lane_adjoint_t(const BackwardParams &q, int sm_count, cudaStream_t s)
+{
+    const TraverseParams &p = q.tp;
+    const int threads = 128;
+    const int smem = lane_smem_bytes(p, threads);
+    auto k = lane_adjoint_kernel<N1, N2, BRICK>;
+    int per_sm = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
+    if (e != cudaSuccess) return (int)e;
+    if (per_sm < 1) per_sm = 1;
+    uint64_t blocks = (uint64_t)sm_count * per_sm;
+    const uint64_t need = (p.n_tiles + (threads / 32) - 1) / (threads / 32);
+    if (need < blocks) blocks = need ? need : 1;
+    k<<<(unsigned)blocks, threads, smem, s>>>(q);
+    return (int)cudaGetLastError();
+}
+static int launch_lane_adjoint(const BackwardParams &q, int sm_count, cudaStream_t s)
+{
+    const int n1 = q.tp.n1, n2 = q.tp.n2;
+    auto go = [&](auto a, auto b) {
+        return q.tp.top ? launch_lane_adjoint_t<a.value, b.value, true>(q, sm_count, s)
+                        : launch_lane_adjoint_t<a.value, b.value, false>(q, sm_count, s);
+    };
+    if (n1 == 31 && n2 == 5) return go(std::integral_constant<int, 31>(), std::integral_constant<int, 5>());
+    if (n1 == 11 && n2 == 5) return go(std::integral_constant<int, 11>(), std::integral_constant<int, 5>());
+    if (n1 == 21 && n2 == 5) return go(std::integral_constant<int, 21>(), std::integral_constant<int, 5>());
+    if (n1 == 31 && n2 == 11) return go(std::integral_constant<int, 31>(), std::integral_constant<int, 11>());
+    return -1;
+}
+
 template <bool ADJ, bool DBG>
 static int launch_fused(const BackwardParams &q, int sm_count, cudaStream_t s)
 {
@@ -1672,6 +1927,7 @@ int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int 
     if (materialised)
         return p.half_table ? launch_sched<TM_TABLE_F16>(p, debug, sm_count, s)
                             : launch_sched<TM_TABLE_F32>(p, debug, sm_count, s);
+    if (p.lanes) return debug ? launch_lane<true>(p, sm_count, s) : launch_lane<false>(p, sm_count, s);
     BackwardParams q{};
     q.tp = p;
     return debug ? launch_fused<false, true>(q, sm_count, s) : launch_fused<false, false>(q, sm_count, s);
@@ -1890,6 +2146,7 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(const VisitList list,
     constexpr int NZ = 9 * N2, NC = N1 + 27 * N2, RN = (NC + 63) / 64;
     const int lane = threadIdx.x & 31;
     const uint32_t n = min(list.count[OVER ? 2 : 0], list.cap);
+    if (OVER && n == 0) return;
     const uint32_t warps = gridDim.x * blockDim.x / 32;
     // the weight and value index of this lane's elements
     int wi[2 * RN], ci[2 * RN];
@@ -1961,6 +2218,7 @@ int launch_grad_scatter_over(const VisitList &list, int n1, int n2, float *grad,
 int launch_backward(const BackwardParams &q, int sm_count, void *stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
+    if (q.dL_dcoeffs64 == nullptr && q.tp.lanes) return launch_lane_adjoint(q, sm_count, s);
     if (q.dL_dcoeffs64 == nullptr) return launch_fused<true, false>(q, sm_count, s);
     const int n1 = q.tp.n1, n2 = q.tp.n2;
     if (n1 == 31 && n2 == 5) return launch_b64<31, 5>(q, sm_count, s);

@@ -320,7 +320,7 @@ def test_grids_asked_for_and_not():
     r.upload(tree)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     rng = np.random.default_rng(4)
-    n = 40 * sms * 32
+    n = 16 * sms * 32  # (fewer than take one lane a ray)
     o = rng.uniform(-0.6, 1.6, (n, 3))
     dev = lambda x: torch.as_tensor(x, dtype=torch.float32, device="cuda")
     o, d, t = dev(o), dev(rng.uniform(0.2, 0.8, (n, 3)) - o), dev(rng.uniform(0, 60, n))

@@ -1,0 +1,115 @@
+"""The fused mode's two ways, a warp evaluating its visits together and one lane
+a ray (large calls on small trees, whole images), against each other."""
+
+import numpy as np
+import pytest
+
+from paper_2202_08614_gb300 import fpo, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+LANES = 1 << 17  # rays from which a tree of fewer than 2^15 leaves takes one lane a ray
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+
+    __graft_entry__.build()
+
+
+def _rays(n, seed):
+    rng = np.random.default_rng(seed)
+    dev = lambda x: torch.as_tensor(x, dtype=torch.float32, device="cuda")
+    o = rng.uniform(-0.6, 1.6, (n, 3))
+    return dev(o), dev(rng.uniform(0.2, 0.8, (n, 3)) - o), dev(rng.uniform(0, 60, n)), dev(rng.normal(size=(n, 3)))
+
+
+def _close_grad(a, b, visits):
+    # FP32 sums of up to `visits` visits a leaf in another order, as a random walk
+    # of roundings: sqrt(visits) * 2^-24 of a sum of |terms| that is up to some
+    # ten times the largest element
+    tol = 40 * visits ** 0.5 * 2.0 ** -24
+    assert float(b.abs().max()) > 0 and float((a - b).abs().max()) <= tol * float(b.abs().max())
+
+
+def _tree(kind, n1, n2):
+    return synth.shell_tree(4, 5, n1, n2) if kind == "bricks" else synth.random_tree(11, max_depth=5, n1=n1, n2=n2)
+
+
+@pytest.mark.parametrize("n1,n2", [(31, 5), (11, 5), (21, 5), (31, 11)])
+@pytest.mark.parametrize("kind", ["bricks", "octree"])
+@pytest.mark.parametrize("own", [True, False])
+def test_lanes_equal_warps(n1, n2, kind, own):
+    tree = _tree(kind, n1, n2)
+    r = fpo.Renderer(n1=n1, n2=n2, idft_mode="fused")
+    r.upload(tree)
+    n = LANES + 33
+    o, d, t, g = _rays(n, n1 + n2)
+    d[:9] = torch.eye(3, device="cuda").repeat(3, 1)  # axis-parallel
+    args = lambda s: dict(rays_o=o[s], rays_d=d[s], t_per_ray=t[s] if own else None, t=7.0)
+    whole = slice(0, n)
+    stats = [torch.zeros(3, dtype=torch.int64, device="cuda") for _ in range(2)]
+    marks = [torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    a = r.render(**args(whole), visit_cap=96, want_T=True, leaf_mark=marks[0], stats=stats[0])
+    plain = r.render(**args(whole))["rgb"]
+    assert torch.equal(plain, a["rgb"])
+    ga, gb = (torch.zeros(tree.coeffs.shape, device="cuda") for _ in range(2))
+    r.render_backward(a["rgb"], g, ga, **args(whole), leaf_mark=marks[2])
+    cuts = [0, 1, n // 2, n - 31, n]
+    for lo, hi in zip(cuts[:-1], cuts[1:]):
+        s = slice(lo, hi)
+        b = r.render(**args(s), visit_cap=96, want_T=True, leaf_mark=marks[1], stats=stats[1])
+        # the same walk; sums of n1 and 27 n2 products in another order, and their
+        # sigmoids and exponentials along at most 96 visits
+        assert float((a["rgb"][s] - b["rgb"]).abs().max()) <= 2e-5
+        assert float((a["T"][s] - b["T"]).abs().max()) <= 2e-5
+        # (a transmittance at stop_T to within that may stop a visit apart)
+        same = (a["visit_count"][s] == b["visit_count"]) & (a["visit_log"][s] == b["visit_log"]).all(1)
+        assert int((~same).sum()) <= 3 + n // 20000
+        r.render_backward(b["rgb"], g[s].contiguous(), gb, **args(s), leaf_mark=marks[3])
+    r.status()
+    r.close()
+    assert torch.equal(stats[0][2:], stats[1][2:]) and int(stats[0][1]) > n
+    assert int((marks[0] != marks[1]).sum()) <= 1 and int((marks[2] != marks[3]).sum()) <= 1
+    assert torch.equal(marks[0], marks[2])
+    _close_grad(ga, gb, 4 * n / tree.n_leaves + 1000)
+
+
+def _camera_rows(cam, y0, y1):
+    """Rows y0 .. y1 of a camera as explicit rays."""
+    from test_grad_gpu import camera_rays
+
+    o, d = camera_rays(cam)
+    s = slice(y0 * cam.width, y1 * cam.width)
+    dev = lambda x: torch.as_tensor(x[s], dtype=torch.float32, device="cuda")
+    return dict(rays_o=dev(o), rays_d=dev(d))
+
+
+@pytest.mark.parametrize("w,h", [(512, 257), (1, 131072), (32769, 4)])
+def test_lanes_of_a_camera_frame(w, h):
+    tree = synth.shell_tree(6)
+    cam = synth.shell_camera(w, h)
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    img = r.render(camera=cam, t=11.0)["rgb"]
+    table = fpo.Renderer()
+    table.upload(tree)
+    assert float((img - table.render(camera=cam, t=11.0)["rgb"]).abs().max()) <= 2e-5
+    g = torch.randn(img.shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    a, b = (torch.zeros(tree.coeffs.shape, device="cuda") for _ in range(2))
+    r.render_backward(img, g, a, camera=cam, t=11.0)
+    for y in range(0, h, max(1, h // 3)):
+        y1 = min(h, y + max(1, h // 3))
+        s = slice(y * w, y1 * w)
+        r.render_backward(img[s].contiguous(), g[s].contiguous(), b, t=11.0, **_camera_rows(cam, y, y1))
+    r.status()
+    r.close()
+    table.close()
+    # (the explicit rays are rounded from the camera's FP64 frame: 2^-24 of a
+    # coordinate moves a segment's ends by as much of a cell)
+    assert float(a.abs().max()) > 0 and float((a - b).abs().max()) <= 2e-3 * float(a.abs().max())
