@@ -522,15 +522,17 @@ static void frame_consts(const FrameParams &fr, int nb, FrameConsts &c)
 }
 
 // Kernel parameters of one render (or adjoint) call from the context, rays
-// and options.
+// and options; of a camera frame, n_rays rays from row y0 on.
 TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
-                               float *out_rgb, uint64_t n_rays)
+                               float *out_rgb, uint64_t n_rays, uint32_t y0)
 {
     const uint32_t fl = opts->flags;
     TraverseParams p{};
     p.fr.mode = rays->mode;
     p.fr.width = rays->width;
     p.fr.height = rays->height;
+    p.fr.y0 = y0;
+    p.fr.rows = rays->mode == FPO_RAYS_CAMERA && rays->width ? (uint32_t)(n_rays / rays->width) : 0;
     p.fr.n_rays = (uint32_t)n_rays;
     for (int k = 0; k < 3; ++k) {
         p.fr.eye[k] = rays->eye[k];
@@ -578,7 +580,7 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
     p.half_table = ctx->half_table;
     if (rays->mode == FPO_RAYS_CAMERA) {
         p.tiles_x = (rays->width + TILE_W - 1) / TILE_W;
-        const uint32_t tiles_y = (rays->height + TILE_H - 1) / TILE_H;
+        const uint32_t tiles_y = (p.fr.rows + TILE_H - 1) / TILE_H;
         p.n_tiles = p.tiles_x * tiles_y;
     } else {
         p.tiles_x = 0;
@@ -1006,14 +1008,38 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     q.dL_dcoeffs = fp64 ? nullptr : dL_dcoeffs;
     q.dL_dcoeffs64 = fp64 ? reinterpret_cast<double *>(dL_dcoeffs) : nullptr;
     q.leaf_mark = mark ? opts->leaf_mark : nullptr;
-    if (!fp64 && !q.tp.lanes) q.list = visit_list(ctx, n_rays, defer, (cudaStream_t)cuda_stream);
-    int ce = launch_backward(q, ctx->sm_count, cuda_stream);
-    if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
-    if (q.list.slot) {
-        ctx->vl_used += (uint32_t)n_rays;
-    } else if (q.list.cap) {
-        ce = launch_grad_scatter(q, ctx->sm_count, cuda_stream);
-        if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "gradient scatter launch");
+    // A batch larger than the list holds goes in equal parts, each with its
+    // pass over the list (whole 32-ray groups, or whole rows of tiles).
+    const bool camera = rays->mode == FPO_RAYS_CAMERA;
+    const uint64_t parts = (n_rays + VL_MAX_RAYS - 1) / VL_MAX_RAYS;
+    const uint64_t unit = camera ? (uint64_t)TILE_H * rays->width : 32;  // rays
+    uint64_t step = ((n_rays + parts - 1) / parts + unit - 1) / unit * unit;
+    if (parts > 1 && step > VL_MAX_RAYS) step = VL_MAX_RAYS / unit * unit;
+    if (!fp64 && !q.tp.lanes && step) q.list = visit_list(ctx, step < n_rays ? step : n_rays, defer && parts == 1, (cudaStream_t)cuda_stream);
+    if (!q.list.cap) step = n_rays;
+    for (uint64_t at = 0; at < n_rays; at += step) {
+        const uint64_t n = n_rays - at < step ? n_rays - at : step;
+        if (n < n_rays) {
+            fpo_rays part = *rays;
+            if (!camera) {
+                part.n = (uint32_t)n;
+                part.o = rays->o + 3 * at;
+                part.d = rays->d + 3 * at;
+                part.t_per_ray = rays->t_per_ray ? rays->t_per_ray + at : nullptr;
+            }
+            q.tp = traverse_params(ctx, &part, &o, nullptr, n, (uint32_t)(camera ? at / rays->width : 0));
+            q.tp.lanes = false;
+            q.out_rgb = out_rgb + 3 * at;
+            q.dL_drgb = dL_drgb + 3 * at;
+        }
+        int ce = launch_backward(q, ctx->sm_count, cuda_stream);
+        if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
+        if (q.list.slot) {
+            ctx->vl_used += (uint32_t)n_rays;
+        } else if (q.list.cap) {
+            ce = launch_grad_scatter(q, ctx->sm_count, cuda_stream);
+            if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "gradient scatter launch");
+        }
     }
     return FPO_OK;
 }

@@ -123,6 +123,7 @@ int validate_and_pack(const fpo_tree_desc *tree, int n1, int n2, PackedTree *out
 struct FrameParams {
     int mode;                 // FPO_RAYS_*
     uint32_t width, height, n_rays;
+    uint32_t y0, rows;        // camera: the rows of this launch, y0 .. y0 + rows - 1 (its rays are numbered from 0)
     double eye[3], target[3], up[3];
     double fov_y_deg;
     double t, period_T;
@@ -197,10 +198,11 @@ __host__ __device__ __forceinline__ bool tile_ray(const TraverseParams &p, uint3
         // row-major tiles: the tiles in flight form one band of rows, whose
         // table lines stay in L2
         const uint32_t tx = tile % p.tiles_x, ty = tile / p.tiles_x;
+        const uint32_t row = ty * TILE_H + k / TILE_W;
         px = (int)(tx * TILE_W + k % TILE_W);
-        py = (int)(ty * TILE_H + k / TILE_W);
-        ray = (uint32_t)py * p.fr.width + (uint32_t)px;
-        return px < (int)p.fr.width && py < (int)p.fr.height;
+        py = (int)(p.fr.y0 + row);
+        ray = row * p.fr.width + (uint32_t)px;
+        return px < (int)p.fr.width && row < p.fr.rows;
     }
     ray = tile * 32 + k;
     return ray < p.fr.n_rays;
@@ -222,7 +224,7 @@ __host__ __device__ __forceinline__ bool slot_ray(const TraverseParams &p, uint3
     if (p.fr.mode != FPO_RAYS_CAMERA || p.tiles_x) return tile_ray(p, slot >> 5, slot & 31u, ray, px, py);
     ray = slot;
     px = (int)(slot % p.fr.width);
-    py = (int)(slot / p.fr.width);
+    py = (int)(p.fr.y0 + slot / p.fr.width);
     return slot < p.fr.n_rays;
 }
 
@@ -273,7 +275,7 @@ int check_render_opts(const fpo_ctx *ctx, const fpo_frame_opts *opts, uint64_t n
 // Kernel parameters of one render (or adjoint) call; p.table is the context's
 // own per-frame table, which a caller may point elsewhere.
 TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
-                               float *out_rgb, uint64_t n_rays);
+                               float *out_rgb, uint64_t n_rays, uint32_t y0 = 0);
 // The per-frame table for time t into `table` on `stream`: the tensor-core
 // decoder for LATENT storage, else the IDFT pass over the stored coefficients
 // (at most max_ctas_per_sm CTAs per SM when > 0; with pipe_stages > 0 the

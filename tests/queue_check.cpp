@@ -16,7 +16,7 @@ int main(int argc, char **argv)
     TraverseParams p{};
     p.fr.mode = FPO_RAYS_CAMERA;
     p.fr.width = (uint32_t)W;
-    p.fr.height = (uint32_t)H;
+    p.fr.height = p.fr.rows = (uint32_t)H;
     p.fr.n_rays = (uint32_t)(W * H);
     p.tiles_x = (uint32_t)((W + TILE_W - 1) / TILE_W);
     const uint64_t tx = p.tiles_x;

@@ -1,5 +1,6 @@
 """The fused mode's two ways, a warp evaluating its visits together and one lane
-a ray (large calls on small trees, whole images), against each other."""
+a ray (large calls on small trees, whole images), against each other, and the
+adjoint of batches larger than its list against that of their parts."""
 
 import numpy as np
 import pytest
@@ -113,3 +114,52 @@ def test_lanes_of_a_camera_frame(w, h):
     # (the explicit rays are rounded from the camera's FP64 frame: 2^-24 of a
     # coordinate moves a segment's ends by as much of a cell)
     assert float(a.abs().max()) > 0 and float((a - b).abs().max()) <= 2e-3 * float(a.abs().max())
+
+
+@pytest.fixture(scope="module")
+def big():
+    """A tree of 2^17 leaves and more: batches past the list's 2^18 rays go in parts."""
+    k = np.arange(52 ** 3)
+    xyz = (6 + np.stack([k % 52, k // 52 % 52, k // 52 ** 2], 1)).astype(np.uint32)
+    rng = np.random.default_rng(2)
+    c = rng.normal(size=(len(xyz), 146)).astype(np.float32) * 0.1
+    c[:, 0] = 10.0
+    tree = synth.Tree(np.full(len(xyz), 6, np.uint8), xyz, c, 6, 11, 5)
+    r = fpo.Renderer(n1=11, n2=5, idft_mode="fused")
+    r.upload(tree)
+    yield tree, r
+    r.close()
+
+
+@pytest.mark.parametrize("n", [(1 << 18) + 1, 500_001])
+def test_large_batches_in_parts(big, n):
+    tree, r = big
+    o, d, t, g = _rays(n, 9)
+    rgb = r.render(rays_o=o, rays_d=d, t_per_ray=t)["rgb"]
+    a, b = (torch.zeros(tree.coeffs.shape, device="cuda") for _ in range(2))
+    ma, mb = (torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda") for _ in range(2))
+    r.render_backward(rgb, g, a, rays_o=o, rays_d=d, t_per_ray=t, leaf_mark=ma, defer=True)
+    for at in range(0, n, 100_000):
+        s = slice(at, min(n, at + 100_000))
+        r.render_backward(rgb[s].contiguous(), g[s].contiguous(), b, rays_o=o[s], rays_d=d[s], t_per_ray=t[s], leaf_mark=mb)
+    r.status()
+    assert torch.equal(ma, mb)
+    _close_grad(a, b, 60 * n / tree.n_leaves + 500)
+
+
+# (a row of tiles of the last is more than the list holds: no parts)
+@pytest.mark.parametrize("w,h,fov", [(640, 480, 40.0), (333, 1001, 40.0), (40000, 7, 0.01)])
+def test_camera_adjoint_in_parts(big, w, h, fov):
+    tree, r = big
+    cam = synth.Camera(eye=(2.2, 0.7, 0.9), width=w, height=h, fov_y_deg=fov)
+    img = r.render(camera=cam, t=5.0)["rgb"]
+    g = torch.randn(img.shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(2))
+    a = torch.zeros(tree.coeffs.shape, device="cuda")
+    r.render_backward(img, g, a, camera=cam, t=5.0)
+    # the FP64 replay takes the frame whole
+    b64 = torch.zeros(tree.coeffs.shape, dtype=torch.float64, device="cuda")
+    r.render_backward(img, g, b64, camera=cam, t=5.0, fp64=True)
+    r.status()
+    assert float(b64.abs().max()) > 0
+    # norm-wise, as the FP32 adjoint against the oracle's
+    assert float((a.double() - b64).norm() / b64.norm()) <= 2e-4
