@@ -280,9 +280,9 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * gradient), which fpo_adam_leaves consumes; the others are ignored.
  * FPO_FLAG_FP64_GRADCHECK selects the FP64 replay, FPO_FLAG_DEFER_GRADIENT
  * leaves the gradient to the next fpo_adam_leaves (see the flags).
- * A call keeps its visits in a workspace of the context (up to 4,096 rays
- * 5 MB of what fpo_upload_tree allocates, grown on the first larger batch, at
- * most 0.4 GB) and adds them to dL_dcoeffs in a second, evenly divided pass;
+ * A call keeps its visits in a workspace of the context (up to 4,096 rays,
+ * on trees of 2 MB of SH records and more, 5 MB of what fpo_upload_tree
+ * allocates; else allocated, and grown on the first larger batch, at most 0.4 GB) and adds them to dL_dcoeffs in a second, evenly divided pass;
  * more than 262,144 rays go in equal parts.  Calls under stream capture (a
  * graph holds nothing of the workspace), large calls on small trees and whole
  * images (131,072 rays or more; by one lane a ray, as fpo_render renders
