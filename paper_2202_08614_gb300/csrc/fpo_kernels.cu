@@ -1320,9 +1320,9 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 //              contiguous 8-byte vector atomics (a row a visit: added from
 //              here, the rows of the rays that run longest came last and
 //              alone).
-// The one-lane-per-ray form that this replaces read 21 scattered 32-byte
-// pieces per visit in each lane, with the whole warp waiting for the few
-// lanes that were inside a leaf, and left most SMs idle below 38,912 rays.
+// With one lane a ray, incoherent rays read 21 scattered 32-byte pieces per
+// visit in each lane, the whole warp waiting for the few lanes that are inside
+// a leaf, and most SMs are idle below 38,912 rays.
 //
 // Adjoint: with w_j = T_j alpha_j and C the forward colour (which includes
 // T_end bg), S_j = C - sum_{k<=j} w_k c_k is the colour behind segment j and

@@ -6,7 +6,8 @@ One step on a batch of explicit rays with per-ray frame times:
   loss      mean over rays of the squared RGB error, dL/drgb = 2 (rgb - y) / B,
   adjoint   fpo_render_backward, which leaves the gradient in the renderer as a
             list of leaf visits (and takes the dense gradient buffer and the
-            marks for visits beyond the list),
+            marks for visits beyond the list, and for batches of more rays than
+            the tree has leaves),
   update    fpo_adam_leaves: Adam on the visited leaves' rows only, written
             straight into the renderer's FP32 records; lists, gradient rows and
             marks are reset in the same pass.
