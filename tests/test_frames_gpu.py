@@ -179,7 +179,10 @@ def test_frames_take_fewer_slots_when_six_tables_do_not_fit():
     table = n * 64
     filler = None
     try:
-        filler = torch.empty(torch.cuda.mem_get_info()[0] - int(3.2 * table), dtype=torch.uint8, device="cuda")
+        try:
+            filler = torch.empty(torch.cuda.mem_get_info()[0] - int(3.2 * table), dtype=torch.uint8, device="cuda")
+        except torch.cuda.OutOfMemoryError:
+            pytest.skip("the rest of the device's memory is not to be had in one piece")
         for _ in range(2):
             r.render_frames(cams, times, out=out)
             r.status()
