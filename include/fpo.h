@@ -286,7 +286,8 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * more than 262,144 rays go in equal parts.  Calls under stream capture (a
  * graph holds nothing of the workspace), large calls on small trees and whole
  * images (131,072 rays or more; by one lane a ray, as fpo_render renders
- * them), and visits beyond the workspace are added from the replay.
+ * them), and visits beyond the workspace are added from the replay (of 65,536
+ * rays or more without a workspace by one lane a ray, too).
  * Errors: INVALID_ARG, NO_TREE, UNSUPPORTED, CUDA. */
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,
                         const float *out_rgb, const float *dL_drgb, float *dL_dcoeffs,

@@ -882,6 +882,15 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames, c
 
 namespace {
 
+// Rays from which an adjoint without a list (capture, no memory, other visits
+// waiting) takes one lane a ray: the lanes' adds follow one another where a
+// warp's wait for its longest ray (us, warps / lanes: camera 160x120 308 / 744,
+// 320x240 956 / 781, 480x360 1786 / 938 on 348,592 leaves, 4730 / 2247 on 3.5M;
+// 65,536 explicit rays 490 / 465 and 1155 / 1057, 131,072 946 / 736 and 2313 /
+// 1756).  (A transmittance within rounding of stop_T may then stop a visit apart
+// from a forward by warps.)
+constexpr uint64_t NO_LIST_LANES = 1u << 16;
+
 // Whether work on s goes into a graph (a stream that cannot be asked counts as such).
 bool capturing(cudaStream_t s)
 {
@@ -1018,7 +1027,10 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     uint64_t step = ((n_rays + parts - 1) / parts + unit - 1) / unit * unit;
     if (parts > 1 && step > VL_MAX_RAYS) step = VL_MAX_RAYS / unit * unit;
     if (!fp64 && !q.tp.lanes && step) q.list = visit_list(ctx, step < n_rays ? step : n_rays, defer && parts == 1, (cudaStream_t)cuda_stream);
-    if (!q.list.cap) step = n_rays;
+    if (!q.list.cap) {
+        step = n_rays;
+        q.tp.lanes |= n_rays >= NO_LIST_LANES;
+    }
     for (uint64_t at = 0; at < n_rays; at += step) {
         const uint64_t n = n_rays - at < step ? n_rays - at : step;
         if (n < n_rays) {

@@ -34,7 +34,7 @@ class Batch:
 
 
 def _close(a, b):
-    # FP32 sums of a few hundred visits a leaf in another order: each within
+    # FP32 sums of up to a few hundred visits a leaf in another order: each within
     # 300 * 2^-24 = 2e-5 of its sum of |terms|, itself a few times the largest element
     assert float(b.abs().max()) > 0 and float((a - b).abs().max()) <= 1e-4 * float(b.abs().max())
 
@@ -47,9 +47,10 @@ def _setup():
     return r, p, torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
 
 
-def test_captured_adjoint_outlives_a_larger_call_and_deferred_visits():
+@pytest.mark.parametrize("n", [300, 70000])  # adds by warps, and by one lane a ray
+def test_captured_adjoint_outlives_a_larger_call_and_deferred_visits(n):
     r, p, mark = _setup()
-    a, b, c = Batch(r, 300, 1), Batch(r, 9000, 2), Batch(r, 500, 3)
+    a, b, c = Batch(r, n, 1), Batch(r, n + 9000, 2), Batch(r, 500, 3)
     m, v = torch.zeros_like(p), torch.zeros_like(p)
     want, got, big, pend = (torch.zeros_like(p) for _ in range(4))
     a.backward(r, want)  # the context has its workspace for 4096 rays now
