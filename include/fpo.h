@@ -285,8 +285,7 @@ int fpo_render_frames(fpo_ctx *ctx, const fpo_rays *frames, uint32_t n_frames,
  * allocates; else allocated, and grown on the first larger batch, at most 0.4 GB) and adds them to dL_dcoeffs in a second, evenly divided pass;
  * more than 262,144 rays go in equal parts.  Calls under stream capture (a
  * graph holds nothing of the workspace), large calls on small trees and whole
- * images (131,072 rays or more; by one lane a ray, as fpo_render renders
- * them), and visits beyond the workspace are added from the replay (of 65,536
+ * images (131,072 rays or more; by one lane a ray), and visits beyond the workspace are added from the replay (of 65,536
  * rays or more without a workspace by one lane a ray, too).
  * Errors: INVALID_ARG, NO_TREE, UNSUPPORTED, CUDA. */
 int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts *opts,

@@ -119,6 +119,7 @@ constexpr uint32_t VL_MAX_RAYS = 1u << 18, VL_PER_RAY = 32;
 // the list had gained.
 constexpr uint32_t VL_BASE_RAYS = 4096;
 constexpr int VL_COUNT = 24, VL_COUNTS = 3;
+constexpr int COHERENT_WORD = 28;  // coherence_kernel's answer
 
 }  // namespace
 
@@ -126,8 +127,9 @@ struct fpo_ctx {
     fpo_config cfg{};
     int sm_count = 0;
     // [0] status bits; [1], [2] tile counter and finished warps of a traversal;
-    // [5], [6] the same for the odd frames of fpo_render_frames, whose
-    // traversals run on a second stream and may overlap the even ones
+    // [1 + 2b], [2 + 2b] the same for slot b of fpo_render_frames, whose
+    // traversals run on streams of their own; [24..26] the visit list's counters;
+    // [28] whether a fused call's rays are coherent
     uint32_t *d_status = nullptr;
     // tree
     bool has_tree = false;
@@ -588,7 +590,8 @@ TraverseParams traverse_params(const fpo_ctx *ctx, const fpo_rays *rays, const f
         p.tiles_x = 0;
         p.n_tiles = (uint32_t)((n_rays + 31) / 32);
     }
-    p.lanes = lane_per_ray(rays->mode == FPO_RAYS_CAMERA, n_rays, ctx->n_leaves);
+    p.form = ray_form(rays->mode == FPO_RAYS_CAMERA, n_rays, ctx->n_leaves);
+    p.coherent = p.form == LANES_IF_COHERENT ? ctx->d_status + COHERENT_WORD : nullptr;
     p.max_steps = ctx->cfg.max_steps > 0 ? (uint32_t)ctx->cfg.max_steps : 3u * (1u << ctx->depth) + 16u;
     p.block_threads = ctx->cfg.traverse_threads ? ctx->cfg.traverse_threads : DEFAULT_TRAVERSE_THREADS;
     p.few_tiles_split = ctx->cfg.traverse_threads == 0;
@@ -1026,11 +1029,18 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
     const uint64_t unit = camera ? (uint64_t)TILE_H * rays->width : 32;  // rays
     uint64_t step = ((n_rays + parts - 1) / parts + unit - 1) / unit * unit;
     if (parts > 1 && step > VL_MAX_RAYS) step = VL_MAX_RAYS / unit * unit;
-    if (!fp64 && !q.tp.lanes && step) q.list = visit_list(ctx, step < n_rays ? step : n_rays, defer && parts == 1, (cudaStream_t)cuda_stream);
+    if (!fp64 && q.tp.form != BY_LANES && step) q.list = visit_list(ctx, step < n_rays ? step : n_rays, defer && parts == 1, (cudaStream_t)cuda_stream);
+    const uint32_t *coherent = nullptr;
     if (!q.list.cap) {
         step = n_rays;
-        q.tp.lanes |= n_rays >= NO_LIST_LANES;
+        if (n_rays >= NO_LIST_LANES) q.tp.form = BY_LANES;
+    } else if (q.tp.form == LANES_IF_COHERENT && parts > 1) {
+        coherent = q.tp.coherent;
+        const int ce = launch_backward(q, ctx->sm_count, cuda_stream);
+        if (ce != cudaSuccess) return cuda_fail((cudaError_t)ce, "backward launch");
     }
+    if (q.tp.form == LANES_IF_COHERENT) q.tp.form = BY_WARPS;
+    q.tp.coherent = coherent;
     for (uint64_t at = 0; at < n_rays; at += step) {
         const uint64_t n = n_rays - at < step ? n_rays - at : step;
         if (n < n_rays) {
@@ -1042,7 +1052,8 @@ int fpo_render_backward(fpo_ctx *ctx, const fpo_rays *rays, const fpo_frame_opts
                 part.t_per_ray = rays->t_per_ray ? rays->t_per_ray + at : nullptr;
             }
             q.tp = traverse_params(ctx, &part, &o, nullptr, n, (uint32_t)(camera ? at / rays->width : 0));
-            q.tp.lanes = false;
+            q.tp.form = BY_WARPS;
+            q.tp.coherent = coherent;
             q.out_rgb = out_rgb + 3 * at;
             q.dL_drgb = dL_drgb + 3 * at;
         }

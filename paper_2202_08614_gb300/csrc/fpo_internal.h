@@ -182,7 +182,8 @@ struct TraverseParams {
     uint32_t inner_steps;     // steps a lane takes between two refill checks
     int block_threads;        // 128 or 256
     int few_tiles_split;      // 1: smaller CTAs when there are few tiles (block_threads is not the user's choice)
-    bool lanes;               // fused mode: one lane a ray (lane_per_ray)
+    int form;                 // fused mode: ray_form
+    const uint32_t *coherent; // LANES_IF_COHERENT: coherence_kernel's answer for this call, else nullptr
     int rays_per_warp, list_cap; // fused mode: rays of one warp and length of its visit list (set by the launcher)
     int max_ctas_per_sm;      // 0: as many as fit
     int carveout;             // preferred shared-memory carveout in percent (0: the driver's default)
@@ -396,6 +397,8 @@ struct MatShape {
 };
 MatShape materialise_pipeline_shape(int storage, int n1, int n2, int smem_budget);
 int materialise_smem_bytes(const MaterialiseParams &p);  // dynamic shared memory of one CTA
+// (form LANES_IF_COHERENT: asks, and launches the lanes' kernel only; the parts by
+// warps, with the same `coherent`, are the caller's)
 int launch_backward(const BackwardParams &q, int sm_count, void *stream);
 // Adds the list's visits to q.dL_dcoeffs and empties it.
 int launch_grad_scatter(const BackwardParams &q, int sm_count, void *stream);
@@ -413,24 +416,31 @@ int traverse_smem_bytes(bool brick, int threads);
 // (refill_min < 32, a tuning option) walks the octree of every tree.
 constexpr bool brick_walk(bool has_index, uint32_t refill_min) { return has_index && refill_min >= 32; }
 bool fused_supported(int n1, int n2);
-// Whether the fused mode (and its adjoint) takes a call with one lane a ray,
-// each reading its visits' records by itself, instead of evaluating a warp's
-// visits together: many rays on a small tree, where neighbours read the same
-// records, or whole images.  Lines and start of the table: rays from which
-// the lanes are the faster way for camera frames (the table's first number)
-// and for images given as explicit rays; random explicit rays gain from the
-// warps up to the larger sizes.  Forward, us, warps / lanes:
+// How the fused mode takes a call: by warps that evaluate their visits
+// together, or with one lane a ray, each reading its visits' records by itself.
+// The lanes are the faster way for many rays on a small tree and for whole
+// images, where neighbours read the same records.  Camera frames are images;
+// of explicit rays only their data tell (an image's rays in pixel order, or a
+// random batch), so that large calls look at some of them on the device first
+// (LANES_IF_COHERENT: coherence_kernel, and both forms launched, of which one
+// returns at once: 5 us).  Forward, us, warps / lanes:
 //   leaves       camera 640x400  800x800     1920x1080    image 800x800  random 400k  random 1M
 //   2,252        106 /   70      265 /   97   545 /  150   293 /  130     281 /  254   660 /  574
 //   5,430        111 /   78      267 /   97   545 /  148   294 /  130     271 /  291   636 /  654
 //   41,929       181 /  201      394 /  221   722 /  304   433 /  271     381 /  461   878 / 1036
 //   348,592      341 /  491      599 /  470  1064 /  561   640 /  557     565 / 1114  1278 / 2541
 //   3,506,408    765 / 1216     1347 / 1381  2199 / 1726  1408 / 1473    1068 / 2432  2414 / 5540
-constexpr bool lane_per_ray(bool camera, uint64_t rays, uint32_t n_leaves)
+// (an image of 400x400 explicit rays: 102 / 84, 104 / 94, 172 / 202 on the first
+// three; 512x512: 141 / 91, 139 / 99, 225 / 210, 378 / 529.)
+enum RayForm { BY_WARPS, BY_LANES, LANES_IF_COHERENT };
+constexpr RayForm ray_form(bool camera, uint64_t rays, uint32_t n_leaves)
 {
-    if (n_leaves < (1u << 15)) return rays >= (1u << 17);
-    if (n_leaves < (1u << 17)) return rays >= (1u << 18);
-    return rays >= (camera ? 1u << 19 : 1u << 20);
+    if (n_leaves < 4096) return rays >= (1u << 17) ? BY_LANES : BY_WARPS;
+    if (camera) {
+        const uint64_t least = n_leaves < (1u << 15) ? 1u << 17 : (n_leaves < (1u << 17) ? 1u << 18 : 1u << 19);
+        return rays >= least ? BY_LANES : BY_WARPS;
+    }
+    return rays >= (n_leaves < (1u << 17) ? 3u << 16 : 1u << 20) ? LANES_IF_COHERENT : BY_WARPS;
 }
 
 }  // namespace fpo

@@ -1106,6 +1106,12 @@ __device__ __forceinline__ void set_lane_basis(const TraverseParams &p, Basis ba
     for (int i = 0; i < nb; ++i) const_cast<float *>(basis.at)[i * basis.stride] = basis_fp32(i, u);
 }
 
+// (true for every thread of a launch that leaves the call to the other form)
+__device__ __forceinline__ bool other_form(const TraverseParams &p, bool lanes)
+{
+    return p.coherent != nullptr && (*p.coherent != 0u) != lanes;
+}
+
 // The last warp of the grid to finish resets the tile counter for the next
 // launch (every warp has made its final grab before counting itself).
 __device__ __forceinline__ void finish_tiles(const TraverseParams &p, int lane)
@@ -1148,7 +1154,10 @@ __global__ void __maxnreg__(REGS) traverse_kernel(const __grid_constant__ Traver
     const int lane = threadIdx.x & 31;
     uint32_t *my_stack = BRICK ? nullptr : smem + threadIdx.x;
     Basis basis = {nullptr, 0};
-    if constexpr (TM == TM_RECORDS) basis = lane_basis(p, smem + (BRICK ? 0 : STACK_LEVELS * stride));
+    if constexpr (TM == TM_RECORDS) {
+        if (other_form(p, true)) return;
+        basis = lane_basis(p, smem + (BRICK ? 0 : STACK_LEVELS * stride));
+    }
 
     auto grab_tile = [&]() -> uint32_t {
         uint32_t tl = 0;
@@ -1296,7 +1305,7 @@ static int launch_sched(const TraverseParams &p, bool debug, int sm_count, cudaS
 // ---------------------------------------------------------------------------
 // Per-visit IDFT (FUSED mode: rays with per-ray times, and frames on request;
 // large calls on small trees and whole images take one lane a ray instead, see
-// lane_per_ray) and its adjoint (Sec. 4.3: back-propagation through the IDFT).
+// ray_form) and its adjoint (Sec. 4.3: back-propagation through the IDFT).
 //
 // A warp owns R rays (lanes 0..R-1) and alternates between four phases, so
 // that the walk, which few lanes of incoherent rays need at the same time, and
@@ -1379,6 +1388,7 @@ __global__ void __maxnreg__(FPO_FUSED_MAXNREG) fused_kernel(const __grid_constan
     using S = FusedSize<N1, N2>;
     extern __shared__ __align__(16) uint32_t smem[];
     const TraverseParams &p = q.tp;
+    if (other_form(p, false)) return;
     const int lane = threadIdx.x & 31;
     const int R = p.rays_per_warp, E = p.list_cap;
     const int G = 1 << p.depth;
@@ -1751,7 +1761,45 @@ static int launch_fused_n(const BackwardParams &q, int sm_count, cudaStream_t s)
     return -1;
 }
 
-// A call of the fused mode with one lane a ray (lane_per_ray).  Bound by the
+// Whether a call's explicit rays come in coherent groups of 32, as an image's
+// do: 32 groups of consecutive rays, spread over the call, each coherent if its
+// rays pass the middle of the cube within a quarter of its side of one another
+// (32 neighbours of an image 400 wide that fills the view: a tenth; random rays:
+// about the side).  Most of them decide.
+__global__ void __launch_bounds__(1024) coherence_kernel(const __grid_constant__ TraverseParams p, uint32_t *coherent)
+{
+    const uint32_t groups = p.fr.n_rays / 32, group = (uint32_t)((uint64_t)groups * (threadIdx.x >> 5) / 32);
+    const size_t ray = (size_t)group * 32 + (threadIdx.x & 31);  // (calls of 2^17 rays and more)
+    const float half = 0.5f * (float)(1u << p.depth) / p.grid_scale;  // half the side
+    float dir[3], to[3], dd = 0.0f, td = 0.0f, extent = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        dir[a] = p.fr.rd[3 * ray + a];
+        to[a] = p.amin[a] + half - p.fr.ro[3 * ray + a];
+        dd = fmaf(dir[a], dir[a], dd);
+        td = fmaf(to[a], dir[a], td);
+    }
+    const float t = td / dd;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        float lo = fmaf(t, dir[a], -to[a]), hi = lo;  // the ray's nearest point to the middle
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        extent = fmaxf(extent, hi - lo);
+    }
+    const int n = __syncthreads_count(extent < 0.5f * half);
+    if (threadIdx.x == 0) *coherent = n > 512;
+}
+static int ask_coherence(const TraverseParams &p, cudaStream_t s)
+{
+    coherence_kernel<<<1, 1024, 0, s>>>(p, const_cast<uint32_t *>(p.coherent));
+    return (int)cudaGetLastError();
+}
+
+// A call of the fused mode with one lane a ray (ray_form).  Bound by the
 // records' trips through L1 and by their 166 multiplications a visit, where the
 // warps' way is bound by instructions: it spreads each visit over four lanes
 // also when the 32 rays of a warp read one record.
@@ -1774,7 +1822,10 @@ static int launch_lane(const TraverseParams &p, int sm_count, cudaStream_t s)
 
 // The adjoint of such a call: each ray is replayed and every visit's gradient
 // row added with 16-byte vector atomics (one 8-byte atomic at an unaligned end).
-// The same stepping and arithmetic as its forward, so the same early stop.
+// The same stepping and arithmetic as a forward by lanes, so the same early stop.
+// (Of explicit rays that are asked, batches that one list holds go by warps:
+// images of 512x512 249 against 310 us on 5,430 leaves, 375 / 414 on 41,929; in
+// parts, 800x800 took 681 / 543 and 975 / 681.)
 // 800x800 camera frame, against the warps' adds: 2,252 leaves 511 -> 421 us,
 // 41,929 966 -> 665, 348,592 2695 -> 1952, 3.5M 8344 -> 5726.
 template <int N1, int N2, bool BRICK>
@@ -1858,6 +1909,7 @@ __global__ void __maxnreg__(LANE_REGS) lane_adjoint_kernel(const __grid_constant
     extern __shared__ __align__(16) uint32_t smem[];
     const TraverseParams &p = q.tp;
     const int lane = threadIdx.x & 31;
+    if (other_form(p, true)) return;
     uint32_t *my_stack = BRICK ? nullptr : smem + threadIdx.x;
     const Basis basis = lane_basis(p, smem + (BRICK ? 0 : STACK_LEVELS * blockDim.x));
     for (;;) {
@@ -1927,7 +1979,14 @@ int launch_traverse(const TraverseParams &p, bool materialised, bool debug, int 
     if (materialised)
         return p.half_table ? launch_sched<TM_TABLE_F16>(p, debug, sm_count, s)
                             : launch_sched<TM_TABLE_F32>(p, debug, sm_count, s);
-    if (p.lanes) return debug ? launch_lane<true>(p, sm_count, s) : launch_lane<false>(p, sm_count, s);
+    if (p.form != BY_WARPS) {
+        if (p.form == LANES_IF_COHERENT) {
+            const int e = ask_coherence(p, s);
+            if (e != cudaSuccess) return e;
+        }
+        const int e = debug ? launch_lane<true>(p, sm_count, s) : launch_lane<false>(p, sm_count, s);
+        if (e != cudaSuccess || p.form == BY_LANES) return e;
+    }
     BackwardParams q{};
     q.tp = p;
     return debug ? launch_fused<false, true>(q, sm_count, s) : launch_fused<false, false>(q, sm_count, s);
@@ -2218,7 +2277,10 @@ int launch_grad_scatter_over(const VisitList &list, int n1, int n2, float *grad,
 int launch_backward(const BackwardParams &q, int sm_count, void *stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
-    if (q.dL_dcoeffs64 == nullptr && q.tp.lanes) return launch_lane_adjoint(q, sm_count, s);
+    if (q.dL_dcoeffs64 == nullptr && q.tp.form != BY_WARPS) {
+        const int e = q.tp.form == LANES_IF_COHERENT ? ask_coherence(q.tp, s) : (int)cudaSuccess;
+        return e != cudaSuccess ? e : launch_lane_adjoint(q, sm_count, s);
+    }
     if (q.dL_dcoeffs64 == nullptr) return launch_fused<true, false>(q, sm_count, s);
     const int n1 = q.tp.n1, n2 = q.tp.n2;
     if (n1 == 31 && n2 == 5) return launch_b64<31, 5>(q, sm_count, s);

@@ -13,7 +13,8 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
-LANES = 1 << 17  # rays from which a tree of fewer than 2^15 leaves takes one lane a ray
+LANES = 1 << 17  # rays from which a tree of fewer than 4096 leaves takes one lane a ray
+ASKED = 3 << 16  # ... and from which explicit rays on one of up to 2^17 leaves do, if they are coherent
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -39,7 +40,10 @@ def _close_grad(a, b, visits):
 
 
 def _tree(kind, n1, n2):
-    return synth.shell_tree(4, 5, n1, n2) if kind == "bricks" else synth.random_tree(11, max_depth=5, n1=n1, n2=n2)
+    if kind == "octree":
+        return synth.random_tree(11, max_depth=5, n1=n1, n2=n2)
+    t = synth.shell_tree(4, 5, n1, n2)  # every other leaf
+    return synth.Tree(t.leaf_depth[::2].copy(), t.leaf_xyz[::2].copy(), t.coeffs[::2].copy(), t.max_depth, n1, n2)
 
 
 @pytest.mark.parametrize("n1,n2", [(31, 5), (11, 5), (21, 5), (31, 11)])
@@ -47,6 +51,7 @@ def _tree(kind, n1, n2):
 @pytest.mark.parametrize("own", [True, False])
 def test_lanes_equal_warps(n1, n2, kind, own):
     tree = _tree(kind, n1, n2)
+    assert tree.n_leaves < 4096
     r = fpo.Renderer(n1=n1, n2=n2, idft_mode="fused")
     r.upload(tree)
     n = LANES + 33
@@ -79,6 +84,38 @@ def test_lanes_equal_warps(n1, n2, kind, own):
     assert int((marks[0] != marks[1]).sum()) <= 1 and int((marks[2] != marks[3]).sum()) <= 1
     assert torch.equal(marks[0], marks[2])
     _close_grad(ga, gb, 4 * n / tree.n_leaves + 1000)
+
+
+@pytest.mark.parametrize("own", [True, False])
+@pytest.mark.parametrize("n", [ASKED - 1, ASKED, (1 << 18) + 41])
+def test_large_calls_look_at_their_rays(n, own):
+    # an image's rays go by lanes from ASKED on (their adjoint, from more than one
+    # list holds on), a random batch by warps; both as parts of them by warps, the
+    # latter in the same bits
+    tree = synth.shell_tree(6)
+    assert tree.n_leaves >= 4096
+    r = fpo.Renderer(idft_mode="fused")
+    r.upload(tree)
+    cam = synth.shell_camera(640, 480)
+    image = _camera_rows(cam, 0, 480)
+    o, d, t, g = _rays(n, 3)
+    for coherent, (o, d) in ((True, (image["rays_o"][:n], image["rays_d"][:n])), (False, (o, d))):
+        args = lambda s: dict(rays_o=o[s], rays_d=d[s], t_per_ray=t[s] if own else None, t=7.0)
+        a = r.render(**args(slice(0, n)))["rgb"]
+        b = torch.cat([r.render(**args(s))["rgb"] for s in (slice(0, n // 2), slice(n // 2, n))])
+        assert float((a - b).abs().max()) <= 2e-5
+        assert torch.equal(a, b) == (not coherent or n < ASKED)
+        log = r.render(**args(slice(0, n)), visit_cap=64, want_T=True)
+        assert torch.equal(log["rgb"], a)
+        ga, gb = (torch.zeros(tree.coeffs.shape, device="cuda") for _ in range(2))
+        r.render_backward(a, g, ga, **args(slice(0, n)))
+        mark = torch.zeros(tree.n_leaves, dtype=torch.uint8, device="cuda")
+        for s in (slice(0, n // 2), slice(n // 2, n)):
+            r.render_backward(b[s], g[s], gb, **args(s), leaf_mark=mark)
+        assert mark.any() and float(ga[mark == 0].abs().sum()) == 0.0
+        _close_grad(ga, gb, 4 * n / tree.n_leaves + 1000)
+    r.status()
+    r.close()
 
 
 def _camera_rows(cam, y0, y1):
